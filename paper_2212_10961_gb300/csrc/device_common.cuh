@@ -160,6 +160,16 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
         : "memory");
 }
 
+// Programmatic dependent launch (launch_chained): the next kernel of the
+// stream may be set up while this one runs; `pdl_wait` returns once the
+// previous kernel has completed and its writes are visible.  Every thread of a
+// chained kernel passes it before its first access to global memory, so that
+// a kernel's completion implies that of all before it.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Hint: bring the 128-byte line holding `p` into L1 (no register, no wait).
 __device__ __forceinline__ void prefetch_l1(const void* p) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
@@ -211,11 +221,14 @@ static inline unsigned long long take_tu_index_faults() {
 // Mismatch epilogue of one cell (kMapMismatch): K = exp(Y), gY = 2 (K - T) K
 // / n_mean with the same FP32 operations as the standalone loss kernel, and
 // the squared difference returned for the loss sum (FP64).
-__device__ __forceinline__ double mismatch_store(const MapDev& m, int64_t o, float y) {
+__device__ __forceinline__ double mismatch_value(const MapDev& m, int64_t o, float y, float target) {
     const float k = expf(y);
-    const float d = k - __ldg(m.T + o);
+    const float d = k - target;
     m.G[o] = m.g_scale * d * k;
     return static_cast<double>(d) * static_cast<double>(d);
+}
+__device__ __forceinline__ double mismatch_store(const MapDev& m, int64_t o, float y) {
+    return mismatch_value(m, o, y, __ldg(m.T + o));
 }
 
 // Map epilogue of one cell (Sec. 3.1 truncation rule, Sec. 4.1 lognormal).

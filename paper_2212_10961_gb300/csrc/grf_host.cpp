@@ -250,6 +250,9 @@ struct PlanMeta {
     // 2 = grid of gn[0] x gn[1] x gn[2] cells.
     int32_t grid_state = 0;
     int32_t gn[3] = {0, 0, 0};
+    // bounds of the cells, once the check has been read
+    bool has_box = false;
+    float box[6] = {0, 0, 0, 0, 0, 0};
     uint64_t tag = 0;
     int32_t slot = -1;
     cudaEvent_t ev = nullptr;
@@ -297,7 +300,9 @@ bool grid_ws_ok(size_t bytes, const GridGeom& gg) {
 // The grid shape of `plan` (single segment), resolving a pending check by
 // waiting for the plan's own event (the planning kernels only).  Returns
 // false when the cells are not a Cartesian grid in x-fastest order.
-bool plan_grid(const void* plan, GridGeom* gg) {
+// box: the bounds of the cells of a single-segment 2-D / 3-D plan (hints only;
+// not finite where they are unknown).
+bool plan_grid(const void* plan, GridGeom* gg, float* box = nullptr) {
     PlanMeta m;
     {
         std::lock_guard<std::mutex> lk(g_reg_mu);
@@ -311,7 +316,10 @@ bool plan_grid(const void* plan, GridGeom* gg) {
         m.layout = it->second.layout;
         m.offsets = it->second.offsets;
         for (int c = 0; c < 3; ++c) m.gn[c] = it->second.gn[c];
+        m.has_box = it->second.has_box;
+        for (int c = 0; c < 6; ++c) m.box[c] = it->second.box[c];
     }
+    for (int c = 0; box && c < 6; ++c) box[c] = m.has_box ? m.box[c] : NAN;
     if (m.grid_state == 0) return false;
     if (m.grid_state == 1) {
         int32_t st = 0, gn[3] = {0, 0, 0};
@@ -320,6 +328,13 @@ bool plan_grid(const void* plan, GridGeom* gg) {
             {
                 std::lock_guard<std::mutex> lk(g_reg_mu);
                 c = g_slots[m.slot];
+            }
+            if (c.tag == m.tag) {
+                m.has_box = true;
+                for (int k = 0; k < 3; ++k) {
+                    m.box[k] = c.lo[k];
+                    m.box[3 + k] = c.hi[k];
+                }
             }
             const int64_t n = m.offsets.back();
             const int64_t nx = static_cast<int64_t>(c.c1);
@@ -339,10 +354,13 @@ bool plan_grid(const void* plan, GridGeom* gg) {
         if (it != g_plans.end() && it->second.tag == m.tag) {
             it->second.grid_state = st;
             for (int c = 0; c < 3; ++c) it->second.gn[c] = gn[c];
+            it->second.has_box = m.has_box;
+            for (int c = 0; c < 6; ++c) it->second.box[c] = m.box[c];
             drop_plan_event(it->second);
         }
         m.grid_state = st;
         for (int c = 0; c < 3; ++c) m.gn[c] = gn[c];
+        for (int c = 0; box && c < 6; ++c) box[c] = m.has_box ? m.box[c] : NAN;
     }
     if (m.grid_state != 2) return false;
     const float* axes = reinterpret_cast<const float*>(static_cast<const unsigned char*>(plan) + m.layout.off_keys_in);
@@ -352,7 +370,58 @@ bool plan_grid(const void* plan, GridGeom* gg) {
     gg->X = axes;
     gg->Y = axes + m.gn[0];
     gg->Z = axes + m.gn[0] + m.gn[1];
+    gg->seg = reinterpret_cast<const SegInfo*>(static_cast<const unsigned char*>(plan) + m.layout.off_segs);
     return true;
+}
+
+// Whether a call is likely to gain from the band path (band.cuh), from the
+// parameters' spectrum, the cells' bounds and the measured rates.  Only a
+// forecast: the device decides on the table's own frequencies, but a call
+// that then finds no lattice has paid kBandTryUs for the attempt.  q: largest
+// |kappa_c| that a fraction 2^-(k+1) of the modes exceeds, by dimension and
+// law (Student t with 1 and 3 degrees of freedom, normal), from 4 10^6 draws.
+// n: cells per axis of a grid, or null.  us_mode: time of one mode summed
+// directly.
+bool band_worth(const grf_params* p, const float* box, const int32_t* n, double us_mode, double us_node,
+                double us_fixed) {
+    static const float q[2][3][12] = {
+        {{1.553f, 3.483f, 7.153f, 14.37f, 28.78f, 57.76f, 116.f, 232.f, 465.f, 916.f, 1853.f, 3539.f},
+         {1.188f, 1.922f, 2.711f, 3.629f, 4.73f, 6.09f, 7.77f, 9.88f, 12.5f, 15.8f, 19.9f, 24.9f},
+         {1.318f, 1.879f, 2.317f, 2.691f, 3.026f, 3.333f, 3.612f, 3.879f, 4.122f, 4.359f, 4.575f, 4.807f}},
+        {{1.874f, 4.121f, 8.416f, 16.88f, 33.81f, 67.67f, 135.f, 277.f, 551.f, 1100.f, 2210.f, 4378.f},
+         {1.43f, 2.213f, 3.066f, 4.07f, 5.287f, 6.784f, 8.62f, 10.9f, 13.8f, 17.6f, 22.2f, 28.1f},
+         {1.584f, 2.115f, 2.53f, 2.888f, 3.206f, 3.5f, 3.773f, 4.029f, 4.273f, 4.503f, 4.729f, 4.947f}}};
+    const double nu = p->family == GRF_GAUSSIAN ? 100.0 : p->family == GRF_EXPONENTIAL ? 0.5 : p->nu;
+    const float* law = q[p->dim > 2 ? 1 : 0][nu < 1.5 ? 0 : nu < 8.0 ? 1 : 2];
+    const double N = static_cast<double>(p->n_modes), direct = us_mode * N;
+    double min_ell = 1e300;
+    for (int c = 0; c < p->dim; ++c) min_ell = std::min(min_ell, p->ell[c]);
+    for (int k = 0; k < 12; ++k) {
+        double heavy = std::ldexp(N, -(k + 1));
+        const bool last = heavy < 2.0 || k == 11;
+        heavy = last ? 0.0 : std::ceil(heavy / 128.0) * 128.0;
+        double nodes = 1.0;
+        for (int c = 0; c < p->dim; ++c) {
+            // a margin for the width of the selection's bins
+            const double a = 1.05 * law[k] / (2.0 * M_PI * (has_rotation(p) ? min_ell : p->ell[c]));
+            double m = 4.0 * a * (static_cast<double>(box[3 + c]) - box[c]) + 9.0;
+            if (n) m = std::min(m, static_cast<double>(n[c]));
+            nodes *= m;
+        }
+        nodes = std::ceil(nodes / 16384.0) * 16384.0;
+        if (heavy * us_mode + (N - heavy) * nodes * us_node + us_fixed < 0.75 * direct) return true;
+        if (last) break;
+    }
+    return false;
+}
+
+// The same for a call on a Cartesian grid, with the workspace it has.
+bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t ws_bytes) {
+    const int64_t n_pad = table_layout(p->n_modes).n_pad;
+    const size_t extra = grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+    if (extra == 0 || ws_bytes < grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra) return false;
+    const int32_t n[3] = {gg.nx, gg.ny, gg.nz};
+    return band_worth(p, box, n, grid_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeUs, kBandFixedUs + kBandTryUs);
 }
 
 bool lookup_plan(const void* plan, PlanMeta& out) {
@@ -846,12 +915,13 @@ int grf_synth_field(const void* table, const grf_params* p, const void* plan, in
     // Cartesian grid handed over x-fastest: tensor-core path when the
     // workspace holds its tables
     GridGeom gg{};
+    float box[6];
     if (n > 0 && workspace && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim &&
-        plan_grid(plan, &gg) && use_grid_path(gg) &&
+        plan_grid(plan, &gg, box) && use_grid_path(gg) &&
         grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
         ws_bytes >= grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad)) {
-        const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, workspace, g_grid_fold.load(), status,
-                                          stream);
+        const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, workspace, grid_band(p, gg, box, ws_bytes),
+                                          g_grid_fold.load(), status, stream);
         if (err != cudaSuccess) return cuda_fail(err, "grid synth kernels");
         return GRF_OK;
     }
@@ -867,8 +937,9 @@ size_t grf_synth_grid_workspace_bytes(const void* plan, int32_t segment, int64_t
         if (!plan || segment != 0 || n_modes < 1 || n_modes > GRF_MAX_MODES) return 0;
         GridGeom gg{};
         if (!plan_grid(plan, &gg)) return 0;
-        const size_t b = grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(n_modes).n_pad);
-        return grid_ws_ok(b, gg) ? b : 0;
+        const int64_t n_pad = table_layout(n_modes).n_pad;
+        const size_t b = grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+        return grid_ws_ok(b, gg) ? b + grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
     } catch (...) {
         return 0;
     }
@@ -937,12 +1008,14 @@ int grf_synth_mismatch(const void* table, const grf_params* p, const void* plan,
     // Cartesian grid: the tensor-core path when the rest of the workspace
     // holds its tables and the loss partials fit
     GridGeom gg{};
-    if (n > 0 && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim && plan_grid(plan, &gg) &&
+    float box[6];
+    if (n > 0 && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim && plan_grid(plan, &gg, box) &&
         use_grid_path(gg) && grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
         ws_bytes - lbytes >= grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad) &&
         grid_loss_partials(gg.nx, gg.ny, gg.nz) <= mismatch_partials(n)) {
-        const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, split_ws, g_grid_fold.load(),
-                                          status, stream);
+        const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, split_ws,
+                                          grid_band(p, gg, box, ws_bytes - lbytes), g_grid_fold.load(), status,
+                                          stream);
         if (err != cudaSuccess) return cuda_fail(err, "grid synth kernels");
         return GRF_OK;
     }

@@ -114,6 +114,7 @@ struct GridCheck {
     int32_t bad;            // some cell is not at (X_i, Y_k, Z_l) of its index
     int32_t pad_;
     uint64_t tag;           // host-assigned plan number
+    float lo[3], hi[3];     // bounds of the cells
 };
 constexpr int kMortonBits = 10;                // quantised coordinate bits per axis
 
@@ -130,7 +131,7 @@ struct PlanHeader {
     // whose z differs (= nx ny), a mismatch flag, and the plan's tag.  The
     // axes X (nx), Y (ny), Z (nz) are written over the keys_in scratch.
     GridCheck grid;
-    int64_t reserved[10];
+    int64_t reserved[7];
 };
 static_assert(sizeof(PlanHeader) <= 256, "plan header must fit in 256 bytes");
 
@@ -216,12 +217,23 @@ struct FwdDesc {
     MapDev map;
 };
 
+struct SegInfo;
+
 // Cartesian grid of a plan: cell n = i + nx (k + ny l) at (X_i, Y_k, Z_l).
 struct GridGeom {
     int32_t nx, ny, nz;
     const float* X;
     const float* Y;
     const float* Z;
+    const SegInfo* seg;  // bounds of the cells
+};
+
+// Coordinates of one axis of a grid synthesis: cell i at p[i], or, on the node
+// lattice of the band path (band.cuh; p null), node i at (n0 + i) h.
+struct AxisSrc {
+    const float* p;
+    float h;
+    int32_t n0;
 };
 
 // Tables of one grid synthesis (workspace) as the prep kernel fills them.
@@ -229,15 +241,43 @@ struct GridPrep {
     const TableHeader* thdr;
     const float4* hot;
     const float4* cold;
-    const float* X;
-    const float* Y;
-    const float* Z;
-    int32_t nx, ny, nz, n_pad, nc, n_mt, n_kt, dim;
+    const int32_t* idx;  // table slots of the modes summed (-1: none), null for all in order
+    AxisSrc ax[3];
+    float gain_h[3];       // node spacings of the axes whose window gain multiplies the amplitudes (0: none)
+    float scale;           // amplitude scale (0: from the table's largest amplitude)
+    int32_t xn;            // x cells of a row block (GridDesc); rows beyond the first block are
+    float zstep;           // shifted by this z distance per block
+    int32_t nx, ny, nz, nc, n_mt, n_kt, dim;
     int32_t form;          // 1: 3-D (B formed from ytab, wztab), 0: B tabulated in btab
     unsigned char* atab;   // x phasors: FP16 hi/lo tiles [n_mt][nc][2][128 x 64]
     unsigned char* btab;   // 2-D: B tiles [n_kt][nc][2][128 x 64]
     float2* ytab;          // 3-D: [nc][ny][32] y phasors
     float2* wztab;         // 3-D: [nc][nz][32] (amplitude, psi, z) phasors
+};
+
+// Sizes of one grid synthesis (grid_tiling.cuh).
+struct GridTiling {
+    int64_t n_tiles;
+    int64_t n_items;  // tiles x splits
+    float scale;      // amplitude scale (0: from the table's largest amplitude)
+    int32_t nx, ny, nz;
+    int32_t nc;       // chunks of 32 modes
+    int32_t fc;       // chunks per fold interval
+    int32_t n_mt, n_kt, n_lt;
+    int32_t pk_log2;  // (y, z) patch: 2^pk_log2 along y, 128 / 2^pk_log2 along z
+    int32_t form;     // 1: B formed in shared memory from the staged table rows
+    int32_t sa;       // stages of the copy ring
+    int32_t a_stage;  // bytes per copy stage
+    int32_t off_b;    // formed B ring (form)
+    int32_t off_bar;  // barriers
+    int32_t n_split;  // mode splits per tile (whole fold intervals each)
+    // rows of a tile: x cell i mod xn in z block i / xn of lz layers (cells:
+    // one block; node lattices of few x nodes fill the 128 rows with several)
+    int32_t xn, lz, zn;
+    // band path, at the cells: the light modes as nl further chunks before the
+    // others, B from light[(l ny + k) lp + node] * l_inv
+    int32_t nl, lp;
+    float l_inv;
 };
 
 // One grid synthesis as the tensor-core kernel sees it.
@@ -247,21 +287,64 @@ struct GridDesc {
     const float2* ytab;
     const float2* wztab;
     const TableHeader* thdr;
-    int32_t nx, ny, nz, n_pad;
-    int32_t nc;       // chunks of 32 modes
-    int32_t fc;       // chunks per fold interval (1, 2 or 4)
-    int32_t n_mt, n_kt, n_lt;
-    int32_t pk_log2;  // (y, z) patch: 2^pk_log2 along y, 128 / 2^pk_log2 along z
-    int64_t n_tiles;
-    int32_t form;     // 1: B formed in shared memory from the staged table rows
-    int32_t sa;       // stages of the copy ring
-    int32_t a_stage;  // bytes per copy stage
-    int32_t off_b;    // formed B ring (form)
-    int32_t off_bar;  // barriers
-    int32_t n_split;  // mode splits per tile (whole fold intervals each); > 1: partial fields in part
-    int64_t n_items;  // tiles x splits
-    float* part;      // [n_split][nx ny nz] partial fields (n_split > 1), summed by the finalize kernel
+    float* part;      // [n_split][xn ny zn] partial fields, summed by the finalize kernel
+    int32_t quiet;    // 1: the tiles are not counted (nodes are not cells)
+    // light chunks: A tiles latab[n_mt][nl] (x weights), first node of an x
+    // tile lstart[n_mt], the rows of x nodes
+    const unsigned char* latab;
+    const int32_t* lstart;
+    const float* light;
+    GridTiling t;
     MapDev map;
+};
+
+// Band path (band.cuh) of one call, chosen on the device by band_select_kernel.
+struct BandAxis {
+    float h, inv_h;  // node spacing (0 with ident)
+    int32_t n0, m;   // nodes (n0 + k) h, k < m
+    int32_t ident;   // 1: not interpolated, the nodes are the axis's cells
+};
+struct BandDesc {
+    int32_t nh;        // modes summed at the cells
+    int32_t n_light;   // modes summed at the nodes (0: band path not taken)
+    int32_t n_splits;  // mode splits whose partials the finalize kernel adds (0: none)
+    int32_t finalize;  // 1: band_finalize_kernel writes the cells
+    int64_t loss_nb;   // loss partials written
+    int32_t lp;        // floats per row of x nodes
+    float lw;          // factor of the x weights' operand tiles: lw l_inv = 1 / (amplitude scale)
+    BandAxis ax[3];
+    GridTiling nodes;  // light modes on the node lattice
+    GridTiling cells;  // direct modes at the cells of a grid
+};
+
+// What the host knows of a band-path call: the table, the cells' axes or
+// bounds, the limits of the workspace and the measured rates.
+struct BandSelect {
+    const float4* hot;
+    const float4* cold;
+    int32_t n_modes, dim;
+    int32_t* idx_h;         // [n_modes padded to 32] table slots of the modes summed at the cells,
+    int32_t* idx_l;         // and of those summed at the nodes, in table order, then -1
+    const SegInfo* seg;     // bounds of the cells
+    const int32_t* status;  // the plan's: bit 1 for cells that are not finite
+    int32_t n[3];           // grid: cells per axis (0 without a grid)
+    const float* X;         // grid: the x axis
+    float us_mode;           // time of one mode summed directly, us
+    float us_node;           // time of one mode at one node, us
+    float us_fixed;          // time of the lattice's own kernels, us
+    int64_t cap_nodes;       // most nodes
+    int64_t cap_part;        // floats of the nodes' partial sums
+    int64_t cap_mid;         // most (x, y) nodes x z cells
+    int32_t cap_mt;          // most 128-row tiles of the nodes' x operand
+    int32_t fold;
+    int32_t n_mt;            // x tiles of the cells
+    int32_t* lstart;         // [n_mt] first x node of a tile (written here; null: no light chunks)
+    int32_t max_split;       // mode splits of the direct sum (1: unsplit)
+    int32_t split_cells;     // 1: the direct sum leaves partial sums to the finalize kernel
+    int32_t loss_per_tile;
+    int64_t loss_nb_finalize;
+    const TableHeader* thdr;
+    GridTiling cells;        // the cells' tiling (all modes)
 };
 
 // Work tile of the batched launch: realisation r, tile index t inside it.
@@ -291,7 +374,8 @@ int launch_synth_fwd(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t
 // Entries of MapDev::lpart a launch of n cells may write (kMapMismatch).
 int64_t mismatch_partials(int64_t n_cells);
 // loss = (sum of the nb partials, fixed order) * inv_n, one block.
-int launch_loss_sum(const double* part, int64_t nb, double inv_n, double* out, void* stream);
+// nb_dev, if not null, holds the count on the device instead of nb.
+int launch_loss_sum(const double* part, int64_t nb, const int64_t* nb_dev, double inv_n, double* out, void* stream);
 
 // Checked builds (-DGRF_CHECKED=1): device accesses skipped since the last
 // call because an index read from device memory was out of range, per
@@ -353,8 +437,25 @@ size_t grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
 int64_t grid_loss_partials(int32_t nx, int32_t ny, int32_t nz);
 // Tiles of 128 x 128 cells of a grid.
 int64_t grid_tiles(int32_t nx, int32_t ny, int32_t nz);
+// band: the band path (band.cuh), whose workspace follows (ws_bytes >=
+// grid_ws_bytes + grid_band_ws_bytes).
 int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const GridGeom& gg, const MapDev& map,
-                      void* ws, int32_t fc, int32_t* status, void* stream);
+                      void* ws, bool band, int32_t fc, int32_t* status, void* stream);
+// Time of one mode summed at the cells of a grid by the grid path, us.
+double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
+// Further workspace of the band path on a grid (0: not taken at these sizes).
+size_t grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
+// Measured times of the band path (us): one mode at one node (tensor cores,
+// whole 128 x 128 tiles), the kernels that the lattice adds, and the kernels
+// that a call pays for when the device finds no lattice worth while.
+constexpr double kBandNodeUs = 1.0 / 22.0e6, kBandFixedUs = 15.0, kBandTryUs = 14.0;
+// Band path kernels (band.cu).
+int launch_band_select(const BandSelect& p, BandDesc* out, void* stream);
+int launch_band_lines(const BandDesc* b, float* part, const GridGeom& gg, float* mid, float* rows, int sms,
+                      void* stream);
+int launch_band_finalize(const BandDesc* b, const float* mid, const float* part, const GridGeom& gg,
+                         const MapDev& map, unsigned long long* tiles, void* stream);
+int64_t band_finalize_blocks(const GridGeom& gg);
 int take_grid_tiles(unsigned long long* tiles);
 int launch_mma_probe(const uint16_t* A, const uint16_t* B, int32_t k_chunks, float* D, int32_t* status,
                      void* stream);

@@ -613,13 +613,17 @@ __device__ __forceinline__ unsigned long long block_min_u64(unsigned long long v
 }
 
 __global__ void __launch_bounds__(kGridThreads) grid_scan_kernel(const float* y, const float* z, int32_t dim,
-                                                                 int64_t n, GridCheck* gc) {
+                                                                 int64_t n, GridCheck* gc, const SegInfo* seg) {
     __shared__ unsigned long long red1[kGridThreads / 32], red2[kGridThreads / 32];
     const int64_t base = static_cast<int64_t>(blockIdx.x) * (kGridThreads * kGridPer);
     // blocks past the current candidates cannot lower them
     const unsigned long long lim =
         dim > 2 ? *reinterpret_cast<volatile unsigned long long*>(&gc->c2)
                 : *reinterpret_cast<volatile unsigned long long*>(&gc->c1);
+    if (blockIdx.x == 0 && threadIdx.x < 3) {
+        gc->lo[threadIdx.x] = seg->lo[threadIdx.x];
+        gc->hi[threadIdx.x] = seg->hi[threadIdx.x];
+    }
     if (static_cast<unsigned long long>(base) >= lim) return;
     const float y0 = __ldg(y);
     const float z0 = dim > 2 ? __ldg(z) : 0.0f;
@@ -679,7 +683,8 @@ int launch_grid_check(int32_t dim, int64_t n, const float* x, const float* y, co
     GridCheck* gc = &reinterpret_cast<PlanHeader*>(base)->grid;
     float* axes = reinterpret_cast<float*>(base + L.off_keys_in);
     const int64_t per = int64_t(kGridThreads) * kGridPer;
-    grid_scan_kernel<<<static_cast<unsigned>((n + per - 1) / per), kGridThreads, 0, st>>>(y, z, dim, n, gc);
+    grid_scan_kernel<<<static_cast<unsigned>((n + per - 1) / per), kGridThreads, 0, st>>>(
+        y, z, dim, n, gc, reinterpret_cast<const SegInfo*>(base + L.off_segs));
     const int64_t vb = std::min<int64_t>((n + kGridThreads - 1) / kGridThreads, 152 * 16);
     grid_verify_kernel<<<static_cast<unsigned>(vb), kGridThreads, 0, st>>>(x, y, z, dim, n, gc, axes);
     count_launches(2);

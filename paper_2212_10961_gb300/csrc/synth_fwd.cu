@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
+#include "launch.cuh"
 
 namespace grf {
 
@@ -558,9 +559,12 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
 // loss = (sum of the nb partial sums of (K - T)^2) / n_mean, one block,
 // fixed order.
 __global__ void __launch_bounds__(256) loss_sum_kernel(const double* __restrict__ part, int64_t nb,
-                                                       double inv_n, double* __restrict__ out) {
+                                                       const int64_t* __restrict__ nb_dev, double inv_n,
+                                                       double* __restrict__ out) {
     __shared__ double red[256];
+    pdl_wait();
     double acc = 0.0;
+    if (nb_dev != nullptr) nb = *nb_dev;
     for (int64_t k = threadIdx.x; k < nb; k += 256) acc += part[k];
     red[threadIdx.x] = acc;
     __syncthreads();
@@ -646,7 +650,7 @@ int launch_fwd_cfg(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* 
     const int64_t grid = (d.n_cells + per_cta - 1) / per_cta;
     if (grid == 0) {
         if (mm) {  // no cells: the loss is 0
-            loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, 0, 0.0, d.map.loss);
+            loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, 0, nullptr, 0.0, d.map.loss);
             count_launches(1);
         }
         return cudaGetLastError();
@@ -669,7 +673,7 @@ int launch_fwd_cfg(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* 
     }
     if (mm) {
         const int64_t nb = n_split > 1 ? fin_blocks : (d.n_cells + 32 * C - 1) / (32 * C);
-        loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, nb, d.map.inv_n_mean, d.map.loss);
+        loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, nb, nullptr, d.map.inv_n_mean, d.map.loss);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -724,10 +728,8 @@ size_t synth_workspace_bytes(int64_t n_cells) {
 // split finalize, whichever is more.
 int64_t mismatch_partials(int64_t n_cells) { return (n_cells + 127) / 128 + 1; }
 
-int launch_loss_sum(const double* part, int64_t nb, double inv_n, double* out, void* stream) {
-    loss_sum_kernel<<<1, 256, 0, static_cast<cudaStream_t>(stream)>>>(part, nb, inv_n, out);
-    count_launches(1);
-    return cudaGetLastError();
+int launch_loss_sum(const double* part, int64_t nb, const int64_t* nb_dev, double inv_n, double* out, void* stream) {
+    return launch_chained(loss_sum_kernel, 1, 256, 0, static_cast<cudaStream_t>(stream), part, nb, nb_dev, inv_n, out);
 }
 
 int launch_synth_fwd(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* status, void* stream) {

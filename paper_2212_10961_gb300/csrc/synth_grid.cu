@@ -48,8 +48,11 @@
 #include <algorithm>
 #include <cmath>
 
+#include "band.cuh"
 #include "device_common.cuh"
 #include "grid_common.cuh"
+#include "grid_tiling.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace grf {
@@ -62,34 +65,7 @@ namespace {
 using gridc::gwait;
 using gridc::psi_z_turns;
 using gridc::tile_off;
-
-constexpr int kGM = 128;                    // x cells per tile (TMEM lanes)
-constexpr int kGN = 128;                    // (y, z) cells per tile (accumulator columns)
-constexpr int kGModes = 32;                 // modes per chunk
-constexpr int kGK = 2 * kGModes;            // K elements per chunk (re, im)
-constexpr int kGOpBytes = kGM * kGK * 2;    // one FP16 operand tile (128 x 64): 16 KB
-constexpr int kGPair = 2 * kGOpBytes;       // hi and lo tiles of one operand
-constexpr int kGRowBytes = kGModes * 8 + 16;  // one table row of a chunk: 32 float2 + 16 bytes of padding
-                                              // (consecutive rows start in different shared-memory banks)
-constexpr int kGMaxSA = 4;
-constexpr int kGSB = 3;                     // formed B stages (3-D)
-constexpr int kGEpiWarps = 16;
-constexpr int kGThreads = 32 * (kGEpiWarps + 2);
-constexpr int kGColsPerWarp = kGN / (kGEpiWarps / 4);    // TMEM columns a warp folds (4 lane quarters)
-// B formation: thread t forms one 4-mode group (t / 64) of two columns that
-// share a y cell (z cells 2 q and 2 q + 1 of the patch, pair t mod 64), so the
-// y row is read once for both
-constexpr int kGFormPairs = kGN / 2;
-static_assert(kGColsPerWarp % 32 == 0 && 32 * kGEpiWarps == kGFormPairs * (kGModes / 4), "epilogue warp layout");
-constexpr uint32_t kGSbo = 1024;            // 8-row groups of a tile: one 128-byte-swizzle atom apart
-constexpr uint32_t kGKStep = 32;            // bytes of 16 K elements inside an atom row
-constexpr uint32_t kGTmemCols = 512;
-constexpr uint32_t kGCorrCol = 256;         // hi.lo + lo.hi accumulator of the tile
-constexpr uint32_t kGSumCol = 384;          // running FP32 sum of the folded hi.hi intervals
-constexpr int kGBarBytes = 256;
-constexpr int kGAlignPad = 1024;            // room to start the stages on a 1024-byte boundary
-constexpr int kGSmemMax = gridc::kSmemMax;
-static_assert(kGM == 128 && kGN == 128, "tile shape is fixed by the TMEM layout");
+using namespace gridt;
 
 // Amplitude scale: the smallest power of two S >= max |A_j| (1 when all
 // amplitudes vanish), so that |W| <= 1.
@@ -131,24 +107,49 @@ __device__ __forceinline__ void form_b(unsigned char* bhi, const float4* ty, con
 struct TileIdx {
     int mt, kt, k0, l0, pkv, plv;  // x tile, y tile, first y and z cell, valid y and z cells of the patch
 };
-__device__ __forceinline__ TileIdx tile_idx(const GridDesc& d, int64_t tile) {
+__device__ __forceinline__ TileIdx tile_idx(const GridTiling& T, int64_t tile) {
     TileIdx t;
-    t.mt = static_cast<int>(tile % d.n_mt);
-    const int64_t rest = tile / d.n_mt;
-    t.kt = static_cast<int>(rest % d.n_kt);
-    t.k0 = t.kt << d.pk_log2;
-    t.l0 = static_cast<int>(rest / d.n_kt) * (kGN >> d.pk_log2);
-    t.pkv = min(1 << d.pk_log2, d.ny - t.k0);
-    t.plv = min(kGN >> d.pk_log2, d.nz - t.l0);
+    t.mt = static_cast<int>(tile % T.n_mt);
+    const int64_t rest = tile / T.n_mt;
+    t.kt = static_cast<int>(rest % T.n_kt);
+    t.k0 = t.kt << T.pk_log2;
+    t.l0 = static_cast<int>(rest / T.n_kt) * (kGN >> T.pk_log2);
+    t.pkv = min(1 << T.pk_log2, T.ny - t.k0);
+    t.plv = min(kGN >> T.pk_log2, T.nz - t.l0);
     return t;
 }
 
-template <bool kSplit>
-__global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int32_t* status) {
-    extern __shared__ __align__(1024) unsigned char gsm_raw[];
+// B of a light chunk: 16 nodes (segments 2 q4, 2 q4 + 1) of column n's row
+// of x nodes, from node `first` of the row, times `inv`.
+__device__ __forceinline__ void form_light(unsigned char* bhi, const float* row, int first, int lp, float inv, int n,
+                                           int q4) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float4 v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int node = first + 16 * q4 + 8 * h + 4 * e;
+            v[e] = node < lp ? __ldg(reinterpret_cast<const float4*>(row + node)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        uint4 H, L;
+        tc::split_f16x2(v[0].x * inv, v[0].y * inv, H.x, L.x);
+        tc::split_f16x2(v[0].z * inv, v[0].w * inv, H.y, L.y);
+        tc::split_f16x2(v[1].x * inv, v[1].y * inv, H.z, L.z);
+        tc::split_f16x2(v[1].z * inv, v[1].w * inv, H.w, L.w);
+        const uint32_t boff = tile_off(n, 2 * q4 + h);
+        *reinterpret_cast<uint4*>(bhi + boff) = H;
+        *reinterpret_cast<uint4*>(bhi + kGOpBytes + boff) = L;
+    }
+}
+
+// kLight: the band path's direct modes at the cells of a 3-D grid; a tile's
+// first interval is the light modes' chunks.
+template <bool kSplit, bool kLight>
+__device__ __forceinline__ void grid_mma_body(const GridDesc& d, const GridTiling& T, unsigned char* gsm_raw,
+                                              int32_t* status) {
     // stages on a 1024-byte boundary of the shared window (swizzle atoms)
     unsigned char* gsm = gsm_raw + ((1024u - (smem_u32(gsm_raw) & 1023u)) & 1023u);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + d.off_bar);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + T.off_bar);
     uint64_t* afull = bars;                // [sa] stage's copies landed (transaction bytes)
     uint64_t* afree = bars + kGMaxSA;      // [sa] stage's MMAs completed
     uint64_t* bfull = bars + 2 * kGMaxSA;  // [kGSB] B formed (one arrival per epilogue warp)
@@ -161,9 +162,9 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
     volatile int32_t* abort = reinterpret_cast<volatile int32_t*>(done + 2);
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const bool form = d.form != 0;
+    const bool form = T.form != 0;
     const bool mm = (d.map.bits & kMapMismatch) != 0;
-    const int SA = d.sa;
+    const int SA = T.sa;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kGMaxSA; ++s) {
@@ -188,9 +189,12 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = *tslot;
-    const int NI = d.nc / d.fc;  // fold intervals per tile
-    const int n_split = kSplit ? d.n_split : 1;
-    const int pkm = (1 << d.pk_log2) - 1;
+    pdl_wait();
+    const int nl = kLight ? T.nl : 0;
+    const int li = nl > 0 ? 1 : 0;    // the light chunks are an interval of their own
+    const int NI = (T.nc + T.fc - 1) / T.fc + li;  // fold intervals per tile
+    const int n_split = kSplit ? T.n_split : 1;
+    const int pkm = (1 << T.pk_log2) - 1;
 
     if (warp < kGEpiWarps) {
         // ---- B formation (3-D), folds, maps ---------------------------------------
@@ -200,24 +204,24 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
         const int fp = t & (kGFormPairs - 1);  // column pair this thread forms
         const int fg = t / kGFormPairs;        // 4-mode group of the chunk it forms
         const int fk = fp & pkm;               // y cell of the pair in the patch
-        const int fz = (fp >> d.pk_log2) * 2;  // first z cell of the pair in the patch
-        const int n0 = fk + (fz << d.pk_log2), n1 = n0 + (1 << d.pk_log2);
+        const int fz = (fp >> T.pk_log2) * 2;  // first z cell of the pair in the patch
+        const int n0 = fk + (fz << T.pk_log2), n1 = n0 + (1 << T.pk_log2);
         const uint32_t lane_off = static_cast<uint32_t>(32 * q) << 16;
-        const float S = grid_scale(d.thdr);
+        const float S = T.scale > 0.0f ? T.scale : grid_scale(d.thdr);
         uint32_t g = 0, gi = 0;
-        for (int64_t item = blockIdx.x; item < (kSplit ? d.n_items : d.n_tiles); item += gridDim.x) {
+        for (int64_t item = blockIdx.x; item < (kSplit ? T.n_items : T.n_tiles); item += gridDim.x) {
             const int64_t tile = kSplit ? item / n_split : item;
             const int split = kSplit ? static_cast<int>(item - tile * n_split) : 0;
             // the item's fold intervals iv0 .. iv1 - 1 (all of the tile's without a split)
             const int iv0 = kSplit ? NI * split / n_split : 0;
             const int NIl = kSplit ? NI * (split + 1) / n_split - iv0 : NI;
-            const TileIdx ti = tile_idx(d, tile);
+            const TileIdx ti = tile_idx(T, tile);
             // staged table rows this thread reads: y row and (amplitude, psi, z) row
             const int ry = min(fk, ti.pkv - 1);
             const int rz0 = min(fz, ti.plv - 1), rz1 = min(fz + 1, ti.plv - 1);
             const int toff_y = kGPair + ry * kGRowBytes + 32 * fg;
-            const int toff_w0 = kGPair + ((1 << d.pk_log2) + rz0) * kGRowBytes + 32 * fg;
-            const int toff_w1 = kGPair + ((1 << d.pk_log2) + rz1) * kGRowBytes + 32 * fg;
+            const int toff_w0 = kGPair + ((1 << T.pk_log2) + rz0) * kGRowBytes + 32 * fg;
+            const int toff_w1 = kGPair + ((1 << T.pk_log2) + rz1) * kGRowBytes + 32 * fg;
 
             // fold of interval gidx: the hi.hi accumulator into the running sum
             // (plain FP32: a few tens of folds per cell); the last fold of a
@@ -249,6 +253,18 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
                     tc::wait_st();
                 } else {
                     const int i = ti.mt * kGM + 32 * q + lane;
+                    // cell of the row: x cell xi of z block zb (one block at the cells)
+                    const int zb = kSplit ? i / T.xn : 0;
+                    const int xi = i - zb * T.xn;
+                    // a plan has fewer than 2^31 cells (and a lattice fewer nodes)
+                    const uint32_t xn = static_cast<uint32_t>(T.xn), xny = xn * static_cast<uint32_t>(T.ny);
+                    const uint32_t o0 = static_cast<uint32_t>(xi) + xn * static_cast<uint32_t>(ti.k0) +
+                                        xny * static_cast<uint32_t>(ti.l0 + zb * T.lz);
+                    // valid columns: y cells below kn, z cells below ln of the patch
+                    const int kn = i < T.nx ? T.ny - ti.k0 : 0;
+                    const int ln = min(T.nz, T.zn - zb * T.lz) - ti.l0;
+                    float* part =
+                        kSplit ? d.part + static_cast<int64_t>(split) * T.xn * T.ny * T.zn : nullptr;
 #pragma unroll 1
                     for (int blk = 0; blk < kGColsPerWarp / 8; ++blk) {  // 8 columns at a time, then the maps
                         const uint32_t col = static_cast<uint32_t>(kGColsPerWarp * h + 8 * blk);
@@ -271,13 +287,11 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
                             if (!first) v = __uint_as_float(sm[cc]) + v;
                             v += __uint_as_float(cr[cc]);
                             const int c = static_cast<int>(col) + cc;
-                            const int k = ti.k0 + (c & pkm);
-                            const int l = ti.l0 + (c >> d.pk_log2);
-                            if (i < d.nx && k < d.ny && l < d.nz) {
-                                const int64_t o = i + static_cast<int64_t>(d.nx) *
-                                                          (k + static_cast<int64_t>(d.ny) * l);
+                            const int kc = c & pkm, lc = c >> T.pk_log2;
+                            if (kc < kn && lc < ln) {
+                                const uint32_t o = o0 + xn * static_cast<uint32_t>(kc) + xny * static_cast<uint32_t>(lc);
                                 if (kSplit) {
-                                    d.part[static_cast<int64_t>(split) * d.nx * d.ny * d.nz + o] = v * S;
+                                    part[o] = v * S;
                                 } else {
                                     const float y = v * S + d.map.mu;
                                     map_store(d.map, o, y);
@@ -292,8 +306,11 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
 
             bool ok = true;
             if (form) {
-                const int c_end = kSplit ? (iv0 + NIl) * d.fc : d.nc;
-                for (int c = kSplit ? iv0 * d.fc : 0; c < c_end; ++c, ++g) {
+                // chunks of the item; light chunks are numbered below 0
+                const int c_end = kSplit ? min((iv0 + NIl) * T.fc, T.nc) : T.nc;
+                const int lcol = t >> 2;  // column whose row of x nodes this thread forms
+                const int lk = min(ti.k0 + (lcol & pkm), T.ny - 1), ll = min(ti.l0 + (lcol >> T.pk_log2), T.nz - 1);
+                for (int c = kSplit ? iv0 * T.fc : -nl; c < c_end; ++c, ++g) {
                     const int sb = static_cast<int>(g % kGSB);
                     const int sa = static_cast<int>(g % SA);
                     if (g >= kGSB &&
@@ -305,15 +322,20 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
                         ok = false;
                         break;
                     }
-                    const unsigned char* st = gsm + sa * d.a_stage;
-                    form_b(gsm + d.off_b + sb * kGPair, reinterpret_cast<const float4*>(st + toff_y),
-                           reinterpret_cast<const float4*>(st + toff_w0), reinterpret_cast<const float4*>(st + toff_w1),
-                           n0, n1, fg);
+                    const unsigned char* st = gsm + sa * T.a_stage;
+                    if (kLight && c < 0)
+                        form_light(gsm + T.off_b + sb * kGPair,
+                                   d.light + (static_cast<int64_t>(ll) * T.ny + lk) * T.lp,
+                                   __ldg(d.lstart + ti.mt) + (c + nl) * kGK, T.lp, T.l_inv, lcol, t & 3);
+                    else
+                        form_b(gsm + T.off_b + sb * kGPair, reinterpret_cast<const float4*>(st + toff_y),
+                               reinterpret_cast<const float4*>(st + toff_w0),
+                               reinterpret_cast<const float4*>(st + toff_w1), n0, n1, fg);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(bfull + sb);
-                    if ((c + 1) % d.fc == 0) {
-                        const int iv = (c + 1) / d.fc - 1 - (kSplit ? iv0 : 0);  // the item's interval whose chunks are all formed
+                    if (c >= -1 && ((c + 1) % T.fc == 0 || c + 1 == c_end)) {
+                        const int iv = (c + T.fc) / T.fc - 1 + li - (kSplit ? iv0 : 0);  // the item's interval whose chunks are all formed
                         if (iv >= 1) {
                             if (!fold(gi, iv == 1, false)) {
                                 ok = false;
@@ -349,12 +371,12 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
             constexpr uint32_t dhi = tc::smem_desc_sw128_hi(kGSbo);
             constexpr uint32_t tstep = kGOpBytes >> 4;  // one operand tile in descriptor units
             const uint32_t alo0 = tc::smem_desc_sw128_lo(smem_u32(gsm));
-            const uint32_t blo0 = tc::smem_desc_sw128_lo(smem_u32(gsm + d.off_b));
+            const uint32_t blo0 = tc::smem_desc_sw128_lo(smem_u32(gsm + T.off_b));
             uint32_t g = 0, gi = 0, tile_count = 0;
             uint32_t sa = 0, pa = 0, sb = 0, pb = 0;  // ring stages and their phase parities
             bool ok = true;
             const uint32_t dc = tbase + kGCorrCol;
-            for (int64_t item = blockIdx.x; item < (kSplit ? d.n_items : d.n_tiles) && ok; item += gridDim.x, ++tile_count) {
+            for (int64_t item = blockIdx.x; item < (kSplit ? T.n_items : T.n_tiles) && ok; item += gridDim.x, ++tile_count) {
                 const int split = kSplit ? static_cast<int>(item % n_split) : 0;
                 const int NIl = kSplit ? NI * (split + 1) / n_split - NI * split / n_split : NI;
                 // the previous item's correction accumulator has been read
@@ -370,13 +392,16 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
                     }
                     tc::fence_after();
                     const uint32_t dt = tbase + b * kGN;
-                    for (int cc = 0; cc < d.fc; ++cc, ++g) {
+                    const int cn = kLight && li && iv == 0
+                                       ? nl
+                                       : min(T.fc, T.nc - (iv - li + (kSplit ? NI * split / n_split : 0)) * T.fc);
+                    for (int cc = 0; cc < cn; ++cc, ++g) {
                         if (!gwait(afull + sa, pa, abort, status) || (form && !gwait(bfull + sb, pb, abort, status))) {
                             ok = false;
                             break;
                         }
                         tc::fence_after();
-                        const uint32_t alo = alo0 + sa * (static_cast<uint32_t>(d.a_stage) >> 4);
+                        const uint32_t alo = alo0 + sa * (static_cast<uint32_t>(T.a_stage) >> 4);
                         const uint32_t blo = form ? blo0 + sb * (kGPair >> 4) : alo + (kGPair >> 4);
 #pragma unroll
                         for (int ks = 0; ks < kGK / 16; ++ks) {
@@ -402,7 +427,7 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
                     }
                     if (ok) tc::commit(accfull + b);
                 }
-                if (ok) atomicAdd(&g_grid_tiles, 1ull);
+                if (ok && !d.quiet) atomicAdd(&g_grid_tiles, 1ull);
             }
             // every MMA this CTA issued has completed before TMEM is released
             tc::commit(done);
@@ -414,34 +439,39 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
         if (lane == 0) {
             uint32_t g = 0;
             bool ok = true;
-            for (int64_t item = blockIdx.x; item < (kSplit ? d.n_items : d.n_tiles) && ok; item += gridDim.x) {
+            for (int64_t item = blockIdx.x; item < (kSplit ? T.n_items : T.n_tiles) && ok; item += gridDim.x) {
                 const int64_t tile = kSplit ? item / n_split : item;
                 const int split = kSplit ? static_cast<int>(item - tile * n_split) : 0;
-                const TileIdx ti = tile_idx(d, tile);
-                const unsigned char* asrc = d.atab + static_cast<int64_t>(ti.mt) * d.nc * kGPair;
-                const int c_end = kSplit ? NI * (split + 1) / n_split * d.fc : d.nc;
-                for (int c = kSplit ? NI * split / n_split * d.fc : 0; c < c_end; ++c, ++g) {
+                const TileIdx ti = tile_idx(T, tile);
+                const unsigned char* asrc = d.atab + static_cast<int64_t>(ti.mt) * T.nc * kGPair;
+                const int c_end = kSplit ? min(NI * (split + 1) / n_split * T.fc, T.nc) : T.nc;
+                for (int c = kSplit ? NI * split / n_split * T.fc : -nl; c < c_end; ++c, ++g) {
                     const int sa = static_cast<int>(g % SA);
                     if (g >= static_cast<uint32_t>(SA) &&
                         !gwait(afree + sa, ((g / SA) - 1u) & 1u, abort, status)) {
                         ok = false;
                         break;
                     }
-                    unsigned char* dst = gsm + sa * d.a_stage;
+                    unsigned char* dst = gsm + sa * T.a_stage;
                     const unsigned char* ac = asrc + static_cast<int64_t>(c) * kGPair;
-                    if (form) {
+                    if (kLight && c < 0) {
+                        ac = d.latab + (static_cast<int64_t>(ti.mt) * nl + (c + nl)) * kGPair;
+                        mbar_arrive_expect_tx(afull + sa, kGPair);
+                        bulk_g2s(dst, ac, kGOpBytes, afull + sa);
+                        bulk_g2s(dst + kGOpBytes, ac + kGOpBytes, kGOpBytes, afull + sa);
+                    } else if (form) {
                         const uint32_t by = static_cast<uint32_t>(ti.pkv) * kGRowBytes;
                         const uint32_t bw = static_cast<uint32_t>(ti.plv) * kGRowBytes;
                         mbar_arrive_expect_tx(afull + sa, kGPair + by + bw);
                         bulk_g2s(dst, ac, kGOpBytes, afull + sa);
                         bulk_g2s(dst + kGOpBytes, ac + kGOpBytes, kGOpBytes, afull + sa);
-                        bulk_g2s(dst + kGPair, d.ytab + (static_cast<int64_t>(c) * d.ny + ti.k0) * (kGRowBytes / 8), by,
+                        bulk_g2s(dst + kGPair, d.ytab + (static_cast<int64_t>(c) * T.ny + ti.k0) * (kGRowBytes / 8), by,
                                  afull + sa);
-                        bulk_g2s(dst + kGPair + (1 << d.pk_log2) * kGRowBytes,
-                                 d.wztab + (static_cast<int64_t>(c) * d.nz + ti.l0) * (kGRowBytes / 8), bw,
+                        bulk_g2s(dst + kGPair + (1 << T.pk_log2) * kGRowBytes,
+                                 d.wztab + (static_cast<int64_t>(c) * T.nz + ti.l0) * (kGRowBytes / 8), bw,
                                  afull + sa);
                     } else {
-                        const unsigned char* bc = d.btab + (static_cast<int64_t>(ti.kt) * d.nc + c) * kGPair;
+                        const unsigned char* bc = d.btab + (static_cast<int64_t>(ti.kt) * T.nc + c) * kGPair;
                         mbar_arrive_expect_tx(afull + sa, 2 * kGPair);
                         bulk_g2s(dst, ac, kGOpBytes, afull + sa);
                         bulk_g2s(dst + kGOpBytes, ac + kGOpBytes, kGOpBytes, afull + sa);
@@ -464,6 +494,27 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
     }
 }
 
+template <bool kSplit>
+__global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int32_t* status) {
+    extern __shared__ __align__(1024) unsigned char gsm_dyn[];
+    grid_mma_body<kSplit, false>(d, d.t, gsm_dyn, status);
+}
+
+// The same with sizes that the device chose: the light modes on the node
+// lattice of the band path or the direct modes at the cells, as partial sums
+// (kSplit) or with the light modes' chunks and the maps.
+template <bool kSplit>
+__global__ void __launch_bounds__(kGThreads, 1) grid_band_kernel(GridDesc d, const GridTiling* src, int32_t* status) {
+    extern __shared__ __align__(1024) unsigned char gsm_dyn[];
+    __shared__ GridTiling T;
+    pdl_wait();
+    if (threadIdx.x < sizeof(GridTiling) / 4)
+        reinterpret_cast<uint32_t*>(&T)[threadIdx.x] = reinterpret_cast<const uint32_t*>(src)[threadIdx.x];
+    __syncthreads();
+    if (blockIdx.x >= T.n_items) return;  // nothing to sum, or fewer items than CTAs
+    grid_mma_body<kSplit, !kSplit>(d, T, gsm_dyn, status);
+}
+
 // Tables of one call (workspace).  Work items, flattened:
 //   A : (mt, chunk, row, quad of 4 modes) -> one 16-byte row segment of the
 //       hi and of the lo tile ((re, -im) pairs of e^{2 pi i a_x X_i}; rows
@@ -472,45 +523,70 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_mma_kernel(GridDesc d, int3
 //                W : (chunk, l, m) -> (A_j / S) e^{2 pi i (psi_j + a_jz Z_l)}, j = 32 chunk + m;
 //   2-D (load):  B : (kt, chunk, column, quad) -> (A_j / S) e^{2 pi i (psi_j + a_jy Y_k + a_jz Z_0)}
 //                as (re, im) hi and lo tiles (columns beyond ny are zero).
-__global__ void grid_prep_kernel(GridPrep p) {
-    const int64_t nA = static_cast<int64_t>(p.n_mt) * p.nc * kGM * 8;
-    const int64_t nY = p.form ? static_cast<int64_t>(p.ny) * p.n_pad : static_cast<int64_t>(p.n_kt) * p.nc * kGN * 8;
-    const int64_t nW = p.form ? static_cast<int64_t>(p.nz) * p.n_pad : 0;
-    const float s_inv = 1.0f / grid_scale(p.thdr);  // exact: a power of two
+// Node lattices of the band path also multiply A_j by the window's gains.
+// Table slot of mode j of the sum; < 0: none (the chunk's padding, amplitude 0).
+__device__ __forceinline__ int prep_slot(const GridPrep& p, int j) { return p.idx != nullptr ? __ldg(p.idx + j) : j; }
+__device__ __forceinline__ float prep_amp(const GridPrep& p, int j, const float4 c0, const float4 c1, float s_inv) {
+    float amp = __ldg(&p.hot[j].w) * s_inv;
+    if (p.gain_h[0] > 0.0f) amp *= band::gain(fabsf(c0.x) * p.gain_h[0]);
+    if (p.gain_h[1] > 0.0f) amp *= band::gain(fabsf(c0.z) * p.gain_h[1]);
+    if (p.gain_h[2] > 0.0f) amp *= band::gain(fabsf(c1.x) * p.gain_h[2]);
+    return amp;
+}
+
+// I: unsigned type that holds the item count (64-bit divisions are slow).
+template <class I>
+__device__ __forceinline__ void grid_prep_items(const GridPrep& p, I nA, I nY, I nW) {
+    const float s_inv = 1.0f / (p.scale > 0.0f ? p.scale : grid_scale(p.thdr));  // exact: a power of two
     const bool has_z = p.dim > 2;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < nA + nY + nW;
-         idx += stride) {
+    const I stride = static_cast<I>(gridDim.x) * blockDim.x;
+    for (I idx = static_cast<I>(blockIdx.x) * blockDim.x + threadIdx.x; idx < nA + nY + nW; idx += stride) {
         if (idx < nA || (!p.form && idx < nA + nY)) {
             // an operand tile row segment: A (x phasors) or, in 2-D, B
             const bool is_a = idx < nA;
-            const int64_t u = is_a ? idx : idx - nA;
+            const I u = is_a ? idx : idx - nA;
             const int quad = static_cast<int>(u & 7);
             const int r = static_cast<int>((u >> 3) & 127);
-            const int64_t rest = u >> 10;
-            const int c = static_cast<int>(rest % p.nc);
-            const int64_t tt = rest / p.nc;  // mt or kt
-            const int64_t i = tt * kGM + r;  // x or y cell
+            const I rest = u >> 10;  // (mt or kt) nc + chunk
+            const int tt = static_cast<int>(rest / static_cast<I>(p.nc));
+            const int c = static_cast<int>(rest - static_cast<I>(tt) * static_cast<I>(p.nc));
+            const int i = tt * kGM + r;  // row or y cell
             float v[8];
+            if (is_a) {
+                const bool in = i < p.nx;
+                const int zb = i / p.xn;  // z block of the row
+                const float x = in ? band::axis_at(p.ax[0], i - zb * p.xn) : 0.0f;
+                const float zs = static_cast<float>(zb) * p.zstep;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int j = c * kGModes + quad * 4 + m;
-                float cs = 0.0f, sn = 0.0f;
-                if (is_a) {
-                    if (i < p.nx) {
+                for (int m = 0; m < 4; ++m) {
+                    const int j = prep_slot(p, c * kGModes + quad * 4 + m);
+                    float cs = 0.0f, sn = 0.0f;
+                    if (in && j >= 0) {
                         const float4 c0 = __ldg(p.cold + 2 * j);
-                        sincospif(2.0f * turns_axis(c0.x, c0.y, __ldg(p.X + i)), &sn, &cs);
+                        float t = turns_axis(c0.x, c0.y, x);
+                        if (zb > 0) {
+                            const float4 c1 = __ldg(p.cold + 2 * j + 1);
+                            t = frac_turn(t + turns_axis(c1.x, c1.y, zs));
+                        }
+                        sincospif(2.0f * t, &sn, &cs);
                     }
                     v[2 * m] = cs;
                     v[2 * m + 1] = -sn;
-                } else {
-                    if (i < p.ny) {
+                }
+            } else {
+                const bool in = i < p.ny;
+                const float y = in ? band::axis_at(p.ax[1], i) : 0.0f;
+                const float z = has_z ? band::axis_at(p.ax[2], 0) : 0.0f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int j = prep_slot(p, c * kGModes + quad * 4 + m);
+                    float cs = 0.0f, sn = 0.0f;
+                    if (in && j >= 0) {
                         const float4 c0 = __ldg(p.cold + 2 * j);
                         const float4 c1 = __ldg(p.cold + 2 * j + 1);
-                        const float tz = psi_z_turns(c1, has_z ? __ldg(p.Z) : 0.0f, has_z);
-                        const float t = frac_turn(turns_axis(c0.z, c0.w, __ldg(p.Y + i)) + tz);
-                        sincospif(2.0f * t, &sn, &cs);
-                        const float amp = __ldg(&p.hot[j].w) * s_inv;
+                        const float tz = psi_z_turns(c1, z, has_z);
+                        sincospif(2.0f * frac_turn(turns_axis(c0.z, c0.w, y) + tz), &sn, &cs);
+                        const float amp = prep_amp(p, j, c0, c1, s_inv);
                         cs *= amp;
                         sn *= amp;
                     }
@@ -523,33 +599,121 @@ __global__ void grid_prep_kernel(GridPrep p) {
             tc::split_f16x2(v[2], v[3], H.y, L.y);
             tc::split_f16x2(v[4], v[5], H.z, L.z);
             tc::split_f16x2(v[6], v[7], H.w, L.w);
-            unsigned char* o = (is_a ? p.atab : p.btab) + (tt * p.nc + c) * static_cast<int64_t>(kGPair) +
-                               tile_off(r, quad);
+            unsigned char* o = (is_a ? p.atab : p.btab) + static_cast<int64_t>(rest) * kGPair + tile_off(r, quad);
             *reinterpret_cast<uint4*>(o) = H;
             *reinterpret_cast<uint4*>(o + kGOpBytes) = L;
-        } else if (idx < nA + nY) {
-            const int64_t u = idx - nA;  // (chunk, k, m)
-            const int m = static_cast<int>(u % kGModes);
-            const int64_t k = (u / kGModes) % p.ny;
-            const int c = static_cast<int>(u / (static_cast<int64_t>(kGModes) * p.ny));
-            const int j = c * kGModes + m;
-            const float4 c0 = __ldg(p.cold + 2 * j);
-            float cs, sn;
-            sincospif(2.0f * turns_axis(c0.z, c0.w, __ldg(p.Y + k)), &sn, &cs);
-            p.ytab[(u / kGModes) * (kGRowBytes / 8) + m] = make_float2(cs, sn);
         } else {
-            const int64_t u = idx - nA - nY;  // (chunk, l, m)
+            const bool is_y = idx < nA + nY;
+            const I u = is_y ? idx - nA : idx - nA - nY;  // (chunk, k or l, m)
             const int m = static_cast<int>(u % kGModes);
-            const int64_t l = (u / kGModes) % p.nz;
-            const int c = static_cast<int>(u / (static_cast<int64_t>(kGModes) * p.nz));
-            const int j = c * kGModes + m;
-            const float4 c1 = __ldg(p.cold + 2 * j + 1);
-            const float amp = __ldg(&p.hot[j].w) * s_inv;
-            float cs, sn;
-            sincospif(2.0f * psi_z_turns(c1, has_z ? __ldg(p.Z + l) : 0.0f, has_z), &sn, &cs);
-            p.wztab[(u / kGModes) * (kGRowBytes / 8) + m] = make_float2(amp * cs, amp * sn);
+            const I row = u / kGModes;
+            const I n = static_cast<I>(is_y ? p.ny : p.nz);
+            const int c = static_cast<int>(row / n);
+            const int k = static_cast<int>(row - static_cast<I>(c) * n);
+            const int j = prep_slot(p, c * kGModes + m);
+            float cs = 0.0f, sn = 0.0f;
+            if (j < 0) {
+                (is_y ? p.ytab : p.wztab)[static_cast<int64_t>(row) * (kGRowBytes / 8) + m] = make_float2(0.0f, 0.0f);
+                continue;
+            }
+            const float4 c0 = __ldg(p.cold + 2 * j);
+            if (is_y) {
+                sincospif(2.0f * turns_axis(c0.z, c0.w, band::axis_at(p.ax[1], k)), &sn, &cs);
+                p.ytab[static_cast<int64_t>(row) * (kGRowBytes / 8) + m] = make_float2(cs, sn);
+            } else {
+                const float4 c1 = __ldg(p.cold + 2 * j + 1);
+                const float amp = prep_amp(p, j, c0, c1, s_inv);
+                sincospif(2.0f * psi_z_turns(c1, has_z ? band::axis_at(p.ax[2], k) : 0.0f, has_z), &sn, &cs);
+                p.wztab[static_cast<int64_t>(row) * (kGRowBytes / 8) + m] = make_float2(amp * cs, amp * sn);
+            }
         }
     }
+}
+
+__device__ __forceinline__ void grid_prep(const GridPrep& p) {
+    const int64_t n_pad = static_cast<int64_t>(p.nc) * kGModes;
+    const int64_t nA = static_cast<int64_t>(p.n_mt) * p.nc * kGM * 8;
+    const int64_t nY = p.form ? static_cast<int64_t>(p.ny) * n_pad : static_cast<int64_t>(p.n_kt) * p.nc * kGN * 8;
+    const int64_t nW = p.form ? static_cast<int64_t>(p.nz) * n_pad : 0;
+    if (nA + nY + nW < (int64_t(1) << 31))
+        grid_prep_items(p, static_cast<uint32_t>(nA), static_cast<uint32_t>(nY), static_cast<uint32_t>(nW));
+    else
+        grid_prep_items(p, static_cast<uint64_t>(nA), static_cast<uint64_t>(nY), static_cast<uint64_t>(nW));
+}
+
+__global__ void __launch_bounds__(256) grid_prep_kernel(GridPrep p) {
+    pdl_wait();
+    grid_prep(p);
+}
+
+// A tiles of the light chunks: row = x cell of the tile, K = x nodes from the
+// tile's first one, the cell's weights times lw.
+__device__ __forceinline__ void light_prep(const BandDesc* b, const float* X, const int32_t* lstart,
+                                           unsigned char* latab) {
+    const BandAxis ax = b->ax[0];
+    const int nl = b->cells.nl;
+    const float lw = b->lw;
+    const uint32_t n = static_cast<uint32_t>(b->cells.n_mt) * nl * kGM * 8;
+    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+        const int seg = static_cast<int>(u & 7), r = static_cast<int>((u >> 3) & 127);
+        const int rest = static_cast<int>(u >> 10);
+        const int mt = rest / nl, lc = rest - mt * nl;
+        const int i = mt * kGM + r;
+        float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        if (i < b->cells.nx) {
+            float w[band::kW];
+            const int s = band::cell_weights(ax, __ldg(X + i), i, w) - (__ldg(lstart + mt) + lc * kGK + 8 * seg);
+            const int nt = band::taps(ax);
+#pragma unroll
+            for (int k = 0; k < band::kW; ++k)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (k < nt && s + k == e) v[e] = w[k] * lw;
+        }
+        uint4 H, L;
+        tc::split_f16x2(v[0], v[1], H.x, L.x);
+        tc::split_f16x2(v[2], v[3], H.y, L.y);
+        tc::split_f16x2(v[4], v[5], H.z, L.z);
+        tc::split_f16x2(v[6], v[7], H.w, L.w);
+        unsigned char* o = latab + static_cast<int64_t>(rest) * kGPair + tile_off(r, seg);
+        *reinterpret_cast<uint4*>(o) = H;
+        *reinterpret_cast<uint4*>(o + kGOpBytes) = L;
+    }
+}
+
+// Tables of a band-path call: those of the direct modes at the cells, those
+// of the light modes at the nodes, whose sizes are the device's choice, and
+// the light chunks' x weights.  `cells`, `nodes`: the host's part (table,
+// table pointers, cell axes).
+__device__ __forceinline__ void prep_sizes(GridPrep& p, const GridTiling& d) {
+    p.nx = d.nx;
+    p.ny = d.ny;
+    p.nz = d.nz;
+    p.nc = d.nc;
+    p.n_mt = d.n_mt;
+    p.n_kt = d.n_kt;
+    p.form = d.form;
+    p.scale = d.scale;
+    p.xn = d.xn;
+}
+__global__ void __launch_bounds__(256) band_prep_kernel(const BandDesc* b, GridPrep cells, GridPrep nodes,
+                                                        const int32_t* lstart, unsigned char* latab) {
+    pdl_wait();
+    if (b->nh > 0 && cells.atab != nullptr) {
+        prep_sizes(cells, b->cells);
+        grid_prep(cells);
+    }
+    if (b->n_light == 0) return;
+    prep_sizes(nodes, b->nodes);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const BandAxis a = b->ax[c];
+        if (!a.ident) nodes.ax[c] = AxisSrc{nullptr, a.h, a.n0};
+        nodes.gain_h[c] = a.ident ? 0.0f : a.h;
+    }
+    nodes.zstep = static_cast<float>(b->nodes.lz) * b->ax[2].h;
+    grid_prep(nodes);
+    if (b->cells.nl > 0) light_prep(b, cells.ax[0].p, lstart, latab);
 }
 
 // Mode-split grids: per cell the partial fields of the splits, added in split
@@ -557,6 +721,7 @@ __global__ void grid_prep_kernel(GridPrep p) {
 // block also writes its sum of (K - T)^2 to lpart.
 __global__ void __launch_bounds__(256) grid_split_finalize(const float* __restrict__ part, int n_split, int64_t n,
                                                            MapDev map) {
+    pdl_wait();
     const int64_t o = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const bool mm = (map.bits & kMapMismatch) != 0;
     double l = 0.0;
@@ -650,76 +815,173 @@ __global__ void __launch_bounds__(128, 1) mma_probe_kernel(const uint16_t* A, co
 
 int g_num_sms = 0;
 
-// Layout of one grid synthesis: mode, patch, tiles, shared-memory rings and
-// workspace tables.
-struct GridPlan {
-    bool form;
-    int pk_log2, n_mt, n_kt, n_lt, nc, sa, a_stage, off_b, off_bar, smem;
-    int max_split;  // mode splits for grids of few tiles (the launch takes at most one per fold interval)
-    int64_t n_tiles, a_bytes, y_bytes, w_bytes, b_bytes, part_bytes;
+}  // namespace
+
+namespace {
+
+int32_t chunks_of(int64_t n_pad) { return static_cast<int32_t>(n_pad / kGModes); }
+int64_t table_bytes(const GridPlan& g) { return g.a_bytes + g.y_bytes + g.w_bytes + g.b_bytes; }
+
+// One list of table slots.
+int64_t idx_bytes(const GridPlan& g) { return align256((int64_t(g.nc) * kGModes + 128) * 4); }
+
+// The nodes' tables: those of a grid of as many y and z cells, with mt row tiles.
+int64_t node_table_bytes(const GridPlan& g, int32_t mt) {
+    return table_bytes(g) - g.a_bytes + align256(int64_t(mt) * g.nc * kGPair);
+}
+
+// Workspace of a band-path call after the grid path's own: the descriptor,
+// the modes' lists, the x tiles' first nodes, the nodes' tables (a node axis is never longer
+// than its cell axis), the light chunks, the nodes' partial sums, the (x, y)
+// nodes at the z cells and the rows of x nodes at the (y, z) cells.
+struct BandLayout {
+    int64_t off_idx, off_lstart, off_tab, off_latab, off_part, off_mid, off_rows, total;
+    int64_t cap_nodes, cap_part, cap_mid;
+    int32_t cap_mt;
 };
+BandLayout band_layout(const GridGeom& gg, const GridPlan& g) {
+    const int64_t n = int64_t(gg.nx) * gg.ny * gg.nz;
+    BandLayout L;
+    L.cap_nodes = n / 4;
+    L.cap_part = n;
+    L.cap_mid = n / 2;
+    // row tiles of the nodes: several z blocks of few x nodes, within 64 MB of tables
+    L.cap_mt = std::max(g.n_mt, static_cast<int>(std::min<int64_t>(8, (int64_t(64) << 20) / (int64_t(g.nc) * kGPair))));
+    L.off_idx = align256(sizeof(BandDesc));
+    L.off_lstart = L.off_idx + 2 * idx_bytes(g);
+    L.off_tab = L.off_lstart + align256(int64_t(g.n_mt) * 4);
+    L.off_latab = L.off_tab + node_table_bytes(g, L.cap_mt);
+    L.off_part = L.off_latab + (g.form ? align256(int64_t(g.n_mt) * ((gg.nx + 3 + kGK - 1) / kGK) * kGPair) : 0);
+    L.off_mid = L.off_part + align256(L.cap_part * 4);
+    L.off_rows = L.off_mid + (g.form ? align256(L.cap_mid * 4) : g.max_split > 1 ? 0 : align256(n * 4));
+    L.total = L.off_rows + align256((int64_t(gg.nx) + 3) * gg.ny * gg.nz * 4);
+    return L;
+}
 
-// Grids of at most 64 tiles split each tile's modes over up to 8 CTAs, so
-// that about 128 work items fill the GPU.
-constexpr int kGMaxSplit = 8;
-constexpr int64_t kGSplitItems = 128;
+// Sizes at which a call on a grid may take the band path: the selection's
+// modes, at least half a finalize block of x cells and 4 rows per block (its
+// loss partials), and a direct sum of at least 50 us, below which the lattice's
+// kernels cost more than they save (512^2 x 4096: 48 us directly, 56 with it).
+constexpr double kBandMinUs = 50.0;
+bool band_sizes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    return n_pad <= band::kMaxModes && nx >= 32 && ny >= 8 &&
+           grid_us_per_mode(nx, ny, nz) * double(n_pad) >= kBandMinUs;
+}
 
-GridPlan grid_plan(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
-    GridPlan g{};
-    g.form = nz > 1;
-    g.nc = static_cast<int>(n_pad / kGModes);
-    g.n_mt = (nx + kGM - 1) / kGM;
+// Table pointers of one synthesis at `w`.
+void set_tables(GridPrep& p, GridDesc& d, const GridPlan& g, unsigned char* w) {
+    p.atab = w;
     if (g.form) {
-        // patch 2^p y-cells by 128 / 2^p z-cells (p = 2 .. 6): fewest wasted
-        // columns, then the fewest staged table rows
-        double best = 1e300;
-        for (int pk = 2; pk <= 6; ++pk) {
-            const int64_t PK = int64_t(1) << pk, PL = kGN / PK;
-            const double cols = double((ny + PK - 1) / PK * PK) * double((nz + PL - 1) / PL * PL);
-            const double w = cols / (double(ny) * double(nz)) + 1e-4 * double(PK + PL);
-            if (w < best) {
-                best = w;
-                g.pk_log2 = pk;
-            }
-        }
-        const int tb = ((1 << g.pk_log2) + (kGN >> g.pk_log2)) * kGRowBytes;
-        g.a_stage = (kGPair + tb + 1023) / 1024 * 1024;  // swizzle atoms start on 1024-byte boundaries
-        g.sa = std::min(kGMaxSA, (kGSmemMax - kGAlignPad - kGBarBytes - kGSB * kGPair) / g.a_stage);
-        g.off_b = g.sa * g.a_stage;
-        g.off_bar = g.off_b + kGSB * kGPair;
+        p.ytab = reinterpret_cast<float2*>(w + g.a_bytes);
+        p.wztab = reinterpret_cast<float2*>(w + g.a_bytes + g.y_bytes);
     } else {
-        g.pk_log2 = 7;
-        g.a_stage = 2 * kGPair;
-        g.sa = std::min(kGMaxSA, (kGSmemMax - kGAlignPad - kGBarBytes) / g.a_stage);
-        g.off_b = g.sa * g.a_stage;
-        g.off_bar = g.off_b;
+        p.btab = w + g.a_bytes;
     }
-    g.smem = g.off_bar + kGBarBytes + kGAlignPad;
-    g.n_kt = (ny + (1 << g.pk_log2) - 1) >> g.pk_log2;
-    const int PL = kGN >> g.pk_log2;
-    g.n_lt = (nz + PL - 1) / PL;
-    g.n_tiles = int64_t(g.n_mt) * g.n_kt * g.n_lt;
-    g.max_split = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kGMaxSplit, kGSplitItems / g.n_tiles)));
-    g.part_bytes = g.max_split > 1 ? align256(int64_t(g.max_split) * nx * ny * nz * 4) : 0;
-    g.a_bytes = align256(int64_t(g.n_mt) * g.nc * kGPair);
-    if (g.form) {
-        g.y_bytes = align256(int64_t(g.nc) * ny * kGRowBytes);
-        g.w_bytes = align256(int64_t(g.nc) * nz * kGRowBytes);
-    } else {
-        g.b_bytes = align256(int64_t(g.n_kt) * g.nc * kGPair);
-    }
-    return g;
+    d.atab = p.atab;
+    d.btab = p.btab;
+    d.ytab = p.ytab;
+    d.wztab = p.wztab;
+}
+
+int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const GridPlan& gp, int64_t n_modes,
+                unsigned char* w, int32_t fc, int32_t* status, cudaStream_t st) {
+    const BandLayout L = band_layout(gg, gp);
+    BandDesc* b = reinterpret_cast<BandDesc*>(w);
+    float* part = reinterpret_cast<float*>(w + L.off_part);
+    float* mid = reinterpret_cast<float*>(w + L.off_mid);
+    float* rows = reinterpret_cast<float*>(w + L.off_rows);
+    unsigned char* latab = w + L.off_latab;
+    // 3-D grids of many tiles add the light modes as chunks of the direct
+    // sum's product; the others leave partial sums to the finalize kernel
+    const bool split = gp.max_split > 1 || !gp.form;
+    GridPrep pc = p, pn = p;
+    BandSelect s{};
+    s.hot = p.hot;
+    s.cold = p.cold;
+    s.n_modes = static_cast<int32_t>(n_modes);
+    s.dim = p.dim;
+    s.idx_h = reinterpret_cast<int32_t*>(w + L.off_idx);
+    s.idx_l = reinterpret_cast<int32_t*>(w + L.off_idx + idx_bytes(gp));
+    s.seg = gg.seg;
+    s.status = status;
+    s.X = gg.X;
+    s.n[0] = gg.nx;
+    s.n[1] = gg.ny;
+    s.n[2] = gg.nz;
+    s.us_mode = static_cast<float>(grid_us_per_mode(gg.nx, gg.ny, gg.nz));
+    s.us_node = static_cast<float>(kBandNodeUs);
+    s.us_fixed = static_cast<float>(kBandFixedUs);
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_part;
+    s.cap_mid = L.cap_mid;
+    s.cap_mt = L.cap_mt;
+    s.fold = fc;
+    s.n_mt = gp.n_mt;
+    s.lstart = split ? nullptr : reinterpret_cast<int32_t*>(w + L.off_lstart);
+    s.max_split = gp.max_split;
+    s.split_cells = split ? 1 : 0;
+    s.loss_per_tile = kGEpiWarps;
+    s.loss_nb_finalize = band_finalize_blocks(gg);
+    s.thdr = p.thdr;
+    pc.idx = s.idx_h;
+    pn.idx = s.idx_l;
+    s.cells = d.t;
+    GridDesc dn = d, dc = d;
+    GridPlan gn = gp;
+    gn.a_bytes = align256(int64_t(L.cap_mt) * gp.nc * kGPair);
+    set_tables(pn, dn, gn, w + L.off_tab);
+    dn.part = part;
+    dn.quiet = 1;
+    // 2-D grids of many tiles: one slice of partial sums, in `mid` (2-D has no other use for it)
+    if (split && dc.part == nullptr) dc.part = mid;
+    dc.latab = latab;
+    dc.lstart = s.lstart;
+    dc.light = rows;
+    unsigned long long* tiles = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void**>(&tiles), g_grid_tiles);
+    if (e != cudaSuccess) return e;
+    int rc = launch_band_select(s, b, st);
+    if (rc != cudaSuccess) return rc;
+    e = launch_chained(band_prep_kernel, g_num_sms * 5, 256, 0, st, b, pc, pn, s.lstart, latab);
+    if (e == cudaSuccess)
+        e = launch_chained(grid_band_kernel<true>, g_num_sms, kGThreads, kGBandSmem, st, dn, &b->nodes, status);
+    if (e != cudaSuccess) return e;
+    rc = launch_band_lines(b, part, gg, mid, split ? nullptr : rows, g_num_sms, st);
+    if (rc != cudaSuccess) return rc;
+    const unsigned grid = static_cast<unsigned>(std::min<int64_t>(d.t.n_tiles * gp.max_split, g_num_sms));
+    e = launch_chained(split ? grid_band_kernel<true> : grid_band_kernel<false>, grid, kGThreads, kGBandSmem, st, dc,
+                       &b->cells, status);
+    if (e != cudaSuccess) return e;
+    rc = launch_band_finalize(b, gp.form ? mid : part, dc.part, gg, d.map, tiles, st);
+    if (rc != cudaSuccess) return rc;
+    if (d.map.bits & kMapMismatch)
+        return launch_loss_sum(d.map.lpart, 0, &b->loss_nb, d.map.inv_n_mean, d.map.loss, st);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
 size_t grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
-    const GridPlan g = grid_plan(nx, ny, nz, n_pad);
-    return static_cast<size_t>(g.a_bytes + g.y_bytes + g.w_bytes + g.b_bytes + g.part_bytes);
+    const GridPlan g = grid_plan(nx, ny, nz, chunks_of(n_pad));
+    return static_cast<size_t>(table_bytes(g) + g.part_bytes);
+}
+
+// Whole tiles, at the rate of the tensor-core kernel on large grids (65
+// Tcell.mode/s in rounds of one tile per SM of 152) or of its mode-split form.
+double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
+    const GridPlan g = grid_plan(nx, ny, nz, 4);
+    const double tile = double(kGM) * kGN;
+    return g.max_split > 1 ? double(g.n_tiles) * tile / 42.0e6 : std::ceil(double(g.n_tiles) / 152.0) * 152.0 * tile / 65.0e6;
+}
+
+size_t grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    if (!band_sizes(nx, ny, nz, n_pad)) return 0;
+    const GridGeom gg{nx, ny, nz, nullptr, nullptr, nullptr, nullptr};
+    return static_cast<size_t>(band_layout(gg, grid_plan(nx, ny, nz, chunks_of(n_pad))).total);
 }
 
 int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const GridGeom& gg, const MapDev& map,
-                      void* ws, int32_t fc, int32_t* status, void* stream) {
+                      void* ws, bool band, int32_t fc, int32_t* status, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const unsigned char* tb = static_cast<const unsigned char*>(table);
     const TableLayout TL = table_layout(n_modes);
@@ -727,88 +989,60 @@ int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const Gri
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(grid_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmemMax);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(grid_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmemMax);
+        auto allow = [&](const void* kern, int bytes) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        };
+        allow(reinterpret_cast<const void*>(grid_mma_kernel<false>), kGSmemMax);
+        allow(reinterpret_cast<const void*>(grid_mma_kernel<true>), kGSmemMax);
+        allow(reinterpret_cast<const void*>(grid_band_kernel<true>), kGBandSmem);
+        allow(reinterpret_cast<const void*>(grid_band_kernel<false>), kGBandSmem);
         if (e != cudaSuccess) return e;
         g_num_sms = sms;
     }
-    const GridPlan gp = grid_plan(gg.nx, gg.ny, gg.nz, TL.n_pad);
+    const GridPlan gp = grid_plan(gg.nx, gg.ny, gg.nz, chunks_of(TL.n_pad));
     unsigned char* w = static_cast<unsigned char*>(ws);
     GridPrep p{};
     p.thdr = reinterpret_cast<const TableHeader*>(tb);
     p.hot = reinterpret_cast<const float4*>(tb + TL.off_hot);
     p.cold = reinterpret_cast<const float4*>(tb + TL.off_cold);
-    p.X = gg.X;
-    p.Y = gg.Y;
-    p.Z = gg.Z;
+    p.ax[0].p = gg.X;
+    p.ax[1].p = gg.Y;
+    p.ax[2].p = gg.Z;
     p.nx = gg.nx;
     p.ny = gg.ny;
     p.nz = gg.nz;
-    p.n_pad = static_cast<int32_t>(TL.n_pad);
     p.nc = gp.nc;
     p.n_mt = gp.n_mt;
     p.n_kt = gp.n_kt;
     p.dim = dim;
     p.form = gp.form ? 1 : 0;
-    p.atab = w;
-    if (gp.form) {
-        p.ytab = reinterpret_cast<float2*>(w + gp.a_bytes);
-        p.wztab = reinterpret_cast<float2*>(w + gp.a_bytes + gp.y_bytes);
-    } else {
-        p.btab = w + gp.a_bytes;
-    }
+    p.xn = gg.nx;
+    GridDesc d{};
+    set_tables(p, d, gp, w);
+    d.thdr = p.thdr;
+    set_tiling(d.t, gp, gg.nx, gg.ny, gg.nz, fc);
+    d.part = gp.max_split > 1 ? reinterpret_cast<float*>(w + table_bytes(gp)) : nullptr;
+    d.map = map;
+    if (band) return launch_band(p, d, gg, gp, n_modes, w + table_bytes(gp) + gp.part_bytes, fc, status, st);
+
     const int64_t items = int64_t(gp.n_mt) * gp.nc * kGM * 8 +
                           (gp.form ? (int64_t(gg.ny) + gg.nz) * TL.n_pad : int64_t(gp.n_kt) * gp.nc * kGN * 8);
     const int pb = 256;
     const int64_t pg = std::min<int64_t>((items + pb - 1) / pb, int64_t(g_num_sms) * 16);
-    grid_prep_kernel<<<static_cast<unsigned>(pg), pb, 0, st>>>(p);
-    count_launches(1);
-
-    GridDesc d{};
-    d.atab = p.atab;
-    d.btab = p.btab;
-    d.ytab = p.ytab;
-    d.wztab = p.wztab;
-    d.thdr = p.thdr;
-    d.nx = gg.nx;
-    d.ny = gg.ny;
-    d.nz = gg.nz;
-    d.n_pad = p.n_pad;
-    d.nc = gp.nc;
-    d.fc = fc;
-    while (d.fc > 1 && gp.nc % d.fc != 0) d.fc >>= 1;  // whole fold intervals per tile
-    d.n_mt = gp.n_mt;
-    d.n_kt = gp.n_kt;
-    d.n_lt = gp.n_lt;
-    d.pk_log2 = gp.pk_log2;
-    d.n_tiles = gp.n_tiles;
-    d.n_split = std::min(gp.max_split, gp.nc / d.fc);  // whole fold intervals per split
-    d.n_items = d.n_tiles * d.n_split;
-    d.part = d.n_split > 1 ? reinterpret_cast<float*>(w + gp.a_bytes + gp.y_bytes + gp.w_bytes + gp.b_bytes)
-                           : nullptr;
-    d.form = p.form;
-    d.sa = gp.sa;
-    d.a_stage = gp.a_stage;
-    d.off_b = gp.off_b;
-    d.off_bar = gp.off_bar;
-    d.map = map;
-    const int64_t grid = std::min<int64_t>(d.n_items, g_num_sms);
-    if (d.n_split > 1)
-        grid_mma_kernel<true><<<static_cast<unsigned>(grid), kGThreads, gp.smem, st>>>(d, status);
-    else
-        grid_mma_kernel<false><<<static_cast<unsigned>(grid), kGThreads, gp.smem, st>>>(d, status);
-    count_launches(1);
+    cudaError_t ce = launch_chained(grid_prep_kernel, static_cast<unsigned>(pg), pb, 0, st, p);
+    const unsigned grid = static_cast<unsigned>(std::min<int64_t>(d.t.n_items, g_num_sms));
+    if (ce == cudaSuccess)
+        ce = launch_chained(d.t.n_split > 1 ? grid_mma_kernel<true> : grid_mma_kernel<false>, grid, kGThreads, gp.smem,
+                            st, d, status);
     const int64_t n = int64_t(gg.nx) * gg.ny * gg.nz;
     const int64_t fin_blocks = (n + 255) / 256;
-    if (d.n_split > 1) {
-        grid_split_finalize<<<static_cast<unsigned>(fin_blocks), 256, 0, st>>>(d.part, d.n_split, n, map);
-        count_launches(1);
-    }
+    if (ce == cudaSuccess && d.t.n_split > 1)
+        ce = launch_chained(grid_split_finalize, static_cast<unsigned>(fin_blocks), 256, 0, st, d.part, d.t.n_split, n,
+                            map);
+    if (ce != cudaSuccess) return ce;
     if (map.bits & kMapMismatch) {
-        const int e = launch_loss_sum(map.lpart, d.n_split > 1 ? fin_blocks : d.n_tiles * kGEpiWarps, map.inv_n_mean,
-                                      map.loss, st);
+        const int e = launch_loss_sum(map.lpart, d.t.n_split > 1 ? fin_blocks : d.t.n_tiles * kGEpiWarps, nullptr,
+                                      map.inv_n_mean, map.loss, st);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -816,11 +1050,11 @@ int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const Gri
 
 int64_t grid_loss_partials(int32_t nx, int32_t ny, int32_t nz) {
     // at most: one per (tile, warp) without a split, one per finalize block with one
-    const GridPlan g = grid_plan(nx, ny, nz, kGModes * 4);
+    const GridPlan g = grid_plan(nx, ny, nz, 4);
     return std::max<int64_t>(g.n_tiles * kGEpiWarps, (int64_t(nx) * ny * nz + 255) / 256);
 }
 
-int64_t grid_tiles(int32_t nx, int32_t ny, int32_t nz) { return grid_plan(nx, ny, nz, kGModes * 4).n_tiles; }
+int64_t grid_tiles(int32_t nx, int32_t ny, int32_t nz) { return grid_plan(nx, ny, nz, 4).n_tiles; }
 
 int take_grid_tiles(unsigned long long* tiles) {
     unsigned long long v = 0ull;

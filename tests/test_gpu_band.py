@@ -1,0 +1,137 @@
+"""GPU tests of the band-limited path (csrc/band.cuh): modes of low frequency
+summed on a coarse node lattice and interpolated to the cells.
+
+The fields are checked against the FP64 oracle at sampled cells with the
+forward tolerance of the other paths (1e-5 sigma): the interpolation's own
+error is at most 1.7e-7 per mode amplitude and adds incoherently over modes.
+The path is taken by size, so the cases are as large as it needs; that it was
+taken shows in the number of kernels launched.
+"""
+import math
+
+import numpy as np
+import pytest
+
+from helpers import check_forward, check_lognormal, gpu_env, oracle_field, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = gpu_env()
+    from paper_2212_10961_gb300 import field as F
+    from paper_2212_10961_gb300 import workloads as W
+    return torch, F, W
+
+
+def _modes(n, dim, ell, law, seed):
+    """Modes with normal ("gaussian") or Student t (1 degree: "rough") kappa."""
+    rng = np.random.default_rng(seed)
+    kappa = rng.standard_normal((n, dim)) * math.sqrt(math.pi / 2)
+    if law == "rough":
+        kappa = rng.standard_normal((n, dim)) / np.sqrt(rng.chisquare(1, n))[:, None]
+    a = kappa / (2 * math.pi * np.asarray(ell))
+    return {"a": a, "amp": rng.rayleigh(1.0, n) * math.sqrt(1.0 / n), "psi": rng.uniform(-0.5, 0.5, n), "kappa": kappa}
+
+
+def _mesh(axes):
+    m = np.meshgrid(*axes[::-1], indexing="ij")
+    return [np.ascontiguousarray(v.ravel().astype(np.float32)) for v in m[::-1]]
+
+
+def _uniform(shape, extent):
+    return [((np.arange(n) + 0.5) * (e / n)).astype(np.float32) for n, e in zip(shape, extent)]
+
+
+def _params(F, n, dim, ell):
+    return F.FieldParams(family="gaussian", sigma2=1.0, mean=0.25, ell=ell, dim=dim, n_modes=n)
+
+
+def _check_grid(env, axes, ell, n, law, seed=3, modes=None):
+    torch, F, W = env
+    dim = len(axes)
+    cells = _mesh(axes)
+    plan = F.CellPlan(*to_dev(torch, cells))
+    assert plan.grid_shape()[:dim] == tuple(len(a) for a in axes)
+    m = modes or _modes(n, dim, ell, law, seed)
+    table = F.ModeTable(m["amp"], m["psi"], m["a"])
+    l0 = F.launch_count()
+    out = F.synth(table, _params(F, n, dim, ell), plan, maps=F.MapSpec(y=True, lognormal=True))
+    torch.cuda.synchronize()
+    assert plan.status() == 0
+    launches = F.launch_count() - l0
+    idx = np.unique(np.concatenate([np.random.default_rng(1).choice(len(cells[0]), 6000), np.arange(300),
+                                    np.arange(len(cells[0]) - 300, len(cells[0]))]))
+    y_or = oracle_field(m, 0.25, cells, idx)
+    check_forward(out["Y"].cpu().numpy()[idx], y_or, 1.0, "band %s" % [len(a) for a in axes])
+    check_lognormal(out["K"].cpu().numpy()[idx], y_or, 1.0)
+    return launches
+
+
+# every route of the grid path: 2-D of few and of many tiles, 3-D of few tiles
+# (partial sums), 3-D of many (the light modes as chunks of the product), with
+# modes left for the direct sum and without
+@pytest.mark.parametrize("shape,extent,ell,n,law", [
+    ((701, 499), (1.4, 1.0), (0.2, 0.1), 6000, "gaussian"),
+    ((701, 499), (1.4, 1.0), (0.2, 0.1), 6001, "rough"),
+    ((1537, 1025), (1.5, 1.0), (0.1, 0.2), 2500, "rough"),
+    ((100, 81, 61), (1.0, 0.8, 0.6), (0.2, 0.2, 0.2), 6000, "gaussian"),
+    ((129, 101, 90), (1.29, 1.0, 0.9), (0.2, 0.15, 0.2), 4097, "rough"),
+    ((257, 131, 65), (1.0, 0.5, 0.25), (0.1, 0.1, 0.1), 3000, "gaussian"),
+    ((33, 40, 301), (0.1, 0.13, 1.0), (0.1, 0.1, 0.1), 4000, "rough"),
+    ((640, 9, 130), (4.0, 0.05, 0.9), (0.1, 0.1, 0.1), 3000, "rough"),
+])
+def test_band_grid_against_oracle(env, shape, extent, ell, n, law):
+    assert _check_grid(env, _uniform(shape, extent), ell, n, law) >= 6
+
+
+def test_band_grid_axes_in_any_order_and_far_away(env):
+    # rectilinear axes: random spacings far from the origin, one axis running
+    # down and one in random order (its cells' nodes lie far apart, so the
+    # staged loads give way to plain ones)
+    rng = np.random.default_rng(5)
+    axes = [np.float32(900.0) + np.cumsum(rng.uniform(0.002, 0.006, 400)).astype(np.float32),
+            np.ascontiguousarray((np.float32(-70.0) + np.cumsum(rng.uniform(0.004, 0.012, 120)).astype(np.float32))[::-1]),
+            rng.permutation(np.linspace(0.0, 1.0, 90).astype(np.float32))]
+    assert _check_grid(env, axes, (0.1, 0.1, 0.1), 3000, "rough") >= 6
+    axes[0] = rng.permutation(axes[0])
+    assert _check_grid(env, axes, (0.1, 0.1, 0.1), 3000, "gaussian") >= 6
+    axes2 = [rng.permutation(np.linspace(0.0, 2.0, 1400).astype(np.float32)), np.linspace(0, 1, 900).astype(np.float32)]
+    assert _check_grid(env, axes2, (0.1, 0.1), 4000, "gaussian") >= 5
+
+
+def test_band_grid_degenerate_frequencies(env):
+    # modes that do not vary along an axis, modes of frequency 0, equal phases
+    # (the light sum far larger than any amplitude) and one very fast mode
+    n = 4000
+    m = _modes(n, 3, (0.2, 0.2, 0.2), "gaussian", 8)
+    m["a"][:, 2] = 0.0
+    m["a"][::7] = 0.0
+    m["a"][11] = (3.0e4, -2.0e5, 17.0)
+    m["psi"][: n // 2] = 0.0
+    m["amp"] = m["amp"] / math.sqrt(n)  # the coherent half would sum to tens of sigma
+    axes = _uniform((180, 160, 70), (1.0, 0.9, 0.4))
+    assert _check_grid(env, axes, (0.2, 0.2, 0.2), n, "gaussian", modes=m) >= 6
+
+
+def test_band_grid_fused_mismatch(env):
+    # the fused loss sees the field of the synthesis (same kernels), on the
+    # routes that finalize and on the one that writes from the product
+    torch, F, W = env
+    for shape, law, n in (((128, 128, 80), "gaussian", 2000), ((160, 128, 90), "rough", 3000), ((900, 700), "rough", 3000)):
+        dim = len(shape)
+        ell = (0.2,) * dim
+        plan = F.CellPlan(*to_dev(torch, _mesh(_uniform(shape, (1.0, 0.9, 0.8)[:dim]))))
+        m = _modes(n, dim, ell, law, 4)
+        table = F.ModeTable(m["amp"], m["psi"], m["a"])
+        p = _params(F, n, dim, ell)
+        ref = F.synth(table, p, plan, maps=F.MapSpec(y=True, lognormal=True))
+        T = torch.full_like(ref["K"], 1.5)
+        loss_u, gY_u = F.mismatch_grad(ref["K"], T)
+        loss, gY, out = F.synth_mismatch(table, p, plan, T, want_Y=True, want_K=True)
+        torch.cuda.synchronize()
+        assert torch.equal(out["Y"], ref["Y"]) and torch.equal(out["K"], ref["K"]) and torch.equal(gY, gY_u)
+        assert loss.item() == pytest.approx(loss_u.item(), rel=1e-12)
+        again = F.synth(table, p, plan, maps=F.MapSpec(y=True))["Y"]
+        assert torch.equal(again, ref["Y"])  # deterministic
