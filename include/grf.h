@@ -361,6 +361,17 @@ size_t grf_synth_workspace_bytes(int64_t n_cells);
  * GRF_EINVAL for NULL pointers or an unknown plan.
  */
 size_t grf_synth_grid_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes);
+
+/*
+ * grf_synth_band_workspace_bytes -- workspace bytes that let grf_synth_field
+ * (and, after the loss partials, grf_synth_mismatch) sum the modes of low
+ * frequency on a coarse lattice of nodes and interpolate them to the cells of
+ * any plan, with room for the mode split of the others; 0 at sizes where all
+ * modes are summed at the cells (or for an unknown plan).  With a smaller
+ * workspace the call sums all modes at the cells.  On grid plans
+ * grf_synth_grid_workspace_bytes() includes the lattice's part.
+ */
+size_t grf_synth_band_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes);
 int grf_plan_grid_shape(const void *plan, int32_t *nx, int32_t *ny, int32_t *nz);
 
 /*

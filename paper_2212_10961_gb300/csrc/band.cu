@@ -30,7 +30,7 @@ namespace {
 using band::kW;
 
 constexpr int kSelThreads = 1024;
-constexpr int kKeep = 4;  // modes a selecting thread keeps in registers
+constexpr int kKeep = 8;  // modes a selecting thread keeps in registers
 constexpr int kNodeSplits = 32;     // most mode splits of a node tile
 constexpr int64_t kNodeItems = 152;  // (tile, mode split) items of the nodes' sum
 // Modes are binned by the largest of their frequencies relative to the axes'
@@ -89,14 +89,15 @@ __device__ __forceinline__ float4 mode_of(const BandSelect& p, int j) {
 // tensor-core tiles of 128 x 128) and `heavy` directly; 3e38 where the
 // lattice does not fit the workspace.
 __device__ float candidate_time(const BandSelect& p, int heavy, int light, int mx, int my, int mz) {
-    const float direct = p.us_mode * static_cast<float>((heavy + gridt::kGModes - 1) / gridt::kGModes * gridt::kGModes);
+    const float direct = p.us_mode * static_cast<float>((heavy + p.chunk - 1) / p.chunk * p.chunk) +
+                         (heavy > 0 ? p.us_heavy : 0.0f);
     if (light == 0) return direct;
     if (max(mx, max(my, mz)) >= 1 << 20) return 3.0e38f;  // the products below fit
     // one node more per axis than estimated: the light modes' own largest
     // frequencies, at most the bin's edge, may place the nodes less favourably
     const int64_t plane = static_cast<int64_t>(mx + 1) * (my + 1);
     if (plane * (mz + 1) > p.cap_nodes || (p.n[2] > 1 && plane * p.n[2] > p.cap_mid)) return 3.0e38f;
-    if ((mx + gridt::kGM) / gridt::kGM > p.cap_mt) return 3.0e38f;
+    if ((mx + gridt::kGM) / gridt::kGM > p.cap_mt || my >= p.cap_yz || mz >= p.cap_yz) return 3.0e38f;
     const int64_t tile = gridt::kGM * gridt::kGN;
     const float nodes = static_cast<float>((static_cast<int64_t>(mx) * my * mz + tile - 1) / tile * tile);
     return direct + p.us_node * nodes * static_cast<float>(light) + p.us_fixed;
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     } else if (warp == 1 && lane == 0) {
         // direct modes at the cells of a grid: the host's tiling with fewer chunks
         GridTiling q = p.cells;
-        q.nc = (nh + gridt::kGModes - 1) / gridt::kGModes;
+        q.nc = (nh + p.chunk - 1) / p.chunk;
         q.fc = max(1, min(p.fold, q.nc));
         q.n_split = max(1, gridt::min2(p.max_split, (q.nc + q.fc - 1) / q.fc));
         q.n_items = nh > 0 ? q.n_tiles * q.n_split : 0;
@@ -404,12 +405,12 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
         frexpf(static_cast<float>(n_light) * 22.0f, &k);
         k = max(0, k - 15);
         q.l_inv = ldexpf(1.0f, -e - k);
-        const int fin = nh == 0 || p.split_cells;
+        const int fin = p.n[0] > 0 ? nh == 0 || p.split_cells : q.n_split > 1;
         out->nh = nh;
         out->n_light = n_light;
-        out->n_splits = nh > 0 && fin ? q.n_split : 0;
+        out->n_splits = p.n[0] > 0 && !(nh > 0 && fin) ? 0 : q.n_split;
         out->finalize = fin;
-        out->loss_nb = fin ? p.loss_nb_finalize : p.cells.n_tiles * p.loss_per_tile;
+        out->loss_nb = fin ? p.loss_nb_finalize : p.loss_nb_tiles;
         out->lp = q.lp;
         out->lw = ldexpf(1.0f, k);
         out->cells = q;
@@ -532,6 +533,212 @@ __global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const
     }
 }
 
+// Cells in the plan's order: add[i] = sum over the 8^DIM nodes around cell i.
+// A block takes kCellsBlock consecutive sorted cells, a compact group: the
+// nodes that they read go to shared memory, and every lane sums one cell with
+// 16-byte loads (12 of the x nodes from a multiple of 4, the weights shifted
+// to them).  The block first puts its cells in the order of their nodes, so
+// that the lanes of a warp read mostly the same addresses: 192 loads per cell
+// in 3-D take 4.3 shared-memory wavefronts each in the plan's order (2M cells:
+// 210 us).  Groups that spread over more nodes than fit read them from memory.
+constexpr int kCellsBlock = 512, kBoxFloats = 10240, kCellBins = 1024;
+template <int DIM>
+__global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, const float* __restrict__ nodes,
+                                                            const float* __restrict__ xs, const float* __restrict__ ys,
+                                                            const float* __restrict__ zs, int64_t n, float* out) {
+    __shared__ __align__(16) float box[kBoxFloats];
+    __shared__ int bins[kCellBins];       // cells per bin, then of the bins before it
+    __shared__ short order[kCellsBlock];  // cells of the block by bin
+    __shared__ int first[3], last[3], warps[8];
+    pdl_wait();
+    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kCellsBlock;
+    const int t = threadIdx.x, lane = t & 31;
+    const int nc = static_cast<int>(min(static_cast<int64_t>(kCellsBlock), n - c0));
+    if (b->n_light == 0) {
+        for (int i = t; i < nc; i += 256) out[c0 + i] = 0.0f;
+        return;
+    }
+    if (t < 3) {
+        first[t] = INT_MAX;
+        last[t] = 0;
+    }
+    for (int k = t; k < kCellBins; k += 256) bins[k] = 0;
+    BandAxis ax[DIM];
+#pragma unroll
+    for (int c = 0; c < DIM; ++c) ax[c] = b->ax[c];
+    const float* src[3] = {xs + c0, ys + c0, zs + c0};
+    __syncthreads();
+    constexpr int kPer = kCellsBlock / 256;
+    int s[kPer][DIM];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int i = min(q * 256 + t, nc - 1);
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) {
+            float v;
+            s[q][c] = band::locate(ax[c], __ldg(src[c] + i), v);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < DIM; ++c) {
+        int lo = s[0][c], hi = s[0][c];
+#pragma unroll
+        for (int q = 1; q < kPer; ++q) {
+            lo = min(lo, s[q][c]);
+            hi = max(hi, s[q][c]);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) {
+            atomicMin(&first[c], lo);
+            atomicMax(&last[c], hi + kW);
+        }
+    }
+    __syncthreads();
+    const int mx = ax[0].m;
+    const int64_t plane = static_cast<int64_t>(mx) * ax[1].m;
+    int f0[3] = {0, 0, 0}, nb[3] = {1, 1, 1};
+#pragma unroll
+    for (int c = 0; c < DIM; ++c) {
+        f0[c] = first[c];
+        nb[c] = last[c] - first[c];
+    }
+    // rows of the box: an odd multiple of 4, so that the 16-byte loads of
+    // neighbouring rows fall in different banks
+    const int bx = nb[0] + 4;  // the last loads reach 4 past the nodes
+    const int px = ((bx + 3) / 4 | 1) * 4;
+    const int rows = nb[1] * nb[2];
+    const bool staged = static_cast<int64_t>(px) * rows <= kBoxFloats;
+    if (staged) {
+        for (int r = t >> 5; r < rows; r += 8) {
+            const int z = DIM > 2 ? r / nb[1] : 0, y = r - z * nb[1];
+            const float* p = nodes + (f0[2] + z) * plane + static_cast<int64_t>(f0[1] + y) * mx + f0[0];
+            for (int x = lane; x < px; x += 32) box[r * px + x] = x < nb[0] ? __ldg(p + x) : 0.0f;
+        }
+    }
+    // ---- order of the cells: counting sort by their first node (bins wrap
+    // where the group has more of them; the order within a bin does not matter)
+    int bin[kPer], rank[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        unsigned key = DIM > 2 ? static_cast<unsigned>(s[q][DIM - 1] - f0[2]) * static_cast<unsigned>(nb[1] - kW + 1) : 0u;
+        key = (key + static_cast<unsigned>(s[q][1] - f0[1])) * static_cast<unsigned>(nb[0] - kW + 1) +
+              static_cast<unsigned>(s[q][0] - f0[0]);
+        bin[q] = static_cast<int>(key & (kCellBins - 1));
+        rank[q] = q * 256 + t < nc ? atomicAdd(&bins[bin[q]], 1) : 0;
+    }
+    __syncthreads();
+    {
+        int v[kCellBins / 256], sum = 0;
+#pragma unroll
+        for (int k = 0; k < kCellBins / 256; ++k) {
+            v[k] = sum;
+            sum += bins[t * (kCellBins / 256) + k];
+        }
+        int run = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, run, off);
+            if (lane >= off) run += o;
+        }
+        if (lane == 31) warps[t >> 5] = run;
+        __syncthreads();
+        int before = run - sum;
+        for (int w = 0; w < (t >> 5); ++w) before += warps[w];
+#pragma unroll
+        for (int k = 0; k < kCellBins / 256; ++k) bins[t * (kCellBins / 256) + k] = before + v[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+        if (q * 256 + t < nc) order[bins[bin[q]] + rank[q]] = static_cast<short>(q * 256 + t);
+    __syncthreads();
+#pragma unroll 1
+    for (int q = 0; q < kPer; ++q) {
+        if (q * 256 + t >= nc) break;
+        const int i = order[q * 256 + t];
+        int at[DIM];
+        float w[kW], wy[kW], wz[kW], v;
+        at[0] = band::locate(ax[0], __ldg(src[0] + i), v);
+        band::weights(v, w);
+        at[1] = band::locate(ax[1], __ldg(src[1] + i), v);
+        band::weights(v, wy);
+        if (DIM > 2) {
+            at[DIM - 1] = band::locate(ax[DIM - 1], __ldg(src[2] + i), v);
+            band::weights(v, wz);
+        }
+        float acc = 0.0f;
+        if (staged) {
+            const int dx = at[0] - f0[0], sh = dx & 3;
+            float w12[12];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                float u = 0.0f;
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (k - h >= 0 && k - h < kW) u = sh == h ? w[k - h] : u;
+                w12[k] = u;
+            }
+            const float* p = box + (dx - sh) + (at[1] - f0[1]) * px + (DIM > 2 ? (at[DIM - 1] - f0[2]) * nb[1] * px : 0);
+#pragma unroll 1
+            for (int kz = 0; kz < (DIM > 2 ? kW : 1); ++kz) {
+                float a = 0.0f;
+#pragma unroll
+                for (int ky = 0; ky < kW; ++ky) {
+                    const float4* r4 = reinterpret_cast<const float4*>(p + ky * px);
+                    const float4 r0 = r4[0], r1 = r4[1], r2 = r4[2];
+                    // the tails first
+                    float u = w12[0] * r0.x;
+                    u = fmaf(w12[11], r2.w, u);
+                    u = fmaf(w12[1], r0.y, u);
+                    u = fmaf(w12[10], r2.z, u);
+                    u = fmaf(w12[2], r0.z, u);
+                    u = fmaf(w12[9], r2.y, u);
+                    u = fmaf(w12[3], r0.w, u);
+                    u = fmaf(w12[8], r2.x, u);
+                    u = fmaf(w12[4], r1.x, u);
+                    u = fmaf(w12[7], r1.w, u);
+                    u = fmaf(w12[5], r1.y, u);
+                    u = fmaf(w12[6], r1.z, u);
+                    a = fmaf(wy[ky], u, a);
+                }
+                if (DIM > 2) {
+                    float u = wz[0];
+#pragma unroll
+                    for (int k = 1; k < kW; ++k) u = kz == k ? wz[k] : u;
+                    acc = fmaf(u, a, acc);
+                } else {
+                    acc = a;
+                }
+                p += nb[1] * px;
+            }
+        } else {
+            const float* p = nodes + (DIM > 2 ? at[DIM - 1] * plane : 0) + static_cast<int64_t>(at[1]) * mx + at[0];
+#pragma unroll 1
+            for (int kz = 0; kz < (DIM > 2 ? kW : 1); ++kz) {
+                float a = 0.0f;
+#pragma unroll
+                for (int ky = 0; ky < kW; ++ky) {
+                    float u = 0.0f;
+#pragma unroll
+                    for (int k = 0; k < kW; ++k) u = fmaf(w[k], __ldg(p + static_cast<int64_t>(ky) * mx + k), u);
+                    a = fmaf(wy[ky], u, a);
+                }
+                if (DIM > 2) {
+                    float u = wz[0];
+#pragma unroll
+                    for (int k = 1; k < kW; ++k) u = kz == k ? wz[k] : u;
+                    acc = fmaf(u, a, acc);
+                } else {
+                    acc = a;
+                }
+                p += plane;
+            }
+        }
+        out[c0 + i] = acc;
+    }
+}
+
 // Cells of a grid: y and x interpolation of the light modes from the (x, y)
 // nodes at the cell's z (2-D: the nodes), plus the direct modes' partial sums
 // (added in split order), mu, the maps and the loss partials.
@@ -544,7 +751,7 @@ __global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const
 constexpr int kFinRows = 8, kFinNodes = 320;
 __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b, const float* __restrict__ mid,
                                                                const float* __restrict__ part, GridGeom gg, int tx,
-                                                               MapDev map, unsigned long long* tiles) {
+                                                               int units, MapDev map, unsigned long long* tiles) {
     __shared__ float rows[kFinRows][kFinNodes];
     __shared__ __align__(16) float wy[kFinRows][kW];
     __shared__ int sy[kFinRows];
@@ -553,20 +760,20 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
     pdl_wait();
     if (!b->finalize) return;
     const int t = threadIdx.x;
+    const int n_light = b->n_light, n_split = b->n_splits;
+    const int nx = gg.nx, ny = gg.ny;
+    const int xb = (nx + tx - 1) / tx, yb = (ny + kFinRows - 1) / kFinRows;
+    const bool mm = (map.bits & kMapMismatch) != 0;
+    if (b->nh == 0 && tiles != nullptr && blockIdx.x == 0 && t == 0)
+        atomicAdd(tiles, static_cast<unsigned long long>(b->cells.n_tiles));
+    for (int u = static_cast<int>(blockIdx.x); u < units; u += static_cast<int>(gridDim.x)) {
+    __syncthreads();  // the previous unit's tables are no longer read
     if (t == 0) {
         first = INT_MAX;
         last = 0;
     }
-    const int n_light = b->n_light, n_split = b->n_splits;
-    const int nx = gg.nx, ny = gg.ny;
-    const int xb = (nx + tx - 1) / tx, yb = (ny + kFinRows - 1) / kFinRows;
-    const int u = static_cast<int>(blockIdx.x);
     const int k0 = (u / xb) % yb * kFinRows, l = u / xb / yb;
     const int i = u % xb * tx + (t & (tx - 1));
-    const bool mm = (map.bits & kMapMismatch) != 0;
-    if (b->nh == 0 && tiles != nullptr && u == 0 && t == 0)
-        atomicAdd(tiles, static_cast<unsigned long long>(b->cells.n_tiles));
-    // targets of the loss: in flight during the interpolation
     const int r0 = t / tx, rstep = 256 / tx;
     float w[kW];
     int s = 0, nt = 0, mx = 0, nty = 0;
@@ -657,6 +864,7 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
             map.lpart[u] = sum;
         }
     }
+    }
 }
 
 }  // namespace
@@ -683,17 +891,26 @@ int launch_band_lines(const BandDesc* b, float* part, const GridGeom& gg, float*
                       void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = launch_chained(band_sum_kernel, sms * 8, 256, 0, st, b, part);
-    if (e == cudaSuccess && gg.nz > 1)
+    if (e == cudaSuccess && mid != nullptr && gg.nz > 1)
         e = launch_chained(band_line_kernel<false>, sms * 4, 256, 0, st, b, part, gg.Z, gg.nz, gg.nz, mid);
     if (e == cudaSuccess && rows != nullptr)
         e = launch_chained(band_line_kernel<true>, sms * 4, 256, 0, st, b, mid, gg.Y, gg.ny, gg.nz, rows);
     return e;
 }
 
+int launch_band_cells(const BandDesc* b, const float* nodes, int32_t dim, const float* xs, const float* ys,
+                      const float* zs, int64_t n, float* out, void* stream) {
+    return launch_chained(dim > 2 ? band_cells_kernel<3> : band_cells_kernel<2>,
+                          static_cast<unsigned>((n + kCellsBlock - 1) / kCellsBlock), 256, 0,
+                          static_cast<cudaStream_t>(stream), b, nodes, xs, ys, zs, n, out);
+}
+
 int launch_band_finalize(const BandDesc* b, const float* mid, const float* part, const GridGeom& gg,
-                         const MapDev& map, unsigned long long* tiles, void* stream) {
-    return launch_chained(band_finalize_kernel, static_cast<unsigned>(band_finalize_blocks(gg)), 256, 0,
-                          static_cast<cudaStream_t>(stream), b, mid, part, gg, finalize_tx(gg.nx), map, tiles);
+                         const MapDev& map, unsigned long long* tiles, int sms, void* stream) {
+    // a few rounds of resident blocks; a launch with nothing to do ends at once
+    const int units = static_cast<int>(band_finalize_blocks(gg));
+    return launch_chained(band_finalize_kernel, std::min(units, sms * 16), 256, 0, static_cast<cudaStream_t>(stream), b,
+                          mid, part, gg, finalize_tx(gg.nx), units, map, tiles);
 }
 
 }  // namespace grf

@@ -50,7 +50,12 @@ __device__ __forceinline__ float gain(float xi) {
     return expf(r) * fmaf(-r, 1.0f / kBeta, 1.0f);
 }
 
-// d ln(gain) / d xi.
+// ln(gain), and its derivative, in FP64.
+__device__ __forceinline__ double log_gain(double xi) {
+    const double q2 = 631.6546816697189 * xi * xi, beta = 18.661060362323371;  // (pi W)^2
+    const double r = q2 / (beta + sqrt(beta * beta - q2));
+    return r + log1p(-r / beta);
+}
 __device__ __forceinline__ double log_gain_slope(double xi) {
     const double pw = 25.132741228718345, beta = 18.661060362323371;
     const double z2 = beta * beta - pw * pw * xi * xi;

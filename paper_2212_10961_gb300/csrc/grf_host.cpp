@@ -380,9 +380,10 @@ bool plan_grid(const void* plan, GridGeom* gg, float* box = nullptr) {
 // that then finds no lattice has paid kBandTryUs for the attempt.  q: largest
 // |kappa_c| that a fraction 2^-(k+1) of the modes exceeds, by dimension and
 // law (Student t with 1 and 3 degrees of freedom, normal), from 4 10^6 draws.
-// n: cells per axis of a grid, or null.  us_mode: time of one mode summed
-// directly.
-bool band_worth(const grf_params* p, const float* box, const int32_t* n, double us_mode, double us_node,
+// n: cells per axis of a grid, or null; cap: most nodes.  us_mode: time of one
+// mode summed directly.  Returns the modes expected to be left for the direct
+// sum, -1 where no gain of a quarter is expected.
+double band_worth(const grf_params* p, const float* box, const int32_t* n, double cap, double us_mode, double us_node,
                 double us_fixed) {
     static const float q[2][3][12] = {
         {{1.553f, 3.483f, 7.153f, 14.37f, 28.78f, 57.76f, 116.f, 232.f, 465.f, 916.f, 1853.f, 3539.f},
@@ -396,6 +397,7 @@ bool band_worth(const grf_params* p, const float* box, const int32_t* n, double 
     const double N = static_cast<double>(p->n_modes), direct = us_mode * N;
     double min_ell = 1e300;
     for (int c = 0; c < p->dim; ++c) min_ell = std::min(min_ell, p->ell[c]);
+    double best = 0.75 * direct, left = -1.0;
     for (int k = 0; k < 12; ++k) {
         double heavy = std::ldexp(N, -(k + 1));
         const bool last = heavy < 2.0 || k == 11;
@@ -408,11 +410,16 @@ bool band_worth(const grf_params* p, const float* box, const int32_t* n, double 
             if (n) m = std::min(m, static_cast<double>(n[c]));
             nodes *= m;
         }
+        const bool fits = nodes < cap;
         nodes = std::ceil(nodes / 16384.0) * 16384.0;
-        if (heavy * us_mode + (N - heavy) * nodes * us_node + us_fixed < 0.75 * direct) return true;
+        const double t = heavy * us_mode + (N - heavy) * nodes * us_node + us_fixed;
+        if (fits && t < best) {
+            best = t;
+            left = heavy;
+        }
         if (last) break;
     }
-    return false;
+    return left;
 }
 
 // The same for a call on a Cartesian grid, with the workspace it has.
@@ -421,7 +428,8 @@ bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t
     const size_t extra = grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
     if (extra == 0 || ws_bytes < grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra) return false;
     const int32_t n[3] = {gg.nx, gg.ny, gg.nz};
-    return band_worth(p, box, n, grid_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeUs, kBandFixedUs + kBandTryUs);
+    return band_worth(p, box, n, 0.25 * gg.nx * gg.ny * gg.nz, grid_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeUs,
+                      kBandFixedUs + kBandTryUs) >= 0.0;
 }
 
 bool lookup_plan(const void* plan, PlanMeta& out) {
@@ -859,6 +867,27 @@ int grf_read_status(const void* plan, int32_t* status_out, void* stream) try {
 // Synthesis
 // ---------------------------------------------------------------------------
 namespace {
+// The segment's bounds on the device where the call takes the band path at
+// the cells of a plan that is not a grid, else null.  Cells whose bounds the
+// host does not know (several segments) try it where the sum is long.  few:
+// whether few modes are expected to be left for the direct sum.
+CellsBand cells_band(const grf_params* p, const void* plan, const PlanMeta& meta, int32_t segment, const float* box,
+                     size_t ws_bytes) {
+    if (g_grid_enabled.load() == 0 || p->dim < 2) return CellsBand{};
+    const int64_t n = meta.offsets[segment + 1] - meta.offsets[segment];
+    const size_t need = cells_band_ws_bytes(n, p->n_modes, p->dim);
+    if (need == 0 || ws_bytes < need) return CellsBand{};
+    const double us = cells_us_per_mode(n), fixed = cells_band_us(n, p->dim) + kBandTryUs;
+    const double N = static_cast<double>(p->n_modes);
+    const double left = std::isfinite(box[0])
+                            ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), us, kBandNodeUs, fixed)
+                            : us * N < 500.0 ? -1.0 : N;
+    if (left < 0.0) return CellsBand{};
+    return CellsBand{
+        reinterpret_cast<const SegInfo*>(static_cast<const unsigned char*>(plan) + meta.layout.off_segs) + segment,
+        left * 16.0 <= N};
+}
+
 int fwd_desc(const void* table, int64_t n_modes, int32_t dim, const void* plan,
              const PlanMeta& meta, int32_t segment, const MapDev& map, FwdDesc& d) {
     if (segment < 0 || segment >= static_cast<int32_t>(meta.offsets.size()) - 1)
@@ -915,7 +944,7 @@ int grf_synth_field(const void* table, const grf_params* p, const void* plan, in
     // Cartesian grid handed over x-fastest: tensor-core path when the
     // workspace holds its tables
     GridGeom gg{};
-    float box[6];
+    float box[6] = {NAN, NAN, NAN, NAN, NAN, NAN};
     if (n > 0 && workspace && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim &&
         plan_grid(plan, &gg, box) && use_grid_path(gg) &&
         grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
@@ -925,11 +954,26 @@ int grf_synth_field(const void* table, const grf_params* p, const void* plan, in
         if (err != cudaSuccess) return cuda_fail(err, "grid synth kernels");
         return GRF_OK;
     }
-    const int err = launch_synth_fwd(d, workspace, workspace ? ws_bytes : 0, status, stream);
+    const int err = launch_synth_fwd(d, table, p->n_modes, cells_band(p, plan, meta, segment, box, workspace ? ws_bytes : 0),
+                                     workspace, workspace ? ws_bytes : 0, status, stream);
     if (err != cudaSuccess) return cuda_fail(err, "synth kernel");
     return GRF_OK;
 } catch (...) {
     return host_exception();
+}
+
+size_t grf_synth_band_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
+    try {
+        PlanMeta meta;
+        if (!plan || n_modes < 1 || n_modes > GRF_MAX_MODES || !lookup_plan(plan, meta)) return 0;
+        if (segment < 0 || segment >= static_cast<int32_t>(meta.offsets.size()) - 1) return 0;
+        const int64_t n = meta.offsets[segment + 1] - meta.offsets[segment];
+        size_t most = 0;
+        for (int32_t dim = 2; dim <= meta.dim; ++dim) most = std::max(most, cells_band_ws_bytes(n, n_modes, dim));
+        return most > 0 ? most + synth_workspace_bytes(n) : 0;
+    } catch (...) {
+        return 0;
+    }
 }
 
 size_t grf_synth_grid_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
@@ -1008,7 +1052,7 @@ int grf_synth_mismatch(const void* table, const grf_params* p, const void* plan,
     // Cartesian grid: the tensor-core path when the rest of the workspace
     // holds its tables and the loss partials fit
     GridGeom gg{};
-    float box[6];
+    float box[6] = {NAN, NAN, NAN, NAN, NAN, NAN};
     if (n > 0 && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim && plan_grid(plan, &gg, box) &&
         use_grid_path(gg) && grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
         ws_bytes - lbytes >= grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad) &&
@@ -1019,7 +1063,8 @@ int grf_synth_mismatch(const void* table, const grf_params* p, const void* plan,
         if (err != cudaSuccess) return cuda_fail(err, "grid synth kernels");
         return GRF_OK;
     }
-    const int err = launch_synth_fwd(d, split_ws, ws_bytes - lbytes, status, stream);
+    const int err = launch_synth_fwd(d, table, p->n_modes, cells_band(p, plan, meta, segment, box, ws_bytes - lbytes),
+                                     split_ws, ws_bytes - lbytes, status, stream);
     if (err != cudaSuccess) return cuda_fail(err, "synth kernel");
     return GRF_OK;
 } catch (...) {

@@ -5,6 +5,8 @@
 #include <cstddef>
 #include <cstdint>
 
+#include <vector_types.h>
+
 #include "grf.h"
 
 #ifndef GRF_CHECKED
@@ -199,6 +201,8 @@ struct MapDev {
     int32_t pad_;
 };
 
+struct BandDesc;
+
 // One realisation as the forward kernel sees it.
 struct FwdDesc {
     const float4* hot;
@@ -214,6 +218,10 @@ struct FwdDesc {
     const int32_t* perm;  // original (plan-global) index of each sorted cell
     int64_t perm_base;    // first plan-global index of the segment
     int64_t n_cells;
+    // band path (band.cuh): the table holds the band->nh direct modes, in
+    // band->n_splits mode splits, and add[sorted cell] the light modes' sum
+    const BandDesc* band;
+    const float* add;
     MapDev map;
 };
 
@@ -332,16 +340,19 @@ struct BandSelect {
     float us_mode;           // time of one mode summed directly, us
     float us_node;           // time of one mode at one node, us
     float us_fixed;          // time of the lattice's own kernels, us
+    float us_heavy;          // time of the direct sum's kernels beside the modes', us
     int64_t cap_nodes;       // most nodes
     int64_t cap_part;        // floats of the nodes' partial sums
     int64_t cap_mid;         // most (x, y) nodes x z cells
     int32_t cap_mt;          // most 128-row tiles of the nodes' x operand
+    int32_t cap_yz;          // the y and z axes have fewer nodes than this
     int32_t fold;
     int32_t n_mt;            // x tiles of the cells
     int32_t* lstart;         // [n_mt] first x node of a tile (written here; null: no light chunks)
+    int32_t chunk;           // the direct sum takes whole chunks of this many modes
     int32_t max_split;       // mode splits of the direct sum (1: unsplit)
     int32_t split_cells;     // 1: the direct sum leaves partial sums to the finalize kernel
-    int32_t loss_per_tile;
+    int64_t loss_nb_tiles;   // loss partials of an unsplit direct sum, and of the finalize kernel
     int64_t loss_nb_finalize;
     const TableHeader* thdr;
     GridTiling cells;        // the cells' tiling (all modes)
@@ -370,7 +381,15 @@ constexpr uint32_t kBatchMagic = 0x48435442u;  // "BTCH"
 // Kernel launchers (defined in the .cu files), all asynchronous on `stream`.
 // Return cudaError_t as int.
 // ---------------------------------------------------------------------------
-int launch_synth_fwd(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* status, void* stream);
+// seg: the segment's bounds, to take the band path with the first
+// cells_band_ws_bytes of the workspace; null: all modes directly.  few: few
+// modes are expected to be left for the direct sum.
+struct CellsBand {
+    const SegInfo* seg = nullptr;
+    bool few = false;
+};
+int launch_synth_fwd(const FwdDesc& d, const void* table, int64_t n_modes, const CellsBand& band, void* workspace,
+                     size_t ws_bytes, int32_t* status, void* stream);
 // Entries of MapDev::lpart a launch of n cells may write (kMapMismatch).
 int64_t mismatch_partials(int64_t n_cells);
 // loss = (sum of the nb partials, fixed order) * inv_n, one block.
@@ -454,8 +473,21 @@ int launch_band_select(const BandSelect& p, BandDesc* out, void* stream);
 int launch_band_lines(const BandDesc* b, float* part, const GridGeom& gg, float* mid, float* rows, int sms,
                       void* stream);
 int launch_band_finalize(const BandDesc* b, const float* mid, const float* part, const GridGeom& gg,
-                         const MapDev& map, unsigned long long* tiles, void* stream);
+                         const MapDev& map, unsigned long long* tiles, int sms, void* stream);
 int64_t band_finalize_blocks(const GridGeom& gg);
+// Band path at the cells of any plan (synth_grid.cu): workspace bytes (0: not
+// taken at these sizes) and the launch up to the light modes' sums at the
+// sorted cells; `d` gets the direct modes' table, `add` and `band`.
+size_t cells_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
+int launch_cells_band(const void* table, int64_t n_modes, FwdDesc& d, const SegInfo* seg, void* ws,
+                      int32_t max_split, int64_t loss_tiles, int64_t loss_finalize, int32_t* status, void* stream);
+// Time of one mode summed at n cells of a plan that is not a grid, and of the
+// interpolation to them, us.
+double cells_us_per_mode(int64_t n_cells);
+int64_t cells_band_cap(int64_t n_cells);
+double cells_band_us(int64_t n_cells, int32_t dim);
+int launch_band_cells(const BandDesc* b, const float* nodes, int32_t dim, const float* xs, const float* ys,
+                      const float* zs, int64_t n, float* out, void* stream);
 int take_grid_tiles(unsigned long long* tiles);
 int launch_mma_probe(const uint16_t* A, const uint16_t* B, int32_t k_chunks, float* D, int32_t* status,
                      void* stream);

@@ -24,6 +24,8 @@
 // Every mbarrier wait is bounded and reports through the status word.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "launch.cuh"
 
@@ -192,7 +194,7 @@ __device__ __forceinline__ float warp_max(float v) {
 // MM: the epilogue also forms the mismatch gradient of every cell and writes
 // the warp's sum of (K - T)^2 to d.map.lpart[wbase / (32 C)] (kMapMismatch).
 template <int DIM, int C, int POLY, bool MM = false, int NS = 0>
-__device__ __forceinline__ bool synth_warp_tile(const FwdDesc& d, int64_t wbase, int cb, int ce,
+__device__ __forceinline__ bool synth_warp_tile(const FwdDesc& d, int n_pad, int64_t wbase, int cb, int ce,
                                                 float2* partial, WarpSmem& ws, uint32_t (&uses)[kStages],
                                                 int32_t* status, float4* stp = nullptr) {
     const int lane = threadIdx.x & 31;
@@ -257,8 +259,8 @@ __device__ __forceinline__ bool synth_warp_tile(const FwdDesc& d, int64_t wbase,
         Ew = fmaxf(Ew, fmaxf(mx - x0[k], x0[k] - mn));
     }
     Et = warp_max(Et);
-    const int k_med = prefix_for(d.kpref, d.n_pad, Ew * d.inv_tau1);
-    const int k_sup = min(k_med, prefix_for(d.kpref, d.n_pad, Et * d.inv_tau2));
+    const int k_med = prefix_for(d.kpref, n_pad, Ew * d.inv_tau1);
+    const int k_sup = min(k_med, prefix_for(d.kpref, n_pad, Et * d.inv_tau2));
 
     float s[C], e[C], p[C];
 #pragma unroll
@@ -469,6 +471,7 @@ __device__ __forceinline__ bool synth_warp_tile(const FwdDesc& d, int64_t wbase,
             if (partial != nullptr) {
                 partial[i] = make_float2(s[c], e[c]);
             } else {
+                if (d.add != nullptr) two_sum_acc(s[c], e[c], __ldg(d.add + i));
                 const float y = (s[c] + e[c]) + d.map.mu;
                 const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
                 if (index_ok(o, d.n_cells)) {
@@ -508,15 +511,18 @@ __global__ void __launch_bounds__(W * 32, (fwd_min_blocks<DIM, C>())) synth_fwd_
     const int warp = threadIdx.x >> 5;
     WarpSmem& ws = sm.w[warp];
     warp_init_barriers(ws);
+    pdl_wait();
     const int64_t wbase = (static_cast<int64_t>(blockIdx.x) * W + warp) * (32 * C);
     if (wbase >= d.n_cells) return;
     uint32_t uses[kStages] = {};
-    const int n_chunks = d.n_pad / kWChunk;
-    const int split = blockIdx.y, n_split = gridDim.y;
+    const int n_pad = d.band != nullptr ? (d.band->nh + kChunk - 1) / kChunk * kChunk : d.n_pad;
+    const int n_chunks = n_pad / kWChunk;
+    const int split = blockIdx.y, n_split = d.band != nullptr ? d.band->n_splits : static_cast<int>(gridDim.y);
+    if (split >= n_split) return;
     const int cb = static_cast<int>(static_cast<int64_t>(n_chunks) * split / n_split);
     const int ce = static_cast<int>(static_cast<int64_t>(n_chunks) * (split + 1) / n_split);
     float2* part = n_split > 1 ? partial + static_cast<int64_t>(split) * d.n_cells : nullptr;
-    const bool ok = synth_warp_tile<DIM, C, 0, MM, NS>(d, wbase, cb, ce, part, ws, uses, status, sm.stp[warp]);
+    const bool ok = synth_warp_tile<DIM, C, 0, MM, NS>(d, n_pad, wbase, cb, ce, part, ws, uses, status, sm.stp[warp]);
     if (MM && !ok && part == nullptr && (threadIdx.x & 31) == 0)
         d.map.lpart[wbase / (32 * C)] = __longlong_as_double(0x7ff8000000000000ll);  // NaN: no loss
 }
@@ -526,7 +532,13 @@ __global__ void __launch_bounds__(W * 32, (fwd_min_blocks<DIM, C>())) synth_fwd_
 // mismatch bit every block also writes its sum of (K - T)^2 to lpart.
 __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const float2* __restrict__ partial,
                                                             int n_split) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    pdl_wait();
+    if (d.band != nullptr) {
+        n_split = d.band->n_splits;
+        if (n_split < 2) return;  // the maps are written
+    }
+    for (int64_t u = blockIdx.x; u * 256 < d.n_cells; u += gridDim.x) {
+    const int64_t i = u * 256 + threadIdx.x;
     double l = 0.0;
     if (i < d.n_cells) {
         float s = 0.0f, e = 0.0f;
@@ -535,6 +547,7 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
             two_sum_acc(s, e, v.x);
             e += v.y;
         }
+        if (d.add != nullptr) two_sum_acc(s, e, __ldg(d.add + i));
         const float y = (s + e) + d.map.mu;
         const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
         if (index_ok(o, d.n_cells)) {
@@ -551,8 +564,10 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
         if (threadIdx.x == 0) {
             double t = 0.0;
             for (int w = 0; w < 8; ++w) t += red[w];
-            d.map.lpart[blockIdx.x] = t;
+            d.map.lpart[u] = t;
         }
+        __syncthreads();
+    }
     }
 }
 
@@ -613,12 +628,12 @@ __global__ void __launch_bounds__(W * 32, C >= 16 ? 4 : 5) synth_batched_kernel(
         bool ok;
         constexpr int NSD = DIM >= 2 ? NS : 0;
         if (DIM > 1 && d.dim == 1)
-            ok = synth_warp_tile<1, C, 1>(d, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status);
+            ok = synth_warp_tile<1, C, 1>(d, d.n_pad, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status);
         else if (DIM > 2 && d.dim == 2)
             ok = synth_warp_tile<(DIM > 2 ? 2 : DIM), C, 1, false, (DIM > 2 ? NS : 0)>(
-                d, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status, sm.stp[warp]);
+                d, d.n_pad, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status, sm.stp[warp]);
         else
-            ok = synth_warp_tile<DIM, C, 1, false, NSD>(d, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status,
+            ok = synth_warp_tile<DIM, C, 1, false, NSD>(d, d.n_pad, wbase, 0, d.n_pad / kWChunk, nullptr, ws, uses, status,
                                                         sm.stp[warp]);
         if (!ok) break;
         __syncwarp();  // every lane is done with the descriptor
@@ -638,8 +653,11 @@ int choose_split(int64_t tiles, int n_chunks, int resident, int64_t n_cells, siz
     return want < 2 ? 1 : static_cast<int>(want);
 }
 
+// band: the plan's bounds of the cells, to take the band path with the
+// workspace's first cells_band_ws_bytes (null: all modes directly).
 template <int DIM, int C, int W>
-int launch_fwd_cfg(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* status, cudaStream_t st) {
+int launch_fwd_cfg(FwdDesc d, const void* table, int64_t n_modes, const SegInfo* band, void* workspace,
+                   size_t ws_bytes, int32_t* status, cudaStream_t st) {
     const size_t smem = sizeof(FwdSmem<W, lattice_ns<DIM, C>()>);
     const bool mm = (d.map.bits & kMapMismatch) != 0;
     auto kern = mm ? synth_fwd_kernel<DIM, C, W, true> : synth_fwd_kernel<DIM, C, W, false>;
@@ -649,33 +667,44 @@ int launch_fwd_cfg(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* 
     const int64_t per_cta = int64_t(W) * 32 * C;
     const int64_t grid = (d.n_cells + per_cta - 1) / per_cta;
     if (grid == 0) {
-        if (mm) {  // no cells: the loss is 0
-            loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, 0, nullptr, 0.0, d.map.loss);
-            count_launches(1);
-        }
-        return cudaGetLastError();
+        // no cells: the loss is 0
+        return mm ? launch_loss_sum(d.map.lpart, 0, nullptr, 0.0, d.map.loss, st) : cudaGetLastError();
+    }
+    unsigned char* split_ws = static_cast<unsigned char*>(workspace);
+    if (band != nullptr) {
+        const size_t used = cells_band_ws_bytes(d.n_cells, n_modes, d.dim);
+        split_ws += used;
+        ws_bytes -= used;
     }
     int n_split = 1;
-    if (workspace != nullptr) {
+    if (split_ws != nullptr) {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem);
         n_split = choose_split(grid, d.n_pad / kWChunk, sms * (per_sm > 0 ? per_sm : 1), d.n_cells, ws_bytes);
     }
-    float2* partial = static_cast<float2*>(workspace);
+    float2* partial = reinterpret_cast<float2*>(split_ws);
+    const int64_t fin_blocks = (d.n_cells + 255) / 256, tiles = (d.n_cells + 32 * C - 1) / (32 * C);
+    if (band != nullptr) {
+        const int e = launch_cells_band(table, n_modes, d, band, workspace, n_split, tiles, fin_blocks, status, st);
+        if (e != cudaSuccess) return e;
+    }
+    // a full launch: blocks that become resident while those of the previous
+    // kernel still are spread unevenly over the SMs, which the few long blocks
+    // of a small field do not make up for (250 x 130 cells: 45 -> 62 us)
     kern<<<dim3(static_cast<unsigned>(grid), n_split), W * 32, smem, st>>>(d, partial, status);
     count_launches(1);
-    const int64_t fin_blocks = (d.n_cells + 255) / 256;
-    if (n_split > 1) {
-        synth_split_finalize<<<static_cast<unsigned>(fin_blocks), 256, 0, st>>>(d, partial, n_split);
-        count_launches(1);
-    }
-    if (mm) {
-        const int64_t nb = n_split > 1 ? fin_blocks : (d.n_cells + 32 * C - 1) / (32 * C);
-        loss_sum_kernel<<<1, 256, 0, st>>>(d.map.lpart, nb, nullptr, d.map.inv_n_mean, d.map.loss);
-        count_launches(1);
-    }
+    err = cudaGetLastError();
+    if (err == cudaSuccess && n_split > 1)
+        // with the band path it may have nothing to do: a few rounds of blocks
+        err = launch_chained(synth_split_finalize,
+                             static_cast<unsigned>(d.band != nullptr ? std::min<int64_t>(fin_blocks, 4096) : fin_blocks),
+                             256, 0, st, d, partial, n_split);
+    if (err != cudaSuccess) return err;
+    if (mm)
+        return launch_loss_sum(d.map.lpart, n_split > 1 ? fin_blocks : tiles,
+                               d.band != nullptr ? &d.band->loss_nb : nullptr, d.map.inv_n_mean, d.map.loss, st);
     return cudaGetLastError();
 }
 
@@ -732,12 +761,18 @@ int launch_loss_sum(const double* part, int64_t nb, const int64_t* nb_dev, doubl
     return launch_chained(loss_sum_kernel, 1, 256, 0, static_cast<cudaStream_t>(stream), part, nb, nb_dev, inv_n, out);
 }
 
-int launch_synth_fwd(const FwdDesc& d, void* workspace, size_t ws_bytes, int32_t* status, void* stream) {
+int launch_synth_fwd(const FwdDesc& d, const void* table, int64_t n_modes, const CellsBand& band, void* workspace,
+                     size_t ws_bytes, int32_t* status, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     switch (d.dim) {
-        case 1: return launch_fwd_cfg<1, 8, 4>(d, workspace, ws_bytes, status, st);
-        case 2: return launch_fwd_cfg<2, 8, 4>(d, workspace, ws_bytes, status, st);
-        case 3: return launch_fwd_cfg<3, 16, 4>(d, workspace, ws_bytes, status, st);
+        case 1: return launch_fwd_cfg<1, 8, 4>(d, table, n_modes, nullptr, workspace, ws_bytes, status, st);
+        case 2: return launch_fwd_cfg<2, 8, 4>(d, table, n_modes, band.seg, workspace, ws_bytes, status, st);
+        // where the band path leaves few modes to sum directly, smaller tiles, of
+        // which more are resident, hide the cells' loads and stores better (128
+        // modes at 2M cells: 145 us with 16 cells per lane, 103 with 8)
+        case 3:
+            return band.few ? launch_fwd_cfg<3, 8, 4>(d, table, n_modes, band.seg, workspace, ws_bytes, status, st)
+                            : launch_fwd_cfg<3, 16, 4>(d, table, n_modes, band.seg, workspace, ws_bytes, status, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -681,6 +681,13 @@ __device__ __forceinline__ void light_prep(const BandDesc* b, const float* X, co
     }
 }
 
+struct SubTable {
+    float4* hot;
+    float4* cold;
+    int32_t* kpref;
+    const int32_t* table_kpref;
+};
+
 // Tables of a band-path call: those of the direct modes at the cells, those
 // of the light modes at the nodes, whose sizes are the device's choice, and
 // the light chunks' x weights.  `cells`, `nodes`: the host's part (table,
@@ -696,9 +703,37 @@ __device__ __forceinline__ void prep_sizes(GridPrep& p, const GridTiling& d) {
     p.scale = d.scale;
     p.xn = d.xn;
 }
+// Table of the direct modes for the kernels that take cells of any plan: the
+// records of the listed slots (in table order, so still by decreasing |a|_1),
+// zeros up to a whole chunk, and the prefix lengths of the extent buckets.
+__device__ __forceinline__ void sub_table(const BandDesc* b, const GridPrep& p, const SubTable& o) {
+    const int n = (b->nh + kChunk - 1) / kChunk * kChunk;
+    const int step = gridDim.x * blockDim.x;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += step) {
+        const int s = __ldg(p.idx + j);
+        const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        o.hot[j] = s >= 0 ? __ldg(p.hot + s) : zero;
+        o.cold[2 * j] = s >= 0 ? __ldg(p.cold + 2 * s) : zero;
+        o.cold[2 * j + 1] = s >= 0 ? __ldg(p.cold + 2 * s + 1) : zero;
+    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < kBuckets; k += step) {
+        const int before = __ldg(o.table_kpref + k);  // slots below this one; how many are listed
+        int lo = 0, hi = b->nh;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (__ldg(p.idx + mid) < before)
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        o.kpref[k] = lo;
+    }
+}
+
 __global__ void __launch_bounds__(256) band_prep_kernel(const BandDesc* b, GridPrep cells, GridPrep nodes,
-                                                        const int32_t* lstart, unsigned char* latab) {
+                                                        const int32_t* lstart, unsigned char* latab, SubTable sub) {
     pdl_wait();
+    if (sub.hot != nullptr) sub_table(b, cells, sub);
     if (b->nh > 0 && cells.atab != nullptr) {
         prep_sizes(cells, b->cells);
         grid_prep(cells);
@@ -817,6 +852,9 @@ int g_num_sms = 0;
 
 }  // namespace
 
+// Most nodes of a lattice for n cells of any plan.
+int64_t cells_band_cap(int64_t n) { return std::max<int64_t>(n, 65536); }
+
 namespace {
 
 int32_t chunks_of(int64_t n_pad) { return static_cast<int32_t>(n_pad / kGModes); }
@@ -868,6 +906,23 @@ bool band_sizes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
            grid_us_per_mode(nx, ny, nz) * double(n_pad) >= kBandMinUs;
 }
 
+// SM count and shared-memory limits of the tensor-core kernels, once.
+int grid_init() {
+    if (g_num_sms != 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto allow = [&](const void* kern, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    allow(reinterpret_cast<const void*>(grid_mma_kernel<false>), kGSmemMax);
+    allow(reinterpret_cast<const void*>(grid_mma_kernel<true>), kGSmemMax);
+    allow(reinterpret_cast<const void*>(grid_band_kernel<true>), kGBandSmem);
+    allow(reinterpret_cast<const void*>(grid_band_kernel<false>), kGBandSmem);
+    if (e == cudaSuccess) g_num_sms = sms;
+    return e;
+}
+
 // Table pointers of one synthesis at `w`.
 void set_tables(GridPrep& p, GridDesc& d, const GridPlan& g, unsigned char* w) {
     p.atab = w;
@@ -911,6 +966,7 @@ int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const 
     s.us_mode = static_cast<float>(grid_us_per_mode(gg.nx, gg.ny, gg.nz));
     s.us_node = static_cast<float>(kBandNodeUs);
     s.us_fixed = static_cast<float>(kBandFixedUs);
+    s.us_heavy = 12.0f;
     s.cap_nodes = L.cap_nodes;
     s.cap_part = L.cap_part;
     s.cap_mid = L.cap_mid;
@@ -920,7 +976,9 @@ int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const 
     s.lstart = split ? nullptr : reinterpret_cast<int32_t*>(w + L.off_lstart);
     s.max_split = gp.max_split;
     s.split_cells = split ? 1 : 0;
-    s.loss_per_tile = kGEpiWarps;
+    s.chunk = kGModes;
+    s.cap_yz = INT32_MAX;
+    s.loss_nb_tiles = d.t.n_tiles * kGEpiWarps;
     s.loss_nb_finalize = band_finalize_blocks(gg);
     s.thdr = p.thdr;
     pc.idx = s.idx_h;
@@ -942,7 +1000,7 @@ int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const 
     if (e != cudaSuccess) return e;
     int rc = launch_band_select(s, b, st);
     if (rc != cudaSuccess) return rc;
-    e = launch_chained(band_prep_kernel, g_num_sms * 5, 256, 0, st, b, pc, pn, s.lstart, latab);
+    e = launch_chained(band_prep_kernel, g_num_sms * 5, 256, 0, st, b, pc, pn, s.lstart, latab, SubTable{});
     if (e == cudaSuccess)
         e = launch_chained(grid_band_kernel<true>, g_num_sms, kGThreads, kGBandSmem, st, dn, &b->nodes, status);
     if (e != cudaSuccess) return e;
@@ -952,11 +1010,53 @@ int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const 
     e = launch_chained(split ? grid_band_kernel<true> : grid_band_kernel<false>, grid, kGThreads, kGBandSmem, st, dc,
                        &b->cells, status);
     if (e != cudaSuccess) return e;
-    rc = launch_band_finalize(b, gp.form ? mid : part, dc.part, gg, d.map, tiles, st);
+    rc = launch_band_finalize(b, gp.form ? mid : part, dc.part, gg, d.map, tiles, g_num_sms, st);
     if (rc != cudaSuccess) return rc;
     if (d.map.bits & kMapMismatch)
         return launch_loss_sum(d.map.lpart, 0, &b->loss_nb, d.map.inv_n_mean, d.map.loss, st);
     return cudaGetLastError();
+}
+
+// Workspace of a band-path call at the cells of any plan: the descriptor, the
+// modes' lists, the nodes' tables, the direct modes' table, the nodes' partial
+// sums and the light modes' sums at the cells.
+struct CellsLayout {
+    int64_t off_idx, idx, off_tab, a_bytes, y_bytes, w_bytes, b_bytes, off_hot, off_cold, off_kpref, off_part, off_add,
+        total;
+    int64_t cap_nodes, cap_part;
+    int32_t cap_mt, cap_yz;
+};
+CellsLayout cells_layout(int64_t n, int64_t n_pad, int32_t dim) {
+    CellsLayout L{};
+    const int64_t nc = n_pad / kGModes;
+    // a node costs about a fifth of a cell; axes of up to four times a cube's
+    // (2-D: a square's)
+    L.cap_nodes = cells_band_cap(n);
+    L.cap_part = std::max<int64_t>(L.cap_nodes, int64_t(1) << 22);
+    const double side = std::pow(double(L.cap_nodes), 1.0 / dim);
+    L.cap_yz = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
+    L.cap_mt = static_cast<int32_t>((L.cap_yz + kGM - 1) / kGM);
+    int64_t off = 0;
+    auto take = [&](int64_t bytes) {
+        const int64_t o = off;
+        off += align256(bytes);
+        return o;
+    };
+    take(sizeof(BandDesc));
+    L.idx = align256((n_pad + 128) * 4);
+    L.off_idx = take(2 * L.idx);
+    L.a_bytes = align256(int64_t(L.cap_mt) * nc * kGPair);
+    L.y_bytes = dim > 2 ? align256(nc * L.cap_yz * kGRowBytes) : 0;
+    L.w_bytes = L.y_bytes;
+    L.b_bytes = dim > 2 ? 0 : align256((L.cap_yz + kGN - 1) / kGN * nc * kGPair);
+    L.off_tab = take(L.a_bytes + L.y_bytes + L.w_bytes + L.b_bytes);
+    L.off_hot = take((n_pad + kChunk) * 16);
+    L.off_cold = take((n_pad + kChunk) * 32);
+    L.off_kpref = take(kBuckets * 4);
+    L.off_part = take(L.cap_part * 4);
+    L.off_add = take(n * 4);
+    L.total = off;
+    return L;
 }
 
 }  // namespace
@@ -974,6 +1074,91 @@ double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
     return g.max_split > 1 ? double(g.n_tiles) * tile / 42.0e6 : std::ceil(double(g.n_tiles) / 152.0) * 152.0 * tile / 65.0e6;
 }
 
+// CUDA-core kernels: 4.2 Tcell.mode/s at the cells of any plan (one hardware
+// cosine each), half of it at 30 000 cells, whose tiles leave SMs idle.  The lattice's interpolation: 50 ps per cell in 3-D, 10 in 2-D.
+double cells_us_per_mode(int64_t n_cells) { return 0.006 + double(n_cells) / 4.2e6; }
+double cells_band_us(int64_t n_cells, int32_t dim) { return 20.0 + double(n_cells) * (dim > 2 ? 5e-5 : 1e-5); }
+
+size_t cells_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim) {
+    const int64_t n_pad = pad_modes(n_modes);
+    if (dim < 2 || n_pad > band::kMaxModes || cells_us_per_mode(n_cells) * double(n_pad) < kBandMinUs) return 0;
+    return static_cast<size_t>(cells_layout(n_cells, n_pad, dim).total);
+}
+
+int launch_cells_band(const void* table, int64_t n_modes, FwdDesc& fd, const SegInfo* seg, void* ws,
+                      int32_t max_split, int64_t loss_tiles, int64_t loss_finalize, int32_t* status, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (const int e = grid_init()) return e;
+    const TableLayout TL = table_layout(n_modes);
+    const unsigned char* tb = static_cast<const unsigned char*>(table);
+    unsigned char* w = static_cast<unsigned char*>(ws);
+    const CellsLayout L = cells_layout(fd.n_cells, TL.n_pad, fd.dim);
+    BandDesc* b = reinterpret_cast<BandDesc*>(w);
+    float* part = reinterpret_cast<float*>(w + L.off_part);
+    float* add = reinterpret_cast<float*>(w + L.off_add);
+    GridPrep pc{};
+    pc.thdr = reinterpret_cast<const TableHeader*>(tb);
+    pc.hot = fd.hot;
+    pc.cold = fd.cold;
+    pc.idx = reinterpret_cast<int32_t*>(w + L.off_idx);
+    pc.dim = fd.dim;
+    GridPrep pn = pc;
+    pn.idx = reinterpret_cast<int32_t*>(w + L.off_idx + L.idx);
+    GridPlan gn{};
+    gn.form = fd.dim > 2;
+    gn.a_bytes = L.a_bytes;
+    gn.y_bytes = L.y_bytes;
+    GridDesc dn{};
+    set_tables(pn, dn, gn, w + L.off_tab);
+    dn.thdr = pc.thdr;
+    dn.part = part;
+    dn.quiet = 1;
+    BandSelect s{};
+    s.hot = fd.hot;
+    s.cold = fd.cold;
+    s.thdr = pc.thdr;
+    s.n_modes = static_cast<int32_t>(n_modes);
+    s.dim = fd.dim;
+    s.idx_h = const_cast<int32_t*>(pc.idx);
+    s.idx_l = const_cast<int32_t*>(pn.idx);
+    s.seg = seg;
+    s.status = status;
+    s.us_mode = static_cast<float>(cells_us_per_mode(fd.n_cells));
+    s.us_node = static_cast<float>(kBandNodeUs);
+    s.us_fixed = static_cast<float>(cells_band_us(fd.n_cells, fd.dim));
+    s.us_heavy = 5.0f;
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_part;
+    s.cap_mt = L.cap_mt;
+    s.cap_yz = L.cap_yz;
+    s.fold = 1;  // as exact as the direct sum (3.0e-7 of sigma); 2 would save 9 of 370 us and give 3.0e-7 to 3.1e-7
+    s.chunk = kChunk;
+    s.max_split = max_split;
+    s.loss_nb_tiles = loss_tiles;
+    s.loss_nb_finalize = loss_finalize;
+    SubTable sub;
+    sub.hot = reinterpret_cast<float4*>(w + L.off_hot);
+    sub.cold = reinterpret_cast<float4*>(w + L.off_cold);
+    sub.kpref = reinterpret_cast<int32_t*>(w + L.off_kpref);
+    sub.table_kpref = fd.kpref;
+    int rc = launch_band_select(s, b, st);
+    if (rc != cudaSuccess) return rc;
+    cudaError_t e = launch_chained(band_prep_kernel, g_num_sms * 5, 256, 0, st, b, pc, pn, nullptr, nullptr, sub);
+    if (e == cudaSuccess)
+        e = launch_chained(grid_band_kernel<true>, g_num_sms, kGThreads, kGBandSmem, st, dn, &b->nodes, status);
+    if (e != cudaSuccess) return e;
+    rc = launch_band_lines(b, part, GridGeom{}, nullptr, nullptr, g_num_sms, st);
+    if (rc != cudaSuccess) return rc;
+    rc = launch_band_cells(b, part, fd.dim, fd.xs, fd.ys, fd.zs, fd.n_cells, add, st);
+    if (rc != cudaSuccess) return rc;
+    fd.hot = sub.hot;
+    fd.cold = sub.cold;
+    fd.kpref = sub.kpref;
+    fd.band = b;
+    fd.add = add;
+    return cudaSuccess;
+}
+
 size_t grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
     if (!band_sizes(nx, ny, nz, n_pad)) return 0;
     const GridGeom gg{nx, ny, nz, nullptr, nullptr, nullptr, nullptr};
@@ -985,20 +1170,7 @@ int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const Gri
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const unsigned char* tb = static_cast<const unsigned char*>(table);
     const TableLayout TL = table_layout(n_modes);
-    if (g_num_sms == 0) {
-        int dev = 0, sms = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        auto allow = [&](const void* kern, int bytes) {
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        };
-        allow(reinterpret_cast<const void*>(grid_mma_kernel<false>), kGSmemMax);
-        allow(reinterpret_cast<const void*>(grid_mma_kernel<true>), kGSmemMax);
-        allow(reinterpret_cast<const void*>(grid_band_kernel<true>), kGBandSmem);
-        allow(reinterpret_cast<const void*>(grid_band_kernel<false>), kGBandSmem);
-        if (e != cudaSuccess) return e;
-        g_num_sms = sms;
-    }
+    if (const int e = grid_init()) return e;
     const GridPlan gp = grid_plan(gg.nx, gg.ny, gg.nz, chunks_of(TL.n_pad));
     unsigned char* w = static_cast<unsigned char*>(ws);
     GridPrep p{};

@@ -445,11 +445,13 @@ def _outputs_struct(out):
 
 
 def synth_workspace_bytes(plan: CellPlan, segment, n_modes):
-    """Workspace that lets grf_synth_field use the mode split and, on a
-    Cartesian-grid plan, the tensor-core grid path (the larger of
-    grf_synth_workspace_bytes and grf_synth_grid_workspace_bytes)."""
-    return max(int(lib().grf_synth_workspace_bytes(plan.segment_size(segment))),
-               int(lib().grf_synth_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes))))
+    """Workspace that lets grf_synth_field use the mode split, the node lattice
+    of low-frequency modes and, on a Cartesian-grid plan, the tensor-core grid
+    path (the largest of grf_synth_workspace_bytes,
+    grf_synth_band_workspace_bytes and grf_synth_grid_workspace_bytes)."""
+    grid = int(lib().grf_synth_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
+    cells = 0 if grid else int(lib().grf_synth_band_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
+    return max(int(lib().grf_synth_workspace_bytes(plan.segment_size(segment))), cells, grid)
 
 
 def synth_mismatch_workspace_bytes(plan: CellPlan, segment, n_modes):

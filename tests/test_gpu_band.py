@@ -135,3 +135,101 @@ def test_band_grid_fused_mismatch(env):
         assert loss.item() == pytest.approx(loss_u.item(), rel=1e-12)
         again = F.synth(table, p, plan, maps=F.MapSpec(y=True))["Y"]
         assert torch.equal(again, ref["Y"])  # deterministic
+
+
+# ---------------------------------------------------------------------------
+# Cells of any plan
+# ---------------------------------------------------------------------------
+def _cloud(kind, n, dim, seed):
+    """Cell centres: "lattice" (jittered), "even" (independent uniform),
+    "clusters" (dense blobs far apart: groups that spread over many nodes)."""
+    rng = np.random.default_rng(seed)
+    if kind == "lattice":
+        side = int(round(n ** (1.0 / dim)))
+        grid = np.stack(np.meshgrid(*[np.arange(side)] * dim, indexing="ij"), -1).reshape(-1, dim)
+        c = (grid + 0.5 + rng.uniform(-0.4, 0.4, grid.shape)) / side
+    elif kind == "even":
+        c = rng.random((n, dim))
+    else:
+        centre = rng.random((40, dim)) * 3.0 - 1.0
+        c = centre[rng.integers(0, 40, n)] + 0.004 * rng.standard_normal((n, dim))
+    return [np.ascontiguousarray(c[:, k].astype(np.float32)) for k in range(dim)]
+
+
+def _check_cells(env, cells, ell, n, law, segments=None, segment=0, seed=6, maps=None):
+    torch, F, W = env
+    dim = len(ell)
+    plan = F.CellPlan(*to_dev(torch, cells), segments=segments)
+    m = _modes(n, dim, ell, law, seed)
+    table = F.ModeTable(m["amp"], m["psi"], m["a"])
+    l0 = F.launch_count()
+    out = F.synth(table, _params(F, n, dim, ell), plan, segment, F.MapSpec(y=True, lognormal=True))
+    torch.cuda.synchronize()
+    launches = F.launch_count() - l0
+    o0 = int(plan.offsets[segment])
+    count = plan.segment_size(segment)
+    idx = np.unique(np.concatenate([np.random.default_rng(1).choice(count, 6000), np.arange(300),
+                                    np.arange(count - 300, count)]))
+    y_or = oracle_field(m, 0.25, [c[:] for c in cells[:dim]], o0 + idx)
+    check_forward(out["Y"].cpu().numpy()[idx], y_or, 1.0, "cells %d" % count)
+    check_lognormal(out["K"].cpu().numpy()[idx], y_or, 1.0)
+    return launches, plan
+
+
+@pytest.mark.parametrize("kind,cells,dim,n,law", [
+    ("lattice", 300_000, 2, 4000, "gaussian"), ("lattice", 300_001, 2, 4100, "rough"),
+    ("even", 150_333, 3, 4000, "gaussian"), ("lattice", 262_144, 3, 5003, "rough"),
+    ("clusters", 400_000, 3, 3000, "gaussian"), ("clusters", 300_000, 2, 4000, "rough"),
+])
+def test_band_cells_against_oracle(env, kind, cells, dim, n, law):
+    launches, plan = _check_cells(env, _cloud(kind, cells, dim, 3), (0.2, 0.25, 0.2)[:dim], n, law)
+    assert launches >= 6 and plan.status() == 0
+
+
+def test_band_cells_segments_and_lower_dimension(env):
+    # the second of three segments, and a 2-D field on the cells of a 3-D plan
+    torch, F, W = env
+    parts = [_cloud("even", k, 3, 10 + k % 7) for k in (1000, 600_000, 37)]
+    cells = [np.concatenate([p[c] for p in parts]) for c in range(3)]
+    launches, _ = _check_cells(env, cells, (0.2, 0.2, 0.2), 6000, "gaussian", segments=[1000, 600_000, 37], segment=1)
+    assert launches >= 6
+    launches, _ = _check_cells(env, cells, (0.2, 0.2), 6000, "gaussian")
+    assert launches >= 6
+
+
+def test_band_cells_not_finite(env):
+    # a cell that is not finite: the plan says so, the path stays with the
+    # direct sum and every other cell keeps its value
+    torch, F, W = env
+    for bad in (np.nan, np.inf):
+        cells = _cloud("even", 200_000, 3, 4)
+        cells[1][77] = bad
+        plan = F.CellPlan(*to_dev(torch, cells))
+        m = _modes(4000, 3, (0.2, 0.2, 0.2), "gaussian", 2)
+        y = F.synth(F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, 4000, 3, (0.2, 0.2, 0.2)), plan)["Y"]
+        torch.cuda.synchronize()
+        assert plan.status() == 1
+        idx = np.setdiff1d(np.random.default_rng(1).choice(200_000, 4000), [77])
+        check_forward(y.cpu().numpy()[idx], oracle_field(m, 0.25, cells, idx), 1.0, "beside a cell at %s" % bad)
+
+
+def test_band_cells_fused_mismatch_and_workspace(env):
+    # the fused loss and gradient are those of the synthesis; without room for
+    # the lattice (workspace=False) all modes are summed at the cells
+    torch, F, W = env
+    for law, n in (("gaussian", 4000), ("rough", 6000)):
+        cells = _cloud("lattice", 262_144, 3, 3)
+        plan = F.CellPlan(*to_dev(torch, cells))
+        m = _modes(n, 3, (0.2, 0.2, 0.2), law, 4)
+        table = F.ModeTable(m["amp"], m["psi"], m["a"])
+        p = _params(F, n, 3, (0.2, 0.2, 0.2))
+        ref = F.synth(table, p, plan, maps=F.MapSpec(y=True, lognormal=True))
+        T = torch.full_like(ref["K"], 1.5)
+        loss_u, gY_u = F.mismatch_grad(ref["K"], T)
+        loss, gY, out = F.synth_mismatch(table, p, plan, T, want_Y=True)
+        direct = F.synth(table, p, plan, workspace=False)["Y"]
+        torch.cuda.synchronize()
+        assert torch.equal(out["Y"], ref["Y"]) and torch.equal(gY, gY_u)
+        assert loss.item() == pytest.approx(loss_u.item(), rel=1e-12)
+        assert not torch.equal(direct, ref["Y"])
+        assert (direct - ref["Y"]).abs().max().item() <= 2e-5
