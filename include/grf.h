@@ -444,6 +444,15 @@ size_t grf_backward_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t di
 size_t grf_backward_grid_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes);
 
 /*
+ * grf_backward_band_workspace_bytes -- workspace bytes that let
+ * grf_synth_backward carry dL/dY to a coarse lattice of nodes for the modes of
+ * low frequency, at the cells of any plan; 0 at sizes where all modes are
+ * summed at the cells.  grf_backward_grid_workspace_bytes() includes the
+ * lattice's part on grid plans.
+ */
+size_t grf_backward_band_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
+
+/*
  * grf_synth_backward -- gradients of a loss L with respect to the mode
  * amplitudes, phases and frequencies, the mean, sigma and the correlation
  * lengths, given gY = dL/dY (device float32, original cell order, cells of
@@ -673,8 +682,8 @@ int grf_take_grid_adjoint_units(int64_t *units);
 /*
  * grf_debug_grid_path -- process-wide setting of the grid path (enable = 0:
  * grid plans take the CUDA-core paths, for comparisons; 1, the default, and
- * 2: every grid plan takes the grid path, forward and adjoint; grids of at
- * most 64 tiles of 128 x 128 cells split each tile's modes over several
+ * 2: every grid plan takes the grid path, forward and adjoint, with all
+ * modes as products (no node lattice); grids of at most 64 tiles of 128 x 128 cells split each tile's modes over several
  * CTAs) and the number of
  * 32-mode chunks the tensor-core accumulator sums before each fold into the
  * running sum (fold_chunks = 1, 2, 4 or 8, lowered to a divisor of the

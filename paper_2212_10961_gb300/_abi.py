@@ -109,6 +109,7 @@ _SIGS = {
                                        ctypes.c_void_p]),
     "grf_synth_workspace_bytes": (ctypes.c_size_t, [ctypes.c_int64]),
     "grf_synth_grid_workspace_bytes": (ctypes.c_size_t, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64]),
+    "grf_backward_band_workspace_bytes": (ctypes.c_size_t, [ctypes.c_int64, ctypes.c_int64, ctypes.c_int32]),
     "grf_synth_band_workspace_bytes": (ctypes.c_size_t, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64]),
     "grf_plan_grid_shape": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32),
                                            ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),

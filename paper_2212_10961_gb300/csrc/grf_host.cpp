@@ -272,7 +272,7 @@ constexpr int kGridSlots = 1024;
 GridCheck* g_slots = nullptr;
 int g_next_slot = 0;
 std::atomic<uint64_t> g_next_tag{1};
-std::atomic<int32_t> g_grid_enabled{1};  // grf_debug_grid_path: 0 off, 1 auto, 2 always
+std::atomic<int32_t> g_grid_enabled{1};  // grf_debug_grid_path: 0 off, 1 auto, 2 always, no node lattice on grids
 std::atomic<int32_t> g_grid_fold{4};     // chunks of 32 modes per fold interval
 
 void drop_plan_event(PlanMeta& m) {
@@ -424,6 +424,7 @@ double band_worth(const grf_params* p, const float* box, const int32_t* n, doubl
 
 // The same for a call on a Cartesian grid, with the workspace it has.
 bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t ws_bytes) {
+    if (g_grid_enabled.load() == 2) return false;
     const int64_t n_pad = table_layout(p->n_modes).n_pad;
     const size_t extra = grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
     if (extra == 0 || ws_bytes < grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra) return false;
@@ -1115,13 +1116,20 @@ size_t grf_backward_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t di
     return bwd_workspace_bytes(n_cells, n_modes, dim);
 }
 
+size_t grf_backward_band_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t dim) {
+    if (n_modes < 1 || n_modes > GRF_MAX_MODES || dim < 1 || dim > 3 || n_cells < 0) return 0;
+    const size_t band = cells_adjoint_band_ws_bytes(n_cells, n_modes, dim);
+    return band > 0 ? band + bwd_workspace_bytes(n_cells, n_modes, dim) : 0;
+}
+
 size_t grf_backward_grid_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
     try {
         if (!plan || segment != 0 || n_modes < 1 || n_modes > GRF_MAX_MODES) return 0;
         GridGeom gg{};
         if (!plan_grid(plan, &gg)) return 0;
-        const size_t b = bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(n_modes).n_pad);
-        return grid_ws_ok(b, gg) ? b : 0;
+        const int64_t n_pad = table_layout(n_modes).n_pad;
+        const size_t b = bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+        return grid_ws_ok(b, gg) ? b + bwd_grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
     } catch (...) {
         return 0;
     }
@@ -1157,22 +1165,39 @@ int grf_synth_backward(const void* table, const grf_params* p, const void* plan,
     // Cartesian grid handed over x-fastest: the tensor-core adjoint when the
     // workspace holds its tables
     GridGeom gg{};
-    if (n > 0 && g_grid_enabled.load() != 0 && meta.offsets.size() == 2 && p->dim >= 2 && plan_grid(plan, &gg) &&
-        use_grid_path(gg) && grid_ws_ok(bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
-        ws_bytes >= bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad)) {
+    float box[6] = {NAN, NAN, NAN, NAN, NAN, NAN};
+    const int64_t n_pad = table_layout(p->n_modes).n_pad;
+    if (n > 0 && g_grid_enabled.load() != 0 && meta.offsets.size() == 2 && p->dim >= 2 && plan_grid(plan, &gg, box) &&
+        use_grid_path(gg) && grid_ws_ok(bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad), gg) &&
+        ws_bytes >= bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad)) {
+        const size_t extra = bwd_grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+        const int32_t cells[3] = {gg.nx, gg.ny, gg.nz};
+        const bool band =
+            extra > 0 && g_grid_enabled.load() != 2 && ws_bytes >= bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra &&
+            band_worth(p, box, cells, 0.25 * static_cast<double>(n), grid_adjoint_us_per_mode(gg.nx, gg.ny, gg.nz),
+                       kBandNodeAdjUs, grid_adjoint_band_us(gg.nx, gg.ny, gg.nz) + kBandTryUs) >= 0.0;
         const int err = launch_synth_bwd_grid(table, p->n_modes, p->dim, gg, gY, std::sqrt(p->sigma2), p->ell, rot,
-                                              periodic, *g, workspace, status, stream);
+                                              periodic, *g, workspace, band, status, stream);
         if (err != cudaSuccess) return cuda_fail(err, "grid backward kernels");
         return GRF_OK;
     }
     const size_t need = bwd_workspace_bytes(n, p->n_modes, p->dim);
     if (ws_bytes < need) return fail(GRF_EWORKSPACE, "backward workspace %zu < %zu bytes", ws_bytes, need);
+    const size_t extra = cells_adjoint_band_ws_bytes(n, p->n_modes, p->dim);
+    const SegInfo* band = nullptr;
+    if (extra > 0 && ws_bytes >= need + extra && g_grid_enabled.load() != 0) {
+        const double us = cells_adjoint_us_per_mode(n);
+        if (std::isfinite(box[0]) ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), us, kBandNodeAdjUs,
+                                               cells_adjoint_band_us(n, p->dim) + kBandTryUs) >= 0.0
+                                  : us * static_cast<double>(p->n_modes) >= 500.0)
+            band = reinterpret_cast<const SegInfo*>(pb + meta.layout.off_segs) + segment;
+    }
     const int err = launch_synth_bwd(
         table, p->n_modes, p->dim, std::sqrt(p->sigma2), p->ell, rot, periodic,
         reinterpret_cast<const float*>(pb + meta.layout.off_xs) + begin,
         reinterpret_cast<const float*>(pb + meta.layout.off_ys) + begin,
         reinterpret_cast<const float*>(pb + meta.layout.off_zs) + begin,
-        reinterpret_cast<const int32_t*>(pb + meta.layout.off_perm) + begin, begin, n, gY, *g,
+        reinterpret_cast<const int32_t*>(pb + meta.layout.off_perm) + begin, begin, n, gY, *g, band,
         workspace, status, stream);
     if (err != cudaSuccess) return cuda_fail(err, "backward kernels");
     return GRF_OK;

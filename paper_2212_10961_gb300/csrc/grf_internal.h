@@ -358,6 +358,74 @@ struct BandSelect {
     GridTiling cells;        // the cells' tiling (all modes)
 };
 
+// Adjoint on the band path (band_bwd.cu): one axis of a grid's transposed
+// interpolation, the phasor tables at the nodes, and the split of the sums.
+struct BandAxisTab {
+    float* w;        // [cells][8] weights
+    int32_t* start;  // [cells] first node
+    int2* range;     // [nodes] first and last cell of a node
+    float* wt;       // [cells of a node][nodes] the same weights by node, from the node's first cell
+    int32_t* most;   // most cells of a node, or 0 where wt does not hold them (axes in no order)
+};
+// Floats of BandAxisTab::wt: a node of an axis in order has about 8 cells /
+// nodes cells.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int64_t band_wt_floats(int64_t cells) { return 16 * cells + 1024; }
+struct BandPhasors {
+    float2* ph[3];   // [nodes][light modes padded to 128]
+    float* off[3];   // [nodes] coordinate from the axis's first node
+    double* gain;    // [4][light modes padded to 128]: the window's gain, and per axis
+                     // (d ln gain / d a_c) / (2 pi)
+    int32_t* rank;   // [table slots] light mode of the slot, or ~ direct mode
+};
+struct BandNodes {
+    int32_t n_mt, n_xc, groups;  // mode tiles, x chunks, groups of lines
+};
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline BandNodes band_nodes_split(int32_t n_light, int32_t mx, int32_t lines, int32_t blocks) {
+    BandNodes s;
+    s.n_mt = (n_light + 127) / 128;
+    s.n_xc = (mx + 63) / 64;
+    const int32_t batches = (lines + 15) / 16, want = blocks / (s.n_mt * s.n_xc);
+    s.groups = want < 1 ? 1 : want > batches ? batches : want;
+    return s;
+}
+// Groups of a grid adjoint's units: one CTA per SM (mode tiles x groups <=
+// SMs), at most kAdjMaxCtas of them.
+constexpr int kAdjMaxCtas = 256;
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int32_t grid_adjoint_groups(int32_t n_mt, int64_t units, int32_t sms) {
+    int64_t g = n_mt > 0 ? sms / n_mt : 1;
+    if (g > units) g = units;
+    const int64_t room = n_mt > 0 && kAdjMaxCtas / n_mt > 1 ? kAdjMaxCtas / n_mt : 1;
+    if (g > room) g = room;
+    return g < 1 ? 1 : static_cast<int32_t>(g);
+}
+// Splits of the cells of band_direct_kernel (blocks for each tile of 128 modes).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int32_t band_direct_splits(int32_t nh, int32_t blocks) {
+    const int32_t tiles = (nh + 127) / 128;
+    return tiles < 1 ? 1 : blocks / tiles > 1 ? blocks / tiles : 1;
+}
+// The band path's part of the adjoint's reduction (null: all modes from part).
+struct BandReduce {
+    const BandDesc* b;
+    const int32_t* rank;
+    const double* gain;
+    const double* part;    // light modes' sums over the nodes
+    int32_t blocks;        // as in band_nodes_split
+    int32_t direct_units;  // > 0: direct sums of the grid adjoint (units, SMs);
+    int32_t direct_sms;    // 0: of band_direct_kernel (its blocks)
+};
+
 // Work tile of the batched launch: realisation r, tile index t inside it.
 struct WorkItem {
     int32_t r;
@@ -418,13 +486,15 @@ int launch_bimap(const grf_bimap& m, int64_t n, const float* Y1, const float* Y2
 // tag: host-assigned plan number, stored with the grid check (GridCheck::tag)
 int launch_plan(int32_t dim, int32_t n_segments, const int64_t* seg_offsets_host, const float* x,
                 const float* y, const float* z, void* plan, const PlanLayout& L, uint64_t tag, void* stream);
+// band: the segment's bounds, to take the band path, whose workspace
+// (cells_adjoint_band_ws_bytes) follows bwd_workspace_bytes; null: all modes directly.
 // periodic_mask: bit c set when axis c is periodic (its frequency is rounded,
 // so its dL/da reaches neither kappa, l nor R).
 int launch_synth_bwd(const void* table, int64_t n_modes, int32_t dim, double sigma,
                      const double* ell, const double* rot, int32_t periodic_mask, const float* xs,
                      const float* ys, const float* zs,
                      const int32_t* perm, int64_t perm_base, int64_t n_cells, const float* gY,
-                     const grf_grads& g, void* workspace, int32_t* status, void* stream);
+                     const grf_grads& g, const SegInfo* band, void* workspace, int32_t* status, void* stream);
 size_t bwd_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
 // Per-mode terms of the scalar gradients the adjoint's reduction writes
 // (contrib rows: (A / sigma) dA, three l terms, nine R terms).
@@ -435,14 +505,41 @@ constexpr int kBwdContrib = 13;
 // partial sums of g, contrib: kBwdContrib x n_pad doubles of scratch.
 int launch_bwd_reduce(const void* table, int64_t n_modes, int32_t dim, double sigma, const double* ell,
                       const double* rot, int32_t periodic_mask, const grf_grads& g, double* part, int32_t splits,
-                      double* gpart, int32_t n_gpart, double* contrib, void* stream);
+                      double* gpart, int32_t n_gpart, double* contrib, const BandReduce& band, void* stream);
 // Tensor-core adjoint on a Cartesian grid in x-fastest order (synth_grid_bwd.cu):
 // workspace bytes, the launch (scan, prep, tensor-core kernel, reduction) and
 // the units computed since the last call (synchronous).
 size_t bwd_grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
 int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const GridGeom& gg, const float* gY,
                           double sigma, const double* ell, const double* rot, int32_t periodic_mask,
-                          const grf_grads& g, void* ws, int32_t* status, void* stream);
+                          const grf_grads& g, void* ws, bool band, int32_t* status, void* stream);
+// band: the band path, whose workspace (bwd_grid_band_ws_bytes) follows.
+size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
+double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
+// Measured times of the adjoint's band path (us): one mode at one node, and the
+// kernels that the lattice adds.
+constexpr double kBandNodeAdjUs = 1.0 / 6.0e6;
+double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz);
+size_t cells_adjoint_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
+double cells_adjoint_us_per_mode(int64_t n_cells);
+double cells_adjoint_band_us(int64_t n_cells, int32_t dim);
+// max |g| (inf if some g is not finite) and compensated sums of g, per block of
+// a fixed partition of n values into adj_scan_blocks().
+int launch_adj_scan(const float* g, int64_t n, const float* X, int32_t nx, float* gmax, double* gsum, float* xmax,
+                    void* stream);
+int adj_scan_blocks();
+// Kernels of band_bwd.cu.
+int launch_band_grid_spread(const BandDesc* b, const GridGeom& gg, const float* g, const BandAxisTab* tab, float* h1,
+                            float* h2, float* nodes, int sms, void* stream);
+int launch_band_spread(const BandDesc* b, int32_t dim, const float* xs, const float* ys, const float* zs,
+                       const int32_t* perm, int64_t perm_base, int64_t n, const float* g, const float* gmax,
+                       int n_gmax, unsigned long long* lattice, float* nodes, int sms, void* stream);
+int launch_band_direct(const BandDesc* b, int32_t dim, const float4* cold, const int32_t* idx, const float* xs,
+                       const float* ys, const float* zs, const int32_t* perm, int64_t perm_base, int64_t n,
+                       const float* g, double* part, int blocks, void* stream);
+int launch_band_nodes(const BandDesc* b, const float4* cold, const int32_t* idx_l, const int32_t* idx_h,
+                      const GridGeom& gg, int32_t dim, const float* nodes, const BandPhasors& t, double* part, int sms,
+                      void* stream);
 int take_grid_adj_units(unsigned long long* units);
 int launch_mismatch(int64_t n, const float* K, const float* T, float* gY, double* loss, void* ws,
                     void* stream);

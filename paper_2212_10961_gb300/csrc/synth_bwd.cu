@@ -25,7 +25,12 @@
 // gradients (sigma, l, mu) in a fixed order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
+#include "band.cuh"
 #include "device_common.cuh"
+#include "launch.cuh"
 
 namespace grf {
 
@@ -81,6 +86,7 @@ struct BwdArgs {
     double inv_sigma;
     double inv_ell[3];
     double inv_2pi_ell[3];
+    BandReduce band;  // band.b null: all modes from part
     grf_grads g;
 };
 
@@ -495,12 +501,37 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
     __shared__ double red[kRedWarps][32][5];
     __shared__ double cts[kContrib][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_wait();
     const int m = blockIdx.x * 32 + lane;  // n_pad is a multiple of 128
+    // this slot's partial sums: rows of `stride` per split; on the band path of
+    // the direct or of the light modes
+    const double* part = args.part + static_cast<int64_t>(m) * 5;
+    int64_t stride = static_cast<int64_t>(args.n_pad) * 5;
+    int splits = args.splits;
+    bool light = false;
+    if (args.band.b != nullptr) {
+        const BandDesc& b = *args.band.b;
+        const int r = m < args.n_modes ? __ldg(args.band.rank + m) : 0;
+        light = m < args.n_modes && r >= 0;
+        if (light) {
+            const BandNodes S = band_nodes_split(b.n_light, b.ax[0].m, b.ax[1].m * b.ax[2].m, args.band.blocks);
+            part = args.band.part + static_cast<int64_t>(r) * 5;
+            stride = static_cast<int64_t>(S.n_mt) * 128 * 5;
+            splits = S.n_xc * S.groups;
+        } else {
+            const int tiles = (b.nh + 127) / 128;
+            part = args.part + static_cast<int64_t>(~r) * 5;
+            stride = static_cast<int64_t>(tiles) * 128 * 5;
+            splits = m >= args.n_modes            ? 0
+                     : args.band.direct_units > 0 ? grid_adjoint_groups(tiles, args.band.direct_units, args.band.direct_sms)
+                                                  : band_direct_splits(b.nh, args.band.direct_sms);
+        }
+    }
     {
         double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
-        for (int s = warp; s < args.splits; s += kRedWarps) {
-            const double* p = args.part + (static_cast<int64_t>(s) * args.n_pad + m) * 5;
+        for (int s = warp; s < splits; s += kRedWarps) {
+            const double* p = part + s * stride;
 #pragma unroll
             for (int q = 0; q < 5; ++q) v[q] += p[q];
         }
@@ -525,6 +556,17 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
             const double a[3] = {static_cast<double>(q0.x) + static_cast<double>(q0.y),
                                  static_cast<double>(q0.z) + static_cast<double>(q0.w),
                                  static_cast<double>(q1.x) + static_cast<double>(q1.y)};
+            if (light) {
+                // from the nodes' sums to the cells': the window's gain, and its
+                // slope where the frequency is differentiated (band_bwd.cu)
+                const int r = __ldg(args.band.rank + m);
+                const int64_t np = (args.band.b->n_light + 127) / 128 * 128;
+                const double gain = args.band.gain[r];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) v[q] *= gain;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) v[2 + c] -= args.band.gain[(1 + c) * np + r] * v[0];
+            }
             const double gs = args.g.gscale != nullptr ? *args.g.gscale : 1.0;
             // the table holds the mode as (-A, psi + 1/2) at odd positions, where the
             // cosine sum v[0] has the opposite sign; A * v[1] and A * v[2..] do not
@@ -580,6 +622,7 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
 constexpr int kScalarRows = kContrib + 1;  // + the sum of g (dmu)
 
 __global__ void __launch_bounds__(32 * kScalarRows) bwd_scalar_kernel(BwdArgs args, int32_t n_blocks) {
+    pdl_wait();
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     double t = 0.0;
     if (q < kContrib) {
@@ -711,10 +754,69 @@ void bwd_common_args(BwdArgs& a, const void* table, int64_t n_modes, int32_t dim
 
 }  // namespace
 
+namespace {
+int launch_reduce(const BwdArgs& a, cudaStream_t st) {
+    cudaError_t e = launch_chained(bwd_reduce_kernel, static_cast<unsigned>(a.n_pad / 32), 32 * kRedWarps, 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(bwd_scalar_kernel, 1, 32 * kScalarRows, 0, st, a, a.n_pad / 32);
+    return e;
+}
+
+// Workspace of the band path after the CUDA-core adjoint's own: the
+// descriptor, the modes' lists, ranks and gains, the scan's partials, the
+// fixed-point lattice and its values, the phasor tables and
+// the partial sums over the nodes.
+struct CellsAdjLayout {
+    int64_t off_idx, idx, off_rank, off_gmax, off_gsum, off_xmax, off_gain, off_fixed, off_nodes,
+        off_ph[3], off_off[3], off_part, total;
+    int64_t cap_nodes;
+    int32_t cap_yz;
+};
+CellsAdjLayout cells_adj_layout(int64_t n, int64_t n_pad, int32_t dim) {
+    CellsAdjLayout L{};
+    L.cap_nodes = std::max<int64_t>(n, 65536);
+    const double side = std::pow(double(L.cap_nodes), 1.0 / dim);
+    L.cap_yz = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
+    int64_t off = 0;
+    auto take = [&](int64_t bytes) {
+        const int64_t o = off;
+        off += align256(bytes);
+        return o;
+    };
+    take(sizeof(BandDesc));
+    L.idx = align256((n_pad + 128) * 4);
+    L.off_idx = take(2 * L.idx);
+    L.off_rank = take(n_pad * 4);
+    L.off_gmax = take(adj_scan_blocks() * 4);
+    L.off_xmax = take(adj_scan_blocks() * 4);
+    L.off_gsum = take(adj_scan_blocks() * 8);
+    L.off_gain = take(4 * n_pad * 8);
+    L.off_fixed = take(L.cap_nodes * 8);
+    L.off_nodes = take(L.cap_nodes * 4);
+    for (int c = 0; c < 3; ++c) {
+        const int64_t m = c < dim ? L.cap_yz : 1;
+        L.off_ph[c] = take(m * n_pad * 8);
+        L.off_off[c] = take(m * 4);
+    }
+    const int64_t tiles = n_pad / 128 * ((int64_t(L.cap_yz) + 63) / 64);
+    L.off_part = take(std::max<int64_t>(256 * 3, tiles) * 128 * 5 * 8);
+    L.total = off;
+    return L;
+}
+}  // namespace
+
+// The direct modes' rate (exact phases, a hardware sine and cosine per pair);
+// the lattice's spread 0.11 ns per cell in 3-D.
+double cells_adjoint_us_per_mode(int64_t n_cells) { return 0.01 + double(n_cells) / 1.0e6; }
+double cells_adjoint_band_us(int64_t n_cells, int32_t dim) { return 30.0 + double(n_cells) * (dim > 2 ? 1.1e-4 : 3e-5); }
+size_t cells_adjoint_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim) {
+    const int64_t n_pad = pad_modes(n_modes);
+    if (dim < 2 || n_pad > band::kMaxModes || cells_adjoint_us_per_mode(n_cells) * double(n_pad) < 60.0) return 0;
+    return static_cast<size_t>(cells_adj_layout(n_cells, n_pad, dim).total);
+}
+
 int launch_bwd_reduce(const void* table, int64_t n_modes, int32_t dim, double sigma, const double* ell,
                       const double* rot, int32_t periodic_mask, const grf_grads& g, double* part, int32_t splits,
-                      double* gpart, int32_t n_gpart, double* contrib, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+                      double* gpart, int32_t n_gpart, double* contrib, const BandReduce& band, void* stream) {
     BwdArgs a{};
     bwd_common_args(a, table, n_modes, dim, sigma, ell, rot, periodic_mask, g);
     a.part = part;
@@ -722,20 +824,19 @@ int launch_bwd_reduce(const void* table, int64_t n_modes, int32_t dim, double si
     a.gpart = gpart;
     a.n_gpart = n_gpart;
     a.contrib = contrib;
-    bwd_reduce_kernel<<<static_cast<unsigned>(a.n_pad / 32), 32 * kRedWarps, 0, st>>>(a);
-    bwd_scalar_kernel<<<1, 32 * kScalarRows, 0, st>>>(a, a.n_pad / 32);
-    count_launches(2);
-    return cudaGetLastError();
+    a.band = band;
+    return launch_reduce(a, static_cast<cudaStream_t>(stream));
 }
 
 int launch_synth_bwd(const void* table, int64_t n_modes, int32_t dim, double sigma,
                      const double* ell, const double* rot, int32_t periodic_mask, const float* xs,
                      const float* ys, const float* zs,
                      const int32_t* perm, int64_t perm_base, int64_t n_cells, const float* gY,
-                     const grf_grads& g, void* workspace, int32_t* status, void* stream) {
+                     const grf_grads& g, const SegInfo* band, void* workspace, int32_t* status, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (const int e = bwd_allow_smem(dim)) return e;
     const TableLayout TL = table_layout(n_modes);
+    const unsigned char* tb = static_cast<const unsigned char*>(table);
     BwdArgs a{};
     bwd_common_args(a, table, n_modes, dim, sigma, ell, rot, periodic_mask, g);
     a.xs = xs;
@@ -745,15 +846,6 @@ int launch_synth_bwd(const void* table, int64_t n_modes, int32_t dim, double sig
     a.perm_base = perm_base;
     a.n_cells = n_cells;
     a.gY = gY;
-    const int mode_blocks = static_cast<int>((TL.n_pad + kBwdThreads * kMPT - 1) / (kBwdThreads * kMPT));
-    a.splits = 1;
-    if (n_cells > 0) {
-        switch (dim) {
-            case 1: a.splits = choose_splits<1>(n_cells, mode_blocks, bwd_max_splits(TL.n_pad)); break;
-            case 2: a.splits = choose_splits<2>(n_cells, mode_blocks, bwd_max_splits(TL.n_pad)); break;
-            default: a.splits = choose_splits<3>(n_cells, mode_blocks, bwd_max_splits(TL.n_pad)); break;
-        }
-    }
     const int64_t n_pad = TL.n_pad;
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     a.part = reinterpret_cast<double*>(ws);
@@ -766,21 +858,92 @@ int launch_synth_bwd(const void* table, int64_t n_modes, int32_t dim, double sig
         if (e == cudaSuccess) e = cudaMemsetAsync(a.gpart, 0, sizeof(double), st);
         if (e != cudaSuccess) return e;
         a.splits = 1;
-    } else {
-        dim3 grid(mode_blocks, a.splits);
-        switch (dim) {
-            case 1: bwd_partial_kernel<1, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
-            case 2: bwd_partial_kernel<2, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
-            case 3: bwd_partial_kernel<3, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
-            default: return cudaErrorInvalidValue;
+        a.n_gpart = 1;
+        return launch_reduce(a, st);
+    }
+    const int64_t most = bwd_max_splits(n_pad);
+    if (band != nullptr) {
+        unsigned char* bw = ws + bwd_workspace_bytes(n_cells, n_modes, dim);
+        const CellsAdjLayout L = cells_adj_layout(n_cells, n_pad, dim);
+        BandDesc* b = reinterpret_cast<BandDesc*>(bw);
+        float* gmax = reinterpret_cast<float*>(bw + L.off_gmax);
+        double* gsum = reinterpret_cast<double*>(bw + L.off_gsum);
+        int rc = launch_adj_scan(gY, n_cells, nullptr, 0, gmax, gsum, reinterpret_cast<float*>(bw + L.off_xmax), st);
+        if (rc != cudaSuccess) return rc;
+        int dev = 0, sms = 148;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        sms = std::min(sms, 256);
+        BandSelect s{};
+        s.hot = a.hot;
+        s.cold = a.cold;
+        s.thdr = reinterpret_cast<const TableHeader*>(tb);
+        s.n_modes = static_cast<int32_t>(n_modes);
+        s.dim = dim;
+        s.idx_h = reinterpret_cast<int32_t*>(bw + L.off_idx);
+        s.idx_l = reinterpret_cast<int32_t*>(bw + L.off_idx + L.idx);
+        s.seg = band;
+        s.status = status;
+        s.us_mode = static_cast<float>(cells_adjoint_us_per_mode(n_cells));
+        s.us_node = static_cast<float>(kBandNodeAdjUs);
+        s.us_fixed = static_cast<float>(cells_adjoint_band_us(n_cells, dim));
+        s.cap_nodes = L.cap_nodes;
+        s.cap_part = L.cap_nodes;
+        s.cap_mt = (L.cap_yz + 127) / 128;
+        s.cap_yz = L.cap_yz;
+        s.fold = 1;
+        s.chunk = 1;
+        s.us_heavy = 5.0f;
+        s.max_split = 1;
+        rc = launch_band_select(s, b, st);
+        if (rc != cudaSuccess) return rc;
+        float* nodes = reinterpret_cast<float*>(bw + L.off_nodes);
+        rc = launch_band_spread(b, dim, xs, ys, zs, perm, perm_base, n_cells, gY, gmax, adj_scan_blocks(),
+                                reinterpret_cast<unsigned long long*>(bw + L.off_fixed), nodes, sms, st);
+        if (rc != cudaSuccess) return rc;
+        BandPhasors ph;
+        for (int c = 0; c < 3; ++c) {
+            ph.ph[c] = reinterpret_cast<float2*>(bw + L.off_ph[c]);
+            ph.off[c] = reinterpret_cast<float*>(bw + L.off_off[c]);
         }
-        count_launches(1);
+        ph.gain = reinterpret_cast<double*>(bw + L.off_gain);
+        ph.rank = reinterpret_cast<int32_t*>(bw + L.off_rank);
+        double* part = reinterpret_cast<double*>(bw + L.off_part);
+        rc = launch_band_nodes(b, a.cold, s.idx_l, s.idx_h, GridGeom{}, dim, nodes, ph, part, sms, st);
+        if (rc != cudaSuccess) return rc;
+        // direct modes: partial sums of at most 4 blocks per SM, within the room
+        // of the CUDA-core adjoint's (a tile of 128 modes per block)
+        const int64_t room = most * n_pad / 128;
+        const int blocks = static_cast<int>(std::min<int64_t>(int64_t(sms) * 4, room));
+        rc = launch_band_direct(b, dim, a.cold, s.idx_h, xs, ys, zs, perm, perm_base, n_cells, gY, a.part, blocks, st);
+        if (rc != cudaSuccess) return rc;
+        a.band.b = b;
+        a.band.rank = ph.rank;
+        a.band.gain = ph.gain;
+        a.band.part = part;
+        a.band.blocks = sms * 3;
+        a.band.direct_sms = blocks;
+        a.gpart = gsum;  // dmu: the scan's sums of g
+        a.n_gpart = adj_scan_blocks();
+        return launch_reduce(a, st);
+    }
+    const int mode_blocks = static_cast<int>((n_pad + kBwdThreads * kMPT - 1) / (kBwdThreads * kMPT));
+    switch (dim) {
+        case 1: a.splits = choose_splits<1>(n_cells, mode_blocks, most); break;
+        case 2: a.splits = choose_splits<2>(n_cells, mode_blocks, most); break;
+        default: a.splits = choose_splits<3>(n_cells, mode_blocks, most); break;
     }
     a.n_gpart = a.splits;
-    bwd_reduce_kernel<<<static_cast<unsigned>(n_pad / 32), 32 * kRedWarps, 0, st>>>(a);
-    bwd_scalar_kernel<<<1, 32 * kScalarRows, 0, st>>>(a, static_cast<int32_t>(n_pad / 32));
-    count_launches(2);
-    return cudaGetLastError();
+    const dim3 grid(mode_blocks, a.splits);
+    switch (dim) {
+        case 1: bwd_partial_kernel<1, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
+        case 2: bwd_partial_kernel<2, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
+        case 3: bwd_partial_kernel<3, kMPT><<<grid, kBwdThreads, kBwdSmemBytes, st>>>(a, status); break;
+        default: return cudaErrorInvalidValue;
+    }
+    count_launches(1);
+    if (const cudaError_t e = cudaGetLastError()) return e;
+    return launch_reduce(a, st);
 }
 
 unsigned long long take_index_faults_bwd() { return take_tu_index_faults(); }

@@ -39,8 +39,10 @@
 #include <algorithm>
 #include <cmath>
 
+#include "band.cuh"
 #include "device_common.cuh"
 #include "grid_common.cuh"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace grf {
@@ -91,6 +93,8 @@ struct AdjDesc {
     double* part;               // [groups][n_pad][5]
     int32_t ny, nz, n_pad, n_kc, n_yb, n_lt, py_log2, n_mt, groups;
     int32_t units;              // per mode tile: n_kc n_yb n_lt
+    const BandDesc* band;       // band path: the modes are its direct ones (device count), else null
+    int32_t sms;
 };
 
 // Walks a CTA's units u0 .. u1 - 1 in order: z block lt fastest, then y
@@ -132,6 +136,8 @@ struct AdjPrep {
     float* scal;
     int32_t nx, ny, nz, n_pad, n_kc, n_yb, n_lt, py_log2, n_mt;
     int64_t units;
+    const BandDesc* band;  // band path: only its direct modes, table slots idx (-1: none)
+    const int32_t* idx;
 };
 
 // Block-wide reduction in a fixed order (warp butterflies, then the warp
@@ -149,20 +155,21 @@ __device__ __forceinline__ T block_reduce(T v, Op op, T* sh) {
     return v;
 }
 
-// Per block: max |g|, the sum of g (compensated per thread, FP64 across the
-// block) and max |X_i - X_0|.
+// Per block: max |g| (infinite where some g is not finite), the sum of g
+// (compensated per thread, FP64 across the block) and max |X_i - X_0|.
 __global__ void __launch_bounds__(256) adj_scan_kernel(const float* g, int64_t n, const float* X, int32_t nx,
                                                         float* gmax, double* gsum, float* xmax) {
     __shared__ float shf[8];
     __shared__ double shd[8];
+    pdl_wait();
     float mx = 0.0f, sh = 0.0f, sl = 0.0f, xm = 0.0f;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float v = __ldg(g + i);
-        mx = fmaxf(mx, fabsf(v));
+        mx = fabsf(v) <= 3.402823466e38f ? fmaxf(mx, fabsf(v)) : INFINITY;
         two_sum_acc(sh, sl, v);
     }
-    const float x0 = __ldg(X);
+    const float x0 = nx > 0 ? __ldg(X) : 0.0f;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nx; i += stride)
         xm = fmaxf(xm, fabsf(__ldg(X + i) - x0));
     const auto fmax_op = [](float a, float b) { return fmaxf(a, b); };
@@ -189,6 +196,12 @@ __global__ void __launch_bounds__(256) adj_scan_kernel(const float* g, int64_t n
 // below 1 (from the scan's per-block maxima; every block derives the same).
 __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
     __shared__ float shf[8];
+    pdl_wait();
+    if (p.band != nullptr) {
+        p.n_mt = (p.band->nh + kAM - 1) / kAM;
+        p.n_pad = p.n_mt * kAM;
+        if (p.n_mt == 0) return;
+    }
     float gm = 0.0f, xm = 0.0f;
     for (int b = threadIdx.x; b < kAScanBlocks; b += blockDim.x) {
         gm = fmaxf(gm, p.gmax[b]);
@@ -224,15 +237,16 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
             const int r = static_cast<int>((idx >> 3) & (kAM - 1));
             const int64_t rest = idx >> 10;  // mode tile * n_kc + x chunk
             const int kc = static_cast<int>(rest % p.n_kc);
-            const int m = static_cast<int>(rest / p.n_kc) * kAM + r;
-            const float4 c0 = __ldg(p.cold + 2 * m);
+            const int row = static_cast<int>(rest / p.n_kc) * kAM + r;
+            const int m = p.idx != nullptr ? __ldg(p.idx + row) : row;
+            const float4 c0 = __ldg(p.cold + 2 * max(m, 0));
             float cs[8], sn[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int x = kc * kAX + kk8 * 8 + e;
                 cs[e] = 0.0f;
                 sn[e] = 0.0f;
-                if (x < p.nx) sincospif(2.0f * turns_axis(c0.x, c0.y, __ldg(p.X + x)), &sn[e], &cs[e]);
+                if (x < p.nx && m >= 0) sincospif(2.0f * turns_axis(c0.x, c0.y, __ldg(p.X + x)), &sn[e], &cs[e]);
             }
             uint4 CH, CL, SH, SL;
             tc::split_f16x2(cs[0], cs[1], CH.x, CL.x);
@@ -250,7 +264,8 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
             *reinterpret_cast<uint4*>(o + 3 * gridc::kTileBytes) = SL;
         } else if (idx < nA + nY) {
             const int64_t u = idx - nA;
-            const int m = static_cast<int>(u % p.n_pad);
+            const int row = static_cast<int>(u % p.n_pad);
+            const int m = p.idx != nullptr ? max(__ldg(p.idx + row), 0) : row;
             const int64_t k = u / p.n_pad;
             const float4 c0 = __ldg(p.cold + 2 * m);
             float cs, sn;
@@ -258,7 +273,8 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
             p.ytab[u] = make_float2(cs, sn);
         } else if (idx < nA + nY + nZ) {
             const int64_t u = idx - nA - nY;
-            const int m = static_cast<int>(u % p.n_pad);
+            const int row = static_cast<int>(u % p.n_pad);
+            const int m = p.idx != nullptr ? max(__ldg(p.idx + row), 0) : row;
             const int64_t l = u / p.n_pad;
             const float4 c1 = __ldg(p.cold + 2 * m + 1);
             float cs, sn;
@@ -331,6 +347,15 @@ __global__ void __launch_bounds__(kAThreads, 1) grid_adj_kernel(AdjDesc d, int32
     volatile int32_t* abort = reinterpret_cast<volatile int32_t*>(done + 2);
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    if (d.band != nullptr) {
+        pdl_wait();
+        d.n_mt = (d.band->nh + kAM - 1) / kAM;
+        d.n_pad = d.n_mt * kAM;
+        d.groups = grid_adjoint_groups(d.n_mt, d.units, d.sms);
+        if (d.n_mt == 0 && blockIdx.x == 0 && threadIdx.x == 0)
+            atomicAdd(&g_grid_adj_units, static_cast<unsigned long long>(d.units));  // all modes at the nodes
+        if (blockIdx.x >= d.n_mt * d.groups) return;  // fewer modes than the launch was made for
+    }
     const int mt = static_cast<int>(blockIdx.x % d.n_mt);
     const int grp = static_cast<int>(blockIdx.x / d.n_mt);
     const int32_t u0 = static_cast<int32_t>(static_cast<int64_t>(d.units) * grp / d.groups);
@@ -358,6 +383,7 @@ __global__ void __launch_bounds__(kAThreads, 1) grid_adj_kernel(AdjDesc d, int32
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = *tslot;
+    pdl_wait();
 
     if (warp < kAEpi) {
         // ---- epilogue: contract the unit's columns with the y and z phasors --------
@@ -672,11 +698,7 @@ AdjPlan adj_plan(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad, int sms) {
     a.n_yb = (ny + PY - 1) / PY;
     a.n_lt = (nz + PZ - 1) / PZ;
     a.units = int64_t(a.n_kc) * a.n_yb * a.n_lt;
-    // groups: as many as fit one CTA per SM (mode tiles x groups <= SMs)
-    int64_t g = sms > 0 ? sms / a.n_mt : 1;
-    g = std::max<int64_t>(1, std::min<int64_t>(g, a.units));
-    g = std::min<int64_t>(g, std::max<int64_t>(1, kAMaxCtas / a.n_mt));
-    a.groups = static_cast<int>(g);
+    a.groups = grid_adjoint_groups(a.n_mt, a.units, sms);
     int64_t off = 0;
     auto take = [&](int64_t bytes) {
         const int64_t o = off;
@@ -706,19 +728,95 @@ size_t bwd_grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
     return static_cast<size_t>(adj_plan(nx, ny, nz, n_pad, 1).total);
 }
 
+namespace {
+
+// Workspace of the band path after the grid adjoint's own: the descriptor, the
+// modes' lists and ranks, the axes' tables, the gradient at (x nodes) x (y, z
+// cells), at (x, y) nodes x z cells and at the nodes, the phasor tables and the
+// partial sums over the nodes.
+struct AdjBandLayout {
+    int64_t off_idx, idx, off_rank, off_tab[3][5], off_gain, off_h1, off_h2, off_nodes, off_ph[3], off_off[3], off_part, total;
+    int64_t cap_nodes, cap_mid;
+};
+AdjBandLayout adj_band_layout(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad, int sms) {
+    AdjBandLayout L{};
+    const int64_t n = int64_t(nx) * ny * nz;
+    L.cap_nodes = n / 4;
+    L.cap_mid = n / 2;
+    int64_t off = 0;
+    auto take = [&](int64_t bytes) {
+        const int64_t o = off;
+        off += align256(bytes);
+        return o;
+    };
+    take(sizeof(BandDesc));
+    L.idx = align256((n_pad + 128) * 4);
+    L.off_idx = take(2 * L.idx);
+    L.off_rank = take(n_pad * 4);
+    const int64_t dims[3] = {nx, ny, nz};  // an axis has no more nodes than cells
+    for (int c = 0; c < 3; ++c) {
+        L.off_tab[c][0] = take(dims[c] * 32);
+        L.off_tab[c][1] = take(dims[c] * 4);
+        L.off_tab[c][2] = take(dims[c] * 8);
+        L.off_tab[c][3] = take(band_wt_floats(dims[c]) * 4);
+        L.off_tab[c][4] = take(4);
+        L.off_ph[c] = take(dims[c] * n_pad * 8);
+        L.off_off[c] = take(dims[c] * 4);
+    }
+    L.off_gain = take(4 * n_pad * 8);
+    L.off_h1 = take(n * 4);
+    L.off_h2 = take(L.cap_mid * 4);
+    L.off_nodes = take(L.cap_nodes * 4);
+    // tiles x chunks x groups is at most the blocks, or one group each
+    const int64_t tiles = n_pad / 128 * ((int64_t(nx) + 63) / 64);
+    L.off_part = take(std::max<int64_t>(int64_t(sms) * 3, tiles) * 128 * 5 * 8);
+    L.total = off;
+    return L;
+}
+
+int adj_init() {
+    if (g_adj_sms != 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(grid_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem);
+    if (e == cudaSuccess) g_adj_sms = sms;
+    return e;
+}
+
+}  // namespace
+
+// Whole units at the tensor-core adjoint's rate; the lattice's transposed
+// interpolation passes over g once more and adds some kernels.
+double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
+    const AdjPlan a = adj_plan(nx, ny, nz, 128, 1);
+    return double(a.units) * kAX * kAYZ / 38.0e6;
+}
+double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz) { return 25.0 + 6e-6 * double(nx) * ny * nz; }
+
+// Below 120 us of direct products the call is bound by the launches of the
+// whole backward pass, and the lattice's ten add to them: 64 x 64 x 64 cells x
+// 4096 modes (forward and backward) took 183 us directly, 206 with the lattice
+// on both ways; 128 x 100 x 90 x 4096 gains, 496 -> 215 to 300 us.
+size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 120.0)
+        return 0;
+    return static_cast<size_t>(adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total);
+}
+
+int adj_scan_blocks() { return kAScanBlocks; }
+int launch_adj_scan(const float* g, int64_t n, const float* X, int32_t nx, float* gmax, double* gsum, float* xmax,
+                    void* stream) {
+    return launch_chained(adj_scan_kernel, kAScanBlocks, 256, 0, static_cast<cudaStream_t>(stream), g, n, X, nx, gmax,
+                          gsum, xmax);
+}
+
 int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const GridGeom& gg, const float* gY,
                           double sigma, const double* ell, const double* rot, int32_t periodic_mask,
-                          const grf_grads& g, void* ws, int32_t* status, void* stream) {
+                          const grf_grads& g, void* ws, bool band, int32_t* status, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (g_adj_sms == 0) {
-        int dev = 0, sms = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(grid_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kASmem);
-        if (e != cudaSuccess) return e;
-        g_adj_sms = sms;
-    }
+    if (const int e = adj_init()) return e;
     const TableLayout TL = table_layout(n_modes);
     const unsigned char* tb = static_cast<const unsigned char*>(table);
     const AdjPlan ap = adj_plan(gg.nx, gg.ny, gg.nz, TL.n_pad, g_adj_sms);
@@ -754,15 +852,6 @@ int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const
     p.n_mt = ap.n_mt;
     p.units = ap.units;
 
-    adj_scan_kernel<<<kAScanBlocks, 256, 0, st>>>(gY, n, gg.X, gg.nx, reinterpret_cast<float*>(w + ap.off_gmax),
-                                                  reinterpret_cast<double*>(w + ap.off_gpart),
-                                                  reinterpret_cast<float*>(w + ap.off_xmax));
-    const int64_t items = int64_t(ap.n_mt) * ap.n_kc * kAM * 8 + (int64_t(gg.ny) + gg.nz) * TL.n_pad +
-                          ap.units * kAYZ * 8 + gg.ny + gg.nz;
-    const int64_t pg = std::min<int64_t>((items + 255) / 256, int64_t(g_adj_sms) * 16);
-    adj_prep_kernel<<<static_cast<unsigned>(pg), 256, 0, st>>>(p);
-    count_launches(2);
-
     AdjDesc d{};
     d.atab = p.atab;
     d.btab = p.btab;
@@ -785,11 +874,87 @@ int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const
     d.n_mt = ap.n_mt;
     d.groups = ap.groups;
     d.units = static_cast<int32_t>(ap.units);
-    grid_adj_kernel<<<static_cast<unsigned>(ap.groups * ap.n_mt), kAThreads, kASmem, st>>>(d, status);
-    count_launches(1);
+    d.sms = g_adj_sms;
+
+    int rc = launch_adj_scan(gY, n, gg.X, gg.nx, reinterpret_cast<float*>(w + ap.off_gmax),
+                             reinterpret_cast<double*>(w + ap.off_gpart), reinterpret_cast<float*>(w + ap.off_xmax),
+                             st);
+    if (rc != cudaSuccess) return rc;
+    BandReduce br{};
+    unsigned grid = static_cast<unsigned>(ap.groups * ap.n_mt);
+    if (band) {
+        unsigned char* bw = w + ap.total;
+        const AdjBandLayout L = adj_band_layout(gg.nx, gg.ny, gg.nz, TL.n_pad, kAMaxCtas);
+        BandDesc* b = reinterpret_cast<BandDesc*>(bw);
+        BandSelect s{};
+        s.hot = reinterpret_cast<const float4*>(tb + TL.off_hot);
+        s.cold = p.cold;
+        s.thdr = p.thdr;
+        s.n_modes = static_cast<int32_t>(n_modes);
+        s.dim = dim;
+        s.idx_h = reinterpret_cast<int32_t*>(bw + L.off_idx);
+        s.idx_l = reinterpret_cast<int32_t*>(bw + L.off_idx + L.idx);
+        s.seg = gg.seg;
+        s.status = status;
+        s.X = gg.X;
+        s.n[0] = gg.nx;
+        s.n[1] = gg.ny;
+        s.n[2] = gg.nz;
+        s.us_mode = static_cast<float>(grid_adjoint_us_per_mode(gg.nx, gg.ny, gg.nz));
+        s.us_node = static_cast<float>(kBandNodeAdjUs);
+        s.us_fixed = static_cast<float>(grid_adjoint_band_us(gg.nx, gg.ny, gg.nz));
+        // the direct modes' tables hold all of g, and their units run at any count
+        s.us_heavy = 10.0f + static_cast<float>(9e-6 * double(n));
+        s.cap_nodes = L.cap_nodes;
+        s.cap_part = L.cap_nodes;
+        s.cap_mid = L.cap_mid;
+        s.cap_mt = INT32_MAX / 256;
+        s.cap_yz = INT32_MAX;
+        s.fold = 1;
+        s.chunk = kAM;
+        s.max_split = 1;
+        rc = launch_band_select(s, b, st);
+        if (rc != cudaSuccess) return rc;
+        BandAxisTab tab[3];
+        BandPhasors ph;
+        for (int c = 0; c < 3; ++c) {
+            tab[c].w = reinterpret_cast<float*>(bw + L.off_tab[c][0]);
+            tab[c].start = reinterpret_cast<int32_t*>(bw + L.off_tab[c][1]);
+            tab[c].range = reinterpret_cast<int2*>(bw + L.off_tab[c][2]);
+            tab[c].wt = reinterpret_cast<float*>(bw + L.off_tab[c][3]);
+            tab[c].most = reinterpret_cast<int32_t*>(bw + L.off_tab[c][4]);
+            ph.ph[c] = reinterpret_cast<float2*>(bw + L.off_ph[c]);
+            ph.off[c] = reinterpret_cast<float*>(bw + L.off_off[c]);
+        }
+        ph.gain = reinterpret_cast<double*>(bw + L.off_gain);
+        ph.rank = reinterpret_cast<int32_t*>(bw + L.off_rank);
+        float* nodes = reinterpret_cast<float*>(bw + L.off_nodes);
+        double* part = reinterpret_cast<double*>(bw + L.off_part);
+        rc = launch_band_grid_spread(b, gg, gY, tab, reinterpret_cast<float*>(bw + L.off_h1),
+                                     reinterpret_cast<float*>(bw + L.off_h2), nodes, g_adj_sms, st);
+        if (rc != cudaSuccess) return rc;
+        rc = launch_band_nodes(b, p.cold, s.idx_l, s.idx_h, gg, dim, nodes, ph, part, g_adj_sms, st);
+        if (rc != cudaSuccess) return rc;
+        p.band = d.band = b;
+        p.idx = s.idx_h;
+        br.b = b;
+        br.rank = ph.rank;
+        br.gain = ph.gain;
+        br.part = part;
+        br.blocks = g_adj_sms * 3;
+        br.direct_sms = g_adj_sms;
+        br.direct_units = d.units;
+        grid = static_cast<unsigned>(std::max(g_adj_sms, ap.n_mt));
+    }
+    const int64_t items = int64_t(ap.n_mt) * ap.n_kc * kAM * 8 + (int64_t(gg.ny) + gg.nz) * TL.n_pad +
+                          ap.units * kAYZ * 8 + gg.ny + gg.nz;
+    const int64_t pg = std::min<int64_t>((items + 255) / 256, int64_t(g_adj_sms) * 16);
+    cudaError_t e = launch_chained(adj_prep_kernel, static_cast<unsigned>(pg), 256, 0, st, p);
+    if (e == cudaSuccess) e = launch_chained(grid_adj_kernel, grid, kAThreads, kASmem, st, d, status);
+    if (e != cudaSuccess) return e;
     return launch_bwd_reduce(table, n_modes, dim, sigma, ell, rot, periodic_mask, g, d.part, ap.groups,
                              reinterpret_cast<double*>(w + ap.off_gpart), kAScanBlocks,
-                             reinterpret_cast<double*>(w + ap.off_contrib), stream);
+                             reinterpret_cast<double*>(w + ap.off_contrib), br, stream);
 }
 
 int take_grid_adj_units(unsigned long long* units) {

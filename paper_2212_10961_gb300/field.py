@@ -592,10 +592,13 @@ _ws_fwd = Workspace()
 
 def backward_workspace_bytes(plan: CellPlan, segment, n_modes, dim):
     """Workspace bytes of grf_synth_backward on this plan: enough for the
-    CUDA-core adjoint and, on a grid plan, for the tensor-core one
-    (grf_backward_workspace_bytes and grf_backward_grid_workspace_bytes)."""
-    return max(int(lib().grf_backward_workspace_bytes(plan.segment_size(segment), int(n_modes), int(dim))),
-               int(lib().grf_backward_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes))))
+    CUDA-core adjoint, with the node lattice of low-frequency modes, or, on a
+    grid plan, for the tensor-core one (grf_backward_workspace_bytes,
+    grf_backward_band_workspace_bytes, grf_backward_grid_workspace_bytes)."""
+    n = plan.segment_size(segment)
+    grid = int(lib().grf_backward_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
+    cells = 0 if grid else int(lib().grf_backward_band_workspace_bytes(n, int(n_modes), int(dim)))
+    return max(int(lib().grf_backward_workspace_bytes(n, int(n_modes), int(dim))), cells, grid)
 
 
 def backward(table: ModeTable, params: FieldParams, plan: CellPlan, gY, segment=0, stream=None,
@@ -922,8 +925,8 @@ def take_grid_adjoint_units():
 
 def grid_path(enable=True, fold_chunks=4):
     """Process-wide setting of the grid path (False: off, True: automatic,
-    "always": every grid plan) and its fold interval in chunks of 32 modes
-    (grf_debug_grid_path)."""
+    "always": every grid plan, all modes as products) and its fold interval
+    in chunks of 32 modes (grf_debug_grid_path)."""
     mode = 2 if enable == "always" else (1 if enable else 0)
     check(lib().grf_debug_grid_path(mode, int(fold_chunks)))
 

@@ -12,7 +12,7 @@ import math
 import numpy as np
 import pytest
 
-from helpers import check_forward, check_lognormal, gpu_env, oracle_field, to_dev
+from helpers import GRAD_TOL, check_forward, check_lognormal, gpu_env, oracle_field, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -233,3 +233,124 @@ def test_band_cells_fused_mismatch_and_workspace(env):
         assert loss.item() == pytest.approx(loss_u.item(), rel=1e-12)
         assert not torch.equal(direct, ref["Y"])
         assert (direct - ref["Y"]).abs().max().item() <= 2e-5
+
+
+# ---------------------------------------------------------------------------
+# The adjoint: g spread onto the lattice, the modes summed there
+# ---------------------------------------------------------------------------
+def _check_adjoint(env, cells, ell, n, law, g=None, segments=None, segment=0, seed=6, modes=None, scale=1.0):
+    """Gradients of a sample of modes (every light/direct class is in it)
+    against the oracle's FP64 sums, sums over all modes against the modes'."""
+    torch, F, W = env
+    from oracle import field as of
+    from oracle import native
+    dim = len(ell)
+    plan = F.CellPlan(*to_dev(torch, cells), segments=segments)
+    o0, count = int(plan.offsets[segment]), plan.segment_size(segment)
+    if g is None:
+        g = np.random.default_rng(seed + 1).standard_normal(count).astype(np.float32)
+    m = modes or _modes(n, dim, ell, law, seed)
+    table = F.ModeTable(m["amp"], m["psi"], m["a"])
+    gd = torch.from_numpy(g).cuda() * scale
+    l0 = F.launch_count()
+    gr = F.backward(table, _params(F, n, dim, ell), plan, gd, segment)
+    torch.cuda.synchronize()
+    launches = F.launch_count() - l0
+    again = F.backward(table, _params(F, n, dim, ell), plan, gd, segment)
+    assert plan.status() == 0
+    for k in ("dA", "dpsi", "da", "dell", "dsigma"):
+        assert torch.equal(gr[k], again[k]), "%s differs from one run to the next" % k
+    fast = np.argsort(np.abs(m["a"] / np.sqrt(np.abs(m["a"])).mean(0).clip(1e-30) ** 2).max(1))
+    idx = np.unique(np.concatenate([fast[:20], fast[-40:], np.random.default_rng(2).choice(n, 200)]))
+    c = np.stack([c[o0:o0 + count] for c in cells[:dim]], axis=-1)
+    g64 = g.astype(np.float64) * scale
+    sums = native.mode_sums(m["a"][idx], m["psi"][idx], c, g64)
+    ref = of.grads_from_sums(*sums, m["amp"][idx], m["a"][idx], 1.0, ell, g64)
+    for k in ("dA", "dpsi", "da"):
+        got = gr[k].cpu().numpy()[idx]
+        for col in ([...],) if got.ndim == 1 else [(slice(None), q) for q in range(dim)]:
+            top = np.abs(ref[k][tuple(col)]).max()
+            err = np.abs(got[tuple(col)] - ref[k][tuple(col)]).max()
+            assert err <= GRAD_TOL * top, "%s %s: %.3e of %.3e" % (k, col, err, top)
+    assert gr["dmu"].item() == pytest.approx(g64.sum(), rel=1e-9, abs=1e-9 * np.abs(g64).sum())
+    dell = -(gr["da"].cpu().numpy() * m["a"]).sum(0) / np.asarray(ell)
+    np.testing.assert_allclose(gr["dell"].cpu().numpy()[:dim], dell, rtol=1e-9, atol=1e-9 * np.abs(dell).max())
+    return launches, {k: v.cpu().numpy() for k, v in gr.items()}
+
+
+# grids: 2-D of few and of many tiles, 3-D with and without modes left for
+# the product, thin grids, an axis that is not interpolated
+@pytest.mark.parametrize("shape,extent,ell,n,law", [
+    ((1401, 999), (1.4, 1.0), (0.2, 0.1), 4001, "rough"),
+    ((1024, 1025), (1.0, 1.0), (0.2, 0.2), 6000, "gaussian"),
+    ((129, 101, 90), (1.29, 1.0, 0.9), (0.2, 0.2, 0.2), 4097, "gaussian"),
+    ((160, 141, 130), (1.6, 1.4, 1.3), (0.2, 0.15, 0.2), 3000, "rough"),
+    ((33, 40, 601), (0.1, 0.13, 2.0), (0.1, 0.1, 0.1), 5000, "rough"),
+    ((640, 9, 260), (4.0, 0.05, 1.8), (0.1, 0.1, 0.1), 3000, "rough"),
+    ((2003, 8, 90), (4.0, 0.05, 0.9), (0.1, 0.1, 0.1), 3000, "gaussian"),
+])
+def test_band_grid_adjoint_against_oracle(env, shape, extent, ell, n, law):
+    launches, _ = _check_adjoint(env, _mesh(_uniform(shape, extent)), ell, n, law)
+    assert launches >= 8
+
+
+def test_band_grid_adjoint_axes_in_any_order_and_far_away(env):
+    # axes in random order and far from the origin, one with a wide gap (the
+    # nodes inside it are read by no cell); modes that do not vary
+    rng = np.random.default_rng(5)
+    axes = [np.float32(900.0) + np.cumsum(rng.uniform(0.002, 0.006, 400)).astype(np.float32),
+            np.ascontiguousarray((np.float32(-70.0) + np.cumsum(rng.uniform(0.004, 0.012, 120)).astype(np.float32))[::-1]),
+            rng.permutation(np.linspace(0.0, 1.0, 90).astype(np.float32))]
+    launches, _ = _check_adjoint(env, _mesh(axes), (0.1, 0.1, 0.1), 3000, "gaussian")
+    assert launches >= 8
+    axes[0] = rng.permutation(np.where(axes[0] > 900.8, axes[0] + np.float32(3.0), axes[0]))
+    m = _modes(3000, 3, (0.1, 0.1, 0.1), "gaussian", 8)
+    m["a"][::7] = 0.0
+    m["a"][11] = (3.0e3, -2.0e4, 17.0)
+    launches, _ = _check_adjoint(env, _mesh(axes), (0.1, 0.1, 0.1), 3000, "gaussian", modes=m)
+    assert launches >= 8
+
+
+@pytest.mark.parametrize("kind,cells,dim,n,law", [
+    ("lattice", 300_000, 2, 4000, "gaussian"), ("lattice", 300_001, 2, 4100, "rough"),
+    ("even", 250_333, 3, 4000, "gaussian"), ("lattice", 262_144, 3, 5003, "rough"),
+    ("clusters", 400_000, 3, 3000, "gaussian"), ("clusters", 300_000, 2, 4000, "rough"),
+])
+def test_band_cells_adjoint_against_oracle(env, kind, cells, dim, n, law):
+    launches, _ = _check_adjoint(env, _cloud(kind, cells, dim, 3), (0.2, 0.25, 0.2)[:dim], n, law)
+    assert launches >= 7
+
+
+def test_band_cells_adjoint_segment_and_coherent_g(env):
+    # the second of three segments, and a g of one sign (the largest sums of
+    # the fixed-point lattice)
+    parts = [_cloud("even", k, 3, 10 + k % 7) for k in (1000, 600_000, 37)]
+    cells = [np.concatenate([p[c] for p in parts]) for c in range(3)]
+    g = np.random.default_rng(3).uniform(0.5, 1.0, 600_000).astype(np.float32)
+    launches, _ = _check_adjoint(env, cells, (0.2, 0.2, 0.2), 6000, "gaussian", g=g, segments=[1000, 600_000, 37],
+                                 segment=1)
+    assert launches >= 7
+
+
+@pytest.mark.parametrize("grid", [False, True])
+def test_band_adjoint_scales_and_carries_what_is_not_finite(env, grid):
+    # g times a power of two gives the same digits times it; a g that holds an
+    # infinity or a NaN gives gradients that are not finite; g = 0 gives 0
+    torch, F, W = env
+    cells = _mesh(_uniform((160, 141, 130), (1.6, 1.4, 1.3))) if grid else _cloud("even", 250_000, 3, 4)
+    ell, n = (0.2, 0.2, 0.2), 4000
+    _, one = _check_adjoint(env, cells, ell, n, "gaussian")
+    for e in (-90, 70):
+        _, big = _check_adjoint(env, cells, ell, n, "gaussian", scale=2.0 ** e)
+        for k in ("dA", "dpsi", "da"):
+            assert np.array_equal(one[k] * 2.0 ** e, big[k])
+    plan = F.CellPlan(*to_dev(torch, cells))
+    m = _modes(n, 3, ell, "gaussian", 6)
+    table = F.ModeTable(m["amp"], m["psi"], m["a"])
+    for bad in (float("nan"), float("inf"), -float("inf")):
+        g = torch.ones(len(cells[0]), device="cuda")
+        g[12345] = bad
+        gr = F.backward(table, _params(F, n, 3, ell), plan, g)
+        assert not torch.isfinite(gr["dA"]).any() and not torch.isfinite(gr["dpsi"]).any()
+    gr = F.backward(table, _params(F, n, 3, ell), plan, torch.zeros(len(cells[0]), device="cuda"))
+    assert all(not v.any() for k, v in gr.items())
