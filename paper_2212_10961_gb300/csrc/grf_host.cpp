@@ -430,7 +430,7 @@ bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t
     if (extra == 0 || ws_bytes < grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra) return false;
     const int32_t n[3] = {gg.nx, gg.ny, gg.nz};
     return band_worth(p, box, n, 0.25 * gg.nx * gg.ny * gg.nz, grid_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeUs,
-                      kBandFixedUs + kBandTryUs) >= 0.0;
+                      kBandFixedUs + kBandTryUs + (gg.nz > 1 ? 8.0 : 0.0)) >= 0.0;
 }
 
 bool lookup_plan(const void* plan, PlanMeta& out) {

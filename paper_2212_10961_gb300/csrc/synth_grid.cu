@@ -559,9 +559,9 @@ __device__ __forceinline__ void grid_prep_items(const GridPrep& p, I nA, I nY, I
                 const float zs = static_cast<float>(zb) * p.zstep;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const int j = prep_slot(p, c * kGModes + quad * 4 + m);
+                    const int j = in ? prep_slot(p, c * kGModes + quad * 4 + m) : -1;
                     float cs = 0.0f, sn = 0.0f;
-                    if (in && j >= 0) {
+                    if (j >= 0) {
                         const float4 c0 = __ldg(p.cold + 2 * j);
                         float t = turns_axis(c0.x, c0.y, x);
                         if (zb > 0) {
@@ -579,9 +579,9 @@ __device__ __forceinline__ void grid_prep_items(const GridPrep& p, I nA, I nY, I
                 const float z = has_z ? band::axis_at(p.ax[2], 0) : 0.0f;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const int j = prep_slot(p, c * kGModes + quad * 4 + m);
+                    const int j = in ? prep_slot(p, c * kGModes + quad * 4 + m) : -1;
                     float cs = 0.0f, sn = 0.0f;
-                    if (in && j >= 0) {
+                    if (j >= 0) {
                         const float4 c0 = __ldg(p.cold + 2 * j);
                         const float4 c1 = __ldg(p.cold + 2 * j + 1);
                         const float tz = psi_z_turns(c1, z, has_z);

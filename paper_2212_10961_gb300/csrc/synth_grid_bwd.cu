@@ -795,12 +795,11 @@ double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
 }
 double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz) { return 25.0 + 6e-6 * double(nx) * ny * nz; }
 
-// Below 120 us of direct products the call is bound by the launches of the
-// whole backward pass, and the lattice's ten add to them: 64 x 64 x 64 cells x
-// 4096 modes (forward and backward) took 183 us directly, 206 with the lattice
-// on both ways; 128 x 100 x 90 x 4096 gains, 496 -> 215 to 300 us.
+// Below 60 us of direct products the lattice's ten launches cost what they
+// save; at 110 us (128 x 128 x 128 cells x 2048 modes, with the forward pass)
+// they gain, 281 -> 241 us.
 size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
-    if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 120.0)
+    if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 60.0)
         return 0;
     return static_cast<size_t>(adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total);
 }
