@@ -222,17 +222,21 @@ __device__ __forceinline__ bool gmax_finite(const float* gmax, int n_gmax) {
     return __all_sync(0xffffffffu, ok);
 }
 
-// A warp takes kSpreadCells consecutive sorted cells and adds them, one after
-// the other, to a box of nodes of its own in shared memory: the lanes hold
-// eight x nodes of four y rows, 16 nodes each.  The cells are first put in the
-// order of their first nodes (a stable counting sort: the order of the sums is
-// fixed), so that cells with the same nodes, about (node spacing / cell
+// A warp takes up to kSpreadCells consecutive sorted cells and adds them, one
+// after the other, to a box of nodes of its own in shared memory: the lanes
+// hold eight x nodes of four y rows, 16 nodes each.  The cells are first put in
+// the order of their first nodes (a stable counting sort: the order of the sums
+// is fixed), so that cells with the same nodes, about (node spacing / cell
 // spacing)^3 of them, add up in registers and the box is read and written once
 // for them: added cell by cell, the box took 133 instructions per cell and 637
 // us for 2M cells.  Then the box goes to the lattice by integer atomics.
-// Groups that spread over more nodes than fit send their values straight to
-// the lattice.
-constexpr int kSpreadCells = 256, kSpreadWarps = 2, kSpreadFloats = 3584, kSpreadBins = 512;
+// A group whose box does not fit (one across a jump of the cells' order) is
+// taken in quarters, down to 32 cells, which then send their values straight to
+// the lattice, 512 atomics a cell: sent so as a whole, the few groups that jump
+// made two thirds of the atomics.  Bound by latency (warps active 15 %, issue
+// 47 %), hence the small box, which lets 14 warps stay on an SM, and the next
+// cell's weights loaded ahead: 579 -> 402 us for 2M cells.
+constexpr int kSpreadCells = 256, kSpreadWarps = 2, kSpreadFloats = 2048, kSpreadBins = 512;
 struct SpreadSmem {
     float box[kSpreadFloats];
     float wts[32][28];  // a round's weights: x (times g), y, z; 16-byte aligned rows
@@ -244,7 +248,7 @@ template <int DIM>
 __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
     const BandDesc* b, const float* __restrict__ xs, const float* __restrict__ ys, const float* __restrict__ zs,
     const int32_t* __restrict__ perm, int64_t perm_base, int64_t n, const float* __restrict__ g,
-    const float* __restrict__ gmax, int n_gmax, unsigned long long* lattice) {
+    const float* __restrict__ gmax, int n_gmax, int cells, unsigned long long* lattice) {
     __shared__ __align__(16) SpreadSmem smem[kSpreadWarps];
     pdl_wait();
     if (b->n_light == 0) return;
@@ -256,9 +260,13 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
     for (int c = 0; c < DIM; ++c) ax[c] = b->ax[c];
     const int mx = ax[0].m;
     const int64_t plane = static_cast<int64_t>(mx) * ax[1].m;
-    const int64_t c0 = (static_cast<int64_t>(blockIdx.x) * kSpreadWarps + warp) * kSpreadCells;
-    if (c0 >= n) return;  // no block-wide barrier below
-    const int nc = static_cast<int>(min(static_cast<int64_t>(kSpreadCells), n - c0));
+    const int64_t first = (static_cast<int64_t>(blockIdx.x) * kSpreadWarps + warp) * cells;
+    if (first >= n) return;  // no block-wide barrier below
+    const int all = static_cast<int>(min(static_cast<int64_t>(cells), n - first));
+    int part = all;
+    for (int at = 0; at < all;) {
+    const int64_t c0 = first + at;
+    const int nc = min(part, all - at);
     const float* src[3] = {xs + c0, ys + c0, zs + c0};
     // ---- the cells' first nodes and the group's box
     constexpr int kPer = kSpreadCells / 32;
@@ -277,10 +285,14 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
         f0[c] = __reduce_min_sync(0xffffffffu, lo);
         nb[c] = __reduce_max_sync(0xffffffffu, hi) + kW - f0[c];
     }
-    // four rows 8 apart in the banks: a pitch of 8 or 24 modulo 32
-    const int pitch = ((nb[0] + 7) / 8 | 1) * 8;
+    const int pitch = (nb[0] + 3) & ~3;
     const int slab = pitch * nb[1];
     const bool staged = static_cast<int64_t>(slab) * nb[2] <= kSpreadFloats;
+    if (!staged && nc > 32) {  // a group across a jump of the order: its quarters
+        part = (nc + 127) / 128 * 32;
+        continue;
+    }
+    __syncwarp();
     const int sx = nb[0] - kW + 1, sy = nb[1] - kW + 1, sz = DIM > 2 ? nb[2] - kW + 1 : 1;
     const bool sorted = staged && static_cast<int64_t>(sx) * sy * sz <= kSpreadBins;
     if (staged)
@@ -369,20 +381,33 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
                                  : static_cast<int>(pz * plane + static_cast<int64_t>(py) * mx + px);
         }
         __syncwarp();
-#pragma unroll 2
-        for (int q = 0; q < m; ++q) {
+        // the next cell's weights are loaded before the current one is added
+        float wx, wa, wb, wn[kz];
+        int next;
+        auto load = [&](int q) {
             const float* w = sm.wts[q];
-            const float wx = w[lx], w0 = wx * w[kW + ly], w1 = wx * w[kW + 4 + ly];
-            float wz[kz];
+            wx = w[lx];
+            wa = w[kW + ly];
+            wb = w[kW + 4 + ly];
             if (DIM > 2) {
                 const float4 a = *reinterpret_cast<const float4*>(w + 2 * kW);
                 const float4 c = *reinterpret_cast<const float4*>(w + 2 * kW + 4);
-                wz[0] = a.x; wz[1 % kz] = a.y; wz[2 % kz] = a.z; wz[3 % kz] = a.w;
-                wz[4 % kz] = c.x; wz[5 % kz] = c.y; wz[6 % kz] = c.z; wz[7 % kz] = c.w;
+                wn[0] = a.x; wn[1 % kz] = a.y; wn[2 % kz] = a.z; wn[3 % kz] = a.w;
+                wn[4 % kz] = c.x; wn[5 % kz] = c.y; wn[6 % kz] = c.z; wn[7 % kz] = c.w;
             } else {
-                wz[0] = 1.0f;
+                wn[0] = 1.0f;
             }
-            const int to = sm.at[q];
+            next = sm.at[q];
+        };
+        load(0);
+#pragma unroll 2
+        for (int q = 0; q < m; ++q) {
+            const float w0 = wx * wa, w1 = wx * wb;
+            float wz[kz];
+#pragma unroll
+            for (int z = 0; z < kz; ++z) wz[z] = wn[z];
+            const int to = next;
+            load(min(q + 1, m - 1));
             if (staged) {
                 if (to != cur) {  // uniform over the warp
                     if (cur >= 0) flush();
@@ -403,7 +428,8 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
             }
         }
     }
-    if (!staged) return;
+    at += nc;
+    if (!staged) continue;
     if (cur >= 0) flush();
     const int rows = nb[1] * nb[2];
     // four rows of up to eight nodes, or one of up to 32, at a time
@@ -415,6 +441,7 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
             const long long v = __float2ll_rn(sm.box[z * slab + y * pitch + x]);
             if (v != 0) atomicAdd(p + x, static_cast<unsigned long long>(v));
         }
+    }
     }
 }
 
@@ -777,12 +804,17 @@ int launch_band_spread(const BandDesc* b, int32_t dim, const float* xs, const fl
                        const int32_t* perm, int64_t perm_base, int64_t n, const float* g, const float* gmax,
                        int n_gmax, unsigned long long* lattice, float* nodes, int sms, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int64_t groups = (n + kSpreadCells - 1) / kSpreadCells;
+    // a warp's group is a chain of sort, sum and write-out: smaller groups where
+    // the warps would not fill the GPU twice (262k cells: 168 us of 64 to a warp
+    // against 146)
+    int cells = kSpreadCells;
+    while (cells > 64 && n / cells < int64_t(sms) * 14 * 2) cells /= 2;
+    const int64_t groups = (n + cells - 1) / cells;
     const unsigned grid = static_cast<unsigned>((groups + kSpreadWarps - 1) / kSpreadWarps);
     cudaError_t e = launch_chained(band_clear_kernel, sms * 4, 256, 0, st, b, lattice);
     if (e == cudaSuccess)
         e = launch_chained(dim > 2 ? band_spread_kernel<3> : band_spread_kernel<2>, grid, 32 * kSpreadWarps, 0, st, b,
-                           xs, ys, zs, perm, perm_base, n, g, gmax, n_gmax, lattice);
+                           xs, ys, zs, perm, perm_base, n, g, gmax, n_gmax, cells, lattice);
     if (e == cudaSuccess)
         e = launch_chained(band_unfix_kernel, sms * 4, 256, 0, st, b, lattice, gmax, n_gmax, n, nodes);
     return e;

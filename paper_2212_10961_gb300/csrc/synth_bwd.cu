@@ -489,13 +489,13 @@ __global__ void __launch_bounds__(kBwdThreads, 4) bwd_partial_kernel(BwdArgs arg
 
 // Kernel 2: per mode, fixed-order sum over splits, chain rule, scatter to the
 // original mode index.  A block owns 32 modes (one per lane); warp w sums
-// the splits w, w + 8, w + 16, ... in increasing order (coalesced rows of the
-// partials, many loads in flight), and warp 0 adds the 8 warp sums in warp
+// the splits w, w + 16, w + 32, ... in increasing order (coalesced rows of the
+// partials, many loads in flight), and warp 0 adds the 16 warp sums in warp
 // order, applies the chain rule (reciprocals of sigma and l precomputed: few
 // FP64 operations, which are slow on this part) and writes the block's sums
 // of the 13 scalar-gradient terms over its 32 modes, in mode order: a fixed
 // order throughout, so the result does not depend on timing.
-constexpr int kRedWarps = 8;
+constexpr int kRedWarps = 16;
 
 __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args) {
     __shared__ double red[kRedWarps][32][5];
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
     }
     {
         double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
+#pragma unroll 8
         for (int s = warp; s < splits; s += kRedWarps) {
             const double* p = part + s * stride;
 #pragma unroll
