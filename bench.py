@@ -787,6 +787,11 @@ GRID_TENSOR_FLOPS_PER_CELL_MODE = 12.0
 # the x-weighted g (4 multiply-adds = 8 flops), each as three FP16 products.
 GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE = 24.0
 
+# Calls large enough sum their modes of low frequency on a coarse node lattice
+# and interpolate: they form fewer cell-mode products than these counts assume.
+EQUIVALENT = ("equivalent rate: counts every mode at every cell; modes of low frequency may be summed on the node "
+              "lattice instead, so frac compares with summing all of them directly and can pass 1")
+
 # Grid-path setting of this run (--grid-path), restored after checks that
 # force the grid path on grids below the automatic threshold.
 GRID_SETTING = True
@@ -798,15 +803,16 @@ def roofline(kern_ms, cell_modes, clocks, sms, traffic=None, lattice_share=0.0, 
     warp tiles): the FP32 pipe at LATTICE_FP32_PER_CELL_MODE instructions per
     cell-mode (1/8 MUFU per cell-mode); the MUFU fraction is kept beside it.
     Grid path: the tensor cores at GRID_TENSOR_FLOPS_PER_CELL_MODE FP16 flops
-    per cell-mode against the measured dense BF16 peak (kern_ms covers the
-    call's two kernels: table preparation and the tensor-core kernel)."""
+    per cell-mode against the measured dense BF16 peak (kern_ms covers all of
+    the call's kernels).  All of them count every mode at every cell
+    (EQUIVALENT)."""
     mufu_peak = MUFU_PER_CLK_PER_SM * sms * 2070e6 / 1e9  # Gcell.mode/s at the maximum SM clock
     achieved = cell_modes / (kern_ms * 1e-3) / 1e9
     if grid:
         tpk, kind = tensor_peak()
         tf = cell_modes * GRID_TENSOR_FLOPS_PER_CELL_MODE / (kern_ms * 1e-3) / 1e12
         return {"bound": "tensor", "achieved": tf, "peak": tpk, "unit": "TFLOP/s", "frac": tf / tpk,
-                "traffic": traffic, "peak_kind": kind,
+                "traffic": traffic, "peak_kind": kind, "note": EQUIVALENT,
                 "peak_basis": ("tensor-core grid path: %.0f FP16 tensor flops per cell-mode (a 2-term real dot "
                                "product as three FP16 products hi.hi + hi.lo + lo.hi) against the %s dense BF16 "
                                "cuBLAS burst peak (FP16 runs at the BF16 rate)" %
@@ -824,7 +830,7 @@ def roofline(kern_ms, cell_modes, clocks, sms, traffic=None, lattice_share=0.0, 
         basis = "%d MUFU cos/clk/SM x %d SMs x 2070 MHz (1 MUFU per cell-mode)" % (MUFU_PER_CLK_PER_SM, sms)
         per_clk = MUFU_PER_CLK_PER_SM
     out = {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "Gcell.mode/s",
-           "frac": achieved / peak_max, "traffic": traffic, "peak_basis": basis,
+           "frac": achieved / peak_max, "traffic": traffic, "peak_basis": basis, "note": EQUIVALENT,
            "frac_of_mufu_roofline": achieved / mufu_peak}
     if clocks.get("sm_mhz"):
         peak_meas = per_clk * sms * clocks["sm_mhz"] * 1e6 / 1e9
@@ -996,7 +1002,7 @@ def main():
                 "peak_basis": ("tensor-core grid adjoint: %.0f FP16 tensor flops per cell-mode (cos and sin "
                                "products of g and of x-weighted g, three FP16 products each) against the %s dense "
                                "BF16 burst peak" % (GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE, kind)),
-                "note": "scan, table preparation, tensor-core kernel and the two reductions"}
+                "note": "scan, table preparation, tensor-core kernel and the two reductions; " + EQUIVALENT}
         elif k_fb.get("adjoint_lattice_share", 0.0) >= 0.5:
             bpk = FP32_PER_CLK_PER_SM * sms * 2070e6 / ADJOINT_LATTICE_FP32_PER_CELL_MODE / 1e9
             basis = ("lattice tiles (%.3f of the tiles): %d FP32 lanes/clk/SM x %d SMs x 2070 MHz / %.1f FP32 "
@@ -1007,7 +1013,7 @@ def main():
         if not k_fb.get("adjoint_grid_path", False):
             k_fb["bwd_roofline"] = {"bound": "alu", "achieved": bw, "peak": bpk, "unit": "Gcell.mode/s",
                                     "frac": bw / bpk, "peak_basis": basis, "frac_of_mufu_roofline": bw / bmufu,
-                                    "note": "adjoint kernel and its two reductions"}
+                                    "note": "adjoint kernel and its two reductions; " + EQUIVALENT}
     if head is None:
         head = next(iter(extra.values()))
         emit(args, {"partial": args.only, "results": extra, "clocks": ck})

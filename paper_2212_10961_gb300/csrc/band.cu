@@ -13,6 +13,9 @@
 //                        light modes' chunks and write the maps
 //   band_finalize_kernel y and x interpolation and maps where the previous
 //                        kernel left partial sums or had no modes
+// At the cells of any plan: the first four, then band_cells_kernel (the light
+// modes' sum at the sorted cells) and synth_fwd_kernel (synth_fwd.cu) for the
+// direct modes, which adds it.
 // Kernels that find nothing to do return at once; all are launched chained.
 #include <cuda_runtime.h>
 

@@ -18,6 +18,7 @@
 //          band_unfix_kernel     fixed point -> FP32
 //   both:  band_phasor_kernel    phasors of the light modes at the nodes' axes
 //          band_nodes_kernel     the sums over the nodes
+//   cells: band_direct_kernel    the direct modes' sums at the cells
 #include <cuda_runtime.h>
 
 #include <algorithm>
