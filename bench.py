@@ -756,12 +756,12 @@ def cpu_baseline(W, name, scale, target_s=10.0, y_gpu=None):
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one full-size call of the
-# headline's grid-path kernels (grid_prep_kernel + grid_mma_kernel, 256^3
-# cells, 4096 modes), one ncu capture (`--metrics dram__bytes_read.sum,
-# dram__bytes_write.sum -k regex:grid`): 0.252 + 0.027 MB and 26.95 + 91.10 MB.
-# Algorithmic: 9 B written per cell (Y, K, facies) = 151 MB plus 26 MB of
-# tables; part of the writes was still in L2 when the launch ended.
-HEAD_TRAFFIC_BYTES = 0.25242e6 + 0.02688e6 + 26.95e6 + 91.10e6
+# headline's kernels (the eight of the node lattice's grid path, 256^3 cells,
+# 4096 modes), one ncu capture (`--metrics dram__bytes_read.sum,
+# dram__bytes_write.sum -k regex:band_`): 31.4 MB read and 89.2 MB written.
+# Algorithmic: 9 B written per cell (Y, K, facies) = 151 MB; part of the writes
+# was still in L2 when the launch ended.
+HEAD_TRAFFIC_BYTES = 31.44e6 + 89.21e6
 
 
 # FP32 instructions per cell-mode of the lattice path (lanes of 4-cell grid
