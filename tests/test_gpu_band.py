@@ -354,3 +354,38 @@ def test_band_adjoint_scales_and_carries_what_is_not_finite(env, grid):
         assert not torch.isfinite(gr["dA"]).any() and not torch.isfinite(gr["dpsi"]).any()
     gr = F.backward(table, _params(F, n, 3, ell), plan, torch.zeros(len(cells[0]), device="cuda"))
     assert all(not v.any() for k, v in gr.items())
+
+
+@pytest.mark.parametrize("grid", [False, True])
+def test_band_captured_with_changing_table(env, grid):
+    # a captured call keeps nothing of the table it was captured with: the
+    # lattice is chosen on the device at every replay, forward and adjoint
+    torch, F, W = env
+    cells = _mesh(_uniform((160, 141, 130), (1.6, 1.4, 1.3))) if grid else _cloud("even", 250_000, 3, 4)
+    ell, n = (0.2, 0.2, 0.2), 4000
+    plan = F.CellPlan(*to_dev(torch, cells))
+    g = torch.from_numpy(np.random.default_rng(2).standard_normal(len(cells[0])).astype(np.float32)).cuda()
+    p = _params(F, n, 3, ell)
+    tables = []
+    for law, seed in (("gaussian", 3), ("rough", 4)):
+        m = _modes(n, 3, ell, law, seed)
+        tables.append(F.ModeTable(m["amp"], m["psi"], m["a"]))
+    call = F.PreparedSynth(p, plan)
+    want = []
+    for t in tables:
+        y = call(t)["Y"].clone()
+        want.append((y, F.backward(t, p, plan, g)["da"].clone()))
+    ws = F.Workspace()
+    F.backward(tables[0], p, plan, g, workspace=ws)
+    torch.cuda.synchronize()
+    table, graph, s = tables[0], torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    keep = table.dev.clone()
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(graph, stream=s):
+            out = call(table, stream=s)
+            da = F.backward(table, p, plan, g, stream=s, workspace=ws)["da"]
+    for k, content in ((0, keep), (1, tables[1].dev), (0, keep)):
+        table.dev.copy_(content)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out["Y"], want[k][0]) and torch.equal(da, want[k][1])
