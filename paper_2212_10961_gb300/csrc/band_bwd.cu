@@ -236,7 +236,7 @@ __device__ __forceinline__ bool gmax_finite(const float* gmax, int n_gmax) {
 // the lattice, 512 atomics a cell: sent so as a whole, the few groups that jump
 // made two thirds of the atomics.  Bound by latency (warps active 15 %, issue
 // 47 %), hence the small box, which lets 14 warps stay on an SM, and the next
-// cell's weights loaded ahead: 579 -> 402 us for 2M cells.
+// cell's weights loaded ahead: 579 -> 397 us for 2M cells.
 constexpr int kSpreadCells = 256, kSpreadWarps = 2, kSpreadFloats = 2048, kSpreadBins = 512;
 struct SpreadSmem {
     float box[kSpreadFloats];
@@ -266,183 +266,183 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
     const int all = static_cast<int>(min(static_cast<int64_t>(cells), n - first));
     int part = all;
     for (int at = 0; at < all;) {
-    const int64_t c0 = first + at;
-    const int nc = min(part, all - at);
-    const float* src[3] = {xs + c0, ys + c0, zs + c0};
-    // ---- the cells' first nodes and the group's box
-    constexpr int kPer = kSpreadCells / 32;
-    int s[kPer][DIM];
-    int f0[3] = {0, 0, 0}, nb[3] = {1, 1, 1};
+        const int64_t c0 = first + at;
+        const int nc = min(part, all - at);
+        const float* src[3] = {xs + c0, ys + c0, zs + c0};
+        // ---- the cells' first nodes and the group's box
+        constexpr int kPer = kSpreadCells / 32;
+        int s[kPer][DIM];
+        int f0[3] = {0, 0, 0}, nb[3] = {1, 1, 1};
 #pragma unroll
-    for (int c = 0; c < DIM; ++c) {
-        int lo = INT_MAX, hi = 0;
+        for (int c = 0; c < DIM; ++c) {
+            int lo = INT_MAX, hi = 0;
 #pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            float v;
-            s[q][c] = band::locate(ax[c], __ldg(src[c] + min(q * 32 + lane, nc - 1)), v);
-            lo = min(lo, s[q][c]);
-            hi = max(hi, s[q][c]);
+            for (int q = 0; q < kPer; ++q) {
+                float v;
+                s[q][c] = band::locate(ax[c], __ldg(src[c] + min(q * 32 + lane, nc - 1)), v);
+                lo = min(lo, s[q][c]);
+                hi = max(hi, s[q][c]);
+            }
+            f0[c] = __reduce_min_sync(0xffffffffu, lo);
+            nb[c] = __reduce_max_sync(0xffffffffu, hi) + kW - f0[c];
         }
-        f0[c] = __reduce_min_sync(0xffffffffu, lo);
-        nb[c] = __reduce_max_sync(0xffffffffu, hi) + kW - f0[c];
-    }
-    const int pitch = (nb[0] + 3) & ~3;
-    const int slab = pitch * nb[1];
-    const bool staged = static_cast<int64_t>(slab) * nb[2] <= kSpreadFloats;
-    if (!staged && nc > 32) {  // a group across a jump of the order: its quarters
-        part = (nc + 127) / 128 * 32;
-        continue;
-    }
-    __syncwarp();
-    const int sx = nb[0] - kW + 1, sy = nb[1] - kW + 1, sz = DIM > 2 ? nb[2] - kW + 1 : 1;
-    const bool sorted = staged && static_cast<int64_t>(sx) * sy * sz <= kSpreadBins;
-    if (staged)
-        for (int k = lane; k < slab * nb[2]; k += 32) sm.box[k] = 0.0f;
-    // ---- order of the cells
-    if (sorted) {
-        for (int k = lane; k < kSpreadBins; k += 32) sm.bins[k] = 0;
+        const int pitch = (nb[0] + 3) & ~3;
+        const int slab = pitch * nb[1];
+        const bool staged = static_cast<int64_t>(slab) * nb[2] <= kSpreadFloats;
+        if (!staged && nc > 32) {  // a group across a jump of the order: its quarters
+            part = (nc + 127) / 128 * 32;
+            continue;
+        }
         __syncwarp();
-        int rank[kPer], key[kPer];
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const bool in = q * 32 + lane < nc;
-            key[q] = ((DIM > 2 ? s[q][DIM - 1] - f0[2] : 0) * sy + s[q][1] - f0[1]) * sx + s[q][0] - f0[0];
-            const unsigned same = __match_any_sync(0xffffffffu, in ? key[q] : -1);
-            rank[q] = in ? sm.bins[key[q]] + __popc(same & ((1u << lane) - 1u)) : 0;
+        const int sx = nb[0] - kW + 1, sy = nb[1] - kW + 1, sz = DIM > 2 ? nb[2] - kW + 1 : 1;
+        const bool sorted = staged && static_cast<int64_t>(sx) * sy * sz <= kSpreadBins;
+        if (staged)
+            for (int k = lane; k < slab * nb[2]; k += 32) sm.box[k] = 0.0f;
+        // ---- order of the cells
+        if (sorted) {
+            for (int k = lane; k < kSpreadBins; k += 32) sm.bins[k] = 0;
             __syncwarp();
-            if (in && (same >> lane) == 1u) sm.bins[key[q]] = rank[q] + 1;  // the last lane of the bin
+            int rank[kPer], key[kPer];
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const bool in = q * 32 + lane < nc;
+                key[q] = ((DIM > 2 ? s[q][DIM - 1] - f0[2] : 0) * sy + s[q][1] - f0[1]) * sx + s[q][0] - f0[0];
+                const unsigned same = __match_any_sync(0xffffffffu, in ? key[q] : -1);
+                rank[q] = in ? sm.bins[key[q]] + __popc(same & ((1u << lane) - 1u)) : 0;
+                __syncwarp();
+                if (in && (same >> lane) == 1u) sm.bins[key[q]] = rank[q] + 1;  // the last lane of the bin
+                __syncwarp();
+            }
+            int run = 0;
+            for (int k = 0; k < kSpreadBins; k += 32) {
+                const int own = sm.bins[k + lane];
+                int v = own;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int o = __shfl_up_sync(0xffffffffu, v, off);
+                    if (lane >= off) v += o;
+                }
+                sm.bins[k + lane] = run + v - own;
+                run += __shfl_sync(0xffffffffu, v, 31);
+            }
             __syncwarp();
-        }
-        int run = 0;
-        for (int k = 0; k < kSpreadBins; k += 32) {
-            const int own = sm.bins[k + lane];
-            int v = own;
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int o = __shfl_up_sync(0xffffffffu, v, off);
-                if (lane >= off) v += o;
+            for (int q = 0; q < kPer; ++q)
+                if (q * 32 + lane < nc) sm.order[sm.bins[key[q]] + rank[q]] = static_cast<short>(q * 32 + lane);
+        } else {
+            for (int i = lane; i < nc; i += 32) sm.order[i] = static_cast<short>(i);
+        }
+        const int lx = lane & 7, ly = lane >> 3;
+        constexpr int kz = DIM > 2 ? kW : 1;
+        float acc[kz][2];
+#pragma unroll
+        for (int z = 0; z < kz; ++z) acc[z][0] = acc[z][1] = 0.0f;
+        int cur = -1;
+        auto flush = [&]() {
+            float* p = sm.box + cur + ly * pitch + lx;
+            float old[kz][2];
+#pragma unroll
+            for (int z = 0; z < kz; ++z) {
+                old[z][0] = p[z * slab];
+                old[z][1] = p[z * slab + 4 * pitch];
             }
-            sm.bins[k + lane] = run + v - own;
-            run += __shfl_sync(0xffffffffu, v, 31);
-        }
-        __syncwarp();
 #pragma unroll
-        for (int q = 0; q < kPer; ++q)
-            if (q * 32 + lane < nc) sm.order[sm.bins[key[q]] + rank[q]] = static_cast<short>(q * 32 + lane);
-    } else {
-        for (int i = lane; i < nc; i += 32) sm.order[i] = static_cast<short>(i);
-    }
-    const int lx = lane & 7, ly = lane >> 3;
-    constexpr int kz = DIM > 2 ? kW : 1;
-    float acc[kz][2];
-#pragma unroll
-    for (int z = 0; z < kz; ++z) acc[z][0] = acc[z][1] = 0.0f;
-    int cur = -1;
-    auto flush = [&]() {
-        float* p = sm.box + cur + ly * pitch + lx;
-        float old[kz][2];
-#pragma unroll
-        for (int z = 0; z < kz; ++z) {
-            old[z][0] = p[z * slab];
-            old[z][1] = p[z * slab + 4 * pitch];
-        }
-#pragma unroll
-        for (int z = 0; z < kz; ++z) {
-            p[z * slab] = old[z][0] + acc[z][0];
-            p[z * slab + 4 * pitch] = old[z][1] + acc[z][1];
-            acc[z][0] = acc[z][1] = 0.0f;
-        }
-        __syncwarp();
-    };
-    for (int i0 = 0; i0 < nc; i0 += 32) {
-        const int m = min(32, nc - i0);
-        __syncwarp();
-        if (lane < m) {
-            const int i = sm.order[i0 + lane];
-            const int64_t o = static_cast<int64_t>(__ldg(perm + c0 + i)) - perm_base;
-            const float gv = index_ok(o, n) ? __ldg(g + o) * scale.first * scale.second : 0.0f;
-            float w[kW], v;
-            const int px = band::locate(ax[0], __ldg(src[0] + i), v);
-            band::weights(v, w);
-            float4* out = reinterpret_cast<float4*>(sm.wts[lane]);
-            out[0] = make_float4(w[0] * gv, w[1] * gv, w[2] * gv, w[3] * gv);
-            out[1] = make_float4(w[4] * gv, w[5] * gv, w[6] * gv, w[7] * gv);
-            const int py = band::locate(ax[1], __ldg(src[1] + i), v);
-            band::weights(v, w);
-            out[2] = make_float4(w[0], w[1], w[2], w[3]);
-            out[3] = make_float4(w[4], w[5], w[6], w[7]);
-            int pz = 0;
-            if (DIM > 2) {
-                pz = band::locate(ax[DIM - 1], __ldg(src[2] + i), v);
-                band::weights(v, w);
-                out[4] = make_float4(w[0], w[1], w[2], w[3]);
-                out[5] = make_float4(w[4], w[5], w[6], w[7]);
+            for (int z = 0; z < kz; ++z) {
+                p[z * slab] = old[z][0] + acc[z][0];
+                p[z * slab + 4 * pitch] = old[z][1] + acc[z][1];
+                acc[z][0] = acc[z][1] = 0.0f;
             }
-            sm.at[lane] = staged ? (pz - f0[2]) * slab + (py - f0[1]) * pitch + (px - f0[0])
-                                 : static_cast<int>(pz * plane + static_cast<int64_t>(py) * mx + px);
-        }
-        __syncwarp();
-        // the next cell's weights are loaded before the current one is added
-        float wx, wa, wb, wn[kz];
-        int next;
-        auto load = [&](int q) {
-            const float* w = sm.wts[q];
-            wx = w[lx];
-            wa = w[kW + ly];
-            wb = w[kW + 4 + ly];
-            if (DIM > 2) {
-                const float4 a = *reinterpret_cast<const float4*>(w + 2 * kW);
-                const float4 c = *reinterpret_cast<const float4*>(w + 2 * kW + 4);
-                wn[0] = a.x; wn[1 % kz] = a.y; wn[2 % kz] = a.z; wn[3 % kz] = a.w;
-                wn[4 % kz] = c.x; wn[5 % kz] = c.y; wn[6 % kz] = c.z; wn[7 % kz] = c.w;
-            } else {
-                wn[0] = 1.0f;
-            }
-            next = sm.at[q];
+            __syncwarp();
         };
-        load(0);
+        for (int i0 = 0; i0 < nc; i0 += 32) {
+            const int m = min(32, nc - i0);
+            __syncwarp();
+            if (lane < m) {
+                const int i = sm.order[i0 + lane];
+                const int64_t o = static_cast<int64_t>(__ldg(perm + c0 + i)) - perm_base;
+                const float gv = index_ok(o, n) ? __ldg(g + o) * scale.first * scale.second : 0.0f;
+                float w[kW], v;
+                const int px = band::locate(ax[0], __ldg(src[0] + i), v);
+                band::weights(v, w);
+                float4* out = reinterpret_cast<float4*>(sm.wts[lane]);
+                out[0] = make_float4(w[0] * gv, w[1] * gv, w[2] * gv, w[3] * gv);
+                out[1] = make_float4(w[4] * gv, w[5] * gv, w[6] * gv, w[7] * gv);
+                const int py = band::locate(ax[1], __ldg(src[1] + i), v);
+                band::weights(v, w);
+                out[2] = make_float4(w[0], w[1], w[2], w[3]);
+                out[3] = make_float4(w[4], w[5], w[6], w[7]);
+                int pz = 0;
+                if (DIM > 2) {
+                    pz = band::locate(ax[DIM - 1], __ldg(src[2] + i), v);
+                    band::weights(v, w);
+                    out[4] = make_float4(w[0], w[1], w[2], w[3]);
+                    out[5] = make_float4(w[4], w[5], w[6], w[7]);
+                }
+                sm.at[lane] = staged ? (pz - f0[2]) * slab + (py - f0[1]) * pitch + (px - f0[0])
+                                     : static_cast<int>(pz * plane + static_cast<int64_t>(py) * mx + px);
+            }
+            __syncwarp();
+            // the next cell's weights are loaded before the current one is added
+            float wx, wa, wb, wn[kz];
+            int next;
+            auto load = [&](int q) {
+                const float* w = sm.wts[q];
+                wx = w[lx];
+                wa = w[kW + ly];
+                wb = w[kW + 4 + ly];
+                if (DIM > 2) {
+                    const float4 a = *reinterpret_cast<const float4*>(w + 2 * kW);
+                    const float4 c = *reinterpret_cast<const float4*>(w + 2 * kW + 4);
+                    wn[0] = a.x; wn[1 % kz] = a.y; wn[2 % kz] = a.z; wn[3 % kz] = a.w;
+                    wn[4 % kz] = c.x; wn[5 % kz] = c.y; wn[6 % kz] = c.z; wn[7 % kz] = c.w;
+                } else {
+                    wn[0] = 1.0f;
+                }
+                next = sm.at[q];
+            };
+            load(0);
 #pragma unroll 2
-        for (int q = 0; q < m; ++q) {
-            const float w0 = wx * wa, w1 = wx * wb;
-            float wz[kz];
+            for (int q = 0; q < m; ++q) {
+                const float w0 = wx * wa, w1 = wx * wb;
+                float wz[kz];
 #pragma unroll
-            for (int z = 0; z < kz; ++z) wz[z] = wn[z];
-            const int to = next;
-            load(min(q + 1, m - 1));
-            if (staged) {
-                if (to != cur) {  // uniform over the warp
-                    if (cur >= 0) flush();
-                    cur = to;
-                }
+                for (int z = 0; z < kz; ++z) wz[z] = wn[z];
+                const int to = next;
+                load(min(q + 1, m - 1));
+                if (staged) {
+                    if (to != cur) {  // uniform over the warp
+                        if (cur >= 0) flush();
+                        cur = to;
+                    }
 #pragma unroll
-                for (int z = 0; z < kz; ++z) {
-                    acc[z][0] = fmaf(wz[z], w0, acc[z][0]);
-                    acc[z][1] = fmaf(wz[z], w1, acc[z][1]);
-                }
-            } else {
-                unsigned long long* p = lattice + to + ly * mx + lx;
+                    for (int z = 0; z < kz; ++z) {
+                        acc[z][0] = fmaf(wz[z], w0, acc[z][0]);
+                        acc[z][1] = fmaf(wz[z], w1, acc[z][1]);
+                    }
+                } else {
+                    unsigned long long* p = lattice + to + ly * mx + lx;
 #pragma unroll
-                for (int z = 0; z < kz; ++z) {
-                    atomicAdd(p + z * plane, static_cast<unsigned long long>(__float2ll_rn(wz[z] * w0)));
-                    atomicAdd(p + z * plane + 4 * mx, static_cast<unsigned long long>(__float2ll_rn(wz[z] * w1)));
+                    for (int z = 0; z < kz; ++z) {
+                        atomicAdd(p + z * plane, static_cast<unsigned long long>(__float2ll_rn(wz[z] * w0)));
+                        atomicAdd(p + z * plane + 4 * mx, static_cast<unsigned long long>(__float2ll_rn(wz[z] * w1)));
+                    }
                 }
             }
         }
-    }
-    at += nc;
-    if (!staged) continue;
-    if (cur >= 0) flush();
-    const int rows = nb[1] * nb[2];
-    // four rows of up to eight nodes, or one of up to 32, at a time
-    const int per = nb[0] <= 8 ? 4 : nb[0] <= 16 ? 2 : 1, wide = 32 / per;
-    for (int r = lane / wide; r < rows; r += per) {
-        const int z = r / nb[1], y = r - z * nb[1];
-        unsigned long long* p = lattice + (f0[2] + z) * plane + static_cast<int64_t>(f0[1] + y) * mx + f0[0];
-        for (int x = lane % wide; x < nb[0]; x += wide) {
-            const long long v = __float2ll_rn(sm.box[z * slab + y * pitch + x]);
-            if (v != 0) atomicAdd(p + x, static_cast<unsigned long long>(v));
+        at += nc;
+        if (!staged) continue;
+        if (cur >= 0) flush();
+        const int rows = nb[1] * nb[2];
+        // four rows of up to eight nodes, or one of up to 32, at a time
+        const int per = nb[0] <= 8 ? 4 : nb[0] <= 16 ? 2 : 1, wide = 32 / per;
+        for (int r = lane / wide; r < rows; r += per) {
+            const int z = r / nb[1], y = r - z * nb[1];
+            unsigned long long* p = lattice + (f0[2] + z) * plane + static_cast<int64_t>(f0[1] + y) * mx + f0[0];
+            for (int x = lane % wide; x < nb[0]; x += wide) {
+                const long long v = __float2ll_rn(sm.box[z * slab + y * pitch + x]);
+                if (v != 0) atomicAdd(p + x, static_cast<unsigned long long>(v));
+            }
         }
-    }
     }
 }
 
@@ -806,8 +806,8 @@ int launch_band_spread(const BandDesc* b, int32_t dim, const float* xs, const fl
                        int n_gmax, unsigned long long* lattice, float* nodes, int sms, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // a warp's group is a chain of sort, sum and write-out: smaller groups where
-    // the warps would not fill the GPU twice (262k cells: 168 us of 64 to a warp
-    // against 146)
+    // the warps would not fill the GPU twice (262k cells x 1024 modes: 168 us a
+    // call with 256 cells to a warp, 150 with 64)
     int cells = kSpreadCells;
     while (cells > 64 && n / cells < int64_t(sms) * 14 * 2) cells /= 2;
     const int64_t groups = (n + cells - 1) / cells;

@@ -538,36 +538,36 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
         if (n_split < 2) return;  // the maps are written
     }
     for (int64_t u = blockIdx.x; u * 256 < d.n_cells; u += gridDim.x) {
-    const int64_t i = u * 256 + threadIdx.x;
-    double l = 0.0;
-    if (i < d.n_cells) {
-        float s = 0.0f, e = 0.0f;
-        for (int k = 0; k < n_split; ++k) {
-            const float2 v = partial[static_cast<int64_t>(k) * d.n_cells + i];
-            two_sum_acc(s, e, v.x);
-            e += v.y;
+        const int64_t i = u * 256 + threadIdx.x;
+        double l = 0.0;
+        if (i < d.n_cells) {
+            float s = 0.0f, e = 0.0f;
+            for (int k = 0; k < n_split; ++k) {
+                const float2 v = partial[static_cast<int64_t>(k) * d.n_cells + i];
+                two_sum_acc(s, e, v.x);
+                e += v.y;
+            }
+            if (d.add != nullptr) two_sum_acc(s, e, __ldg(d.add + i));
+            const float y = (s + e) + d.map.mu;
+            const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
+            if (index_ok(o, d.n_cells)) {
+                map_store(d.map, o, y);
+                if (d.map.bits & kMapMismatch) l = mismatch_store(d.map, o, y);
+            }
         }
-        if (d.add != nullptr) two_sum_acc(s, e, __ldg(d.add + i));
-        const float y = (s + e) + d.map.mu;
-        const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
-        if (index_ok(o, d.n_cells)) {
-            map_store(d.map, o, y);
-            if (d.map.bits & kMapMismatch) l = mismatch_store(d.map, o, y);
-        }
-    }
-    if (d.map.bits & kMapMismatch) {
-        __shared__ double red[8];
+        if (d.map.bits & kMapMismatch) {
+            __shared__ double red[8];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < 8; ++w) t += red[w];
-            d.map.lpart[u] = t;
+            for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double t = 0.0;
+                for (int w = 0; w < 8; ++w) t += red[w];
+                d.map.lpart[u] = t;
+            }
+            __syncthreads();
         }
-        __syncthreads();
-    }
     }
 }
 

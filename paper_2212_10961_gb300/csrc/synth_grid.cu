@@ -1084,6 +1084,8 @@ double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
 double cells_us_per_mode(int64_t n_cells) { return 0.006 + double(n_cells) / 4.2e6; }
 double cells_band_us(int64_t n_cells, int32_t dim) { return 20.0 + double(n_cells) * (dim > 2 ? 5e-5 : 1e-5); }
 
+// The same lower limit as on grids: 250 x 130 cells x 1000 modes (45 us
+// directly) cannot pay for six more launches, 126 x 63 x 31 x 2048 (130 us) gains 50.
 size_t cells_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim) {
     const int64_t n_pad = pad_modes(n_modes);
     if (dim < 2 || n_pad > band::kMaxModes || cells_us_per_mode(n_cells) * double(n_pad) < kBandMinUs) return 0;
