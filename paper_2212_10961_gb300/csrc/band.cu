@@ -100,7 +100,7 @@ __device__ float candidate_time(const BandSelect& p, int heavy, int light, int m
     // frequencies, at most the bin's edge, may place the nodes less favourably
     const int64_t plane = static_cast<int64_t>(mx + 1) * (my + 1);
     if (plane * (mz + 1) > p.cap_nodes || (p.n[2] > 1 && plane * p.n[2] > p.cap_mid)) return 3.0e38f;
-    if ((mx + gridt::kGM) / gridt::kGM > p.cap_mt || my >= p.cap_yz || mz >= p.cap_yz) return 3.0e38f;
+    if (mx >= p.cap_ax[0] || my >= p.cap_ax[1] || mz >= p.cap_ax[2]) return 3.0e38f;
     const int64_t tile = gridt::kGM * gridt::kGN;
     const float nodes = static_cast<float>((static_cast<int64_t>(mx) * my * mz + tile - 1) / tile * tile);
     return direct + p.us_node * nodes * static_cast<float>(light) + p.us_fixed;

@@ -1732,6 +1732,34 @@ int grf_debug_grid_path(int32_t enable, int32_t fold_chunks) {
     return GRF_OK;
 }
 
+int grf_debug_lattice_room(int32_t kind, int32_t dim, const int64_t* cells, int64_t n_modes, int64_t* out) try {
+    if (!cells || !out) return fail(GRF_EINVAL, "NULL argument");
+    if (kind < 0 || kind > 3 || dim < 2 || dim > 3 || n_modes < 1 || n_modes > GRF_MAX_MODES)
+        return fail(GRF_EINVAL, "kind must be in 0..3, dim 2 or 3, n_modes in range");
+    int64_t n = 1;
+    for (int c = 0; c < (kind < 2 ? 1 : 3); ++c) {
+        if (cells[c] < 1 || cells[c] > INT32_MAX / n) return fail(GRF_EINVAL, "cell counts out of range");
+        n *= cells[c];
+    }
+    const int64_t n_pad = table_layout(n_modes).n_pad;
+    const int32_t g[3] = {static_cast<int32_t>(cells[0]), static_cast<int32_t>(kind < 2 ? 1 : cells[1]),
+                          static_cast<int32_t>(kind < 2 ? 1 : cells[2])};
+    const LatticeRoom r = kind == 0   ? cells_room(n, n_modes, dim)
+                          : kind == 1 ? cells_adjoint_room(n, n_modes, dim)
+                          : kind == 2 ? grid_room(g[0], g[1], g[2], n_pad)
+                                      : grid_adjoint_room(g[0], g[1], g[2], n_pad);
+    for (int c = 0; c < 3; ++c) {
+        out[c] = r.limit[c];
+        out[3 + c] = r.held[c];
+    }
+    out[6] = r.nodes;
+    out[7] = r.nodes_held;
+    out[8] = r.bytes;
+    return GRF_OK;
+} catch (...) {
+    return host_exception();
+}
+
 int grf_debug_mma_f16(const uint16_t* A, const uint16_t* B, int32_t k_chunks, float* D, int32_t* status_dev,
                       void* stream) try {
     if (!A || !B || !D || !status_dev) return fail(GRF_EINVAL, "NULL argument");

@@ -345,7 +345,7 @@ struct BandSelect {
     int64_t cap_part;        // floats of the nodes' partial sums
     int64_t cap_mid;         // most (x, y) nodes x z cells
     int32_t cap_mt;          // most 128-row tiles of the nodes' x operand
-    int32_t cap_yz;          // the y and z axes have fewer nodes than this
+    int32_t cap_ax[3];       // most nodes of an axis (grids: at most its cells besides)
     int32_t fold;
     int32_t n_mt;            // x tiles of the cells
     int32_t* lstart;         // [n_mt] first x node of a tile (written here; null: no light chunks)
@@ -356,6 +356,15 @@ struct BandSelect {
     int64_t loss_nb_finalize;
     const TableHeader* thdr;
     GridTiling cells;        // the cells' tiling (all modes)
+};
+
+// Room of a band-path call's workspace for the lattice's tables, next to what
+// the selection accepts (grf_debug_lattice_room).
+struct LatticeRoom {
+    int64_t limit[3];  // most nodes of an axis that the selection accepts
+    int64_t held[3];   // nodes of an axis that the tables hold
+    int64_t nodes, nodes_held;
+    int64_t bytes;     // the lattice's part of the workspace (0: not offered)
 };
 
 // Adjoint on the band path (band_bwd.cu): one axis of a grid's transposed
@@ -521,6 +530,10 @@ double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
 constexpr double kBandNodeAdjUs = 1.0 / 6.0e6;
 double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz);
 size_t cells_adjoint_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
+LatticeRoom cells_adjoint_room(int64_t n_cells, int64_t n_modes, int32_t dim);
+LatticeRoom cells_room(int64_t n_cells, int64_t n_modes, int32_t dim);
+LatticeRoom grid_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
+LatticeRoom grid_adjoint_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
 double cells_adjoint_us_per_mode(int64_t n_cells);
 double cells_adjoint_band_us(int64_t n_cells, int32_t dim);
 // max |g| (inf if some g is not finite) and compensated sums of g, per block of

@@ -772,13 +772,13 @@ struct CellsAdjLayout {
     int64_t off_idx, idx, off_rank, off_gmax, off_gsum, off_xmax, off_gain, off_fixed, off_nodes,
         off_ph[3], off_off[3], off_part, total;
     int64_t cap_nodes;
-    int32_t cap_yz;
+    int32_t cap_ax;  // nodes of an axis that the phasor tables and the partial sums hold
 };
 CellsAdjLayout cells_adj_layout(int64_t n, int64_t n_pad, int32_t dim) {
     CellsAdjLayout L{};
     L.cap_nodes = std::max<int64_t>(n, 65536);
     const double side = std::pow(double(L.cap_nodes), 1.0 / dim);
-    L.cap_yz = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
+    L.cap_ax = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
     int64_t off = 0;
     auto take = [&](int64_t bytes) {
         const int64_t o = off;
@@ -796,16 +796,40 @@ CellsAdjLayout cells_adj_layout(int64_t n, int64_t n_pad, int32_t dim) {
     L.off_fixed = take(L.cap_nodes * 8);
     L.off_nodes = take(L.cap_nodes * 4);
     for (int c = 0; c < 3; ++c) {
-        const int64_t m = c < dim ? L.cap_yz : 1;
+        const int64_t m = c < dim ? L.cap_ax : 1;
         L.off_ph[c] = take(m * n_pad * 8);
         L.off_off[c] = take(m * 4);
     }
-    const int64_t tiles = n_pad / 128 * ((int64_t(L.cap_yz) + 63) / 64);
+    const int64_t tiles = n_pad / 128 * ((int64_t(L.cap_ax) + 63) / 64);
     L.off_part = take(std::max<int64_t>(256 * 3, tiles) * 128 * 5 * 8);
     L.total = off;
     return L;
 }
+
+void set_limits(BandSelect& s, const CellsAdjLayout& L) {
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_nodes;
+    s.cap_mt = INT32_MAX / 256;  // no operand tiles at the nodes
+    for (int c = 0; c < 3; ++c) s.cap_ax[c] = L.cap_ax;
+}
 }  // namespace
+
+LatticeRoom cells_adjoint_room(int64_t n_cells, int64_t n_modes, int32_t dim) {
+    LatticeRoom r{};
+    r.bytes = static_cast<int64_t>(cells_adjoint_band_ws_bytes(n_cells, n_modes, dim));
+    if (r.bytes == 0) return r;
+    const int64_t n_pad = pad_modes(n_modes);
+    const CellsAdjLayout L = cells_adj_layout(n_cells, n_pad, dim);
+    BandSelect s{};
+    set_limits(s, L);
+    for (int c = 0; c < 3; ++c) {
+        r.limit[c] = c < dim ? s.cap_ax[c] : 1;
+        r.held[c] = (L.off_off[c] - L.off_ph[c]) / (n_pad * 8);
+    }
+    r.nodes = s.cap_nodes;
+    r.nodes_held = (L.off_ph[0] - L.off_nodes) / 4;
+    return r;
+}
 
 // The direct modes' rate (exact phases, a hardware sine and cosine per pair);
 // the lattice's spread 0.11 ns per cell in 3-D.
@@ -890,10 +914,7 @@ int launch_synth_bwd(const void* table, int64_t n_modes, int32_t dim, double sig
         s.us_mode = static_cast<float>(cells_adjoint_us_per_mode(n_cells));
         s.us_node = static_cast<float>(kBandNodeAdjUs);
         s.us_fixed = static_cast<float>(cells_adjoint_band_us(n_cells, dim));
-        s.cap_nodes = L.cap_nodes;
-        s.cap_part = L.cap_nodes;
-        s.cap_mt = (L.cap_yz + 127) / 128;
-        s.cap_yz = L.cap_yz;
+        set_limits(s, L);
         s.fold = 1;
         s.chunk = 1;
         s.us_heavy = 5.0f;

@@ -901,6 +901,17 @@ BandLayout band_layout(const GridGeom& gg, const GridPlan& g) {
     return L;
 }
 
+// What the selection may choose, from what the layout holds: the rows of the
+// x operand; the y and z tables have a row per cell.
+void set_limits(BandSelect& s, const BandLayout& L) {
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_part;
+    s.cap_mid = L.cap_mid;
+    s.cap_mt = L.cap_mt;
+    s.cap_ax[0] = L.cap_mt * kGM;
+    s.cap_ax[1] = s.cap_ax[2] = INT32_MAX;
+}
+
 // Sizes at which a call on a grid may take the band path: the selection's
 // modes, at least half a finalize block of x cells and 4 rows per block (its
 // loss partials), and a direct sum of at least 50 us, below which the lattice's
@@ -972,17 +983,13 @@ int launch_band(const GridPrep& p, const GridDesc& d, const GridGeom& gg, const 
     s.us_node = static_cast<float>(kBandNodeUs);
     s.us_fixed = static_cast<float>(kBandFixedUs);
     s.us_heavy = 12.0f;
-    s.cap_nodes = L.cap_nodes;
-    s.cap_part = L.cap_part;
-    s.cap_mid = L.cap_mid;
-    s.cap_mt = L.cap_mt;
+    set_limits(s, L);
     s.fold = fc;
     s.n_mt = gp.n_mt;
     s.lstart = split ? nullptr : reinterpret_cast<int32_t*>(w + L.off_lstart);
     s.max_split = gp.max_split;
     s.split_cells = split ? 1 : 0;
     s.chunk = kGModes;
-    s.cap_yz = INT32_MAX;
     s.loss_nb_tiles = d.t.n_tiles * kGEpiWarps;
     s.loss_nb_finalize = band_finalize_blocks(gg);
     s.thdr = p.thdr;
@@ -1064,7 +1071,50 @@ CellsLayout cells_layout(int64_t n, int64_t n_pad, int32_t dim) {
     return L;
 }
 
+void set_limits(BandSelect& s, const CellsLayout& L) {
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_part;
+    s.cap_mt = L.cap_mt;
+    s.cap_ax[0] = L.cap_mt * kGM;
+    s.cap_ax[1] = s.cap_ax[2] = L.cap_yz;
+}
+
 }  // namespace
+
+LatticeRoom cells_room(int64_t n, int64_t n_modes, int32_t dim) {
+    LatticeRoom r{};
+    const int64_t n_pad = pad_modes(n_modes), nc = n_pad / kGModes;
+    r.bytes = static_cast<int64_t>(cells_band_ws_bytes(n, n_modes, dim));
+    if (r.bytes == 0) return r;
+    const CellsLayout L = cells_layout(n, n_pad, dim);
+    BandSelect s{};
+    set_limits(s, L);
+    for (int c = 0; c < 3; ++c) r.limit[c] = c < dim ? s.cap_ax[c] : 1;
+    r.held[0] = L.a_bytes / (nc * kGPair) * kGM;
+    r.held[1] = dim > 2 ? L.y_bytes / (nc * kGRowBytes) : L.b_bytes / (nc * kGPair) * kGN;
+    r.held[2] = dim > 2 ? L.w_bytes / (nc * kGRowBytes) : 1;
+    r.nodes = s.cap_nodes;
+    r.nodes_held = (L.off_add - L.off_part) / 4;
+    return r;
+}
+
+LatticeRoom grid_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    LatticeRoom r{};
+    r.bytes = static_cast<int64_t>(grid_band_ws_bytes(nx, ny, nz, n_pad));
+    if (r.bytes == 0) return r;
+    const GridPlan g = grid_plan(nx, ny, nz, chunks_of(n_pad));
+    const BandLayout L = band_layout(GridGeom{nx, ny, nz, nullptr, nullptr, nullptr, nullptr}, g);
+    BandSelect s{};
+    set_limits(s, L);
+    const int64_t n[3] = {nx, ny, nz};
+    for (int c = 0; c < 3; ++c) r.limit[c] = std::min<int64_t>(s.cap_ax[c], n[c]);
+    r.held[0] = int64_t(L.cap_mt) * kGM;
+    r.held[1] = g.form ? g.y_bytes / (g.nc * kGRowBytes) : g.b_bytes / (int64_t(g.nc) * kGPair) * kGN;
+    r.held[2] = g.form ? g.w_bytes / (g.nc * kGRowBytes) : 1;
+    r.nodes = s.cap_nodes;
+    r.nodes_held = (L.off_mid - L.off_part) / 4;
+    return r;
+}
 
 size_t grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
     const GridPlan g = grid_plan(nx, ny, nz, chunks_of(n_pad));
@@ -1134,10 +1184,7 @@ int launch_cells_band(const void* table, int64_t n_modes, FwdDesc& fd, const Seg
     s.us_node = static_cast<float>(kBandNodeUs);
     s.us_fixed = static_cast<float>(cells_band_us(fd.n_cells, fd.dim));
     s.us_heavy = 5.0f;
-    s.cap_nodes = L.cap_nodes;
-    s.cap_part = L.cap_part;
-    s.cap_mt = L.cap_mt;
-    s.cap_yz = L.cap_yz;
+    set_limits(s, L);
     s.fold = 1;  // as exact as the direct sum (3.0e-7 of sigma); 2 would save 9 of 370 us and give 3.0e-7 to 3.1e-7
     s.chunk = kChunk;
     s.max_split = max_split;

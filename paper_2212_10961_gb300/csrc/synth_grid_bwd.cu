@@ -774,6 +774,14 @@ AdjBandLayout adj_band_layout(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad,
     return L;
 }
 
+void set_limits(BandSelect& s, const AdjBandLayout& L) {
+    s.cap_nodes = L.cap_nodes;
+    s.cap_part = L.cap_nodes;
+    s.cap_mid = L.cap_mid;
+    s.cap_mt = INT32_MAX / 256;  // no operand tiles at the nodes
+    for (int c = 0; c < 3; ++c) s.cap_ax[c] = INT32_MAX;  // tables by cells
+}
+
 int adj_init() {
     if (g_adj_sms != 0) return cudaSuccess;
     int dev = 0, sms = 0;
@@ -802,6 +810,23 @@ size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad)
     if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 60.0)
         return 0;
     return static_cast<size_t>(adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total);
+}
+
+LatticeRoom grid_adjoint_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    LatticeRoom r{};
+    r.bytes = static_cast<int64_t>(bwd_grid_band_ws_bytes(nx, ny, nz, n_pad));
+    if (r.bytes == 0) return r;
+    const AdjBandLayout L = adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas);
+    BandSelect s{};
+    set_limits(s, L);
+    const int64_t n[3] = {nx, ny, nz};
+    for (int c = 0; c < 3; ++c) {
+        r.limit[c] = std::min<int64_t>(s.cap_ax[c], n[c]);
+        r.held[c] = (L.off_off[c] - L.off_ph[c]) / (n_pad * 8);
+    }
+    r.nodes = s.cap_nodes;
+    r.nodes_held = (L.off_part - L.off_nodes) / 4;
+    return r;
 }
 
 int adj_scan_blocks() { return kAScanBlocks; }
@@ -904,11 +929,7 @@ int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const
         s.us_fixed = static_cast<float>(grid_adjoint_band_us(gg.nx, gg.ny, gg.nz));
         // the direct modes' tables hold all of g, and their units run at any count
         s.us_heavy = 10.0f + static_cast<float>(9e-6 * double(n));
-        s.cap_nodes = L.cap_nodes;
-        s.cap_part = L.cap_nodes;
-        s.cap_mid = L.cap_mid;
-        s.cap_mt = INT32_MAX / 256;
-        s.cap_yz = INT32_MAX;
+        set_limits(s, L);
         s.fold = 1;
         s.chunk = kAM;
         s.max_split = 1;

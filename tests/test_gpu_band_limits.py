@@ -1,0 +1,53 @@
+"""GPU tests of the node lattice near the limits of its tables: cells of any
+plan whose field varies much faster along one axis than along the others, so
+that one axis takes as many nodes as the selection allows."""
+import numpy as np
+import pytest
+
+from helpers import check_forward, oracle_field, to_dev
+from test_gpu_band import _check_adjoint, _modes, _params, env  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+GUARD = 1 << 20
+
+
+class _Guarded:
+    """A workspace of exactly the bytes asked for, inside a larger allocation
+    whose other bytes must stay as they are."""
+
+    def __init__(self, torch):
+        self.torch, self.all = torch, None
+
+    def get(self, nbytes, device):
+        n = (int(nbytes) + 255) // 256 * 256
+        self.all = self.torch.full((n + 2 * GUARD,), 0xa5, dtype=self.torch.uint8, device=device)
+        return self.all[GUARD:GUARD + n]
+
+    def untouched(self):
+        return bool((self.all[:GUARD] == 0xa5).all()) and bool((self.all[-GUARD:] == 0xa5).all())
+
+
+@pytest.mark.parametrize("fine", [0, 1, 2])
+@pytest.mark.parametrize("cells", [100_000, 262_144])
+def test_one_fine_axis(env, cells, fine):  # noqa: F811
+    torch, F, W = env
+    ell = [0.3, 0.3, 0.3]
+    ell[fine] = 0.01
+    c = [np.ascontiguousarray(v) for v in np.random.default_rng(5).random((cells, 3)).astype(np.float32).T]
+    n = 4096
+    _check_adjoint(env, c, tuple(ell), n, "gaussian")
+    plan = F.CellPlan(*to_dev(torch, c))
+    m = _modes(n, 3, tuple(ell), "gaussian", 6)
+    table, p = F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, n, 3, tuple(ell))
+    g = torch.randn(cells, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    ws = _Guarded(torch)
+    guarded = F.backward(table, p, plan, g, workspace=ws)
+    assert ws.untouched()
+    plain = F.backward(table, p, plan, g)
+    assert all(torch.equal(guarded[k], plain[k]) for k in ("dA", "dpsi", "da"))
+    ws = _Guarded(torch)
+    y = F.synth(table, p, plan, workspace=ws)["Y"].cpu().numpy()
+    assert ws.untouched()
+    idx = np.random.default_rng(2).choice(cells, 6000, replace=False)
+    check_forward(y[idx], oracle_field(m, 0.25, c, idx), 1.0, "fine axis %d" % fine)
