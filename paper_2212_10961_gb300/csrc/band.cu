@@ -88,6 +88,14 @@ __device__ __forceinline__ float4 mode_of(const BandSelect& p, int j) {
     return make_float4(fabsf(c0.x), fabsf(c0.z), fabsf(c1.x), fabsf(__ldg(&p.hot[j].w)));
 }
 
+// Whether the workspace holds a lattice of mx x my x mz nodes.
+__device__ __forceinline__ bool lattice_fits(const BandSelect& p, int mx, int my, int mz) {
+    if (max(mx, max(my, mz)) >= 1 << 20) return false;  // the products below fit
+    const int64_t plane = static_cast<int64_t>(mx) * my;
+    return mx <= p.cap_ax[0] && my <= p.cap_ax[1] && mz <= p.cap_ax[2] && plane * mz <= p.cap_nodes &&
+           (p.n[2] <= 1 || plane * p.n[2] <= p.cap_mid);
+}
+
 // Estimated time of summing `light` modes at mx x my x mz nodes (whole
 // tensor-core tiles of 128 x 128) and `heavy` directly; 3e38 where the
 // lattice does not fit the workspace.
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     }
     __syncthreads();
     const int pick = static_cast<int>(best & 0xffffffffu);
-    const int n_light = pick < kBins ? count[pick] : 0, nh = n - n_light;
+    int n_light = pick < kBins ? count[pick] : 0;
     // the light modes' own largest frequencies, at most the bin's edges
     if (n_light > 0) {
         float a[3] = {0.0f, 0.0f, 0.0f};
@@ -280,13 +288,20 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     }
     __syncthreads();
     if (t < 3) {
-        BandAxis ax{0.0f, 0.0f, 0, n_light > 0 ? 1 : 0, 1};
+        BandAxis ax{0.0f, 0.0f, 0, 1, 1};
         if (n_light > 0 && t < dim) node_axis(__int_as_float(amax[t]), lo[t], hi[t], p.n[t], ax);
         axs[t] = ax;
-        out->ax[t] = ax;
     }
     __syncthreads();
-    const BandAxis ax[3] = {axs[0], axs[1], axs[2]};
+    // The candidates' sizes come from the bins' edges, which a mode at an edge
+    // may pass by a rounding, and from typical frequencies that underflow where
+    // all are tiny: what is taken is what fits with the modes' own frequencies.
+    if (n_light > 0 && !lattice_fits(p, axs[0].m, axs[1].m, axs[2].m)) n_light = 0;
+    const int nh = n - n_light;
+    const BandAxis none{0.0f, 0.0f, 0, 0, 1};
+    const BandAxis ax[3] = {n_light > 0 ? axs[0] : none, n_light > 0 ? axs[1] : none, n_light > 0 ? axs[2] : none};
+    if (t == 0)
+        for (int c = 0; c < 3; ++c) out->ax[c] = ax[c];
     // ---- slots of the light and the other modes, in table order, and a bound
     // of the light ones' amplitudes with their gains
     float top = 0.0f;

@@ -51,3 +51,23 @@ def test_one_fine_axis(env, cells, fine):  # noqa: F811
     assert ws.untouched()
     idx = np.random.default_rng(2).choice(cells, 6000, replace=False)
     check_forward(y[idx], oracle_field(m, 0.25, c, idx), 1.0, "fine axis %d" % fine)
+
+
+def test_frequencies_whose_scale_underflows(env):  # noqa: F811
+    # one mode of 2e-36 turns per unit among constant ones, over 3e38 units: the
+    # squared mean of the roots underflows, so that every mode looks constant
+    # and the selection's estimate is 9 nodes an axis; the mode needs 2000
+    torch, F, W = env
+    cells, n = 300_000, 60_000
+    c = [np.ascontiguousarray(v) for v in (np.random.default_rng(5).random((cells, 3)) * 3e38).astype(np.float32).T]
+    ell = (1e35,) * 3
+    m = _modes(n, 3, ell, "gaussian", 6)
+    m["a"][:] = 0.0
+    m["a"][17, 0] = 2e-36
+    m["amp"][17] = 1.0
+    plan = F.CellPlan(*to_dev(torch, c))
+    ws = _Guarded(torch)
+    y = F.synth(F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, n, 3, ell), plan, workspace=ws)["Y"].cpu().numpy()
+    assert ws.untouched() and plan.status() == 0
+    idx = np.random.default_rng(2).choice(cells, 6000, replace=False)
+    check_forward(y[idx], oracle_field(m, 0.25, c, idx), 1.0, "underflowing frequencies")
