@@ -805,8 +805,10 @@ double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz) { return 25.0 + 
 
 // Below 60 us of direct products the lattice's ten launches cost what they
 // save; at 110 us (128 x 128 x 128 cells x 2048 modes, with the forward pass)
-// they gain, 281 -> 241 us.
+// they gain, 281 -> 241 us.  The phasor tables are indexed in 32 bits: an axis
+// of 2^31 cells x modes (17 GB of table) keeps the products, which index in 64.
 size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
+    if (std::max(nx, std::max(ny, nz)) * n_pad >= int64_t(1) << 31) return 0;
     if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 60.0)
         return 0;
     return static_cast<size_t>(adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total);

@@ -44,6 +44,14 @@ def test_tables_hold_every_lattice_the_selection_accepts(kind, dim, cells, modes
     assert r["nodes"] <= r["nodes_held"]
 
 
+@pytest.mark.parametrize("shape,modes", [((66_000, 16_384), 65_000), ((70_000, 30_000), 40_000), ((16, 70_000, 500), 50_000),
+                                         ((9, 900, 70_000), 33_000), ((32_768, 2048), 65_536), ((16_384, 2048), 65_536)])
+def test_adjoint_tables_stay_within_32_bit_indices(shape, modes):
+    r = room(GRID_ADJOINT, len(shape), shape, modes)
+    n_pad = (modes + 127) // 128 * 128
+    assert all(r["held_" + c] * n_pad < 2 ** 31 for c in "xyz")
+
+
 def test_large_calls_are_offered_the_lattice():
     # so that the cases above are not all empty
     assert all(room(k, 3, c, 4096)["bytes"] > 0
