@@ -695,9 +695,10 @@ int grf_debug_grid_path(int32_t enable, int32_t fold_chunks);
  * grf_debug_lattice_room -- sizes of the node lattice's part of a workspace,
  * for tests.  kind: 0 synthesis at any cells, 1 its adjoint (cells[0] cells of
  * a dim-dimensional field), 2 synthesis on a grid, 3 its adjoint (cells[0..2]
- * per axis).  out (9): most nodes per axis that the selection accepts, nodes
- * per axis that the tables hold, most nodes accepted, nodes held, bytes; all
- * zero where the lattice is not offered.  GRF_EINVAL for NULL pointers or
+ * per axis).  out (10): most nodes per axis that the selection accepts, nodes
+ * per axis that the tables hold, most nodes accepted, nodes held, bytes of the
+ * lattice's part, bytes of a grid call's other part; all zero where the
+ * lattice is not offered.  GRF_EINVAL for NULL pointers or
  * values out of range.  Needs no device.
  */
 int grf_debug_lattice_room(int32_t kind, int32_t dim, const int64_t *cells, int64_t n_modes, int64_t *out);

@@ -297,6 +297,28 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     // may pass by a rounding, and from typical frequencies that underflow where
     // all are tiny: what is taken is what fits with the modes' own frequencies.
     if (n_light > 0 && !lattice_fits(p, axs[0].m, axs[1].m, axs[2].m)) n_light = 0;
+    // ---- light chunks: first x node of every tile, a multiple of 4 (16-byte
+    // loads of the rows), and the most nodes of a tile
+    if (p.lstart != nullptr && n_light > 0 && n_light < n) {
+        const BandAxis ax = axs[0];
+        for (int mt = warp; mt < p.n_mt; mt += kSelThreads / 32) {
+            int s0 = INT_MAX, s1 = 0;
+            for (int i = mt * gridt::kGM + lane; i < min((mt + 1) * gridt::kGM, p.n[0]); i += 32) {
+                float v;
+                const int s = ax.ident ? max(0, min(i, ax.m - kW)) : band::locate(ax, __ldg(p.X + i), v);
+                s0 = min(s0, s);
+                s1 = max(s1, s);
+            }
+            s0 = __reduce_min_sync(0xffffffffu, s0) & ~3;
+            s1 = __reduce_max_sync(0xffffffffu, s1);
+            if (lane == 0) {
+                p.lstart[mt] = s0;
+                atomicMax(&width, s1 + kW - s0);
+            }
+        }
+        __syncthreads();
+        if (width > p.cap_nl * gridt::kGK) n_light = 0;  // an axis in no order may need more than there is room for
+    }
     const int nh = n - n_light;
     const BandAxis none{0.0f, 0.0f, 0, 0, 1};
     const BandAxis ax[3] = {n_light > 0 ? axs[0] : none, n_light > 0 ? axs[1] : none, n_light > 0 ? axs[2] : none};
@@ -358,26 +380,6 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     {
         const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
         if (lane == 0) atomicMax(&gmax, static_cast<int>(w));
-    }
-    // ---- light chunks: first x node of every tile, a multiple of 4 (16-byte
-    // loads of the rows), and the most nodes of a tile
-    if (p.lstart != nullptr && n_light > 0 && nh > 0) {
-        for (int mt = warp; mt < p.n_mt; mt += kSelThreads / 32) {
-            int s0 = INT_MAX, s1 = 0;
-            for (int i = mt * gridt::kGM + lane; i < min((mt + 1) * gridt::kGM, p.n[0]); i += 32) {
-                float v;
-                const int s = ax[0].ident ? max(0, min(i, ax[0].m - kW))
-                                          : band::locate(ax[0], __ldg(p.X + i), v);
-                s0 = min(s0, s);
-                s1 = max(s1, s);
-            }
-            s0 = __reduce_min_sync(0xffffffffu, s0) & ~3;
-            s1 = __reduce_max_sync(0xffffffffu, s1);
-            if (lane == 0) {
-                p.lstart[mt] = s0;
-                atomicMax(&width, s1 + kW - s0);
-            }
-        }
     }
     __syncthreads();
     if (warp == 0) {

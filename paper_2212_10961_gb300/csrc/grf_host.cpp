@@ -293,8 +293,7 @@ bool use_grid_path(const GridGeom& gg) {
 // times N; beyond max(1 GB, 64 B per cell) -- N far above the cell count,
 // where the CUDA-core kernels need no tables -- it is not offered.
 bool grid_ws_ok(size_t bytes, const GridGeom& gg) {
-    const double cells = static_cast<double>(gg.nx) * gg.ny * gg.nz;
-    return static_cast<double>(bytes) <= std::max(double(1u << 30), 64.0 * cells);
+    return bytes <= static_cast<size_t>(ws_most(int64_t(gg.nx) * gg.ny * gg.nz));
 }
 
 // The grid shape of `plan` (single segment), resolving a pending check by
@@ -1755,6 +1754,7 @@ int grf_debug_lattice_room(int32_t kind, int32_t dim, const int64_t* cells, int6
     out[6] = r.nodes;
     out[7] = r.nodes_held;
     out[8] = r.bytes;
+    out[9] = r.base;
     return GRF_OK;
 } catch (...) {
     return host_exception();

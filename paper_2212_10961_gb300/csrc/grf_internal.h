@@ -227,6 +227,12 @@ struct FwdDesc {
 
 struct SegInfo;
 
+// Most bytes of a call's tables and partial sums beside the direct sums' own:
+// 1 GB, or 64 bytes per cell where that is more.
+inline int64_t ws_most(int64_t n_cells) {
+    return n_cells > (int64_t(1) << 24) ? 64 * n_cells : int64_t(1) << 30;
+}
+
 // Cartesian grid of a plan: cell n = i + nx (k + ny l) at (X_i, Y_k, Z_l).
 struct GridGeom {
     int32_t nx, ny, nz;
@@ -345,6 +351,7 @@ struct BandSelect {
     int64_t cap_part;        // floats of the nodes' partial sums
     int64_t cap_mid;         // most (x, y) nodes x z cells
     int32_t cap_mt;          // most 128-row tiles of the nodes' x operand
+    int32_t cap_nl;          // most light chunks of an x tile
     int32_t cap_ax[3];       // most nodes of an axis (grids: at most its cells besides)
     int32_t fold;
     int32_t n_mt;            // x tiles of the cells
@@ -365,6 +372,7 @@ struct LatticeRoom {
     int64_t held[3];   // nodes of an axis that the tables hold
     int64_t nodes, nodes_held;
     int64_t bytes;     // the lattice's part of the workspace (0: not offered)
+    int64_t base;      // a grid path's own part; 0 at any cells
 };
 
 // Adjoint on the band path (band_bwd.cu): one axis of a grid's transposed

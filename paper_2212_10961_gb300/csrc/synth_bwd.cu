@@ -777,8 +777,12 @@ struct CellsAdjLayout {
 CellsAdjLayout cells_adj_layout(int64_t n, int64_t n_pad, int32_t dim) {
     CellsAdjLayout L{};
     L.cap_nodes = std::max<int64_t>(n, 65536);
+    // within the bound on the workspace: 8 bytes per axis, node and mode, and 40
+    // per 64 x nodes and mode for the partial sums
     const double side = std::pow(double(L.cap_nodes), 1.0 / dim);
-    L.cap_ax = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
+    const int64_t fixed = n_pad * (4 * 3 + 32 + 40) + L.cap_nodes * 12 + (int64_t(1) << 22);
+    L.cap_ax = static_cast<int32_t>(std::min({4096.0, 4.0 * side, double((ws_most(n) - fixed) / (n_pad * (8 * dim + 1)) - 16)})) + 16;
+    if (L.cap_ax < 64) return L;  // total 0: not offered
     int64_t off = 0;
     auto take = [&](int64_t bytes) {
         const int64_t o = off;

@@ -868,36 +868,49 @@ int64_t table_bytes(const GridPlan& g) { return g.a_bytes + g.y_bytes + g.w_byte
 // One list of table slots.
 int64_t idx_bytes(const GridPlan& g) { return align256((int64_t(g.nc) * kGModes + 128) * 4); }
 
-// The nodes' tables: those of a grid of as many y and z cells, with mt row tiles.
-int64_t node_table_bytes(const GridPlan& g, int32_t mt) {
-    return table_bytes(g) - g.a_bytes + align256(int64_t(mt) * g.nc * kGPair);
-}
-
 // Workspace of a band-path call after the grid path's own: the descriptor,
-// the modes' lists, the x tiles' first nodes, the nodes' tables (a node axis is never longer
-// than its cell axis), the light chunks, the nodes' partial sums, the (x, y)
+// the modes' lists, the x tiles' first nodes, the nodes' tables (those of a
+// grid of as many y and z cells, with cap_mt row tiles), the light chunks, the nodes' partial sums, the (x, y)
 // nodes at the z cells and the rows of x nodes at the (y, z) cells.
 struct BandLayout {
     int64_t off_idx, off_lstart, off_tab, off_latab, off_part, off_mid, off_rows, total;
     int64_t cap_nodes, cap_part, cap_mid;
-    int32_t cap_mt;
+    int32_t cap_mt, cap_nl;
 };
+// All of it stays, with the grid path's own part, within ws_most.  Two parts
+// give way: the nodes' x operand, down to a quarter of the cells' row tiles,
+// and the light chunks' operand tiles, which have a row per cell and a column
+// per x node that its tile of 128 cells reads.  That is at most all of them,
+// quadratic in the x axis (65 536 x 16 x 16 cells: 17 GB), but 140 on an evenly
+// spaced axis in order: at least 3 chunks of 64; a call whose tiles read more
+// than there is room for sums all modes directly.
+constexpr int64_t kMinLight = 3;
 BandLayout band_layout(const GridGeom& gg, const GridPlan& g) {
     const int64_t n = int64_t(gg.nx) * gg.ny * gg.nz;
-    BandLayout L;
+    BandLayout L{};
     L.cap_nodes = n / 4;
     L.cap_part = n;
     L.cap_mid = n / 2;
-    // row tiles of the nodes: several z blocks of few x nodes, within 64 MB of tables
-    L.cap_mt = std::max(g.n_mt, static_cast<int>(std::min<int64_t>(8, (int64_t(64) << 20) / (int64_t(g.nc) * kGPair))));
     L.off_idx = align256(sizeof(BandDesc));
     L.off_lstart = L.off_idx + 2 * idx_bytes(g);
     L.off_tab = L.off_lstart + align256(int64_t(g.n_mt) * 4);
-    L.off_latab = L.off_tab + node_table_bytes(g, L.cap_mt);
-    L.off_part = L.off_latab + (g.form ? align256(int64_t(g.n_mt) * ((gg.nx + 3 + kGK - 1) / kGK) * kGPair) : 0);
-    L.off_mid = L.off_part + align256(L.cap_part * 4);
-    L.off_rows = L.off_mid + (g.form ? align256(L.cap_mid * 4) : g.max_split > 1 ? 0 : align256(n * 4));
-    L.total = L.off_rows + align256((int64_t(gg.nx) + 3) * gg.ny * gg.nz * 4);
+    const int64_t yz = table_bytes(g) - g.a_bytes;
+    const int64_t part = align256(L.cap_part * 4);
+    const int64_t mid = g.form ? align256(L.cap_mid * 4) : g.max_split > 1 ? 0 : align256(n * 4);
+    const int64_t rows = align256((int64_t(gg.nx) + 3) * gg.ny * gg.nz * 4);
+    const int64_t tile = int64_t(g.nc) * kGPair, chunk = int64_t(g.n_mt) * kGPair;
+    const int64_t chunks = g.form ? (gg.nx + 3 + kGK - 1) / kGK : 0;  // the most an x tile can read
+    const int64_t left = ws_most(n) - (table_bytes(g) + g.part_bytes) - (L.off_tab + yz + part + mid + rows);
+    // row tiles of the nodes: several z blocks of few x nodes, within 64 MB of tables
+    const int64_t mt = std::max<int64_t>(g.n_mt, std::min<int64_t>(8, (int64_t(64) << 20) / tile));
+    L.cap_mt = static_cast<int32_t>(std::min(mt, (left - std::min(chunks, kMinLight) * chunk) / tile));
+    if (L.cap_mt < (g.n_mt + 3) / 4) return L;  // total 0: not offered
+    L.cap_nl = static_cast<int32_t>(std::min(chunks, (left - L.cap_mt * tile) / chunk));
+    L.off_latab = L.off_tab + yz + L.cap_mt * tile;
+    L.off_part = L.off_latab + L.cap_nl * chunk;
+    L.off_mid = L.off_part + part;
+    L.off_rows = L.off_mid + mid;
+    L.total = L.off_rows + rows;
     return L;
 }
 
@@ -908,6 +921,7 @@ void set_limits(BandSelect& s, const BandLayout& L) {
     s.cap_part = L.cap_part;
     s.cap_mid = L.cap_mid;
     s.cap_mt = L.cap_mt;
+    s.cap_nl = L.cap_nl;
     s.cap_ax[0] = L.cap_mt * kGM;
     s.cap_ax[1] = s.cap_ax[2] = INT32_MAX;
 }
@@ -1045,8 +1059,13 @@ CellsLayout cells_layout(int64_t n, int64_t n_pad, int32_t dim) {
     // (2-D: a square's)
     L.cap_nodes = cells_band_cap(n);
     L.cap_part = std::max<int64_t>(L.cap_nodes, int64_t(1) << 22);
+    // within the bound on the workspace: 8 bytes per node and mode and operand,
+    // tiles of 128 nodes
     const double side = std::pow(double(L.cap_nodes), 1.0 / dim);
-    L.cap_yz = static_cast<int32_t>(std::min(4096.0, 4.0 * side)) + 16;
+    const int64_t fixed = n_pad * 60 + L.cap_part * 4 + n * 4 + 65536;
+    const int64_t per_node = dim > 2 ? n_pad * 8 + 2 * nc * kGRowBytes : n_pad * 16;
+    L.cap_yz = static_cast<int32_t>(std::min({4096.0, 4.0 * side, double((ws_most(n) - fixed) / per_node - kGM - 16)})) + 16;
+    if (L.cap_yz < 64) return L;  // total 0: not offered
     L.cap_mt = static_cast<int32_t>((L.cap_yz + kGM - 1) / kGM);
     int64_t off = 0;
     auto take = [&](int64_t bytes) {
@@ -1113,6 +1132,7 @@ LatticeRoom grid_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
     r.held[2] = g.form ? g.w_bytes / (g.nc * kGRowBytes) : 1;
     r.nodes = s.cap_nodes;
     r.nodes_held = (L.off_mid - L.off_part) / 4;
+    r.base = static_cast<int64_t>(grid_ws_bytes(nx, ny, nz, n_pad));
     return r;
 }
 

@@ -811,7 +811,8 @@ size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad)
     if (std::max(nx, std::max(ny, nz)) * n_pad >= int64_t(1) << 31) return 0;
     if (n_pad > band::kMaxModes || nx < 32 || ny < 8 || grid_adjoint_us_per_mode(nx, ny, nz) * double(n_pad) < 60.0)
         return 0;
-    return static_cast<size_t>(adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total);
+    const int64_t total = adj_band_layout(nx, ny, nz, n_pad, kAMaxCtas).total;
+    return adj_plan(nx, ny, nz, n_pad, 1).total + total <= ws_most(int64_t(nx) * ny * nz) ? static_cast<size_t>(total) : 0;
 }
 
 LatticeRoom grid_adjoint_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad) {
@@ -828,6 +829,7 @@ LatticeRoom grid_adjoint_room(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad)
     }
     r.nodes = s.cap_nodes;
     r.nodes_held = (L.off_part - L.off_nodes) / 4;
+    r.base = static_cast<int64_t>(bwd_grid_ws_bytes(nx, ny, nz, n_pad));
     return r;
 }
 

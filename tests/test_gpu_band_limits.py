@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from helpers import check_forward, oracle_field, to_dev
-from test_gpu_band import _check_adjoint, _modes, _params, env  # noqa: F401
+from test_gpu_band import _check_adjoint, _check_grid, _modes, _params, env  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -71,3 +71,14 @@ def test_frequencies_whose_scale_underflows(env):  # noqa: F811
     assert ws.untouched() and plan.status() == 0
     idx = np.random.default_rng(2).choice(cells, 6000, replace=False)
     check_forward(y[idx], oracle_field(m, 0.25, c, idx), 1.0, "underflowing frequencies")
+
+
+@pytest.mark.parametrize("order", ["running", "random"])
+def test_long_x_axis(env, order):  # noqa: F811
+    # 32,768 x cells: the light modes' chunks get part of what an axis in no
+    # order would need (each tile of it reads nearly all nodes)
+    axes = [np.linspace(0.0, 400.0, 32_768).astype(np.float32), np.linspace(0.0, 0.4, 32).astype(np.float32),
+            np.linspace(0.0, 0.2, 16).astype(np.float32)]
+    if order == "random":
+        axes[0] = np.random.default_rng(3).permutation(axes[0])
+    _check_grid(env, axes, (0.3, 0.3, 0.3), 1000, "rough")

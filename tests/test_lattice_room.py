@@ -8,7 +8,7 @@ import pytest
 from paper_2212_10961_gb300 import _abi
 
 CELLS, CELLS_ADJOINT, GRID, GRID_ADJOINT = range(4)
-FIELDS = ("limit_x", "limit_y", "limit_z", "held_x", "held_y", "held_z", "nodes", "nodes_held", "bytes")
+FIELDS = ("limit_x", "limit_y", "limit_z", "held_x", "held_y", "held_z", "nodes", "nodes_held", "bytes", "base")
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -19,7 +19,7 @@ def _built():
 
 def room(kind, dim, cells, n_modes):
     cells = (list(cells) + [1, 1, 1])[:3]
-    out = (ctypes.c_int64 * 9)()
+    out = (ctypes.c_int64 * 10)()
     _abi.check(_abi.lib().grf_debug_lattice_room(kind, dim, (ctypes.c_int64 * 3)(*cells), n_modes, out))
     return dict(zip(FIELDS, out))
 
@@ -50,6 +50,31 @@ def test_adjoint_tables_stay_within_32_bit_indices(shape, modes):
     r = room(GRID_ADJOINT, len(shape), shape, modes)
     n_pad = (modes + 127) // 128 * 128
     assert all(r["held_" + c] * n_pad < 2 ** 31 for c in "xyz")
+
+
+BIG = [(GRID, (s, 1024)) for s in ((32_768, 32, 16), (65_536, 16, 16), (262_144, 16, 16), (1_000_000, 32, 16))]
+BIG += [(k, (s, m)) for k in (GRID, GRID_ADJOINT) for s in ((256, 256, 256), (70_000, 40), (65_536, 16, 16))
+        for m in (4096, 60_000)]
+BIG += [(k, ((n,), m)) for k in (CELLS, CELLS_ADJOINT) for n in (70_000, 2_000_376, 2 ** 26) for m in (8192, 65_536)]
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("kind,call", BIG)
+def test_workspace_stays_within_its_bound(kind, dim, call):
+    # 1 GB, or 64 bytes per cell where that is more (grids: with the grid path's own tables)
+    cells, modes = call
+    if len(cells) > 1 and dim != len(cells):
+        pytest.skip("the grid's own dimension")
+    r = room(kind, dim, cells, modes)
+    n = 1
+    for c in cells:
+        n *= c
+    assert r["bytes"] + r["base"] <= max(2 ** 30, 64 * n)
+
+
+@pytest.mark.parametrize("shape,modes", [((256, 256, 256), 8192), ((65_536, 16, 16), 1024), ((262_144, 16, 16), 1024)])
+def test_long_grids_keep_the_lattice(shape, modes):
+    assert room(GRID, 3, shape, modes)["bytes"] > 0
 
 
 def test_large_calls_are_offered_the_lattice():
