@@ -464,8 +464,8 @@ __global__ void __launch_bounds__(256) band_sum_kernel(const BandDesc* b, float*
 // memory.
 constexpr int kCols = 64, kLineNodes = 96, kLineRun = 64;
 template <bool kY>
-__global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const float* __restrict__ src,
-                                                        const float* cells, int n, int nz, float* out) {
+__global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const float* src, const float* cells,
+                                                        int n, int nz, float* __restrict__ out) {
     __shared__ float nodes[kLineNodes][kCols];
     __shared__ __align__(16) float wts[kLineRun][kW];
     __shared__ int start[kLineRun];
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const
         const bool staged = nn <= kLineNodes;
         if (staged && c < columns) {
 #pragma unroll 8
-            for (int q = row; q < nn; q += 256 / kCols) nodes[q][lane] = zero ? 0.0f : __ldg(col + (n0 + q) * stride);
+            for (int q = row; q < nn; q += 256 / kCols) nodes[q][lane] = zero ? 0.0f : col[(n0 + q) * stride];
         }
         __syncthreads();
         if (c < columns) {
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const
                         if (staged)
                             f[q] = nodes[s + q][lane];
                         else if (!zero)
-                            f[q] = __ldg(col + (n0 + s + q) * stride);
+                            f[q] = col[(n0 + s + q) * stride];
                     }
                 }
                 // pairs from the tails inwards: the small terms first
@@ -563,9 +563,10 @@ __global__ void __launch_bounds__(256) band_line_kernel(const BandDesc* b, const
 // 210 us).  Groups that spread over more nodes than fit read them from memory.
 constexpr int kCellsBlock = 512, kBoxFloats = 10240, kCellBins = 1024;
 template <int DIM>
-__global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, const float* __restrict__ nodes,
+__global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, const float* nodes,
                                                             const float* __restrict__ xs, const float* __restrict__ ys,
-                                                            const float* __restrict__ zs, int64_t n, float* out) {
+                                                            const float* __restrict__ zs, int64_t n,
+                                                            float* __restrict__ out) {
     __shared__ __align__(16) float box[kBoxFloats];
     __shared__ int bins[kCellBins];       // cells per bin, then of the bins before it
     __shared__ short order[kCellsBlock];  // cells of the block by bin
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, c
         for (int r = t >> 5; r < rows; r += 8) {
             const int z = DIM > 2 ? r / nb[1] : 0, y = r - z * nb[1];
             const float* p = nodes + (f0[2] + z) * plane + static_cast<int64_t>(f0[1] + y) * mx + f0[0];
-            for (int x = lane; x < px; x += 32) box[r * px + x] = x < nb[0] ? __ldg(p + x) : 0.0f;
+            for (int x = lane; x < px; x += 32) box[r * px + x] = x < nb[0] ? p[x] : 0.0f;
         }
     }
     // ---- order of the cells: counting sort by their first node (bins wrap
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, c
                 for (int ky = 0; ky < kW; ++ky) {
                     float u = 0.0f;
 #pragma unroll
-                    for (int k = 0; k < kW; ++k) u = fmaf(w[k], __ldg(p + static_cast<int64_t>(ky) * mx + k), u);
+                    for (int k = 0; k < kW; ++k) u = fmaf(w[k], p[static_cast<int64_t>(ky) * mx + k], u);
                     a = fmaf(wy[ky], u, a);
                 }
                 if (DIM > 2) {
@@ -769,9 +770,9 @@ __global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, c
 // their 64 values straight from memory.  Memory-bound on the outputs where
 // the maps are many, else on latency: all loads of a phase are independent.
 constexpr int kFinRows = 8, kFinNodes = 320;
-__global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b, const float* __restrict__ mid,
-                                                               const float* __restrict__ part, GridGeom gg, int tx,
-                                                               int units, MapDev map, unsigned long long* tiles) {
+__global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b, const float* mid, const float* part,
+                                                               GridGeom gg, int tx, int units, MapDev map,
+                                                               unsigned long long* tiles) {
     __shared__ float rows[kFinRows][kFinNodes];
     __shared__ __align__(16) float wy[kFinRows][kW];
     __shared__ int sy[kFinRows];
@@ -831,7 +832,7 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
             const float* p = base + static_cast<int64_t>(sy[r]) * mx + n0 + c;
             float f[kW];
 #pragma unroll
-            for (int q = 0; q < kW; ++q) f[q] = q < nty ? __ldg(p + static_cast<int64_t>(q) * mx) : 0.0f;
+            for (int q = 0; q < kW; ++q) f[q] = q < nty ? p[static_cast<int64_t>(q) * mx] : 0.0f;
             float v = 0.0f;
 #pragma unroll
             for (int q = 0; q < kW / 2; ++q) v = fmaf(wy[r][q], f[q], fmaf(wy[r][kW - 1 - q], f[kW - 1 - q], v));
@@ -845,7 +846,7 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
 #pragma unroll 2
         for (int r = r0; r < min(kFinRows, ny - k0); r += rstep) {
             const int64_t o = (static_cast<int64_t>(l) * ny + k0 + r) * nx + i;
-            const float target = mm ? __ldg(map.T + o) : 0.0f;
+            const float target = mm ? map.T[o] : 0.0f;
             float v = 0.0f;
             if (staged) {
                 const float* p = &rows[r][s - n0];
@@ -858,7 +859,7 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
                 for (int q = 0; q < nt; ++q) {
                     float f = 0.0f;
                     for (int k = 0; k < nty; ++k)
-                        f = fmaf(wy[r][k], __ldg(base + static_cast<int64_t>(sy[r] + k) * mx + s + q), f);
+                        f = fmaf(wy[r][k], base[static_cast<int64_t>(sy[r] + k) * mx + s + q], f);
                     float wq = 0.0f;
 #pragma unroll
                     for (int k = 0; k < kW; ++k) wq = k == q ? w[k] : wq;
@@ -867,7 +868,7 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
             }
             float e = 0.0f;
 #pragma unroll 4
-            for (int k = 0; k < n_split; ++k) two_sum_acc(v, e, __ldg(part + k * n + o));
+            for (int k = 0; k < n_split; ++k) two_sum_acc(v, e, part[k * n + o]);
             const float y = (v + e) + map.mu;
             map_store(map, o, y);
             if (mm) loss += mismatch_value(map, o, y, target);

@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
 // lanes are nodes, warps groups of rows, a thread kTxPer rows of one node (a
 // weight is read once for them).  Bound by the read of g and by latency.
 constexpr int kTxRows = 32, kTxPer = 4, kTxCells = 256;
-__global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const float* __restrict__ g, int nx,
-                                                      int64_t n_rows, BandAxisTab tab, float* out) {
+__global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const float* g, int nx, int64_t n_rows,
+                                                      BandAxisTab tab, float* __restrict__ out) {
     __shared__ float gs[kTxRows / kTxPer][kTxCells][kTxPer];
     pdl_wait();
     if (b->n_light == 0) return;
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
                     for (int r = warp; r < kTxRows; r += 8)
 #pragma unroll 4
                         for (int i = lane; i < nc; i += 32)
-                            gs[r / kTxPer][i][r % kTxPer] = r < nr ? __ldg(g + (r0 + r) * nx + c0 + i) : 0.0f;
+                            gs[r / kTxPer][i][r % kTxPer] = r < nr ? g[(r0 + r) * nx + c0 + i] : 0.0f;
                     __syncthreads();
                 }
                 const int ca = max(range.x, c0), cb = min(range.y, c0 + nc - 1);
@@ -127,10 +127,10 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
                 for (int i = ca; i <= cb; ++i) {
                     float w = 0.0f;
                     if (most > 0) {
-                        w = __ldg(tab.wt + (i - range.x) * mx + node);
+                        w = tab.wt[(i - range.x) * mx + node];
                     } else {
-                        const unsigned k = static_cast<unsigned>(node - __ldg(tab.start + i));
-                        if (k < kW) w = __ldg(tab.w + static_cast<int64_t>(i) * kW + k);
+                        const unsigned k = static_cast<unsigned>(node - tab.start[i]);
+                        if (k < kW) w = tab.w[static_cast<int64_t>(i) * kW + k];
                     }
                     const float4 v = *reinterpret_cast<const float4*>(gs[warp][i - c0]);
                     acc.x = fmaf(w, v.x, acc.x);
@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
 // out[(l m_y + node) m_x + i]; z: columns are the (x, y) nodes.  One thread per
 // value, contiguous over the columns; all loads of a value are independent.
 template <bool kY>
-__global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, const float* __restrict__ in, int n, int nz,
-                                                         BandAxisTab tab, float* out) {
+__global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, const float* in, int n, int nz,
+                                                         BandAxisTab tab, float* __restrict__ out) {
     pdl_wait();
     if (b->n_light == 0) return;
     const int mx = b->ax[0].m, m = kY ? b->ax[1].m : b->ax[2].m, most = *tab.most;
@@ -183,11 +183,11 @@ __global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, cons
         if (most > 0) {
 #pragma unroll 8
             for (int i = range.x; i <= range.y; ++i)
-                acc = fmaf(__ldg(tab.wt + (i - range.x) * m + node), __ldg(src + i * stride), acc);
+                acc = fmaf(tab.wt[(i - range.x) * m + node], src[i * stride], acc);
         } else {
             for (int i = range.x; i <= range.y; ++i) {
-                const unsigned k = static_cast<unsigned>(node - __ldg(tab.start + i));
-                if (k < kW) acc = fmaf(__ldg(tab.w + static_cast<int64_t>(i) * kW + k), __ldg(src + i * stride), acc);
+                const unsigned k = static_cast<unsigned>(node - tab.start[i]);
+                if (k < kW) acc = fmaf(tab.w[static_cast<int64_t>(i) * kW + k], src[i * stride], acc);
             }
         }
         out[u] = acc;
@@ -208,7 +208,7 @@ struct FixedScale {
 };
 __device__ __forceinline__ FixedScale fixed_scale(const float* gmax, int n_gmax, int64_t n) {
     float m = 0.0f;
-    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) m = fmaxf(m, __ldg(gmax + k));
+    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) m = fmaxf(m, gmax[k]);
     m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
     if (!(m > 0.0f) || !(m < 3.0e38f)) return FixedScale{1.0f, 1.0f};
     int e = 0, c = 0;
@@ -219,7 +219,7 @@ __device__ __forceinline__ FixedScale fixed_scale(const float* gmax, int n_gmax,
 
 __device__ __forceinline__ bool gmax_finite(const float* gmax, int n_gmax) {
     bool ok = true;
-    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) ok = ok && __ldg(gmax + k) < 3.0e38f;
+    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) ok = ok && gmax[k] < 3.0e38f;
     return __all_sync(0xffffffffu, ok);
 }
 
@@ -248,8 +248,8 @@ struct SpreadSmem {
 template <int DIM>
 __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
     const BandDesc* b, const float* __restrict__ xs, const float* __restrict__ ys, const float* __restrict__ zs,
-    const int32_t* __restrict__ perm, int64_t perm_base, int64_t n, const float* __restrict__ g,
-    const float* __restrict__ gmax, int n_gmax, int cells, unsigned long long* lattice) {
+    const int32_t* __restrict__ perm, int64_t perm_base, int64_t n, const float* g, const float* gmax, int n_gmax,
+    int cells, unsigned long long* lattice) {
     __shared__ __align__(16) SpreadSmem smem[kSpreadWarps];
     pdl_wait();
     if (b->n_light == 0) return;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) band_spread_kernel(
             if (lane < m) {
                 const int i = sm.order[i0 + lane];
                 const int64_t o = static_cast<int64_t>(__ldg(perm + c0 + i)) - perm_base;
-                const float gv = index_ok(o, n) ? __ldg(g + o) * scale.first * scale.second : 0.0f;
+                const float gv = index_ok(o, n) ? g[o] * scale.first * scale.second : 0.0f;
                 float w[kW], v;
                 const int px = band::locate(ax[0], __ldg(src[0] + i), v);
                 band::weights(v, w);
@@ -479,8 +479,7 @@ __global__ void __launch_bounds__(256) band_unfix_kernel(const BandDesc* b, cons
 // (z: with psi) and the coordinates off[node] relative to the axis's first
 // node; and rank[slot], the light mode of a table slot or ~ the direct one.
 __global__ void __launch_bounds__(256) band_phasor_kernel(const BandDesc* b, const float4* __restrict__ cold,
-                                                          const int32_t* __restrict__ idx_l,
-                                                          const int32_t* __restrict__ idx_h, GridGeom gg, int dim,
+                                                          const int32_t* idx_l, const int32_t* idx_h, GridGeom gg, int dim,
                                                           BandPhasors t) {
     pdl_wait();
     const int nl = b->n_light, nh = b->nh;
@@ -554,7 +553,7 @@ __global__ void __launch_bounds__(256) band_phasor_kernel(const BandDesc* b, con
 // once per mode tile from L2.
 constexpr int kNLines = 16, kNX = 64, kNModes = 128;
 constexpr int kNSmem = kNX * kNModes * 8 + kNX * kNLines * 4 + kNX * 4;
-__global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* b, const float* __restrict__ G,
+__global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* b, const float* G,
                                                                 BandPhasors t, int dim, GridGeom gg, int blocks,
                                                                 double* part) {
     extern __shared__ __align__(16) unsigned char nsm[];
@@ -576,7 +575,7 @@ __global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* 
         const int i0 = xc * kNX, ni = min(kNX, mx - i0);
         __syncthreads();
 #pragma unroll 8
-        for (int i = 0; i < ni; ++i) xp[i * kNModes + tid] = __ldg(t.ph[0] + static_cast<int64_t>(i0 + i) * np + m);
+        for (int i = 0; i < ni; ++i) xp[i * kNModes + tid] = t.ph[0][static_cast<int64_t>(i0 + i) * np + m];
         if (tid < kNX) xw[tid] = tid < ni ? t.off[0][i0 + tid] : 0.0f;
         float hi[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, lo[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         const int nb = (lines + kNLines - 1) / kNLines;
@@ -588,7 +587,7 @@ __global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* 
 #pragma unroll
             for (int e = tid; e < kNX * kNLines; e += kNModes) {
                 const int r = e / kNX, i = e - r * kNX;
-                if (i < ni) gs[i * kNLines + r] = r < nr ? __ldg(G + static_cast<int64_t>(l0 + r) * mx + i0 + i) : 0.0f;
+                if (i < ni) gs[i * kNLines + r] = r < nr ? G[static_cast<int64_t>(l0 + r) * mx + i0 + i] : 0.0f;
             }
             __syncthreads();
             float dr[kNLines], di[kNLines], er[kNLines], ei[kNLines];
@@ -615,15 +614,15 @@ __global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* 
 #pragma unroll
             for (int r = 0; r < kNLines; ++r) {
                 if (r < nr) {
-                    const float2 y = __ldg(t.ph[1] + static_cast<int64_t>(k) * np + m);
-                    const float2 z = __ldg(t.ph[2] + static_cast<int64_t>(l) * np + m);
+                    const float2 y = t.ph[1][static_cast<int64_t>(k) * np + m];
+                    const float2 z = t.ph[2][static_cast<int64_t>(l) * np + m];
                     const float pr = fmaf(y.x, z.x, -y.y * z.y), pi = fmaf(y.x, z.y, y.y * z.x);
                     const float im = fmaf(dr[r], pi, di[r] * pr);
                     s[0] += fmaf(dr[r], pr, -di[r] * pi);
                     s[1] += im;
                     s[2] += fmaf(er[r], pi, ei[r] * pr);
-                    s[3] = fmaf(__ldg(t.off[1] + k), im, s[3]);
-                    s[4] = fmaf(__ldg(t.off[2] + l), im, s[4]);
+                    s[3] = fmaf(t.off[1][k], im, s[3]);
+                    s[4] = fmaf(t.off[2][l], im, s[4]);
                     if (++k == my) {
                         k = 0;
                         ++l;
@@ -661,9 +660,9 @@ __global__ void __launch_bounds__(kNModes, 3) band_nodes_kernel(const BandDesc* 
 constexpr int kDirCells = 256, kDirModes = 128, kDirWarps = 4;
 template <int DIM>
 __global__ void __launch_bounds__(32 * kDirWarps, 4) band_direct_kernel(
-    const BandDesc* b, const float4* __restrict__ cold, const int32_t* __restrict__ idx, const float* __restrict__ xs,
+    const BandDesc* b, const float4* __restrict__ cold, const int32_t* idx, const float* __restrict__ xs,
     const float* __restrict__ ys, const float* __restrict__ zs, const int32_t* __restrict__ perm, int64_t perm_base,
-    int64_t n, const float* __restrict__ g, double* part) {
+    int64_t n, const float* g, double* part) {
     __shared__ float4 mode[kDirModes][2];
     __shared__ float2 acc[kDirWarps][kDirModes][5];
     pdl_wait();
@@ -677,7 +676,7 @@ __global__ void __launch_bounds__(32 * kDirWarps, 4) band_direct_kernel(
         const int nm = min(kDirModes, nh - mt * kDirModes);
         __syncthreads();
         for (int k = threadIdx.x; k < nm; k += blockDim.x) {
-            const int s = __ldg(idx + mt * kDirModes + k);
+            const int s = idx[mt * kDirModes + k];
             mode[k][0] = __ldg(cold + 2 * s);
             mode[k][1] = __ldg(cold + 2 * s + 1);
         }
@@ -694,7 +693,7 @@ __global__ void __launch_bounds__(32 * kDirWarps, 4) band_direct_kernel(
             for (int q = 0; q < kPer; ++q) {
                 const int64_t i = c0 + q * 32 + lane;
                 const int64_t o = i < n ? static_cast<int64_t>(__ldg(perm + i)) - perm_base : 0;
-                gv[q] = i < n && index_ok(o, n) ? __ldg(g + o) : 0.0f;
+                gv[q] = i < n && index_ok(o, n) ? g[o] : 0.0f;
 #pragma unroll
                 for (int c = 0; c < DIM; ++c) x[q][c] = __ldg(src[c] + (i < n ? i : c0));
             }

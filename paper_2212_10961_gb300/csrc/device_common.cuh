@@ -164,7 +164,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
 // stream may be set up while this one runs; `pdl_wait` returns once the
 // previous kernel has completed and its writes are visible.  Every thread of a
 // chained kernel passes it before its first access to global memory, so that
-// a kernel's completion implies that of all before it.
+// a kernel's completion implies that of all before it.  Since it may start
+// before they end, it reads what a chained kernel may have written -- the
+// workspace, and outputs of earlier calls such as dL/dY -- with plain loads:
+// read-only ones (__ldg, const __restrict__) need data that is constant while
+// the kernel runs, as the mode table and the plan are.
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -228,7 +232,7 @@ __device__ __forceinline__ double mismatch_value(const MapDev& m, int64_t o, flo
     return static_cast<double>(d) * static_cast<double>(d);
 }
 __device__ __forceinline__ double mismatch_store(const MapDev& m, int64_t o, float y) {
-    return mismatch_value(m, o, y, __ldg(m.T + o));
+    return mismatch_value(m, o, y, m.T[o]);
 }
 
 // Map epilogue of one cell (Sec. 3.1 truncation rule, Sec. 4.1 lognormal).

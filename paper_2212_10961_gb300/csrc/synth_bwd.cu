@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
     bool light = false;
     if (args.band.b != nullptr) {
         const BandDesc& b = *args.band.b;
-        const int r = m < args.n_modes ? __ldg(args.band.rank + m) : 0;
+        const int r = m < args.n_modes ? args.band.rank[m] : 0;
         light = m < args.n_modes && r >= 0;
         if (light) {
             const BandNodes S = band_nodes_split(b.n_light, b.ax[0].m, b.ax[1].m * b.ax[2].m, args.band.blocks);
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(32 * kRedWarps) bwd_reduce_kernel(BwdArgs args
             if (light) {
                 // from the nodes' sums to the cells': the window's gain, and its
                 // slope where the frequency is differentiated (band_bwd.cu)
-                const int r = __ldg(args.band.rank + m);
+                const int r = args.band.rank[m];
                 const int64_t np = (args.band.b->n_light + 127) / 128 * 128;
                 const double gain = args.band.gain[r];
 #pragma unroll

@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(W * 32, (fwd_min_blocks<DIM, C>())) synth_fwd_
 // Combine the per-split partials of every sorted cell in split order (a
 // fixed order, so results are deterministic) and apply the maps; with the
 // mismatch bit every block also writes its sum of (K - T)^2 to lpart.
-__global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const float2* __restrict__ partial,
+__global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const float2* partial,
                                                             int n_split) {
     pdl_wait();
     if (d.band != nullptr) {
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
                 two_sum_acc(s, e, v.x);
                 e += v.y;
             }
-            if (d.add != nullptr) two_sum_acc(s, e, __ldg(d.add + i));
+            if (d.add != nullptr) two_sum_acc(s, e, d.add[i]);
             const float y = (s + e) + d.map.mu;
             const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
             if (index_ok(o, d.n_cells)) {
@@ -573,9 +573,8 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
 
 // loss = (sum of the nb partial sums of (K - T)^2) / n_mean, one block,
 // fixed order.
-__global__ void __launch_bounds__(256) loss_sum_kernel(const double* __restrict__ part, int64_t nb,
-                                                       const int64_t* __restrict__ nb_dev, double inv_n,
-                                                       double* __restrict__ out) {
+__global__ void __launch_bounds__(256) loss_sum_kernel(const double* part, int64_t nb, const int64_t* nb_dev,
+                                                       double inv_n, double* __restrict__ out) {
     __shared__ double red[256];
     pdl_wait();
     double acc = 0.0;

@@ -134,7 +134,7 @@ __device__ __forceinline__ void form_light(unsigned char* bhi, const float* row,
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int node = first + 16 * q4 + 8 * h + 4 * e;
-            v[e] = node < lp ? __ldg(reinterpret_cast<const float4*>(row + node)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            v[e] = node < lp ? *reinterpret_cast<const float4*>(row + node) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         uint4 H, L;
         tc::split_f16x2(v[0].x * inv, v[0].y * inv, H.x, L.x);
@@ -331,7 +331,7 @@ __device__ __forceinline__ void grid_mma_body(const GridDesc& d, const GridTilin
                     if (kLight && c < 0)
                         form_light(gsm + T.off_b + sb * kGPair,
                                    d.light + (static_cast<int64_t>(ll) * T.ny + lk) * T.lp,
-                                   __ldg(d.lstart + ti.mt) + (c + nl) * kGK, T.lp, T.l_inv, lcol, t & 3);
+                                   d.lstart[ti.mt] + (c + nl) * kGK, T.lp, T.l_inv, lcol, t & 3);
                     else
                         form_b(gsm + T.off_b + sb * kGPair, reinterpret_cast<const float4*>(st + toff_y),
                                reinterpret_cast<const float4*>(st + toff_w0),
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kGThreads, 1) grid_band_kernel(GridDesc d, con
 //                as (re, im) hi and lo tiles (columns beyond ny are zero).
 // Node lattices of the band path also multiply A_j by the window's gains.
 // Table slot of mode j of the sum; < 0: none (the chunk's padding, amplitude 0).
-__device__ __forceinline__ int prep_slot(const GridPrep& p, int j) { return p.idx != nullptr ? __ldg(p.idx + j) : j; }
+__device__ __forceinline__ int prep_slot(const GridPrep& p, int j) { return p.idx != nullptr ? p.idx[j] : j; }
 __device__ __forceinline__ float prep_amp(const GridPrep& p, int j, const float4 c0, const float4 c1, float s_inv) {
     float amp = __ldg(&p.hot[j].w) * s_inv;
     if (p.gain_h[0] > 0.0f) amp *= band::gain(fabsf(c0.x) * p.gain_h[0]);
@@ -667,7 +667,7 @@ __device__ __forceinline__ void light_prep(const BandDesc* b, const float* X, co
         float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         if (i < b->cells.nx) {
             float w[band::kW];
-            const int s = band::cell_weights(ax, __ldg(X + i), i, w) - (__ldg(lstart + mt) + lc * kGK + 8 * seg);
+            const int s = band::cell_weights(ax, __ldg(X + i), i, w) - (lstart[mt] + lc * kGK + 8 * seg);
             const int nt = band::taps(ax);
 #pragma unroll
             for (int k = 0; k < band::kW; ++k)
@@ -715,7 +715,7 @@ __device__ __forceinline__ void sub_table(const BandDesc* b, const GridPrep& p, 
     const int n = (b->nh + kChunk - 1) / kChunk * kChunk;
     const int step = gridDim.x * blockDim.x;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += step) {
-        const int s = __ldg(p.idx + j);
+        const int s = p.idx[j];
         const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         o.hot[j] = s >= 0 ? __ldg(p.hot + s) : zero;
         o.cold[2 * j] = s >= 0 ? __ldg(p.cold + 2 * s) : zero;
@@ -726,7 +726,7 @@ __device__ __forceinline__ void sub_table(const BandDesc* b, const GridPrep& p, 
         int lo = 0, hi = b->nh;
         while (lo < hi) {
             const int mid = (lo + hi) / 2;
-            if (__ldg(p.idx + mid) < before)
+            if (p.idx[mid] < before)
                 lo = mid + 1;
             else
                 hi = mid;
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(256) band_prep_kernel(const BandDesc* b, GridP
 // Mode-split grids: per cell the partial fields of the splits, added in split
 // order (a fixed order), plus mu, then the maps; with the mismatch bit every
 // block also writes its sum of (K - T)^2 to lpart.
-__global__ void __launch_bounds__(256) grid_split_finalize(const float* __restrict__ part, int n_split, int64_t n,
+__global__ void __launch_bounds__(256) grid_split_finalize(const float* part, int n_split, int64_t n,
                                                            MapDev map) {
     pdl_wait();
     const int64_t o = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(256) adj_scan_kernel(const float* g, int64_t n
     float mx = 0.0f, sh = 0.0f, sl = 0.0f, xm = 0.0f;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float v = __ldg(g + i);
+        const float v = g[i];
         mx = fabsf(v) <= 3.402823466e38f ? fmaxf(mx, fabsf(v)) : INFINITY;
         two_sum_acc(sh, sl, v);
     }
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
             const int64_t rest = idx >> 10;  // mode tile * n_kc + x chunk
             const int kc = static_cast<int>(rest % p.n_kc);
             const int row = static_cast<int>(rest / p.n_kc) * kAM + r;
-            const int m = p.idx != nullptr ? __ldg(p.idx + row) : row;
+            const int m = p.idx != nullptr ? p.idx[row] : row;
             const float4 c0 = __ldg(p.cold + 2 * max(m, 0));
             float cs[8], sn[8];
 #pragma unroll
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
         } else if (idx < nA + nY) {
             const int64_t u = idx - nA;
             const int row = static_cast<int>(u % p.n_pad);
-            const int m = p.idx != nullptr ? max(__ldg(p.idx + row), 0) : row;
+            const int m = p.idx != nullptr ? max(p.idx[row], 0) : row;
             const int64_t k = u / p.n_pad;
             const float4 c0 = __ldg(p.cold + 2 * m);
             float cs, sn;
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
         } else if (idx < nA + nY + nZ) {
             const int64_t u = idx - nA - nY;
             const int row = static_cast<int>(u % p.n_pad);
-            const int m = p.idx != nullptr ? max(__ldg(p.idx + row), 0) : row;
+            const int m = p.idx != nullptr ? max(p.idx[row], 0) : row;
             const int64_t l = u / p.n_pad;
             const float4 c1 = __ldg(p.cold + 2 * m + 1);
             float cs, sn;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(256) adj_prep_kernel(AdjPrep p) {
                 gv[e] = 0.0f;
                 wv[e] = 0.0f;
                 if (valid && x < p.nx) {
-                    gv[e] = __ldg(p.gY + row + x) * gs;
+                    gv[e] = p.gY[row + x] * gs;
                     wv[e] = gv[e] * ((__ldg(p.X + x) - x0) * xs);
                 }
             }
@@ -427,8 +427,8 @@ __global__ void __launch_bounds__(kAThreads, 1) grid_adj_kernel(AdjDesc d, int32
                 // consecutive y cells of z cell lt
                 const int c0 = kACols * h;
                 const int nv = min(kACols, d.ny - yb * kAYZ - c0);  // valid columns (warp-uniform)
-                const float2 zv = __ldg(d.ztab + static_cast<int64_t>(lt) * d.n_pad + m);
-                const float zwl = __ldg(d.zw + lt);
+                const float2 zv = d.ztab[static_cast<int64_t>(lt) * d.n_pad + m];
+                const float zwl = d.zw[lt];
                 // four groups of 4 columns; the next group's TMEM loads are in
                 // flight while the current group is contracted
                 float qr = 0.0f, qi = 0.0f, qxr = 0.0f, qxi = 0.0f, qyr = 0.0f, qyi = 0.0f;
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kAThreads, 1) grid_adj_kernel(AdjDesc d, int32
                         const float c = __uint_as_float(dc[cc]), s = __uint_as_float(ds[cc]);
                         const float xc = __uint_as_float(dxc[cc]), xsn = __uint_as_float(dxs[cc]);
                         const float pr = fmaf(c, y.x, -s * y.y), pi = fmaf(c, y.y, s * y.x);
-                        const float w = __ldg(d.yw + k);
+                        const float w = d.yw[k];
                         qr += pr;
                         qi += pi;
                         qyr = fmaf(w, pr, qyr);
@@ -524,13 +524,13 @@ __global__ void __launch_bounds__(kAThreads, 1) grid_adj_kernel(AdjDesc d, int32
                     // end of a run of one z cell: multiply by its z phasor
                     if (kl == py - 1 || (half == 1 && cc == 7)) {
                         if (l < d.nz) {
-                            const float2 z = __ldg(d.ztab + static_cast<int64_t>(l) * d.n_pad + m);
+                            const float2 z = d.ztab[static_cast<int64_t>(l) * d.n_pad + m];
                             const float er = fmaf(qr, z.x, -qi * z.y), ei = fmaf(qr, z.y, qi * z.x);
                             uc += er;
                             us += ei;
                             ux += fmaf(qxr, z.y, qxi * z.x);
                             uy += fmaf(qyr, z.y, qyi * z.x);
-                            uz = fmaf(__ldg(d.zw + l), ei, uz);
+                            uz = fmaf(d.zw[l], ei, uz);
                         }
                         qr = qi = qxr = qxi = qyr = qyi = 0.0f;
                     }
