@@ -372,6 +372,14 @@ size_t grf_synth_grid_workspace_bytes(const void *plan, int32_t segment, int64_t
  * grf_synth_grid_workspace_bytes() includes the lattice's part.
  */
 size_t grf_synth_band_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes);
+
+/*
+ * grf_synth_plan_workspace_bytes -- the most workspace that grf_synth_field can
+ * use on a segment of the plan: the largest of grf_synth_workspace_bytes and,
+ * on a grid plan that has one, grf_synth_grid_workspace_bytes, otherwise
+ * grf_synth_band_workspace_bytes, in one call; 0 for an unknown plan.
+ */
+size_t grf_synth_plan_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes);
 int grf_plan_grid_shape(const void *plan, int32_t *nx, int32_t *ny, int32_t *nz);
 
 /*
@@ -451,6 +459,15 @@ size_t grf_backward_grid_workspace_bytes(const void *plan, int32_t segment, int6
  * lattice's part on grid plans.
  */
 size_t grf_backward_band_workspace_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
+
+/*
+ * grf_backward_plan_workspace_bytes -- the same for grf_synth_backward: the
+ * largest of grf_backward_workspace_bytes and, on a grid plan that has one,
+ * grf_backward_grid_workspace_bytes, otherwise
+ * grf_backward_band_workspace_bytes; 0 for an unknown plan or values out of
+ * range.
+ */
+size_t grf_backward_plan_workspace_bytes(const void *plan, int32_t segment, int64_t n_modes, int32_t dim);
 
 /*
  * grf_synth_backward -- gradients of a loss L with respect to the mode

@@ -889,6 +889,24 @@ CellsBand cells_band(const grf_params* p, const void* plan, const PlanMeta& meta
         left * 16.0 <= N};
 }
 
+// Workspace of a synthesis at any cells with the node lattice, and of one on a
+// grid (0: not offered).
+size_t cells_workspace(int64_t n, int64_t n_modes, int32_t plan_dim) {
+    size_t most = 0;
+    for (int32_t dim = 2; dim <= plan_dim; ++dim) most = std::max(most, cells_band_ws_bytes(n, n_modes, dim));
+    return most > 0 ? most + synth_workspace_bytes(n) : 0;
+}
+size_t grid_workspace(const GridGeom& gg, int64_t n_modes) {
+    const int64_t n_pad = table_layout(n_modes).n_pad;
+    const size_t b = grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+    return grid_ws_ok(b, gg) ? b + grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+}
+size_t grid_adjoint_workspace(const GridGeom& gg, int64_t n_modes) {
+    const int64_t n_pad = table_layout(n_modes).n_pad;
+    const size_t b = bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
+    return grid_ws_ok(b, gg) ? b + bwd_grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+}
+
 int fwd_desc(const void* table, int64_t n_modes, int32_t dim, const void* plan,
              const PlanMeta& meta, int32_t segment, const MapDev& map, FwdDesc& d) {
     if (segment < 0 || segment >= static_cast<int32_t>(meta.offsets.size()) - 1)
@@ -968,10 +986,24 @@ size_t grf_synth_band_workspace_bytes(const void* plan, int32_t segment, int64_t
         PlanMeta meta;
         if (!plan || n_modes < 1 || n_modes > GRF_MAX_MODES || !lookup_plan(plan, meta)) return 0;
         if (segment < 0 || segment >= static_cast<int32_t>(meta.offsets.size()) - 1) return 0;
-        const int64_t n = meta.offsets[segment + 1] - meta.offsets[segment];
-        size_t most = 0;
-        for (int32_t dim = 2; dim <= meta.dim; ++dim) most = std::max(most, cells_band_ws_bytes(n, n_modes, dim));
-        return most > 0 ? most + synth_workspace_bytes(n) : 0;
+        return cells_workspace(meta.offsets[segment + 1] - meta.offsets[segment], n_modes, meta.dim);
+    } catch (...) {
+        return 0;
+    }
+}
+
+size_t grf_synth_plan_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
+    try {
+        PlanMeta meta;
+        if (!plan || !lookup_plan(plan, meta)) return 0;
+        const bool in = segment >= 0 && segment < static_cast<int32_t>(meta.offsets.size()) - 1;
+        const int64_t n = in ? meta.offsets[segment + 1] - meta.offsets[segment] : 0;
+        const size_t split = synth_workspace_bytes(n);
+        if (!in || n_modes < 1 || n_modes > GRF_MAX_MODES) return split;
+        GridGeom gg{};
+        if (segment == 0 && plan_grid(plan, &gg))
+            if (const size_t grid = grid_workspace(gg, n_modes)) return std::max(split, grid);
+        return std::max(split, cells_workspace(n, n_modes, meta.dim));
     } catch (...) {
         return 0;
     }
@@ -981,10 +1013,7 @@ size_t grf_synth_grid_workspace_bytes(const void* plan, int32_t segment, int64_t
     try {
         if (!plan || segment != 0 || n_modes < 1 || n_modes > GRF_MAX_MODES) return 0;
         GridGeom gg{};
-        if (!plan_grid(plan, &gg)) return 0;
-        const int64_t n_pad = table_layout(n_modes).n_pad;
-        const size_t b = grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
-        return grid_ws_ok(b, gg) ? b + grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+        return plan_grid(plan, &gg) ? grid_workspace(gg, n_modes) : 0;
     } catch (...) {
         return 0;
     }
@@ -1122,14 +1151,28 @@ size_t grf_backward_band_workspace_bytes(int64_t n_cells, int64_t n_modes, int32
     return band > 0 ? band + bwd_workspace_bytes(n_cells, n_modes, dim) : 0;
 }
 
+size_t grf_backward_plan_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes, int32_t dim) {
+    try {
+        PlanMeta meta;
+        if (!plan || !lookup_plan(plan, meta) || n_modes < 1 || n_modes > GRF_MAX_MODES || dim < 1 || dim > 3) return 0;
+        const bool in = segment >= 0 && segment < static_cast<int32_t>(meta.offsets.size()) - 1;
+        const int64_t n = in ? meta.offsets[segment + 1] - meta.offsets[segment] : 0;
+        const size_t cells = bwd_workspace_bytes(n, n_modes, dim);
+        if (!in) return cells;
+        GridGeom gg{};
+        if (segment == 0 && plan_grid(plan, &gg))
+            if (const size_t grid = grid_adjoint_workspace(gg, n_modes)) return std::max(cells, grid);
+        return cells + cells_adjoint_band_ws_bytes(n, n_modes, dim);
+    } catch (...) {
+        return 0;
+    }
+}
+
 size_t grf_backward_grid_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
     try {
         if (!plan || segment != 0 || n_modes < 1 || n_modes > GRF_MAX_MODES) return 0;
         GridGeom gg{};
-        if (!plan_grid(plan, &gg)) return 0;
-        const int64_t n_pad = table_layout(n_modes).n_pad;
-        const size_t b = bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
-        return grid_ws_ok(b, gg) ? b + bwd_grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+        return plan_grid(plan, &gg) ? grid_adjoint_workspace(gg, n_modes) : 0;
     } catch (...) {
         return 0;
     }

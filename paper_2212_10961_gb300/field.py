@@ -447,11 +447,8 @@ def _outputs_struct(out):
 def synth_workspace_bytes(plan: CellPlan, segment, n_modes):
     """Workspace that lets grf_synth_field use the mode split, the node lattice
     of low-frequency modes and, on a Cartesian-grid plan, the tensor-core grid
-    path (the largest of grf_synth_workspace_bytes,
-    grf_synth_band_workspace_bytes and grf_synth_grid_workspace_bytes)."""
-    grid = int(lib().grf_synth_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
-    cells = 0 if grid else int(lib().grf_synth_band_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
-    return max(int(lib().grf_synth_workspace_bytes(plan.segment_size(segment))), cells, grid)
+    path (grf_synth_plan_workspace_bytes)."""
+    return lib().grf_synth_plan_workspace_bytes(plan.ptr, int(segment), int(n_modes))
 
 
 def synth_mismatch_workspace_bytes(plan: CellPlan, segment, n_modes):
@@ -593,12 +590,8 @@ _ws_fwd = Workspace()
 def backward_workspace_bytes(plan: CellPlan, segment, n_modes, dim):
     """Workspace bytes of grf_synth_backward on this plan: enough for the
     CUDA-core adjoint, with the node lattice of low-frequency modes, or, on a
-    grid plan, for the tensor-core one (grf_backward_workspace_bytes,
-    grf_backward_band_workspace_bytes, grf_backward_grid_workspace_bytes)."""
-    n = plan.segment_size(segment)
-    grid = int(lib().grf_backward_grid_workspace_bytes(plan.ptr, int(segment), int(n_modes)))
-    cells = 0 if grid else int(lib().grf_backward_band_workspace_bytes(n, int(n_modes), int(dim)))
-    return max(int(lib().grf_backward_workspace_bytes(n, int(n_modes), int(dim))), cells, grid)
+    grid plan, for the tensor-core one (grf_backward_plan_workspace_bytes)."""
+    return lib().grf_backward_plan_workspace_bytes(plan.ptr, int(segment), int(n_modes), int(dim))
 
 
 def backward(table: ModeTable, params: FieldParams, plan: CellPlan, gY, segment=0, stream=None,
