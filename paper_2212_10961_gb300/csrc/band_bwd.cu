@@ -56,17 +56,25 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
     for (int k = threadIdx.x; k < ax.m; k += blockDim.x) t.range[k] = make_int2(INT_MAX, -1);
     __syncthreads();
     const int nt = band::taps(ax);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        const bool in = i < n;
         float w[kW];
-        const int s = band::cell_weights(ax, __ldg(X + i), i, w);
+        const int s = in ? band::cell_weights(ax, __ldg(X + min(i, n - 1)), i, w) : -1;
+        // of neighbours with the same nodes the first and the last count
+        const int before = __shfl_up_sync(0xffffffffu, s, 1), after = __shfl_down_sync(0xffffffffu, s, 1);
+        const bool low = (threadIdx.x & 31) == 0 || before != s, high = (threadIdx.x & 31) == 31 || after != s;
+        if (!in) continue;  // no warp-wide step below
         t.start[i] = s;
+        float4* o = reinterpret_cast<float4*>(t.w + static_cast<int64_t>(i) * kW);
+#pragma unroll
+        for (int k = 0; k < kW; ++k) w[k] = k < nt ? w[k] : 0.0f;
+        o[0] = make_float4(w[0], w[1], w[2], w[3]);
+        o[1] = make_float4(w[4], w[5], w[6], w[7]);
 #pragma unroll
         for (int k = 0; k < kW; ++k) {
-            t.w[static_cast<int64_t>(i) * kW + k] = k < nt ? w[k] : 0.0f;
-            if (k < nt) {
-                atomicMin(&t.range[s + k].x, i);
-                atomicMax(&t.range[s + k].y, i);
-            }
+            if (k < nt && low) atomicMin(&t.range[s + k].x, i);
+            if (k < nt && high) atomicMax(&t.range[s + k].y, i);
         }
     }
     __syncthreads();
@@ -80,23 +88,32 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
     if (threadIdx.x == 0) *t.most = fits ? most : 0;
     if (!fits) return;
     __syncthreads();
-    for (int u = threadIdx.x; u < most * ax.m; u += blockDim.x) {
-        const int q = u / ax.m, node = u - q * ax.m;
-        const int2 r = t.range[node];
-        float w = 0.0f;
-        if (q <= r.y - r.x) {
-            const int i = r.x + q;
+    constexpr int kAt = 4;  // values in flight of a thread: each is a chain of three loads
+    const int all = most * ax.m;
+    for (int u0 = threadIdx.x; u0 < all; u0 += kAt * blockDim.x) {
+        float w[kAt];
+#pragma unroll
+        for (int e = 0; e < kAt; ++e) {
+            const int u = min(u0 + e * static_cast<int>(blockDim.x), all - 1);
+            const int q = u / ax.m, node = u - q * ax.m;
+            const int2 r = t.range[node];
+            const int i = min(r.x + q, n - 1);
             const unsigned k = static_cast<unsigned>(node - t.start[i]);
-            if (k < kW) w = t.w[static_cast<int64_t>(i) * kW + k];
+            w[e] = q <= r.y - r.x && k < kW ? t.w[static_cast<int64_t>(i) * kW + (k & (kW - 1))] : 0.0f;
         }
-        t.wt[u] = w;
+#pragma unroll
+        for (int e = 0; e < kAt; ++e)
+            if (u0 + e * static_cast<int>(blockDim.x) < all) t.wt[u0 + e * static_cast<int>(blockDim.x)] = w[e];
     }
 }
 
 // x: out[row][node] = sum over the node's cells of w g[row][cell].  A block
 // takes kTxRows rows of cells, staged in shared memory in pieces of kTxCells:
 // lanes are nodes, warps groups of rows, a thread kTxPer rows of one node (a
-// weight is read once for them).  Bound by the read of g and by latency.
+// weight is read once for them).  Of a row of more than one piece, 32 nodes
+// take only the cells that they weigh: staged whole for each 32 nodes, a row of
+// 16 384 cells and 520 nodes was read 17 times.  Bound by the read of g and by
+// latency.
 constexpr int kTxRows = 32, kTxPer = 4, kTxCells = 256;
 __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const float* g, int nx, int64_t n_rows,
                                                       BandAxisTab tab, float* __restrict__ out) {
@@ -105,16 +122,28 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
     if (b->n_light == 0) return;
     const int mx = b->ax[0].m, most = *tab.most;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kTxRows; r0 < n_rows;
-         r0 += static_cast<int64_t>(gridDim.x) * kTxRows) {
+    // a row of one piece stays for all its nodes; of a longer one a unit takes
+    // 32 nodes
+    const bool whole = nx <= kTxCells;
+    const int passes = whole ? 1 : (mx + 31) / 32;
+    const int64_t units = (n_rows + kTxRows - 1) / kTxRows * passes;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const int64_t r0 = u / passes * kTxRows;
+        const int first = static_cast<int>(u % passes) * 32, last = whole ? mx : min(first + 32, mx);
         const int nr = static_cast<int>(min(static_cast<int64_t>(kTxRows), n_rows - r0));
-        for (int n0 = 0; n0 < mx; n0 += 32) {
+        for (int n0 = first; n0 < last; n0 += 32) {
             const int node = n0 + lane;
             const int2 range = node < mx ? tab.range[node] : make_int2(0, -1);
             float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            for (int c0 = 0; c0 < nx; c0 += kTxCells) {
-                const int nc = min(kTxCells, nx - c0);
-                if (n0 == 0 || nx > kTxCells) {
+            // the cells of the row that these nodes need (the same in every warp)
+            int lo = 0, hi = nx - 1;
+            if (!whole) {
+                lo = __reduce_min_sync(0xffffffffu, range.y < range.x ? INT_MAX : range.x) & ~31;
+                hi = __reduce_max_sync(0xffffffffu, range.y);
+            }
+            for (int c0 = lo; c0 <= hi; c0 += kTxCells) {
+                const int nc = min(kTxCells, hi + 1 - c0);
+                if (n0 == 0 || !whole) {
                     __syncthreads();
                     for (int r = warp; r < kTxRows; r += 8)
 #pragma unroll 4
@@ -790,7 +819,11 @@ int launch_band_grid_spread(const BandDesc* b, const GridGeom& gg, const float* 
     const int64_t rows = int64_t(gg.ny) * gg.nz;
     cudaError_t e = launch_chained(band_axis_kernel, gg.nz > 1 ? 3 : 2, 1024, 0, st, b, gg, tab[0], tab[1], tab[2]);
     if (e == cudaSuccess)
-        e = launch_chained(band_tx_kernel, static_cast<unsigned>(std::min<int64_t>((rows + kTxRows - 1) / kTxRows, sms * 64)),
+        // long rows: a unit per 32 nodes, of which there are at most as many as cells
+        e = launch_chained(band_tx_kernel,
+                           static_cast<unsigned>(std::min<int64_t>(
+                               (rows + kTxRows - 1) / kTxRows * (gg.nx > kTxCells ? (gg.nx + 31) / 32 : 1),
+                               gg.nx > kTxCells ? sms * 7 : sms * 64)),
                            256, 0, st, b, g, gg.nx, rows, tab[0], h1);
     if (e == cudaSuccess)
         e = launch_chained(band_tline_kernel<true>, sms * 16, 256, 0, st, b, h1, gg.ny, gg.nz, tab[1],

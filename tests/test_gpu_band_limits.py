@@ -82,3 +82,18 @@ def test_long_x_axis(env, order):  # noqa: F811
     if order == "random":
         axes[0] = np.random.default_rng(3).permutation(axes[0])
     _check_grid(env, axes, (0.3, 0.3, 0.3), 1000, "rough")
+
+
+@pytest.mark.parametrize("order", ["running", "random", "gap"])
+def test_long_x_axis_adjoint(env, order):  # noqa: F811
+    # rows of several staged pieces: each 32 nodes take the cells that they
+    # weigh, all of them on an axis in no order, none for nodes inside a gap
+    x = np.linspace(0.0, 40.0, 5003).astype(np.float32)
+    if order == "random":
+        x = np.random.default_rng(3).permutation(x)
+    if order == "gap":
+        x = np.where(x > 20.0, x + np.float32(30.0), x)
+    axes = [x, np.linspace(0.0, 0.4, 37).astype(np.float32), np.linspace(0.0, 0.2, 31).astype(np.float32)]
+    m = np.meshgrid(*axes[::-1], indexing="ij")
+    cells = [np.ascontiguousarray(v.ravel()) for v in m[::-1]]
+    _check_adjoint(env, cells, (0.3, 0.3, 0.3), 2000, "gaussian")
