@@ -766,10 +766,12 @@ __global__ void __launch_bounds__(256, 3) band_cells_kernel(const BandDesc* b, c
 // A block takes tx x cells of kFinRows y cells of one layer: the rows' values
 // at the x nodes its cells read go to shared memory (a few values per cell,
 // since nodes are wider apart than cells), then every cell takes eight of
-// them.  Cells of an axis in no order may need more nodes than fit: they sum
-// their 64 values straight from memory.  Memory-bound on the outputs where
-// the maps are many, else on latency: all loads of a phase are independent.
-constexpr int kFinRows = 8, kFinNodes = 320;
+// them.  Cells of an axis in no order may need more nodes than fit: the block
+// then takes window after window of them (4096 x 4096 cells of a rough field, x
+// in random order: 1320 us a call with the 64 values of a cell summed from
+// memory, 408 so).  Memory-bound on the outputs where the maps are many, else on
+// latency: all loads of a phase are independent.
+constexpr int kFinRows = 8, kFinNodes = 320, kFinStep = kFinNodes - (kW - 1);
 __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b, const float* mid, const float* part,
                                                                GridGeom gg, int tx, int units, MapDev map,
                                                                unsigned long long* tiles) {
@@ -824,46 +826,39 @@ __global__ void __launch_bounds__(256, 4) band_finalize_kernel(const BandDesc* b
         }
     }
     __syncthreads();
-    const int n0 = first, nn = last - first;
-    const bool staged = n_light > 0 && nn <= kFinNodes;
-    if (staged) {
-        for (int e = t; e < kFinRows * nn; e += 256) {
-            const int r = e / nn, c = e - r * nn;
-            const float* p = base + static_cast<int64_t>(sy[r]) * mx + n0 + c;
-            float f[kW];
-#pragma unroll
-            for (int q = 0; q < kW; ++q) f[q] = q < nty ? p[static_cast<int64_t>(q) * mx] : 0.0f;
-            float v = 0.0f;
-#pragma unroll
-            for (int q = 0; q < kW / 2; ++q) v = fmaf(wy[r][q], f[q], fmaf(wy[r][kW - 1 - q], f[kW - 1 - q], v));
-            rows[r][c] = v;
-        }
-    }
-    __syncthreads();
     double loss = 0.0;
-    if (i < nx) {
-        const int64_t n = static_cast<int64_t>(nx) * ny * gg.nz;
+    const int64_t n = static_cast<int64_t>(nx) * ny * gg.nz;
+    // windows of nodes: a cell belongs to the one that holds its first node
+    const int n_end = n_light > 0 ? last - nt + 1 : 1;
+    for (int n0 = n_light > 0 ? first : 0; n0 < n_end; n0 += kFinStep) {
+        if (n_light > 0) {
+            const int nn = min(kFinNodes, last - n0);
+            __syncthreads();  // the previous window is no longer read
+            for (int e = t; e < kFinRows * nn; e += 256) {
+                const int r = e / nn, c = e - r * nn;
+                const float* p = base + static_cast<int64_t>(sy[r]) * mx + n0 + c;
+                float f[kW];
+#pragma unroll
+                for (int q = 0; q < kW; ++q) f[q] = q < nty ? p[static_cast<int64_t>(q) * mx] : 0.0f;
+                float v = 0.0f;
+#pragma unroll
+                for (int q = 0; q < kW / 2; ++q) v = fmaf(wy[r][q], f[q], fmaf(wy[r][kW - 1 - q], f[kW - 1 - q], v));
+                rows[r][c] = v;
+            }
+            __syncthreads();
+        }
+        if (i >= nx || static_cast<unsigned>(s - n0) >= static_cast<unsigned>(kFinStep)) continue;
 #pragma unroll 2
         for (int r = r0; r < min(kFinRows, ny - k0); r += rstep) {
             const int64_t o = (static_cast<int64_t>(l) * ny + k0 + r) * nx + i;
             const float target = mm ? map.T[o] : 0.0f;
             float v = 0.0f;
-            if (staged) {
+            if (n_light > 0) {
                 const float* p = &rows[r][s - n0];
 #pragma unroll
                 for (int q = 0; q < kW / 2; ++q) {
                     if (kW - 1 - q < nt) v = fmaf(w[kW - 1 - q], p[kW - 1 - q], v);
                     if (q < nt) v = fmaf(w[q], p[q], v);
-                }
-            } else if (n_light > 0) {
-                for (int q = 0; q < nt; ++q) {
-                    float f = 0.0f;
-                    for (int k = 0; k < nty; ++k)
-                        f = fmaf(wy[r][k], base[static_cast<int64_t>(sy[r] + k) * mx + s + q], f);
-                    float wq = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < kW; ++k) wq = k == q ? w[k] : wq;
-                    v = fmaf(wq, f, v);
                 }
             }
             float e = 0.0f;

@@ -97,3 +97,11 @@ def test_long_x_axis_adjoint(env, order):  # noqa: F811
     m = np.meshgrid(*axes[::-1], indexing="ij")
     cells = [np.ascontiguousarray(v.ravel()) for v in m[::-1]]
     _check_adjoint(env, cells, (0.3, 0.3, 0.3), 2000, "gaussian")
+
+
+@pytest.mark.parametrize("law", ["gaussian", "rough"])
+def test_wide_random_x_axis(env, law):  # noqa: F811
+    # 2-D: a block's cells read more x nodes than it stages at a time
+    axes = [np.random.default_rng(3).permutation(np.linspace(0.0, 60.0, 3001).astype(np.float32)),
+            np.linspace(0.0, 0.4, 400).astype(np.float32)]
+    _check_grid(env, axes, (0.3, 0.3), 2000, law)
