@@ -39,12 +39,18 @@ using band::kW;
 // ---------------------------------------------------------------------------
 
 // Block c: the cells' weights of axis c, their first nodes, for every node the
-// first and last cell that reads it, and the weights by node. Where the axis is
-// in no order a node's cells lie far apart: wt then does not hold them and the
-// sums run over all cells between, skipping those that do not read the node.
+// first and last of the cells that read it, and the weights by node.  The
+// cells are counted in the axis's own order where it runs one way; on an axis
+// in no order by their first nodes (`ord`, a counting sort), so that a node's
+// cells are neighbours there too: read as they come, a node takes the whole
+// axis (2048 x 128 x 64 cells of a rough field, all axes in random order: 1363
+// us a call, 680 so).  Where the cells crowd at few nodes that order would take long
+// and wt may not hold the weights: the sums then run over all cells between
+// the first and the last, skipping those that do not read the node.
+constexpr int kCrowd = 64;  // most cells with the same first node that are put in order
 __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, GridGeom gg, BandAxisTab tx, BandAxisTab ty,
                                                          BandAxisTab tz) {
-    __shared__ int most;
+    __shared__ int most, ups, downs, crowd, warps[32];
     pdl_wait();
     if (b->n_light == 0) return;
     const int c = blockIdx.x;
@@ -52,29 +58,84 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
     const float* X = c == 0 ? gg.X : c == 1 ? gg.Y : gg.Z;
     const int n = c == 0 ? gg.nx : c == 1 ? gg.ny : gg.nz;
     const BandAxisTab t = c == 0 ? tx : c == 1 ? ty : tz;
-    if (threadIdx.x == 0) most = 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) most = ups = downs = crowd = 0;
     for (int k = threadIdx.x; k < ax.m; k += blockDim.x) t.range[k] = make_int2(INT_MAX, -1);
     __syncthreads();
     const int nt = band::taps(ax);
-    for (int i0 = 0; i0 < n; i0 += blockDim.x) {
-        const int i = i0 + threadIdx.x;
-        const bool in = i < n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
         float w[kW];
-        const int s = in ? band::cell_weights(ax, __ldg(X + min(i, n - 1)), i, w) : -1;
-        // of neighbours with the same nodes the first and the last count
-        const int before = __shfl_up_sync(0xffffffffu, s, 1), after = __shfl_down_sync(0xffffffffu, s, 1);
-        const bool low = (threadIdx.x & 31) == 0 || before != s, high = (threadIdx.x & 31) == 31 || after != s;
-        if (!in) continue;  // no warp-wide step below
+        const float x = __ldg(X + i), before = __ldg(X + max(i - 1, 0));
+        const int s = band::cell_weights(ax, x, i, w);
+        if (!ax.ident && x > before) ups = 1;
+        if (!ax.ident && x < before) downs = 1;
         t.start[i] = s;
-        float4* o = reinterpret_cast<float4*>(t.w + static_cast<int64_t>(i) * kW);
 #pragma unroll
         for (int k = 0; k < kW; ++k) w[k] = k < nt ? w[k] : 0.0f;
+        float4* o = reinterpret_cast<float4*>(t.w + static_cast<int64_t>(i) * kW);
         o[0] = make_float4(w[0], w[1], w[2], w[3]);
         o[1] = make_float4(w[4], w[5], w[6], w[7]);
+    }
+    __syncthreads();
+    bool sorted = ups != 0 && downs != 0;
+    if (sorted) {
+        // cells per first node, then of the nodes before it
+        for (int k = threadIdx.x; k < ax.m; k += blockDim.x) t.pos[k] = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&t.pos[t.start[i]], 1);
+        __syncthreads();
+        int carry = 0;
+        for (int k0 = 0; k0 < ax.m; k0 += blockDim.x) {
+            const int k = k0 + threadIdx.x, own = k < ax.m ? t.pos[k] : 0;
+            if (own > kCrowd) crowd = 1;
+            int v = own;
 #pragma unroll
-        for (int k = 0; k < kW; ++k) {
-            if (k < nt && low) atomicMin(&t.range[s + k].x, i);
-            if (k < nt && high) atomicMax(&t.range[s + k].y, i);
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, v, off);
+                if (lane >= off) v += o;
+            }
+            if (lane == 31) warps[warp] = v;
+            __syncthreads();
+            int sum = warps[lane];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, sum, off);
+                if (lane >= off) sum += o;
+            }
+            const int until = __shfl_sync(0xffffffffu, sum, max(warp - 1, 0));
+            if (k < ax.m) t.pos[k] = carry + (warp > 0 ? until : 0) + v - own;
+            carry += __shfl_sync(0xffffffffu, sum, 31);
+            __syncthreads();
+        }
+        sorted = crowd == 0;
+    }
+    if (sorted) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) t.ord[atomicAdd(&t.pos[t.start[i]], 1)] = i;
+        __syncthreads();
+        // pos[k] is now the end of node k's cells; they get a fixed order
+        for (int k = threadIdx.x; k < ax.m; k += blockDim.x) {
+            const int p0 = k > 0 ? t.pos[k - 1] : 0, p1 = t.pos[k];
+            for (int p = p0 + 1; p < p1; ++p) {
+                const int v = t.ord[p];
+                int q = p;
+                for (; q > p0 && t.ord[q - 1] > v; --q) t.ord[q] = t.ord[q - 1];
+                t.ord[q] = v;
+            }
+            // read by the cells whose first node is k - 7 to k
+            t.range[k] = make_int2(k >= kW ? t.pos[k - kW] : 0, p1 - 1);
+        }
+    } else {
+        for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+            const int i = i0 + threadIdx.x;
+            const int s = i < n ? t.start[i] : -1;
+            // of neighbours with the same nodes the first and the last count
+            const int prev = __shfl_up_sync(0xffffffffu, s, 1), next = __shfl_down_sync(0xffffffffu, s, 1);
+            const bool low = lane == 0 || prev != s, high = lane == 31 || next != s;
+            if (i >= n) continue;  // the last round
+            for (int k = 0; k < nt; ++k) {
+                if (low) atomicMin(&t.range[s + k].x, i);
+                if (high) atomicMax(&t.range[s + k].y, i);
+            }
         }
     }
     __syncthreads();
@@ -85,10 +146,13 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
     for (int k = threadIdx.x; k < ax.m; k += blockDim.x)
         if (t.range[k].x > t.range[k].y) t.range[k] = make_int2(0, -1);
     const bool fits = static_cast<int64_t>(most) * ax.m <= band_wt_floats(n);
-    if (threadIdx.x == 0) *t.most = fits ? most : 0;
+    if (threadIdx.x == 0) {
+        t.most[0] = fits ? most : 0;
+        t.most[1] = sorted ? 1 : 0;
+    }
     if (!fits) return;
     __syncthreads();
-    constexpr int kAt = 4;  // values in flight of a thread: each is a chain of three loads
+    constexpr int kAt = 4;  // values in flight of a thread: each is a chain of loads
     const int all = most * ax.m;
     for (int u0 = threadIdx.x; u0 < all; u0 += kAt * blockDim.x) {
         float w[kAt];
@@ -97,7 +161,7 @@ __global__ void __launch_bounds__(1024) band_axis_kernel(const BandDesc* b, Grid
             const int u = min(u0 + e * static_cast<int>(blockDim.x), all - 1);
             const int q = u / ax.m, node = u - q * ax.m;
             const int2 r = t.range[node];
-            const int i = min(r.x + q, n - 1);
+            const int p = min(r.x + q, n - 1), i = sorted ? t.ord[p] : p;
             const unsigned k = static_cast<unsigned>(node - t.start[i]);
             w[e] = q <= r.y - r.x && k < kW ? t.w[static_cast<int64_t>(i) * kW + (k & (kW - 1))] : 0.0f;
         }
@@ -120,7 +184,8 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
     __shared__ float gs[kTxRows / kTxPer][kTxCells][kTxPer];
     pdl_wait();
     if (b->n_light == 0) return;
-    const int mx = b->ax[0].m, most = *tab.most;
+    const int mx = b->ax[0].m, most = tab.most[0];
+    const int32_t* ord = tab.most[1] ? tab.ord : nullptr;  // cells in the order of their nodes
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // a row of one piece stays for all its nodes; of a longer one a unit takes
     // 32 nodes
@@ -145,27 +210,38 @@ __global__ void __launch_bounds__(256) band_tx_kernel(const BandDesc* b, const f
                 const int nc = min(kTxCells, hi + 1 - c0);
                 if (n0 == 0 || !whole) {
                     __syncthreads();
-                    for (int r = warp; r < kTxRows; r += 8)
+                    if (ord == nullptr) {
+                        for (int r = warp; r < kTxRows; r += 8)
 #pragma unroll 4
-                        for (int i = lane; i < nc; i += 32)
-                            gs[r / kTxPer][i][r % kTxPer] = r < nr ? g[(r0 + r) * nx + c0 + i] : 0.0f;
+                            for (int i = lane; i < nc; i += 32)
+                                gs[r / kTxPer][i][r % kTxPer] = r < nr ? g[(r0 + r) * nx + c0 + i] : 0.0f;
+                    } else {
+                        for (int i = lane; i < nc; i += 32) {
+                            const int cell = ord[c0 + i];
+                            for (int r = warp; r < kTxRows; r += 8)
+                                gs[r / kTxPer][i][r % kTxPer] = r < nr ? g[(r0 + r) * nx + cell] : 0.0f;
+                        }
+                    }
                     __syncthreads();
                 }
                 const int ca = max(range.x, c0), cb = min(range.y, c0 + nc - 1);
-#pragma unroll 4
-                for (int i = ca; i <= cb; ++i) {
-                    float w = 0.0f;
-                    if (most > 0) {
-                        w = tab.wt[(i - range.x) * mx + node];
-                    } else {
-                        const unsigned k = static_cast<unsigned>(node - tab.start[i]);
-                        if (k < kW) w = tab.w[static_cast<int64_t>(i) * kW + k];
-                    }
+                auto add = [&](float w, int i) {
                     const float4 v = *reinterpret_cast<const float4*>(gs[warp][i - c0]);
                     acc.x = fmaf(w, v.x, acc.x);
                     acc.y = fmaf(w, v.y, acc.y);
                     acc.z = fmaf(w, v.z, acc.z);
                     acc.w = fmaf(w, v.w, acc.w);
+                };
+                if (most > 0) {
+                    const float* wt = tab.wt + (ca - range.x) * mx + node;
+#pragma unroll 8
+                    for (int i = ca; i <= cb; ++i, wt += mx) add(*wt, i);
+                } else {
+                    for (int i = ca; i <= cb; ++i) {
+                        const int cell = ord != nullptr ? ord[i] : i;
+                        const unsigned k = static_cast<unsigned>(node - tab.start[cell]);
+                        if (k < kW) add(tab.w[static_cast<int64_t>(cell) * kW + k], i);
+                    }
                 }
             }
             if (node < mx) {
@@ -190,7 +266,8 @@ __global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, cons
                                                          BandAxisTab tab, float* __restrict__ out) {
     pdl_wait();
     if (b->n_light == 0) return;
-    const int mx = b->ax[0].m, m = kY ? b->ax[1].m : b->ax[2].m, most = *tab.most;
+    const int mx = b->ax[0].m, m = kY ? b->ax[1].m : b->ax[2].m, most = tab.most[0];
+    const int32_t* ord = tab.most[1] ? tab.ord : nullptr;  // cells in the order of their nodes
     const int64_t plane = static_cast<int64_t>(mx) * b->ax[1].m;
     const int64_t all = kY ? plane * nz : plane * m;
     const int64_t stride = kY ? mx : plane;
@@ -209,14 +286,19 @@ __global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, cons
         }
         const int2 range = tab.range[node];
         float acc = 0.0f;
-        if (most > 0) {
+        if (most > 0 && ord == nullptr) {
 #pragma unroll 8
             for (int i = range.x; i <= range.y; ++i)
                 acc = fmaf(tab.wt[(i - range.x) * m + node], src[i * stride], acc);
+        } else if (most > 0) {
+#pragma unroll 8
+            for (int i = range.x; i <= range.y; ++i)
+                acc = fmaf(tab.wt[(i - range.x) * m + node], src[ord[i] * stride], acc);
         } else {
             for (int i = range.x; i <= range.y; ++i) {
-                const unsigned k = static_cast<unsigned>(node - tab.start[i]);
-                if (k < kW) acc = fmaf(tab.w[static_cast<int64_t>(i) * kW + k], src[i * stride], acc);
+                const int cell = ord != nullptr ? ord[i] : i;
+                const unsigned k = static_cast<unsigned>(node - tab.start[cell]);
+                if (k < kW) acc = fmaf(tab.w[static_cast<int64_t>(cell) * kW + k], src[cell * stride], acc);
             }
         }
         out[u] = acc;

@@ -380,9 +380,11 @@ struct LatticeRoom {
 struct BandAxisTab {
     float* w;        // [cells][8] weights
     int32_t* start;  // [cells] first node
-    int2* range;     // [nodes] first and last cell of a node
+    int2* range;     // [nodes] first and last cell of a node, counted as ord says
     float* wt;       // [cells of a node][nodes] the same weights by node, from the node's first cell
-    int32_t* most;   // most cells of a node, or 0 where wt does not hold them (axes in no order)
+    int32_t* most;   // [2] most cells of a node, or 0 where wt does not hold them; 1 where ord counts
+    int32_t* ord;    // [cells] axes in no order: the cells in the order of their nodes
+    int32_t* pos;    // [nodes] scratch of that order
 };
 // Floats of BandAxisTab::wt: a node of an axis in order has about 8 cells /
 // nodes cells.

@@ -735,7 +735,7 @@ namespace {
 // cells), at (x, y) nodes x z cells and at the nodes, the phasor tables and the
 // partial sums over the nodes.
 struct AdjBandLayout {
-    int64_t off_idx, idx, off_rank, off_tab[3][5], off_gain, off_h1, off_h2, off_nodes, off_ph[3], off_off[3], off_part, total;
+    int64_t off_idx, idx, off_rank, off_tab[3][7], off_gain, off_h1, off_h2, off_nodes, off_ph[3], off_off[3], off_part, total;
     int64_t cap_nodes, cap_mid;
 };
 AdjBandLayout adj_band_layout(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad, int sms) {
@@ -759,7 +759,9 @@ AdjBandLayout adj_band_layout(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad,
         L.off_tab[c][1] = take(dims[c] * 4);
         L.off_tab[c][2] = take(dims[c] * 8);
         L.off_tab[c][3] = take(band_wt_floats(dims[c]) * 4);
-        L.off_tab[c][4] = take(4);
+        L.off_tab[c][4] = take(8);
+        L.off_tab[c][5] = take(dims[c] * 4);
+        L.off_tab[c][6] = take(dims[c] * 4);
         L.off_ph[c] = take(dims[c] * n_pad * 8);
         L.off_off[c] = take(dims[c] * 4);
     }
@@ -947,6 +949,8 @@ int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const
             tab[c].range = reinterpret_cast<int2*>(bw + L.off_tab[c][2]);
             tab[c].wt = reinterpret_cast<float*>(bw + L.off_tab[c][3]);
             tab[c].most = reinterpret_cast<int32_t*>(bw + L.off_tab[c][4]);
+            tab[c].ord = reinterpret_cast<int32_t*>(bw + L.off_tab[c][5]);
+            tab[c].pos = reinterpret_cast<int32_t*>(bw + L.off_tab[c][6]);
             ph.ph[c] = reinterpret_cast<float2*>(bw + L.off_ph[c]);
             ph.off[c] = reinterpret_cast<float*>(bw + L.off_off[c]);
         }

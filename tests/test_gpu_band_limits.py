@@ -84,11 +84,17 @@ def test_long_x_axis(env, order):  # noqa: F811
     _check_grid(env, axes, (0.3, 0.3, 0.3), 1000, "rough")
 
 
-@pytest.mark.parametrize("order", ["running", "random", "gap"])
+@pytest.mark.parametrize("order", ["running", "back", "random", "gap", "crowd"])
 def test_long_x_axis_adjoint(env, order):  # noqa: F811
     # rows of several staged pieces: each 32 nodes take the cells that they
-    # weigh, all of them on an axis in no order, none for nodes inside a gap
+    # weigh, ordered by node on an axis in no order (unless they crowd at few
+    # nodes), none for nodes inside a gap
     x = np.linspace(0.0, 40.0, 5003).astype(np.float32)
+    if order == "back":
+        x = np.ascontiguousarray(x[::-1])
+    if order == "crowd":
+        x[::2] *= np.float32(1e-3)
+        x = np.random.default_rng(3).permutation(x)
     if order == "random":
         x = np.random.default_rng(3).permutation(x)
     if order == "gap":
@@ -97,6 +103,15 @@ def test_long_x_axis_adjoint(env, order):  # noqa: F811
     m = np.meshgrid(*axes[::-1], indexing="ij")
     cells = [np.ascontiguousarray(v.ravel()) for v in m[::-1]]
     _check_adjoint(env, cells, (0.3, 0.3, 0.3), 2000, "gaussian")
+
+
+def test_adjoint_with_every_axis_in_random_order(env):  # noqa: F811
+    rng = np.random.default_rng(7)
+    axes = [rng.permutation(np.linspace(0.0, e, n).astype(np.float32)) for n, e in ((300, 1.0), (141, 0.9), (130, 0.8))]
+    m = np.meshgrid(*axes[::-1], indexing="ij")
+    cells = [np.ascontiguousarray(v.ravel()) for v in m[::-1]]
+    for law in ("gaussian", "rough"):
+        _check_adjoint(env, cells, (0.15, 0.2, 0.2), 3000, law)
 
 
 @pytest.mark.parametrize("law", ["gaussian", "rough"])
