@@ -379,11 +379,17 @@ bool plan_grid(const void* plan, GridGeom* gg, float* box = nullptr) {
 // that then finds no lattice has paid kBandTryUs for the attempt.  q: largest
 // |kappa_c| that a fraction 2^-(k+1) of the modes exceeds, by dimension and
 // law (Student t with 1 and 3 degrees of freedom, normal), from 4 10^6 draws.
-// n: cells per axis of a grid, or null; cap: most nodes.  us_mode: time of one
-// mode summed directly.  Returns the modes expected to be left for the direct
-// sum, -1 where no gain of a quarter is expected.
-double band_worth(const grf_params* p, const float* box, const int32_t* n, double cap, double us_mode, double us_node,
-                double us_fixed) {
+// n: cells per axis of a grid, or null; cap: most nodes.  Returns the modes
+// expected to be left for the direct sum, -1 where no gain beyond the margin
+// is expected.
+struct BandCost {
+    double us_mode, us_node;  // one mode summed directly, one mode at one node
+    double fixed;             // the lattice's own kernels and the attempt
+    double direct0 = 0.0;     // a direct sum beside its modes
+    double heavy0 = 0.0;      // the kernels of the modes left for it
+    double margin = 0.75;     // of the direct time that the forecast must stay below
+};
+double band_worth(const grf_params* p, const float* box, const int32_t* n, double cap, const BandCost& cost) {
     static const float q[2][3][12] = {
         {{1.553f, 3.483f, 7.153f, 14.37f, 28.78f, 57.76f, 116.f, 232.f, 465.f, 916.f, 1853.f, 3539.f},
          {1.188f, 1.922f, 2.711f, 3.629f, 4.73f, 6.09f, 7.77f, 9.88f, 12.5f, 15.8f, 19.9f, 24.9f},
@@ -393,10 +399,10 @@ double band_worth(const grf_params* p, const float* box, const int32_t* n, doubl
          {1.584f, 2.115f, 2.53f, 2.888f, 3.206f, 3.5f, 3.773f, 4.029f, 4.273f, 4.503f, 4.729f, 4.947f}}};
     const double nu = p->family == GRF_GAUSSIAN ? 100.0 : p->family == GRF_EXPONENTIAL ? 0.5 : p->nu;
     const float* law = q[p->dim > 2 ? 1 : 0][nu < 1.5 ? 0 : nu < 8.0 ? 1 : 2];
-    const double N = static_cast<double>(p->n_modes), direct = us_mode * N;
+    const double N = static_cast<double>(p->n_modes);
     double min_ell = 1e300;
     for (int c = 0; c < p->dim; ++c) min_ell = std::min(min_ell, p->ell[c]);
-    double best = 0.75 * direct, left = -1.0;
+    double best = cost.margin * (cost.direct0 + cost.us_mode * N), left = -1.0;
     for (int k = 0; k < 12; ++k) {
         double heavy = std::ldexp(N, -(k + 1));
         const bool last = heavy < 2.0 || k == 11;
@@ -411,7 +417,8 @@ double band_worth(const grf_params* p, const float* box, const int32_t* n, doubl
         }
         const bool fits = nodes < cap;
         nodes = std::ceil(nodes / 16384.0) * 16384.0;
-        const double t = heavy * us_mode + (N - heavy) * nodes * us_node + us_fixed;
+        const double t = heavy * cost.us_mode + (heavy > 0.0 ? cost.heavy0 : 0.0) +
+                         (N - heavy) * nodes * cost.us_node + cost.fixed;
         if (fits && t < best) {
             best = t;
             left = heavy;
@@ -428,9 +435,14 @@ bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t
     const size_t extra = grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad);
     if (extra == 0 || ws_bytes < grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra) return false;
     const int32_t n[3] = {gg.nx, gg.ny, gg.nz};
-    // 3-D: two line kernels more (64^3 cells x 4096 modes gain nothing: 49.6 us directly, 49.7)
-    return band_worth(p, box, n, 0.25 * gg.nx * gg.ny * gg.nz, grid_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeUs,
-                      kBandFixedUs + kBandTryUs + (gg.nz > 1 ? 8.0 : 0.0)) >= 0.0;
+    const double us = grid_us_per_mode(gg.nx, gg.ny, gg.nz), N = static_cast<double>(p->n_modes);
+    // 3-D: two line kernels more
+    BandCost cost{us, kBandNodeUs, kBandFixedUs + kBandTryUs + (gg.nz > 1 ? 8.0 : 0.0)};
+    // 3-D grids of few tiles: whole calls as measured (GPU time, 64^3 to 128 x
+    // 128 x 64 cells x 1000 to 8000 modes, to 15 %), where both sides lie close
+    // (64^3 x 8000: 87 us as products, smooth 60 and Matern 95 with the lattice)
+    if (gg.nz > 1 && grid_splits(gg.nx, gg.ny, gg.nz)) cost = {0.72 * us, kBandNodeUs, 39.0 + 0.0025 * N, 13.0, 14.0, 1.0};
+    return band_worth(p, box, n, 0.25 * gg.nx * gg.ny * gg.nz, cost) >= 0.0;
 }
 
 bool lookup_plan(const void* plan, PlanMeta& out) {
@@ -868,6 +880,30 @@ int grf_read_status(const void* plan, int32_t* status_out, void* stream) try {
 // Synthesis
 // ---------------------------------------------------------------------------
 namespace {
+// Times of a synthesis at n cells of any plan.  Where the field is smooth at
+// the scale of the cells the direct kernel's time follows from the sizes alone
+// (fits of 16 thousand to 192 thousand cells x 700 to 8192 modes, GPU time, to
+// 15 %) and the chain's own from the modes: with its kernels charged as they
+// are, 128 x 128 cells x 5600 modes of a smooth field (47 us directly, 51 to
+// 54 with the lattice) and 42^3 x 2800, Matern (83 and 111) stay direct.  A
+// rougher field has modes that need exact phases at some or all tiles, which
+// double to quadruple the direct time; there the lattice's cost counts less.
+BandCost cells_cost(const grf_params* p, int64_t n, const float* box) {
+    const bool flat = p->dim == 2;
+    double volume = 1.0, ell = 1.0;
+    for (int c = 0; c < p->dim; ++c) {
+        volume *= static_cast<double>(box[3 + c]) - box[c];
+        ell *= p->ell[c];
+    }
+    const double N = static_cast<double>(p->n_modes), M = static_cast<double>(n);
+    const double step = std::pow(volume / M, 1.0 / p->dim) / std::pow(ell, 1.0 / p->dim);  // cell size / length
+    const bool matern = p->family == GRF_MATERN && p->nu >= 1.5;
+    if (p->family == GRF_GAUSSIAN ? step < 0.35 : matern && !flat && step < 0.25)
+        return flat ? BandCost{0.002 + M / 4.6e6, kBandNodeUs, 41.0 + 0.0023 * N + 1e-5 * M, 15.0, 4.0 + 0.0025 * N, 0.95}
+                    : BandCost{0.003 + M / 3.6e6, kBandNodeUs, 55.0 + 0.0023 * N + 3e-5 * M, 22.0, 15.0, 0.95};
+    return {cells_us_per_mode(n) * (flat ? 0.88 : 1.0), kBandNodeUs, cells_band_us(n, p->dim) + kBandTryUs};
+}
+
 // The segment's bounds on the device where the call takes the band path at
 // the cells of a plan that is not a grid, else null.  Cells whose bounds the
 // host does not know (several segments) try it where the sum is long.  few:
@@ -878,11 +914,10 @@ CellsBand cells_band(const grf_params* p, const void* plan, const PlanMeta& meta
     const int64_t n = meta.offsets[segment + 1] - meta.offsets[segment];
     const size_t need = cells_band_ws_bytes(n, p->n_modes, p->dim);
     if (need == 0 || ws_bytes < need) return CellsBand{};
-    const double us = cells_us_per_mode(n), fixed = cells_band_us(n, p->dim) + kBandTryUs;
     const double N = static_cast<double>(p->n_modes);
     const double left = std::isfinite(box[0])
-                            ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), us, kBandNodeUs, fixed)
-                            : us * N < 500.0 ? -1.0 : N;
+                            ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), cells_cost(p, n, box))
+                            : cells_us_per_mode(n) * N < 500.0 ? -1.0 : N;
     if (left < 0.0) return CellsBand{};
     return CellsBand{
         reinterpret_cast<const SegInfo*>(static_cast<const unsigned char*>(plan) + meta.layout.off_segs) + segment,
@@ -1217,8 +1252,10 @@ int grf_synth_backward(const void* table, const grf_params* p, const void* plan,
         const int32_t cells[3] = {gg.nx, gg.ny, gg.nz};
         const bool band =
             extra > 0 && g_grid_enabled.load() != 2 && ws_bytes >= bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) + extra &&
-            band_worth(p, box, cells, 0.25 * static_cast<double>(n), grid_adjoint_us_per_mode(gg.nx, gg.ny, gg.nz),
-                       kBandNodeAdjUs, grid_adjoint_band_us(gg.nx, gg.ny, gg.nz) + kBandTryUs) >= 0.0;
+            band_worth(p, box, cells, 0.25 * static_cast<double>(n),
+                       {grid_adjoint_call_us_per_mode(gg.nx, gg.ny, gg.nz), kBandNodeAdjUs,
+                        grid_adjoint_band_us(gg.nx, gg.ny, gg.nz) + kAdjBandCallUs, kAdjCallUs, grid_adjoint_heavy_us(n),
+                        0.9}) >= 0.0;
         const int err = launch_synth_bwd_grid(table, p->n_modes, p->dim, gg, gY, std::sqrt(p->sigma2), p->ell, rot,
                                               periodic, *g, workspace, band, status, stream);
         if (err != cudaSuccess) return cuda_fail(err, "grid backward kernels");
@@ -1230,8 +1267,8 @@ int grf_synth_backward(const void* table, const grf_params* p, const void* plan,
     const SegInfo* band = nullptr;
     if (extra > 0 && ws_bytes >= need + extra && g_grid_enabled.load() != 0) {
         const double us = cells_adjoint_us_per_mode(n);
-        if (std::isfinite(box[0]) ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), us, kBandNodeAdjUs,
-                                               cells_adjoint_band_us(n, p->dim) + kBandTryUs) >= 0.0
+        if (std::isfinite(box[0]) ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)),
+                                               {us, kBandNodeAdjUs, cells_adjoint_band_us(n, p->dim) + kBandTryUs}) >= 0.0
                                   : us * static_cast<double>(p->n_modes) >= 500.0)
             band = reinterpret_cast<const SegInfo*>(pb + meta.layout.off_segs) + segment;
     }

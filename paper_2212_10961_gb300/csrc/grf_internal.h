@@ -532,6 +532,10 @@ size_t bwd_grid_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
 int launch_synth_bwd_grid(const void* table, int64_t n_modes, int32_t dim, const GridGeom& gg, const float* gY,
                           double sigma, const double* ell, const double* rot, int32_t periodic_mask,
                           const grf_grads& g, void* ws, bool band, int32_t* status, void* stream);
+// Measured times of the band path (us): one mode at one node (tensor cores,
+// whole 128 x 128 tiles), the kernels that the lattice adds, and the kernels
+// that a call pays for when the device finds no lattice worth while.
+constexpr double kBandNodeUs = 1.0 / 22.0e6, kBandFixedUs = 15.0, kBandTryUs = 14.0;
 // band: the band path, whose workspace (bwd_grid_band_ws_bytes) follows.
 size_t bwd_grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
 double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
@@ -539,6 +543,12 @@ double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
 // kernels that the lattice adds.
 constexpr double kBandNodeAdjUs = 1.0 / 6.0e6;
 double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz);
+// The same as a forecast of whole calls: a mode as products, the other kernels
+// of a call with all of them so, what those and the lattice's chain take
+// beside grid_adjoint_band_us, and the kernels of modes left for the products.
+double grid_adjoint_call_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
+constexpr double kAdjCallUs = 35.0, kAdjBandCallUs = 40.0 + kBandTryUs;
+double grid_adjoint_heavy_us(int64_t n_cells);
 size_t cells_adjoint_band_ws_bytes(int64_t n_cells, int64_t n_modes, int32_t dim);
 LatticeRoom cells_adjoint_room(int64_t n_cells, int64_t n_modes, int32_t dim);
 LatticeRoom cells_room(int64_t n_cells, int64_t n_modes, int32_t dim);
@@ -582,12 +592,10 @@ int launch_synth_grid(const void* table, int64_t n_modes, int32_t dim, const Gri
                       void* ws, bool band, int32_t fc, int32_t* status, void* stream);
 // Time of one mode summed at the cells of a grid by the grid path, us.
 double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz);
+// Whether the grid path splits the modes of this grid's tiles over several CTAs.
+bool grid_splits(int32_t nx, int32_t ny, int32_t nz);
 // Further workspace of the band path on a grid (0: not taken at these sizes).
 size_t grid_band_ws_bytes(int32_t nx, int32_t ny, int32_t nz, int64_t n_pad);
-// Measured times of the band path (us): one mode at one node (tensor cores,
-// whole 128 x 128 tiles), the kernels that the lattice adds, and the kernels
-// that a call pays for when the device finds no lattice worth while.
-constexpr double kBandNodeUs = 1.0 / 22.0e6, kBandFixedUs = 15.0, kBandTryUs = 14.0;
 // Band path kernels (band.cu).
 int launch_band_select(const BandSelect& p, BandDesc* out, void* stream);
 int launch_band_lines(const BandDesc* b, float* part, const GridGeom& gg, float* mid, float* rows, int sms,

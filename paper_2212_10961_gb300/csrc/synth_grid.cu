@@ -1149,6 +1149,8 @@ double grid_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
     return g.max_split > 1 ? double(g.n_tiles) * tile / 42.0e6 : std::ceil(double(g.n_tiles) / 152.0) * 152.0 * tile / 65.0e6;
 }
 
+bool grid_splits(int32_t nx, int32_t ny, int32_t nz) { return grid_plan(nx, ny, nz, 4).max_split > 1; }
+
 // CUDA-core kernels: 4.2 Tcell.mode/s at the cells of any plan (one hardware
 // cosine each), half of it at 30 000 cells, whose tiles leave SMs idle.  The lattice's interpolation: 50 ps per cell in 3-D, 10 in 2-D.
 double cells_us_per_mode(int64_t n_cells) { return 0.006 + double(n_cells) / 4.2e6; }

@@ -803,6 +803,17 @@ double grid_adjoint_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
     const AdjPlan a = adj_plan(nx, ny, nz, 128, 1);
     return double(a.units) * kAX * kAYZ / 38.0e6;
 }
+// Measured over whole calls (GPU time, 1000 to 8000 modes): units of one z
+// cell a column, as all of 2-D grids, take 3.8 times as long (1024 x 512: 0.053
+// us a mode), patches of fewer than 64 y cells 1.5 to 1.7 times (250 x 130 x 65: 0.105).
+double grid_adjoint_call_us_per_mode(int32_t nx, int32_t ny, int32_t nz) {
+    const double us = grid_adjoint_us_per_mode(nx, ny, nz);
+    return us * (nz == 1 ? 3.8 : adj_plan(nx, ny, nz, 128, 1).py_log2 < 6 ? 1.5 : 1.0);
+}
+// The direct modes' tables hold all of g, and their units run at any count: 46
+// us more at 2.1M cells (128^3 x 2000 modes, Matern: 145 us as products, 160
+// with 128 modes left).
+double grid_adjoint_heavy_us(int64_t n) { return 15.0 + 1.5e-5 * double(n); }
 double grid_adjoint_band_us(int32_t nx, int32_t ny, int32_t nz) { return 25.0 + 6e-6 * double(nx) * ny * nz; }
 
 // Below 60 us of direct products the lattice's ten launches cost what they

@@ -120,3 +120,35 @@ def test_wide_random_x_axis(env, law):  # noqa: F811
     axes = [np.random.default_rng(3).permutation(np.linspace(0.0, 60.0, 3001).astype(np.float32)),
             np.linspace(0.0, 0.4, 400).astype(np.float32)]
     _check_grid(env, axes, (0.3, 0.3), 2000, law)
+
+
+def _launches(F, torch, table, p, plan):
+    n = F.launch_count()
+    F.synth(table, p, plan)
+    torch.cuda.synchronize()
+    return F.launch_count() - n
+
+
+@pytest.mark.parametrize("shape,ell,n,law,offset,lattice", [
+    ((128, 128), 0.2, 5600, "gaussian", 0.0, False),       # 47 us directly, 51 with the lattice
+    ((250, 130), 0.2, 3700, "gaussian", 0.0, False),       # 50 and 52
+    ((250, 130), 0.2, 5600, "gaussian", 0.0, True),        # 68 and 51
+    ((64, 60, 50), 0.2, 1400, "gaussian", 0.0, True),      # 111 and 62
+])
+def test_calls_that_cannot_gain_are_not_tried(env, shape, ell, n, law, offset, lattice):  # noqa: F811
+    torch, F, W = env
+    dim = len(shape)
+    rng = np.random.default_rng(4)
+    h = 1.0 / max(shape)
+    axes = np.meshgrid(*[(np.arange(k) + 0.5) * h for k in shape[::-1]], indexing="ij")[::-1]
+    cells = [(v.ravel() + offset + (0.0 if law == "grid" else 0.4 * h) * rng.uniform(-1, 1, v.size)).astype(np.float32) for v in axes]
+    plan = F.CellPlan(*to_dev(torch, [np.ascontiguousarray(c) for c in cells]))
+    m = _modes(n, dim, (ell,) * dim, "gaussian", 6)
+    table, p = F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, n, dim, (ell,) * dim)
+    taken = _launches(F, torch, table, p, plan)
+    try:
+        F.grid_path("always" if law == "grid" else False)
+        direct = _launches(F, torch, table, p, plan)
+    finally:
+        F.grid_path(True)
+    assert (taken > direct) == lattice
