@@ -408,14 +408,18 @@ double band_worth(const grf_params* p, const float* box, const int32_t* n, doubl
         const bool last = heavy < 2.0 || k == 11;
         heavy = last ? 0.0 : std::ceil(heavy / 128.0) * 128.0;
         double nodes = 1.0;
+        bool exact = true;  // node coordinates are, within 2^16 spacings of 0 (band.cuh)
         for (int c = 0; c < p->dim; ++c) {
             // a margin for the width of the selection's bins
             const double a = 1.05 * law[k] / (2.0 * M_PI * (has_rotation(p) ? min_ell : p->ell[c]));
             double m = 4.0 * a * (static_cast<double>(box[3 + c]) - box[c]) + 9.0;
-            if (n) m = std::min(m, static_cast<double>(n[c]));
+            if (n && m >= n[c])
+                m = n[c];  // not interpolated
+            else
+                exact = exact && 4.0 * a * std::max(std::fabs(box[c]), std::fabs(box[3 + c])) < 65000.0;
             nodes *= m;
         }
-        const bool fits = nodes < cap;
+        const bool fits = exact && nodes < cap;
         nodes = std::ceil(nodes / 16384.0) * 16384.0;
         const double t = heavy * cost.us_mode + (heavy > 0.0 ? cost.heavy0 : 0.0) +
                          (N - heavy) * nodes * cost.us_node + cost.fixed;

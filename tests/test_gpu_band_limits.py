@@ -134,6 +134,8 @@ def _launches(F, torch, table, p, plan):
     ((250, 130), 0.2, 3700, "gaussian", 0.0, False),       # 50 and 52
     ((250, 130), 0.2, 5600, "gaussian", 0.0, True),        # 68 and 51
     ((64, 60, 50), 0.2, 1400, "gaussian", 0.0, True),      # 111 and 62
+    ((64, 60, 50), 0.2, 1400, "gaussian", 2.0e4, False),   # nodes beyond 2^16 spacings from 0: the device refuses
+    ((96, 80, 70), 0.2, 4000, "grid", 2.0e4, False),       # the same on a grid
 ])
 def test_calls_that_cannot_gain_are_not_tried(env, shape, ell, n, law, offset, lattice):  # noqa: F811
     torch, F, W = env
