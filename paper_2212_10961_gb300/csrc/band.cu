@@ -437,8 +437,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     }
 }
 
-// The nodes' partial sums of the mode splits, added in split order into the
-// first one's place.
+// The nodes' partial sums of the mode splits, added in split order and
+// compensated, as the cells' are, into the first one's place (bound by the read).
 __global__ void __launch_bounds__(256) band_sum_kernel(const BandDesc* b, float* part) {
     pdl_wait();
     const int n_split = b->nodes.n_split;
@@ -446,16 +446,16 @@ __global__ void __launch_bounds__(256) band_sum_kernel(const BandDesc* b, float*
     const int64_t all = static_cast<int64_t>(b->ax[0].m) * b->ax[1].m * b->ax[2].m;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < all;
          i += static_cast<int64_t>(gridDim.x) * 256) {
-        float v = 0.0f;
+        float v = 0.0f, e = 0.0f;
 #pragma unroll 16
-        for (int q = 0; q < n_split; ++q) v += part[q * all + i];
-        part[i] = v;
+        for (int q = 0; q < n_split; ++q) two_sum_acc(v, e, part[q * all + i]);
+        part[i] = v + e;
     }
 }
 
 // Interpolation along one axis.  kY = false (z): mid[l][y node][x node] from
-// the nodes; kY = true: rows[(l ny + k) lp + x node] from mid (or, in 2-D, from
-// the nodes), zero for the x nodes up to lp (a multiple of 4).
+// the nodes; kY = true (3-D): rows[(l ny + k) lp + x node] from mid, zero for
+// the x nodes up to lp (a multiple of 4).
 // A block takes 64 columns (the values of one axis position, contiguous in
 // memory) and a run of cells of the axis: the run's nodes go to shared memory,
 // each read once per block, and the cells' weights, shared by the columns;
