@@ -317,11 +317,12 @@ __global__ void __launch_bounds__(256) band_tline_kernel(const BandDesc* b, cons
 struct FixedScale {
     float first, second;
 };
+constexpr float kFiniteMax = 3.402823466e38f;
 __device__ __forceinline__ FixedScale fixed_scale(const float* gmax, int n_gmax, int64_t n) {
     float m = 0.0f;
     for (int k = threadIdx.x & 31; k < n_gmax; k += 32) m = fmaxf(m, gmax[k]);
     m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
-    if (!(m > 0.0f) || !(m < 3.0e38f)) return FixedScale{1.0f, 1.0f};
+    if (!(m > 0.0f) || !(m <= kFiniteMax)) return FixedScale{1.0f, 1.0f};
     int e = 0, c = 0;
     frexpf(m, &e);
     frexpf(static_cast<float>(n), &c);
@@ -330,7 +331,7 @@ __device__ __forceinline__ FixedScale fixed_scale(const float* gmax, int n_gmax,
 
 __device__ __forceinline__ bool gmax_finite(const float* gmax, int n_gmax) {
     bool ok = true;
-    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) ok = ok && gmax[k] < 3.0e38f;
+    for (int k = threadIdx.x & 31; k < n_gmax; k += 32) ok = ok && gmax[k] <= kFiniteMax;
     return __all_sync(0xffffffffu, ok);
 }
 

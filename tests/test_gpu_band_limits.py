@@ -154,3 +154,11 @@ def test_calls_that_cannot_gain_are_not_tried(env, shape, ell, n, law, offset, l
     finally:
         F.grid_path(True)
     assert (taken > direct) == lattice
+
+
+def test_adjoint_of_the_largest_finite_gradient(env):  # noqa: F811
+    # max |g| just below the largest float is finite
+    c = [np.ascontiguousarray(v) for v in np.random.default_rng(5).random((250_000, 3)).astype(np.float32).T]
+    g = np.zeros(250_000, dtype=np.float32)
+    g[1234] = 3.1e38
+    _check_adjoint(env, c, (0.2, 0.2, 0.2), 4000, "gaussian", g=g)
