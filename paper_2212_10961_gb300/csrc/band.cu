@@ -446,9 +446,12 @@ __global__ void __launch_bounds__(256) band_sum_kernel(const BandDesc* b, float*
     const int64_t all = static_cast<int64_t>(b->ax[0].m) * b->ax[1].m * b->ax[2].m;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < all;
          i += static_cast<int64_t>(gridDim.x) * 256) {
-        float v = 0.0f, e = 0.0f;
-#pragma unroll 16
-        for (int q = 0; q < n_split; ++q) two_sum_acc(v, e, part[q * all + i]);
+        float x[kNodeSplits];  // all loads in flight: summed as they come, 1024 x 512 cells took 5 us more
+#pragma unroll
+        for (int q = 0; q < kNodeSplits; ++q) x[q] = q < n_split ? part[q * all + i] : 0.0f;
+        float v = x[0], e = 0.0f;
+#pragma unroll
+        for (int q = 1; q < kNodeSplits; ++q) two_sum_acc(v, e, x[q]);
         part[i] = v + e;
     }
 }
