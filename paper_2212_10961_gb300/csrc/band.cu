@@ -322,8 +322,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) band_select_kernel(const __gri
     const int nh = n - n_light;
     const BandAxis none{0.0f, 0.0f, 0, 0, 1};
     const BandAxis ax[3] = {n_light > 0 ? axs[0] : none, n_light > 0 ? axs[1] : none, n_light > 0 ? axs[2] : none};
-    if (t == 0)
-        for (int c = 0; c < 3; ++c) out->ax[c] = ax[c];
+    if (t < 3) out->ax[t] = n_light > 0 ? axs[t] : none;
     // ---- slots of the light and the other modes, in table order, and a bound
     // of the light ones' amplitudes with their gains
     float top = 0.0f;
