@@ -541,15 +541,22 @@ __global__ void __launch_bounds__(256) synth_split_finalize(FwdDesc d, const flo
         const int64_t i = u * 256 + threadIdx.x;
         double l = 0.0;
         if (i < d.n_cells) {
-            float s = 0.0f, e = 0.0f;
-            for (int k = 0; k < n_split; ++k) {
-                const float2 v = partial[static_cast<int64_t>(k) * d.n_cells + i];
-                two_sum_acc(s, e, v.x);
-                e += v.y;
-            }
-            if (d.add != nullptr) two_sum_acc(s, e, d.add[i]);
-            const float y = (s + e) + d.map.mu;
             const int64_t o = static_cast<int64_t>(__ldg(d.perm + i)) - d.perm_base;
+            const float add = d.add != nullptr ? d.add[i] : 0.0f;
+            float s = 0.0f, e = 0.0f;
+            for (int k0 = 0; k0 < n_split; k0 += 8) {  // 8 splits' loads in flight
+                float2 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    v[k] = k0 + k < n_split ? partial[static_cast<int64_t>(k0 + k) * d.n_cells + i] : make_float2(0.0f, 0.0f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    two_sum_acc(s, e, v[k].x);
+                    e += v[k].y;
+                }
+            }
+            if (d.add != nullptr) two_sum_acc(s, e, add);
+            const float y = (s + e) + d.map.mu;
             if (index_ok(o, d.n_cells)) {
                 map_store(d.map, o, y);
                 if (d.map.bits & kMapMismatch) l = mismatch_store(d.map, o, y);

@@ -767,7 +767,11 @@ __global__ void __launch_bounds__(256) grid_split_finalize(const float* part, in
     double l = 0.0;
     if (o < n) {
         float s = 0.0f, e = 0.0f;
-        for (int k = 0; k < n_split; ++k) two_sum_acc(s, e, part[static_cast<int64_t>(k) * n + o]);
+        float v[kGMaxSplit];  // all splits' loads in flight
+#pragma unroll
+        for (int k = 0; k < kGMaxSplit; ++k) v[k] = k < n_split ? part[static_cast<int64_t>(k) * n + o] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < kGMaxSplit; ++k) two_sum_acc(s, e, v[k]);
         const float y = (s + e) + map.mu;
         map_store(map, o, y);
         if (mm) l = mismatch_store(map, o, y);
