@@ -458,6 +458,18 @@ bool lookup_plan(const void* plan, PlanMeta& out) {
     return true;
 }
 
+// Dimension of a plan and cells of a segment (-1: out of range), without a copy
+// of the plan's record: the workspace queries allocate nothing.
+bool plan_segment(const void* plan, int32_t segment, int32_t& dim, int64_t& n) {
+    std::lock_guard<std::mutex> lk(g_reg_mu);
+    auto it = g_plans.find(plan);
+    if (it == g_plans.end()) return false;
+    const auto& o = it->second.offsets;
+    dim = it->second.dim;
+    n = segment >= 0 && segment < static_cast<int32_t>(o.size()) - 1 ? o[segment + 1] - o[segment] : -1;
+    return true;
+}
+
 struct BatchMeta {
     BatchHeader hdr;
     int32_t plan_dim;
@@ -1022,10 +1034,10 @@ int grf_synth_field(const void* table, const grf_params* p, const void* plan, in
 
 size_t grf_synth_band_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
     try {
-        PlanMeta meta;
-        if (!plan || n_modes < 1 || n_modes > GRF_MAX_MODES || !lookup_plan(plan, meta)) return 0;
-        if (segment < 0 || segment >= static_cast<int32_t>(meta.offsets.size()) - 1) return 0;
-        return cells_workspace(meta.offsets[segment + 1] - meta.offsets[segment], n_modes, meta.dim);
+        int32_t dim = 0;
+        int64_t n = 0;
+        if (!plan || n_modes < 1 || n_modes > GRF_MAX_MODES || !plan_segment(plan, segment, dim, n) || n < 0) return 0;
+        return cells_workspace(n, n_modes, dim);
     } catch (...) {
         return 0;
     }
@@ -1033,16 +1045,15 @@ size_t grf_synth_band_workspace_bytes(const void* plan, int32_t segment, int64_t
 
 size_t grf_synth_plan_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes) {
     try {
-        PlanMeta meta;
-        if (!plan || !lookup_plan(plan, meta)) return 0;
-        const bool in = segment >= 0 && segment < static_cast<int32_t>(meta.offsets.size()) - 1;
-        const int64_t n = in ? meta.offsets[segment + 1] - meta.offsets[segment] : 0;
-        const size_t split = synth_workspace_bytes(n);
-        if (!in || n_modes < 1 || n_modes > GRF_MAX_MODES) return split;
+        int32_t dim = 0;
+        int64_t n = 0;
+        if (!plan || !plan_segment(plan, segment, dim, n)) return 0;
+        const size_t split = synth_workspace_bytes(std::max<int64_t>(n, 0));
+        if (n < 0 || n_modes < 1 || n_modes > GRF_MAX_MODES) return split;
         GridGeom gg{};
         if (segment == 0 && plan_grid(plan, &gg))
             if (const size_t grid = grid_workspace(gg, n_modes)) return std::max(split, grid);
-        return std::max(split, cells_workspace(n, n_modes, meta.dim));
+        return std::max(split, cells_workspace(n, n_modes, dim));
     } catch (...) {
         return 0;
     }
@@ -1192,12 +1203,12 @@ size_t grf_backward_band_workspace_bytes(int64_t n_cells, int64_t n_modes, int32
 
 size_t grf_backward_plan_workspace_bytes(const void* plan, int32_t segment, int64_t n_modes, int32_t dim) {
     try {
-        PlanMeta meta;
-        if (!plan || !lookup_plan(plan, meta) || n_modes < 1 || n_modes > GRF_MAX_MODES || dim < 1 || dim > 3) return 0;
-        const bool in = segment >= 0 && segment < static_cast<int32_t>(meta.offsets.size()) - 1;
-        const int64_t n = in ? meta.offsets[segment + 1] - meta.offsets[segment] : 0;
-        const size_t cells = bwd_workspace_bytes(n, n_modes, dim);
-        if (!in) return cells;
+        int32_t plan_dim = 0;
+        int64_t n = 0;
+        if (!plan || n_modes < 1 || n_modes > GRF_MAX_MODES || dim < 1 || dim > 3 || !plan_segment(plan, segment, plan_dim, n))
+            return 0;
+        const size_t cells = bwd_workspace_bytes(std::max<int64_t>(n, 0), n_modes, dim);
+        if (n < 0) return cells;
         GridGeom gg{};
         if (segment == 0 && plan_grid(plan, &gg))
             if (const size_t grid = grid_adjoint_workspace(gg, n_modes)) return std::max(cells, grid);
