@@ -432,6 +432,12 @@ double band_worth(const grf_params* p, const float* box, const int32_t* n, doubl
     return left;
 }
 
+// Whether a workspace holds the grid path of a synthesis.
+bool grid_fits(const GridGeom& gg, int64_t n_modes, size_t ws_bytes) {
+    const size_t b = grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(n_modes).n_pad);
+    return grid_ws_ok(b, gg) && ws_bytes >= b;
+}
+
 // The same for a call on a Cartesian grid, with the workspace it has.
 bool grid_band(const grf_params* p, const GridGeom& gg, const float* box, size_t ws_bytes) {
     if (g_grid_enabled.load() == 2) return false;
@@ -1016,9 +1022,7 @@ int grf_synth_field(const void* table, const grf_params* p, const void* plan, in
     GridGeom gg{};
     float box[6] = {NAN, NAN, NAN, NAN, NAN, NAN};
     if (n > 0 && workspace && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim &&
-        plan_grid(plan, &gg, box) && use_grid_path(gg) &&
-        grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
-        ws_bytes >= grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad)) {
+        plan_grid(plan, &gg, box) && use_grid_path(gg) && grid_fits(gg, p->n_modes, ws_bytes)) {
         const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, workspace, grid_band(p, gg, box, ws_bytes),
                                           g_grid_fold.load(), status, stream);
         if (err != cudaSuccess) return cuda_fail(err, "grid synth kernels");
@@ -1134,8 +1138,7 @@ int grf_synth_mismatch(const void* table, const grf_params* p, const void* plan,
     GridGeom gg{};
     float box[6] = {NAN, NAN, NAN, NAN, NAN, NAN};
     if (n > 0 && g_grid_enabled.load() != 0 && n_seg == 1 && p->dim == meta.dim && plan_grid(plan, &gg, box) &&
-        use_grid_path(gg) && grid_ws_ok(grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad), gg) &&
-        ws_bytes - lbytes >= grid_ws_bytes(gg.nx, gg.ny, gg.nz, table_layout(p->n_modes).n_pad) &&
+        use_grid_path(gg) && grid_fits(gg, p->n_modes, ws_bytes - lbytes) &&
         grid_loss_partials(gg.nx, gg.ny, gg.nz) <= mismatch_partials(n)) {
         const int err = launch_synth_grid(table, p->n_modes, p->dim, gg, d.map, split_ws,
                                           grid_band(p, gg, box, ws_bytes - lbytes), g_grid_fold.load(), status,
@@ -1282,8 +1285,14 @@ int grf_synth_backward(const void* table, const grf_params* p, const void* plan,
     const SegInfo* band = nullptr;
     if (extra > 0 && ws_bytes >= need + extra && g_grid_enabled.load() != 0) {
         const double us = cells_adjoint_us_per_mode(n);
-        if (std::isfinite(box[0]) ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)),
-                                               {us, kBandNodeAdjUs, cells_adjoint_band_us(n, p->dim) + kBandTryUs}) >= 0.0
+        BandCost cost{us, kBandNodeAdjUs, cells_adjoint_band_us(n, p->dim) + kBandTryUs};
+        // few cells in 3-D: whole calls as measured (16 thousand cells x 2600 and
+        // 4000 modes); modes left for the direct sum walk it one after the other
+        // (24 x 26 x 27 x 4000: 254 us directly, 318 with 512 modes left, 143 with none)
+        if (p->dim > 2 && n < 20000)
+            cost = {0.03 + static_cast<double>(n) / 2.8e6, kBandNodeAdjUs, 105.0 + 0.005 * static_cast<double>(p->n_modes),
+                    100.0, 130.0, 0.95};
+        if (std::isfinite(box[0]) ? band_worth(p, box, nullptr, static_cast<double>(cells_band_cap(n)), cost) >= 0.0
                                   : us * static_cast<double>(p->n_modes) >= 500.0)
             band = reinterpret_cast<const SegInfo*>(pb + meta.layout.off_segs) + segment;
     }

@@ -162,3 +162,25 @@ def test_adjoint_of_the_largest_finite_gradient(env):  # noqa: F811
     g = np.zeros(250_000, dtype=np.float32)
     g[1234] = 3.1e38
     _check_adjoint(env, c, (0.2, 0.2, 0.2), 4000, "gaussian", g=g)
+
+
+@pytest.mark.parametrize("ell,lattice", [(0.08, False), (0.2, True)])  # 254 us directly, 318 with the lattice; 244 and 143
+def test_adjoints_that_cannot_gain_are_not_tried(env, ell, lattice):  # noqa: F811
+    torch, F, W = env
+    rng = np.random.default_rng(3)
+    axes = np.stack(np.meshgrid(np.arange(24), np.arange(26), np.arange(27), indexing="ij"), 0).reshape(3, -1)
+    c = ((axes + 0.5 + rng.uniform(-0.4, 0.4, axes.shape)) / 27).astype(np.float32)
+    plan = F.CellPlan(*to_dev(torch, list(c)))
+    m = _modes(4000, 3, (ell,) * 3, "gaussian", 6)
+    table, p = F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, 4000, 3, (ell,) * 3)
+    g = torch.ones(c.shape[1], device="cuda")
+    counts = []
+    for setting in (True, False):
+        F.grid_path(setting)
+        try:
+            n = F.launch_count()
+            F.backward(table, p, plan, g)
+            counts.append(F.launch_count() - n)
+        finally:
+            F.grid_path(True)
+    assert (counts[0] > counts[1]) == lattice
