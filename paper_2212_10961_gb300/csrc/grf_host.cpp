@@ -907,7 +907,8 @@ namespace {
 // (fits of 16 thousand to 192 thousand cells x 700 to 8192 modes, GPU time, to
 // 15 %) and the chain's own from the modes: with its kernels charged as they
 // are, 128 x 128 cells x 5600 modes of a smooth field (47 us directly, 51 to
-// 54 with the lattice) and 42^3 x 2800, Matern (83 and 111) stay direct.  A
+// 54 with the lattice), 186 x 192 x 4000, Matern (47 and 57), and 42^3 x 2800,
+// Matern (83 and 111) stay direct.  A
 // rougher field has modes that need exact phases at some or all tiles, which
 // double to quadruple the direct time; there the lattice's cost counts less.
 BandCost cells_cost(const grf_params* p, int64_t n, const float* box) {
@@ -920,8 +921,9 @@ BandCost cells_cost(const grf_params* p, int64_t n, const float* box) {
     const double N = static_cast<double>(p->n_modes), M = static_cast<double>(n);
     const double step = std::pow(volume / M, 1.0 / p->dim) / std::pow(ell, 1.0 / p->dim);  // cell size / length
     const bool matern = p->family == GRF_MATERN && p->nu >= 1.5;
-    if (p->family == GRF_GAUSSIAN ? step < 0.35 : matern && !flat && step < 0.25)
-        return flat ? BandCost{0.002 + M / 4.6e6, kBandNodeUs, 41.0 + 0.0023 * N + 1e-5 * M, 15.0, 4.0 + 0.0025 * N, 0.95}
+    if (p->family == GRF_GAUSSIAN ? step < 0.35 : matern && step < (flat ? 0.07 : 0.25))
+        return flat ? BandCost{0.002 + M / 4.6e6, kBandNodeUs, 41.0 + 0.0023 * N + 1e-5 * M, 15.0, 1.0 + 0.0016 * N,
+                               matern ? 0.93 : 0.95}
                     : BandCost{0.003 + M / 3.6e6, kBandNodeUs, 55.0 + 0.0023 * N + 3e-5 * M, 22.0, 15.0, 0.95};
     return {cells_us_per_mode(n) * (flat ? 0.88 : 1.0), kBandNodeUs, cells_band_us(n, p->dim) + kBandTryUs};
 }
