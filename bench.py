@@ -324,6 +324,7 @@ def bench_forward(torch, F, W, name, rank, world, steps, warmup, scale, with_e2e
     torch.cuda.synchronize()
     pf.close()
     paths = take_paths(F)
+    formed = formed_products(F, "synth", plan, ps.params, ps.workspace, launches / float(steps + warmup), M)
     kern_all = [a.elapsed_time(b) for a, b in kev[warmup:]]
     kern_ms = float(np.mean(kern_all))
     assert plan.status() == 0
@@ -341,7 +342,7 @@ def bench_forward(torch, F, W, name, rank, world, steps, warmup, scale, with_e2e
            "kernel_ms_median": max_over_ranks(torch, world, float(np.median(kern_all))),
            "kernel_ms_best": max_over_ranks(torch, world, float(np.min(kern_all))), "plan_ms": plan_ms,
            "cell_modes_per_step": float(M) * N, "launches_in_timed_region": int(round(per_step * steps)),
-           "launches_per_step": per_step, "y_seed": y_seed, **path_fields(paths)}
+           "launches_per_step": per_step, "y_seed": y_seed, **path_fields(paths), **formed}
     if check and rank == 0:
         res["fp64_check"] = fp64_check(cells, y_seed, oracle_modes_for(w, dim, w["seed"]), w["mean"], sig,
                                        thresholds=thr, facies=fac_seed)
@@ -484,6 +485,7 @@ def bench_fwd_bwd(torch, F, W, rank, world, steps, warmup, scale):
     T = F.GaussianField(pt).synth(plan, F.MapSpec(y=False, lognormal=True))["K"]
     base = w["seed"] + 1000 * rank
     ring = [F.ModeTable.from_modes(F.gen_modes(params_for(F, w, 3, base + k))) for k in range(2)]
+    ws = F.Workspace(), F.Workspace()
     st = torch.cuda.current_stream()
     kev = []
 
@@ -494,9 +496,9 @@ def bench_fwd_bwd(torch, F, W, rank, world, steps, warmup, scale):
         b = torch.cuda.Event(enable_timing=True)
         c = torch.cuda.Event(enable_timing=True)
         a.record(st)
-        loss, gY, _ = F.synth_mismatch(tab, p, plan, T)
+        loss, gY, _ = F.synth_mismatch(tab, p, plan, T, workspace=ws[0])
         b.record(st)
-        F.backward(tab, p, plan, gY)
+        F.backward(tab, p, plan, gY, workspace=ws[1])
         c.record(st)
         kev.append((a, b, c))
 
@@ -509,12 +511,16 @@ def bench_fwd_bwd(torch, F, W, rank, world, steps, warmup, scale):
     paths = take_paths(F)
     bgen, blat = F.take_adjoint_path_counts()
     bgrid = F.take_grid_adjoint_units()
+    # more than 14 launches: both calls on the node lattice
+    pf, lf = params_for(F, w, 3, base), launches / float(steps + warmup) - 10
+    formed = [formed_products(F, k, plan, pf, b, lf, M) for k, b in zip(("mismatch", "backward"), ws)]
     fwd_ms = float(np.mean([a.elapsed_time(b) for a, b, c in kev[warmup:]]))
     bwd_ms = float(np.mean([b.elapsed_time(c) for a, b, c in kev[warmup:]]))
     res = {"workload": "diff128" if scale == 1 else "diff128/%d" % scale, "cells": M, "modes": N,
            "ms_per_step": ms, "fwd_ms": fwd_ms, "bwd_ms": bwd_ms, "cell_modes_per_step": float(M) * N,
            "launches_per_step": launches / float(steps + warmup),
            "forward": "fused synthesis + lognormal mismatch loss and gradient (grf_synth_mismatch)",
+           "fwd_products": formed[0], "bwd_products": formed[1],
            **path_fields(paths),
            "adjoint_path_tiles": {"general": bgen, "lattice": blat, "grid_units": bgrid},
            "adjoint_lattice_share": blat / float(bgen + blat) if bgen + blat else 0.0,
@@ -788,37 +794,52 @@ GRID_TENSOR_FLOPS_PER_CELL_MODE = 12.0
 GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE = 24.0
 
 # Calls large enough sum their modes of low frequency on a coarse node lattice
-# and interpolate: they form fewer cell-mode products than these counts assume.
-EQUIVALENT = ("equivalent rate: counts every mode at every cell; modes of low frequency may be summed on the node "
-              "lattice instead, so frac compares with summing all of them directly and can pass 1")
+# and interpolate: rates in cell-modes count every mode at every cell, fractions
+# of a peak count the products that the last timed call formed.
+EQUIVALENT = ("achieved and frac count the products formed (direct modes at the cells, modes of low frequency at the "
+              "nodes of a coarse lattice); gcell_modes_per_s counts every mode at every cell")
+
+
+def formed_products(F, kind, plan, params, workspace, launches, cells):
+    """Mode products of one call with the node lattice: direct modes at the
+    cells and light ones at the nodes (the interpolation not counted), and how
+    the modes were divided; {} where the call has none."""
+    if launches < 5:
+        return {}
+    c = F.lattice_choice(kind, plan, params, workspace)
+    if c["light"] == 0:
+        return {}
+    nodes = c["nodes"][0] * c["nodes"][1] * max(1, c["nodes"][2])
+    return {"node_lattice": c, "products_formed": float(cells) * c["direct"] + float(nodes) * c["light"]}
 
 # Grid-path setting of this run (--grid-path), restored after checks that
 # force the grid path on grids below the automatic threshold.
 GRID_SETTING = True
 
 
-def roofline(kern_ms, cell_modes, clocks, sms, traffic=None, lattice_share=0.0, grid=False):
+def roofline(kern_ms, cell_modes, clocks, sms, traffic=None, lattice_share=0.0, grid=False, formed=None):
     """Roofline of a synthesis kernel.  General path: the MUFU pipe, 1
     hardware cosine per cell-mode.  Lattice path (lattice_share >= 1/2 of the
     warp tiles): the FP32 pipe at LATTICE_FP32_PER_CELL_MODE instructions per
     cell-mode (1/8 MUFU per cell-mode); the MUFU fraction is kept beside it.
     Grid path: the tensor cores at GRID_TENSOR_FLOPS_PER_CELL_MODE FP16 flops
     per cell-mode against the measured dense BF16 peak (kern_ms covers all of
-    the call's kernels).  All of them count every mode at every cell
-    (EQUIVALENT)."""
+    the call's kernels).  formed: products that the call formed, where it
+    took the node lattice (EQUIVALENT); all of its time is charged to them."""
     mufu_peak = MUFU_PER_CLK_PER_SM * sms * 2070e6 / 1e9  # Gcell.mode/s at the maximum SM clock
     achieved = cell_modes / (kern_ms * 1e-3) / 1e9
+    done = formed or cell_modes
     if grid:
         tpk, kind = tensor_peak()
-        tf = cell_modes * GRID_TENSOR_FLOPS_PER_CELL_MODE / (kern_ms * 1e-3) / 1e12
+        tf = done * GRID_TENSOR_FLOPS_PER_CELL_MODE / (kern_ms * 1e-3) / 1e12
         return {"bound": "tensor", "achieved": tf, "peak": tpk, "unit": "TFLOP/s", "frac": tf / tpk,
                 "traffic": traffic, "peak_kind": kind, "note": EQUIVALENT,
                 "peak_basis": ("tensor-core grid path: %.0f FP16 tensor flops per cell-mode (a 2-term real dot "
                                "product as three FP16 products hi.hi + hi.lo + lo.hi) against the %s dense BF16 "
                                "cuBLAS burst peak (FP16 runs at the BF16 rate)" %
                                (GRID_TENSOR_FLOPS_PER_CELL_MODE, kind)),
-                "gcell_modes_per_s": achieved, "frac_of_mufu_roofline": achieved / mufu_peak,
-                "frac_of_lattice_fp32_roofline": achieved / (FP32_PER_CLK_PER_SM * sms * 2070e6 /
+                "gcell_modes_per_s": achieved, "frac_of_mufu_roofline": done / cell_modes * achieved / mufu_peak,
+                "frac_of_lattice_fp32_roofline": done / cell_modes * achieved / (FP32_PER_CLK_PER_SM * sms * 2070e6 /
                                                              LATTICE_FP32_PER_CELL_MODE / 1e9)}
     if lattice_share >= 0.5:
         peak_max = FP32_PER_CLK_PER_SM * sms * 2070e6 / LATTICE_FP32_PER_CELL_MODE / 1e9
@@ -829,12 +850,13 @@ def roofline(kern_ms, cell_modes, clocks, sms, traffic=None, lattice_share=0.0, 
         peak_max = mufu_peak
         basis = "%d MUFU cos/clk/SM x %d SMs x 2070 MHz (1 MUFU per cell-mode)" % (MUFU_PER_CLK_PER_SM, sms)
         per_clk = MUFU_PER_CLK_PER_SM
-    out = {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "Gcell.mode/s",
-           "frac": achieved / peak_max, "traffic": traffic, "peak_basis": basis, "note": EQUIVALENT,
-           "frac_of_mufu_roofline": achieved / mufu_peak}
+    rate = done / (kern_ms * 1e-3) / 1e9
+    out = {"bound": "alu", "achieved": rate, "peak": peak_max, "unit": "Gcell.mode/s",
+           "frac": rate / peak_max, "traffic": traffic, "peak_basis": basis, "note": EQUIVALENT,
+           "gcell_modes_per_s": achieved, "frac_of_mufu_roofline": rate / mufu_peak}
     if clocks.get("sm_mhz"):
         peak_meas = per_clk * sms * clocks["sm_mhz"] * 1e6 / 1e9
-        out["frac_at_measured_clock"] = achieved / peak_meas
+        out["frac_at_measured_clock"] = rate / peak_meas
     return out
 
 
@@ -966,7 +988,8 @@ def main():
         v["gcell_modes_per_s"] = v["cell_modes_per_step"] * world / (v["ms_per_step"] * 1e-3) / 1e9
         if "kernel_ms" in v:
             v["roofline"] = roofline(v["kernel_ms"], v["cell_modes_per_step"], ck, sms,
-                                     lattice_share=v.get("lattice_share", 0.0), grid=v.get("grid_path", False))
+                                     lattice_share=v.get("lattice_share", 0.0), grid=v.get("grid_path", False),
+                                     formed=v.get("products_formed"))
     if k_b := extra.get("batched"):
         # one cosine per lane of the general path comes from the FMA pipe: the
         # MUFU pipe's share of that path's work; the lattice lanes (the 64^3
@@ -984,21 +1007,26 @@ def main():
         k_fb["roofline_fwd_bwd"] = {
             "achieved": k_fb["cell_modes_per_step"] / ((k_fb["fwd_ms"] + k_fb["bwd_ms"]) * 1e-3) / 1e9,
             "peak": MUFU_PER_CLK_PER_SM * sms * 2070e6 / 3 / 1e9, "unit": "Gcell.mode/s"}
-        k_fb["roofline_fwd_bwd"]["frac"] = k_fb["roofline_fwd_bwd"]["achieved"] / k_fb["roofline_fwd_bwd"]["peak"]
+        # no fraction: with the node lattice the step forms far fewer products
+        k_fb["roofline_fwd_bwd"]["times_every_mode_at_every_cell"] = (k_fb["roofline_fwd_bwd"]["achieved"] /
+                                                                       k_fb["roofline_fwd_bwd"]["peak"])
         k_fb["roofline_fwd_bwd"]["peak_basis"] = ("3 MUFU per cell-mode (1 forward cosine, adjoint sine and "
                                                   "cosine); the forward's own bound is in fwd_roofline")
         # each half against its own bound
         k_fb["fwd_roofline"] = roofline(k_fb["fwd_ms"], k_fb["cell_modes_per_step"], ck, sms,
                                         lattice_share=k_fb.get("lattice_share", 0.0),
-                                        grid=k_fb.get("grid_path", False))
+                                        grid=k_fb.get("grid_path", False),
+                                        formed=k_fb["fwd_products"].get("products_formed"))
         bw = k_fb["cell_modes_per_step"] / (k_fb["bwd_ms"] * 1e-3) / 1e9
         bmufu = MUFU_PER_CLK_PER_SM * sms * 2070e6 / 2 / 1e9
         if k_fb.get("adjoint_grid_path", False):
             tpk, kind = tensor_peak()
-            tf = k_fb["cell_modes_per_step"] * GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE / (k_fb["bwd_ms"] * 1e-3) / 1e12
+            done = k_fb["bwd_products"].get("products_formed", k_fb["cell_modes_per_step"])
+            tf = done * GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE / (k_fb["bwd_ms"] * 1e-3) / 1e12
             k_fb["bwd_roofline"] = {
                 "bound": "tensor", "achieved": tf, "peak": tpk, "unit": "TFLOP/s", "frac": tf / tpk,
-                "peak_kind": kind, "gcell_modes_per_s": bw, "frac_of_mufu_roofline": bw / bmufu,
+                "peak_kind": kind, "gcell_modes_per_s": bw,
+                "frac_of_mufu_roofline": done / k_fb["cell_modes_per_step"] * bw / bmufu,
                 "peak_basis": ("tensor-core grid adjoint: %.0f FP16 tensor flops per cell-mode (cos and sin "
                                "products of g and of x-weighted g, three FP16 products each) against the %s dense "
                                "BF16 burst peak" % (GRID_ADJ_TENSOR_FLOPS_PER_CELL_MODE, kind)),
@@ -1029,7 +1057,8 @@ def main():
         "plan_ms_once_per_mesh": head["plan_ms"],
         "roofline": roofline(head["kernel_ms"], head["cell_modes_per_step"], ck, sms,
                              HEAD_TRAFFIC_BYTES if args.scale == 1 and HEAD_TRAFFIC_BYTES else None,
-                             head.get("lattice_share", 0.0), grid=head.get("grid_path", False)),
+                             head.get("lattice_share", 0.0), grid=head.get("grid_path", False),
+                             formed=head.get("products_formed")),
         "grid_path": head.get("grid_path", False),
         "path_warps": head.get("path_warps"),
         "kernel_ms": head["kernel_ms"], "kernel_ms_median": head["kernel_ms_median"],

@@ -709,6 +709,18 @@ int grf_take_grid_adjoint_units(int64_t *units);
 int grf_debug_grid_path(int32_t enable, int32_t fold_chunks);
 
 /*
+ * grf_debug_lattice_choice -- what the last call of a kind chose: the modes
+ * summed at the nodes, those summed at the cells, and the nodes per axis.
+ * kind: 0 grf_synth_field, 1 grf_synth_mismatch, 2 grf_synth_backward; plan,
+ * segment, n_modes, dim and workspace are that call's.  out (5): all zero at
+ * sizes where no lattice is offered; meaningful only after a call that
+ * launched the lattice's kernels.  Synchronises the device.  GRF_EINVAL for
+ * NULL pointers, unknown plans or values out of range.
+ */
+int grf_debug_lattice_choice(int32_t kind, const void *plan, int32_t segment, int64_t n_modes, int32_t dim,
+                             const void *workspace, int64_t *out);
+
+/*
  * grf_debug_lattice_room -- sizes of the node lattice's part of a workspace,
  * for tests.  kind: 0 synthesis at any cells, 1 its adjoint (cells[0] cells of
  * a dim-dimensional field), 2 synthesis on a grid, 3 its adjoint (cells[0..2]

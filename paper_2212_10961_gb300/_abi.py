@@ -156,6 +156,8 @@ _SIGS = {
     "grf_take_grid_tiles": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int64)]),
     "grf_take_grid_adjoint_units": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int64)]),
     "grf_debug_grid_path": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32]),
+    "grf_debug_lattice_choice": (ctypes.c_int, [ctypes.c_int32, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64,
+                                                ctypes.c_int32, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64)]),
     "grf_debug_lattice_room": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, ctypes.POINTER(ctypes.c_int64),
                                               ctypes.c_int64, ctypes.POINTER(ctypes.c_int64)]),
     "grf_debug_mma_f16": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p,

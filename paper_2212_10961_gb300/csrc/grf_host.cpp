@@ -1837,6 +1837,46 @@ int grf_debug_grid_path(int32_t enable, int32_t fold_chunks) {
     return GRF_OK;
 }
 
+int grf_debug_lattice_choice(int32_t kind, const void* plan, int32_t segment, int64_t n_modes, int32_t dim,
+                             const void* workspace, int64_t* out) try {
+    if (!plan || !workspace || !out) return fail(GRF_EINVAL, "NULL argument");
+    int32_t plan_dim = 0;
+    int64_t n = 0;
+    if (!plan_segment(plan, segment, plan_dim, n) || n < 0) return fail(GRF_EINVAL, "unknown plan or segment");
+    if (kind < 0 || kind > 2 || dim < 2 || dim > plan_dim || n_modes < 1 || n_modes > GRF_MAX_MODES)
+        return fail(GRF_EINVAL, "kind must be in 0..2, dim and n_modes those of the call");
+    const int64_t n_pad = table_layout(n_modes).n_pad;
+    GridGeom gg{};
+    const bool grid = segment == 0 && dim == plan_dim && g_grid_enabled.load() != 0 && plan_grid(plan, &gg);
+    // the descriptor comes first in the lattice's part of the workspace
+    size_t at = kind == 1 ? static_cast<size_t>(align256(mismatch_partials(n) * 8)) : 0;
+    bool offered;
+    if (kind == 2) {
+        const size_t b = grid ? bwd_grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+        const bool on_grid = grid && grid_ws_ok(b, gg);
+        offered = on_grid ? bwd_grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) > 0
+                          : cells_adjoint_band_ws_bytes(n, n_modes, dim) > 0;
+        at = on_grid ? b : bwd_workspace_bytes(n, n_modes, dim);
+    } else {
+        const size_t b = grid ? grid_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) : 0;
+        const bool on_grid = grid && grid_ws_ok(b, gg);
+        offered = on_grid ? grid_band_ws_bytes(gg.nx, gg.ny, gg.nz, n_pad) > 0 : cells_band_ws_bytes(n, n_modes, dim) > 0;
+        if (on_grid) at += b;
+    }
+    for (int k = 0; k < 5; ++k) out[k] = 0;
+    if (!offered) return GRF_OK;
+    BandDesc b;
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(&b, static_cast<const unsigned char*>(workspace) + at, sizeof(b), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "lattice descriptor");
+    out[0] = b.n_light;
+    out[1] = b.nh;
+    for (int c = 0; c < 3; ++c) out[2 + c] = b.ax[c].m;
+    return GRF_OK;
+} catch (...) {
+    return host_exception();
+}
+
 int grf_debug_lattice_room(int32_t kind, int32_t dim, const int64_t* cells, int64_t n_modes, int64_t* out) try {
     if (!cells || !out) return fail(GRF_EINVAL, "NULL argument");
     if (kind < 0 || kind > 3 || dim < 2 || dim > 3 || n_modes < 1 || n_modes > GRF_MAX_MODES)

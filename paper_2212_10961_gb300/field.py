@@ -463,8 +463,9 @@ def synth(table: ModeTable, params: FieldParams, plan: CellPlan, segment=0, maps
           stream=None, workspace=None):
     """Field and fused maps at every cell of `segment` (original cell order).
 
-    workspace: a Workspace for the mode split of small segments (default: a
-    module-level one; pass workspace=False for none)."""
+    workspace: a Workspace for what the call can use (synth_workspace_bytes:
+    the mode split, the grid path's tables, the node lattice); default: a
+    module-level one.  workspace=False: none, all modes summed at the cells."""
     maps = maps or MapSpec()
     n = plan.segment_size(segment)
     if out is None:
@@ -490,6 +491,7 @@ class PreparedSynth:
         n = plan.segment_size(segment)
         self.out = out if out is not None else maps.allocate(n, plan.buf.device)
         self.plan = plan
+        self.params = params
         self._p = params.to_c()
         self._m = maps.to_c()
         self._o = _outputs_struct(self.out)
@@ -498,6 +500,10 @@ class PreparedSynth:
         self._stream = None if stream is None else _stream_handle(stream)
         self._args = (ctypes.byref(self._p), plan.ptr, int(segment), ctypes.byref(self._m), ctypes.byref(self._o),
                       _ptr(self._ws), self._nbytes)
+
+    @property
+    def workspace(self):
+        return self._ws
 
     def __call__(self, table: ModeTable, stream=None):
         st = _stream_handle(stream) if stream is not None else (self._stream or _stream_handle(None))
@@ -897,6 +903,18 @@ def take_adjoint_path_counts():
     g, l_ = ctypes.c_int64(0), ctypes.c_int64(0)
     check(lib().grf_take_adjoint_path_counts(ctypes.byref(g), ctypes.byref(l_)))
     return g.value, l_.value
+
+
+def lattice_choice(kind, plan, params, workspace, segment=0):
+    """What the last call of a kind ("synth", "mismatch" or "backward") with
+    this workspace (a Workspace or its tensor) chose on the node lattice
+    (grf_debug_lattice_choice): dict with light and direct mode counts and the
+    nodes per axis; synchronises the device."""
+    buf = workspace.buf if isinstance(workspace, Workspace) else workspace
+    out = (ctypes.c_int64 * 5)()
+    check(lib().grf_debug_lattice_choice(("synth", "mismatch", "backward").index(kind), plan.ptr, int(segment),
+                                         int(params.n_modes), int(params.dim), _ptr(buf), out))
+    return {"light": out[0], "direct": out[1], "nodes": tuple(out[2:5])}
 
 
 def take_grid_tiles():

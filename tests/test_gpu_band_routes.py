@@ -24,7 +24,7 @@ ROUTES = [("grid 2-D", _uniform((701, 499), (1.4, 1.0)), (0.2, 0.1), 6000),
           ("cells 2-D", None, (0.2, 0.25), 4000), ("cells 3-D", None, (0.2, 0.25, 0.2), 4000)]
 
 
-# "rough" leaves modes for the direct sum on every route, "gaussian" mostly none
+# "rough" leaves modes for the direct sum on every route, "gaussian" none
 @pytest.mark.parametrize("law", ["gaussian", "rough"])
 @pytest.mark.parametrize("name,axes,ell,n", ROUTES, ids=[r[0] for r in ROUTES])
 def test_large_calls_run_on_the_lattice(env, name, axes, ell, n, law):  # noqa: F811
@@ -36,10 +36,19 @@ def test_large_calls_run_on_the_lattice(env, name, axes, ell, n, law):  # noqa: 
     table, p = F.ModeTable(m["amp"], m["psi"], m["a"]), _params(F, n, dim, ell)
     g = torch.randn(len(cells[0]), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
 
+    ws, wb = F.Workspace(), F.Workspace()
+
     def call():
-        return F.synth(table, p, plan)["Y"], F.backward(table, p, plan, g)["dA"]
+        return F.synth(table, p, plan, workspace=ws)["Y"], F.backward(table, p, plan, g, workspace=wb)["dA"]
 
     y, da = call()
+    chosen = [F.lattice_choice("synth", plan, p, ws)]
+    if name not in ("grid 2-D", "grid 3-D, few tiles"):  # their adjoints keep the products
+        chosen.append(F.lattice_choice("backward", plan, p, wb))
+    for c in chosen:
+        assert c["light"] > 0 and c["light"] + c["direct"] == n
+        assert (c["direct"] > 0) == (law == "rough")
+        assert all(k >= 8 for k in c["nodes"][:dim])
     try:
         F.grid_path("always" if axes else False)
         y0, da0 = call()
@@ -48,8 +57,8 @@ def test_large_calls_run_on_the_lattice(env, name, axes, ell, n, law):  # noqa: 
     torch.cuda.synchronize()
     assert not torch.equal(y, y0)
     assert (y - y0).abs().max().item() <= 2e-5  # twice the forward tolerance of either
-    if name in ("grid 2-D", "grid 3-D, few tiles"):
-        return  # the adjoint of these sizes keeps the products
+    if len(chosen) == 1:
+        return
     assert not torch.equal(da, da0)
     assert (da - da0).abs().max().item() <= 2e-4 * da0.abs().max().item()
 
