@@ -629,9 +629,17 @@ def bench_bitruncated(torch, F, W, rank, world, steps, warmup, scale):
     ms = timed_steps(torch, world, steps, warmup, lambda i: pg.synth(plan, t, (0.0,), rule, values))
     launches = F.launch_count() - l0
     paths = take_paths(F)
+    # the two fields' own divisions of the modes, from a call each
+    formed = []
+    for f in (pg.f1, pg.f2):
+        ws, l0 = F.Workspace(), F.launch_count()
+        F.synth(f.table, f.params, plan, workspace=ws)
+        formed.append(formed_products(F, "synth", plan, f.params, ws, F.launch_count() - l0, M))
+    products = [f.get("products_formed", float(M) * N) for f in formed]
     res = {"workload": "grid3d_256 bitruncated: exponential l=(0.2,0.2,0.05) x Gaussian l=0.1, 3 x 2 rule",
            "cells": M, "modes_per_field": N, "ms_per_step": ms, "cell_modes_per_step": 2.0 * M * N,
-           "launches_per_step": launches / float(steps + warmup), "kernel_ms": ms, **path_fields(paths)}
+           "launches_per_step": launches / float(steps + warmup), "kernel_ms": ms, **path_fields(paths),
+           "node_lattices": [f.get("node_lattice") for f in formed], "products_formed": sum(products)}
     if rank == 0:
         # both fields against the oracle's own draws (streams 0 and 1), and the
         # merged facies against the rule applied to the oracle fields

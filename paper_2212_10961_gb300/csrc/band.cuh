@@ -13,10 +13,13 @@
 // cell takes W^dim node values; the others are summed at the cells as before.
 // The adjoint applies the same weights transposed.
 //
-// Error.  With beta = 0.99 pi W (1 - xi) the aliased copies of a mode are
-// below 1.7e-7 of its amplitude anywhere in the band and 3e-8 at half of it
-// (gen_band_weights.py), for every phase and position: less than the FP32
-// rounding of the direct sums (3e-7 to 4e-7 of sigma).  Node coordinates
+// Error.  With beta = 0.99 pi W (1 - xi) the aliased copies of a mode along
+// one axis are, relative to its amplitude, at most 1.6e-7 in RMS over the
+// positions and 2.5e-7 at the worst one anywhere in the band, 3e-8 and 4e-8 at
+// half of it (gen_band_weights.py).  The axes' errors add: at a corner of the
+// band in 3-D 2.8e-7 in RMS, 7.5e-7 at worst.  Few modes lie there and their
+// errors are unrelated, so that fields stay below the FP32 rounding of the
+// direct sums (2.0e-7 to 3.5e-7 of sigma in RMS against 2.7e-7 to 4.1e-7).  Node coordinates
 // n h are exact FP32 numbers (h has 8 significant bits, |n| < 2^16), so node
 // phases are reduced exactly like cell phases, and x - n h is exact.
 //

@@ -4,14 +4,14 @@ The Kaiser-Bessel window of width W = 8 nodes (Kaiser and Schafer, "On the use
 of the I0-sinh window for spectrum analysis", 1980),
     phi(t) = I0(beta sqrt(1 - (2 t / W)^2)) / I0(beta),  |t| <= W / 2,
 with beta = 0.99 pi W (1 - xi), xi = 1/4 the largest frequency in turns per node (the factor puts the zero of the
-nearest alias inside the band edge: the largest aliasing error falls from 6.8e-7 to 1.6e-7),
+nearest alias inside the band edge: the RMS aliasing error falls from 6.8e-7 to 1.6e-7),
 divided by its integral phihat(0) = W sinh(beta) / (beta I0(beta)).  A cell at
 u = v + 1/2 in [0, 1) between the nodes 3 and 4 of its eight takes the weight
 phi(v + 7/2 - k) at node k; with p_k(v) that function for k = 0 .. 3 the other
 four are p_{7-k}(v) = p_k(-v).  Each p_k is the least-squares polynomial of
 degree 9 on Chebyshev nodes of [-1/2, 1/2], computed in FP64 and rounded to
 FP32.  The script prints the coefficients, the error of their FP32 Horner
-evaluation, and the largest aliasing error over the frequencies |xi| <= 1/4.
+evaluation, and the aliasing error over the frequencies |xi| <= 1/4, RMS and largest over the positions.
 
 Run: python gen_band_weights.py   (numpy and scipy)
 """
@@ -56,9 +56,18 @@ def main():
         err = np.max(np.abs(acc - phi(dense.astype(np.float32).astype(np.float64) + 3.5 - k)))
         print("{%s},  // node %d: %.1e" % (", ".join("%.9ef" % q for q in c), k, err))
     xi = np.linspace(0.0, XI, 1001)
-    alias = np.sqrt(sum((transform(xi + m) / transform(xi)) ** 2 for m in range(-200, 201) if m))
-    print("beta = %.9f, gain at xi: %.4f, aliasing error: at most %.2e, %.2e at xi / 2" %
-          (BETA, transform(0.0) / transform(XI), np.max(alias), alias[500]))
+    # relative error of a mode e^{2 pi i xi t} at position t: its aliases'
+    # sum_{m != 0} r_m e^{2 pi i m t}, r_m = phihat(xi + m) / phihat(xi)
+    ratios = {m: transform(xi + m) / transform(xi) for m in range(-200, 201) if m}
+    rms = np.sqrt(sum(r ** 2 for r in ratios.values()))
+    t = np.linspace(0.0, 1.0, 2001)
+    most = np.array([np.max(np.abs(sum(r[i] * np.exp(2j * np.pi * m * t) for m, r in ratios.items())))
+                     for i in range(0, 1001, 20)])
+    print("beta = %.9f, gain at xi: %.4f, aliasing error over the positions: RMS at most %.2e (%.2e at xi / 2), largest "
+          "%.2e (%.2e)" % (BETA, transform(0.0) / transform(XI), np.max(rms), rms[500], np.max(most), most[25]))
+    # in 3-D at a corner of the band the axes' errors add: three times the
+    # largest, sqrt(3) times the RMS
+    print("3-D corner: RMS %.2e, largest %.2e" % (np.sqrt(3.0) * np.max(rms), 3.0 * np.max(most)))
 
 
 if __name__ == "__main__":

@@ -25,7 +25,7 @@
 // gradients (sigma, l, mu) in a fixed order.
 //
 // Large calls carry g to a node lattice and take the sums of the modes of low
-// frequency there (band_bwd.cu): 2.0M cells x 2048 modes 8994 -> 715 us.
+// frequency there (band_bwd.cu): 2.0M cells x 2048 modes 8994 -> 694 to 774 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
